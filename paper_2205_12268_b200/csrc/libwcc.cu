@@ -5,8 +5,7 @@
 #include "regather.cuh"
 #include "select.cuh"
 #include "contract.cuh"
-#include "fused.cuh"
-#include "fused_tiles.cuh"
+#include "pass2.cuh"
 #include "wavelet.cuh"
 
 namespace wcc {
@@ -35,11 +34,21 @@ static wcc_status check_forward_args(int N, int Cin, int Cout, int H, int W, int
     return WCC_OK;
 }
 
-// Can one of the two fused second-pass kernels run this problem?  (x only enters through its alignment.)
-static bool fused_fits(const void* x, int Cout, int W, int bits, wcc_dtype dt, int Cin)
+// Run the second pass as one kernel, or gather the kept columns and contract only those (wide_impl)?  One kernel, unless its
+// operand has to be rebuilt for many chunks of output channels, or the channel loop of a few CTAs gets long (bf16 input,
+// one kernel / gathered, us): 256 -> 256 on 2 x 128 x 256 81 / 83, 320 -> 64 there 56 / 69, 128 -> 1024 on 2 x 64 x 128
+// 54 / 65, 180 -> 512 on 2 x 64 x 64 48 / 50; the other way 256 -> 320 on 2 x 64 x 128 65 / 57, 192 -> 1024 there 89 / 65,
+// 512 -> 64 there 69 / 59, 384 -> 384 on 2 x 64 x 64 80 / 55.
+static bool one_kernel(int N, int Cin, int Cout, int H, int W, int L, int bits)
 {
-    const int esz = (dt == WCC_BF16) ? 2 : 4, kpad = wcc_kpad(Cin, bits);
-    return ft_plan(x, esz, W, Cout, kpad, bits).ok || fz_plan(esz, Cout, kpad, bits).ok;
+    const bool i8 = bits >= 2;
+    const int krow = wcc_kpad(Cin, bits) * (i8 ? 1 : 2), ksteps = krow / 32;
+    const P2Plan p = p2_plan_of(4, Cout, krow, i8, L);
+    if (!p.ok) return false;
+    const int chunks = ceil_div(p.npad, p.nchunk);
+    if (p.ksteps_part == ksteps) return chunks * ksteps <= 72;
+    if (ksteps <= 10) return chunks * ksteps <= 40;
+    return chunks == 1 && ksteps <= 16 && (long long)N * H * W >= 64 * p2::ROWS;
 }
 
 // Can the staged contraction kernel run it?  (Mirrors launch_contract: K is a loop and N is tiled, so only the
@@ -300,10 +309,19 @@ static WideWs carve_wide_ws(void* ws, int N, int Cin, int Cout, int H, int W, in
 }
 
 // One cluster per image in the selection (it reads the first pass's histograms), vector loads of whole patches.
-static bool wide_fits(const void* x, int Cin, int Cout, int H, int W, int bits, wcc_dtype dt)
+static bool wide_fits(int Cin, int Cout, int H, int W, int bits)
 {
-    (void)x; (void)dt;
     return staged_fits(Cin, Cout, bits) && select_in_cluster(H * W) && (W % 4) == 0;
+}
+
+// Does wcc_forward run the fused kernels?  Where the gathered pipeline cannot run, they also take the layers that it would
+// be faster for (up to eight K steps; beyond, stage by stage).
+static bool fused_fits(int N, int Cin, int Cout, int H, int W, int L, int bits)
+{
+    if (one_kernel(N, Cin, Cout, H, W, L, bits)) return true;
+    const bool i8 = bits >= 2;
+    const int krow = wcc_kpad(Cin, bits) * (i8 ? 1 : 2);
+    return !wide_fits(Cin, Cout, H, W, bits) && krow <= 256 && p2_plan_of(4, Cout, krow, i8, L).ok;
 }
 
 static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int Cout, int H, int W,
@@ -364,29 +382,9 @@ static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int 
     return WCC_OK;
 }
 
-// Chain fusion hooks of forward_impl: norms_ready = the previous layer's second pass has already produced this layer's
-// norms, per-position maxima and histograms in this workspace (no first pass; the weights are quantized by a launch of
-// their own); next_ws = workspace of the next layer, whose first pass this layer's second pass performs.
-struct ChainHooks { bool norms_ready; void* next_ws; int next_cout; };
-
-// Can the second pass of layer (Cin -> Cout) also be the first pass of a next layer?  (The four-tile kernel with room
-// for the tokens, one cluster per image in the selection.)
-// It pays while the next layer's input is narrow: the extra transform and norm chain cost the second pass about 0.2 us
-// per output channel on a 2 x 256 x 512 map (192 channels: +41 us against a 31 us first pass of its own; 32 channels:
-// +12 us against 18 us), because the pass is bound by instruction issue, not by the bytes the fusion saves.
-constexpr int CHAIN_FUSE_MAX_CHANNELS = 64;
-
-static bool chain_fusable(const void* x, int Cin, int Cout, int H, int W, int bits, wcc_dtype dt)
-{
-    const int esz = (dt == WCC_BF16) ? 2 : 4;
-    return Cout <= CHAIN_FUSE_MAX_CHANNELS && select_in_cluster(H * W) &&
-           ft_plan(x, esz, W, Cout, wcc_kpad(Cin, bits), bits, true).ok;
-}
-
 static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, int Cout, int H, int W,
                                int L, int k, int bits, void* y, wcc_dtype dt, void* ws, size_t ws_bytes,
-                               cudaStream_t st, const wcc_taps* taps, const wcc_options* opt = nullptr,
-                               const ChainHooks* hooks = nullptr)
+                               cudaStream_t st, const wcc_taps* taps, const wcc_options* opt = nullptr)
 {
     const bool own_codes = opt && opt->Wq;             // weights arrive quantized: Wt is not read
     if (!x || (!Wt && !own_codes) || !y || !ws) return WCC_ERR_NULL;
@@ -396,9 +394,11 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     if (!aligned16(x) || !aligned16(Wt) || !aligned16(y) || (reinterpret_cast<uintptr_t>(ws) & 255u)) return WCC_ERR_ALIGN;
     if (taps && (!aligned16(taps->coef) || !aligned16(taps->Xq) || !aligned16(taps->Xb) || !aligned16(taps->acc)))
         return WCC_ERR_ALIGN;
-    if (!fused_fits(x, Cout, W, bits, dt, Cin)) {      // decided before anything is launched: channel counts beyond one
-        if (own_codes) return WCC_ERR_SHAPE;           // operand tile run stage by stage (the contraction there tiles K and N)
-        if (wide_fits(x, Cin, Cout, H, W, bits, dt) && !(taps && taps->coef))
+    if (own_codes) {                                   // codes only enter the fused kernels
+        const int krow = wcc_kpad(Cin, bits);
+        if (!p2_plan_of(4, Cout, krow, true, L).ok) return WCC_ERR_SHAPE;
+    } else if (!fused_fits(N, Cin, Cout, H, W, L, bits)) {                     // decided before anything is launched
+        if (wide_fits(Cin, Cout, H, W, bits) && !(taps && taps->coef))
             return wide_impl(x, Wt, N, Cin, Cout, H, W, L, k, bits, y, dt, ws, ws_bytes, st, taps, opt);
         return staged_impl(x, Wt, N, Cin, Cout, H, W, L, k, bits, y, dt, ws, ws_bytes, st, taps, opt);
     }
@@ -411,9 +411,7 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     // coefficient map is written only when a test asks for it).  The same launch fills round 1 of the select's
     // histogram and quantizes the weights in a few extra CTAs.
     const SelectWs sw = carve_select_ws(f.sel, N, P);
-    const bool norms_ready = hooks && hooks->norms_ready;
-    if (!norms_ready)
-        WCC_CUDA_TRY(cudaMemsetAsync(f.fine, 0, f.fine_bytes + sw.zero_bytes, st));   // histograms, max |kept|, barrier counters
+    WCC_CUDA_TRY(cudaMemsetAsync(f.fine, 0, f.fine_bytes + sw.zero_bytes, st));       // histograms, max |kept|, barrier counters
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
     NormsExtra ex = {};
     ex.coef = taps ? taps->coef : nullptr;
@@ -424,15 +422,8 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     const void* Wq_use = own_codes ? static_cast<const void*>(opt->Wq) : f.Wq;
     const float* scale_w_use = own_codes ? opt->scale_w : f.scale_w;
     const FusedExtra fx = {opt ? opt->alpha : 0.0f, opt ? opt->relu : 0, opt ? opt->residual : nullptr};
-    if (norms_ready) {
-        if (!own_codes) {
-            s = launch_weight_prep(Wt, Cout, Cin, f.kpad, wbits, f.Wq, f.scale_w, st);
-            if (s != WCC_OK) return s;
-        }
-    } else {
-        s = launch_haar_norms(x, N, Cin, H, W, L, dt, f.nrm2, f.amaxpos, ex, st);
-        if (s != WCC_OK) return s;
-    }
+    s = launch_haar_norms(x, N, Cin, H, W, L, dt, f.nrm2, f.amaxpos, ex, st);
+    if (s != WCC_OK) return s;
     if ((s = profile_mark(2, st)) != WCC_OK) return s;
     // joint shrinkage: index list, rank map, max |kept|
     s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, f.amaxpos, true, f.sel, f.sel_bytes, st, true,
@@ -441,22 +432,8 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     if ((s = profile_mark(3, st)) != WCC_OK) return s;
     // second pass over x: transform, mask + quantize, tensor-core contraction, dequantize, inverse, store
     void* xq_tap = taps ? (bits >= 2 ? static_cast<void*>(taps->Xq) : taps->Xb) : nullptr;
-    ft::NextNorms nx = {};
-    const bool feeds_next = hooks && hooks->next_ws;
-    if (feeds_next) {
-        // the next layer's workspace (its input has Cout channels): clear its histograms, then let this layer's second
-        // pass fill its norms, maxima and histograms
-        const FusedWs g = carve_fused_ws(hooks->next_ws, N, Cout, hooks->next_cout, H, W, k, bits);
-        const SelectWs gs = carve_select_ws(g.sel, N, P);
-        WCC_CUDA_TRY(cudaMemsetAsync(g.fine, 0, g.fine_bytes + gs.zero_bytes, st));
-        nx.nrm2 = g.nrm2; nx.amaxpos = g.amaxpos; nx.hist1 = gs.hist; nx.fine = g.fine;
-    }
-    s = launch_fused_tiles(x, Wq_use, f.rank, f.nrm2, f.thr, f.amax_kept, bits, scale_w_use, N, Cin, Cout, H, W, L, k, f.kpad, dt, y,
-                           xq_tap, taps ? taps->acc : nullptr, fx, st, feeds_next ? &nx : nullptr);
-    if (feeds_next && s != WCC_OK) return s == WCC_ERR_SHAPE ? WCC_ERR_CUDA : s;       // (chain_fusable said it fits)
-    if (s == WCC_ERR_SHAPE)                            // shapes the four-tile kernel does not cover (nothing was launched)
-        s = launch_fused_pass2(x, Wq_use, f.rank, f.nrm2, f.thr, f.amax_kept, bits, scale_w_use, N, Cin, Cout, H, W, L, k, f.kpad, dt, y,
-                               xq_tap, taps ? taps->acc : nullptr, fx, st);
+    s = launch_pass2(x, Wq_use, f.rank, f.nrm2, f.thr, f.amax_kept, bits, scale_w_use, N, Cin, Cout, H, W, L, k, f.kpad, dt, y,
+                     xq_tap, taps ? taps->acc : nullptr, fx, st);
     if (s != WCC_OK) return s;
     for (int i = 4; i <= WCC_NUM_STAGES; ++i)
         if ((s = profile_mark(i, st)) != WCC_OK) return s;
@@ -599,7 +576,7 @@ static BlockWs carve_block_ws(void* ws, int N, int C, int E, int H, int W, int L
 }
 
 // ---- chain of layers -------------------------------------------------------------------------------
-struct ChainWs { void* act[2]; void* layer_ws[2]; size_t layer_ws_bytes; size_t total; };
+struct ChainWs { void* act[2]; void* layer_ws; size_t layer_ws_bytes; size_t total; };
 
 static wcc_status chain_shapes_ok(const wcc_chain_layer* layers, int n_layers)
 {
@@ -628,8 +605,7 @@ static ChainWs carve_chain_ws(void* ws, const wcc_chain_layer* layers, int n_lay
     c.act[0] = take(act);
     c.act[1] = take(act);
     c.layer_ws_bytes = lw;
-    c.layer_ws[0] = take(lw);                          // consecutive layers alternate: a fused second pass writes the next
-    c.layer_ws[1] = take(lw);                          // layer's norms while it still reads its own
+    c.layer_ws = take(lw);
     c.total = off;
     return c;
 }
@@ -649,7 +625,7 @@ int wcc_kpad(int Cin, int bits)
 size_t wcc_workspace_bytes(int N, int Cin, int Cout, int H, int Wd, int levels, int k, int bits, wcc_dtype dt)
 {
     if (check_forward_args(N, Cin, Cout, H, Wd, levels, k, bits, dt) != WCC_OK) return 0;
-    if (!fused_fits(nullptr, Cout, Wd, bits, dt, Cin)) {                       // these shapes run around the tiled contraction
+    if (!fused_fits(N, Cin, Cout, H, Wd, levels, bits)) {                      // these shapes run around the tiled contraction
         if (!staged_fits(Cin, Cout, bits)) return 0;
         const size_t a = carve_forward_ws(nullptr, N, Cin, Cout, H, Wd, k, bits).total;
         const size_t b = carve_wide_ws(nullptr, N, Cin, Cout, H, Wd, k, bits).total;
@@ -958,24 +934,15 @@ wcc_status wcc_chain_forward(const void* x, const wcc_chain_layer* layers, int n
     const ChainWs c = carve_chain_ws(ws, layers, n_layers, N, H, Wd, levels, k, bits, dt);
     if (c.total == 0) return WCC_ERR_SHAPE;
     if (ws_bytes < c.total) return WCC_ERR_WORKSPACE;
-    // Layer i's second pass doubles as layer i+1's first pass (inverse transform, ReLU and the next forward transform
-    // on the same tile while it is in registers) wherever both layers run the four-tile kernel.
     const void* in = x;
-    bool norms_ready = false;
     for (int i = 0; i < n_layers; ++i) {
         void* out = (i + 1 == n_layers) ? y : c.act[i & 1];
         wcc_options o = {};
         o.alpha = layers[i].alpha;
         o.relu = layers[i].relu;
-        const bool this_fused = fused_fits(in, layers[i].Cout, Wd, bits, dt, layers[i].Cin);
-        const bool feed = this_fused && i + 1 < n_layers && chain_fusable(in, layers[i].Cin, layers[i].Cout, H, Wd, bits, dt) &&
-                          fused_fits(out, layers[i + 1].Cout, Wd, bits, dt, layers[i + 1].Cin) &&
-                          tc::tma_ok_x(out, dt == WCC_BF16 ? 2 : 4, Wd);
-        const ChainHooks hooks = {norms_ready, feed ? c.layer_ws[(i + 1) & 1] : nullptr, feed ? layers[i + 1].Cout : 0};
-        s = forward_impl(in, layers[i].Wt, N, layers[i].Cin, layers[i].Cout, H, Wd, levels, k, bits, out, dt,
-                         c.layer_ws[i & 1], c.layer_ws_bytes, static_cast<cudaStream_t>(stream), nullptr, &o, &hooks);
+        s = forward_impl(in, layers[i].Wt, N, layers[i].Cin, layers[i].Cout, H, Wd, levels, k, bits, out, dt, c.layer_ws,
+                         c.layer_ws_bytes, static_cast<cudaStream_t>(stream), nullptr, &o);
         if (s != WCC_OK) return s;
-        norms_ready = feed;
         in = out;
     }
     return WCC_OK;
