@@ -66,7 +66,7 @@ def stage_bytes(w, stage: str) -> float:
     NP, Nk = w.N * w.P, w.N * w.k
     es = 2 if w.bits == 0 else 1
     return {
-        "clear": w.N * (65536 + 3 * 2048) * 4,                                  # the select's histograms, zeroed (a memset node)
+        "clear": w.N * (65536 + 3 * 2048) * 4,                                  # the select's histograms, zeroed
         "haar_norms": NP * w.Cin * s + 8 * NP + 5 * w.Cout * w.Cin,             # x once; norms and per-position max out; weights
         "fused_pass2": NP * w.Cin * s + 4 * NP + s * NP * w.Cout,               # x again, norms (or rank map), y once
         "haar_fwd_norms": NP * w.Cin * (s + 4) + 4 * NP,
@@ -576,7 +576,7 @@ def run_ours(args):
     # per-stage device times with CUDA events recorded inside the call (eager launches of the same configuration)
     peak, peak_kind = _peaks()
     stage_ms = case.stage_times(flush, max(50, min(args.steps, 200)))
-    dom = max((n for n in stage_ms if n != "clear"), key=stage_ms.get)      # a memset node is not one of our kernels
+    dom = max((n for n in stage_ms if n != "clear"), key=stage_ms.get)      # clearing moves no input or output
     achieved = stage_bytes(w, dom) / (stage_ms[dom] * 1e-3) / 1e9
     tr = NCU_TRAFFIC.get((w.name, dom))
     traffic = tr["bytes"] if tr and tr.get("src") == _source_hash() and not args.batch else None

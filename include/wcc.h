@@ -136,7 +136,8 @@ wcc_status wcc_select_topk_static(const float* nrm2, int N, int P, int k, int32_
  *            0: no quantization; columns and weights rounded to bf16, fp32 accumulation.
  *   y   out: [N][Cout][H][Wd] of dt; must not overlap x
  *   ws     : scratch of at least wcc_workspace_bytes(...) bytes, 256-byte aligned; contents undefined afterwards
- * Execution: three launches, two passes over x around the selection.  Pass 1 transforms x in registers and keeps
+ * Execution: four launches (one clears the histograms), two passes over x around the selection; each kernel may start
+ * while the one before it drains.  Pass 1 transforms x in registers and keeps
  * only the channel norms, the per-position max |coefficient| and two histograms of the norms' leading bits below the sign (it
  * also quantizes the weights); the selection finds the threshold norm, max|kept| and, only if ties at the threshold
  * are kept in part, the rank of every position; pass 2 transforms x again, zeroes the dropped positions, quantizes
@@ -325,14 +326,14 @@ wcc_status wcc_debug_wait_selftest(void* stream);
  * stream around each stage; wcc_profile_read waits for the last recorded call and writes, to the HOST array ms, the
  * milliseconds of, for wcc_forward_staged: 0 Haar transform + norms, 1 top-k select + compaction, 2 weight
  * quantization, 3 gather + quantize, 4 tensor-core contraction, 5 dequantize + scatter + inverse Haar; for wcc_forward:
- * 0 clearing of the select's histograms (a memset node), 1 pass 1 (transform + norms, select histograms, weight
+ * 0 clearing of the select's histograms, 1 pass 1 (transform + norms, select histograms, weight
  * quantization), 2 select, 3 fused pass 2, 4 and 5 zero.
  * Off by default; not thread-safe.
  */
 #define WCC_NUM_STAGES 6
 wcc_status wcc_profile_enable(int on);
 wcc_status wcc_profile_read(float* ms);
-/* Number of kernels this library has launched in this process so far (memset nodes not counted). */
+/* Number of kernels this library has launched in this process so far. */
 unsigned long long wcc_kernel_launches(void);
 
 #ifdef __cplusplus

@@ -35,6 +35,59 @@ static unsigned long long g_launches = 0;
         }                                                    \
     } while (0)
 
+// ---- kernels that overlap the launch and the set-up of their successor -------------------------
+// A layer is a chain of short kernels: clear -> pass 1 -> selection -> pass 2 (-> the next layer's clear).  Each is launched with
+// the programmatic attribute, so that it may become resident while its predecessor drains; an ordinary launch boundary cost
+// 1.5 to 2.5 us between kernels of 2 to 40 us.  What makes it safe:
+//  - pdl_wait() returns when every earlier kernel's memory operations are complete and visible, provided each kernel of the
+//    chain calls it before it signals pdl_launch() (or signals at all only by ending).  Clear and selection do so first
+//    thing: once pass 1 runs, everything before the layer is complete, and once pass 2 runs, pass 1 is.
+//  - Pass 1 reads x and the weights and writes only what nothing in flight uses; it waits before it touches the histograms
+//    that clear zeroes.  Pass 2 reads x, the quantized weights and the norms early and waits before it reads what the
+//    selection writes.
+//  - A kernel that reads anything early has such a kernel as its predecessor (never the caller's own kernels).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// `overlap` false: an ordinary launch.  cluster > 1: cluster size along x.
+template <typename... KArgs, typename... Args>
+static wcc_status launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
+                                    int cluster, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (cluster > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = (unsigned)cluster; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    if (overlap) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    cfg.attrs = attr; cfg.numAttrs = (unsigned)na;
+    WCC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
+    WCC_LAUNCH_CHECK();
+    return WCC_OK;
+}
+
+// Zeroes `n16` 16-byte words (the selection's histograms and counters of one call).
+__global__ void __launch_bounds__(256) clear_kernel(uint4* __restrict__ p, size_t n16)
+{
+    pdl_wait();
+    pdl_launch();
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n16; i += (size_t)gridDim.x * 256) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+static wcc_status launch_clear(void* p, size_t bytes, cudaStream_t st)
+{
+    const size_t n16 = bytes / 16;                     // (256-byte multiples)
+    const size_t want = (n16 + 1023) / 1024;
+    return launch_overlapped(clear_kernel, dim3((unsigned)(want < 592 ? want : 592)), dim3(256), 0, st, true, 1, static_cast<uint4*>(p), n16);
+}
+
 // ---- element access -------------------------------------------------------------------------
 __device__ __forceinline__ float bf16lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }

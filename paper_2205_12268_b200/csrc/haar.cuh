@@ -943,6 +943,7 @@ __global__ void __launch_bounds__(NORMS_WARPS * 32)
 haar_norms_kernel(const T* __restrict__ x, int N, int C, int H, int W,
                   float* __restrict__ nrm2, float* __restrict__ amaxpos, const NormsExtra ex)
 {
+    pdl_launch();
     if ((int)blockIdx.x >= ex.tiles) {                 // weight preparation CTAs
         const int o = ((int)blockIdx.x - ex.tiles) * NORMS_WARPS + (int)(threadIdx.x >> 5);
         if (o < ex.Cout) weight_prep_row(ex.Wt, o, C, ex.kpad, ex.bits, ex.Wq, ex.scale_w);
@@ -1014,6 +1015,7 @@ haar_norms_kernel(const T* __restrict__ x, int N, int C, int H, int W,
     }
     if (VEC) Ring::template wait<0>();
     if (warp >= 4) return;
+    pdl_wait();                                        // the histograms are cleared
     norms_finish<L, VEC>(lp, warp, n, P, nn.x, nn.y, a0, a1, nrm2, amaxpos, ex);
 }
 
@@ -1144,6 +1146,7 @@ haar_norms_token_kernel(const __grid_constant__ CUtensorMap tmx, int N, int C, i
     using Ring = typename Cfg::Ring;
     constexpr int CB = Cfg::CB, S = Cfg::S, NW = Cfg::W;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_launch();
     if ((int)blockIdx.x >= tile_ctas) {                // weight preparation CTAs
         const int o = ((int)blockIdx.x - tile_ctas) * NW + warp;
         if (o < ex.Cout) weight_prep_row(ex.Wt, o, C, ex.kpad, ex.bits, ex.Wq, ex.scale_w);
@@ -1270,6 +1273,7 @@ haar_norms_token_kernel(const __grid_constant__ CUtensorMap tmx, int N, int C, i
                     nacc[2 * i] = __fmul_rn(acc[i].x, __fmul_rn(sc[2 * i], sc[2 * i]));
                     nacc[2 * i + 1] = __fmul_rn(acc[i].y, __fmul_rn(sc[2 * i + 1], sc[2 * i + 1]));
                 }
+                pdl_wait();                            // the histograms are cleared
                 store_slots<L, true>(nrm2 + (size_t)n * P, lp, nacc);
                 // Norms that are exactly zero are not counted: after a ReLU whole regions of a map are zero, and their
                 // positions would all hit one bin (thousands of atomics on one address).  The selection knows the number
@@ -1486,9 +1490,8 @@ static wcc_status haar_norms_dispatch(const void* x, int N, int C, int H, int W,
             const long long resident = warps / Cfg::W;                  // every tile CTA is resident at once
             const int tile_ctas = (int)(tiles < resident ? tiles : resident);
             const long long grid = tile_ctas + (ex.Wt ? ceil_div(ex.Cout, Cfg::W) : 0);
-            kern<<<(unsigned)grid, Cfg::W * 32, Cfg::SMEM, st>>>(tmx, N, C, H, W, (int)tiles, tile_ctas, nrm2, amaxpos, ex, status);
-            WCC_LAUNCH_CHECK();
-            return WCC_OK;
+            return launch_overlapped(kern, dim3((unsigned)grid), dim3(Cfg::W * 32), Cfg::SMEM, st, ex.hist1 != nullptr, 1,
+                                     tmx, N, C, H, W, (int)tiles, tile_ctas, nrm2, amaxpos, ex, status);
         };
         if (tiles * 2 > warps) return launch(haar_norms_token_kernel<T, L, 1>, NormsTokCfg<T, L, 1>{});
         if (tiles * 4 > warps) return launch(haar_norms_token_kernel<T, L, 2>, NormsTokCfg<T, L, 2>{});
@@ -1496,12 +1499,12 @@ static wcc_status haar_norms_dispatch(const void* x, int N, int C, int H, int W,
     }
     ex.tiles = (int)tiles;
     const long long grid = tiles + (ex.Wt ? ceil_div(ex.Cout, NORMS_WARPS) : 0);
-    haar_norms_kernel<T, L, VEC><<<(unsigned)grid, NORMS_WARPS * 32, 0, st>>>(static_cast<const T*>(x), N, C, H, W, nrm2, amaxpos, ex);
-    WCC_LAUNCH_CHECK();
-    return WCC_OK;
+    return launch_overlapped(haar_norms_kernel<T, L, VEC>, dim3((unsigned)grid), dim3(NORMS_WARPS * 32), 0, st, ex.hist1 != nullptr, 1,
+                             static_cast<const T*>(x), N, C, H, W, nrm2, amaxpos, ex);
 }
 
-// First pass of the fused layer (see haar_norms_kernel); ex.tiles is filled in here.
+// First pass of the fused layer (see haar_norms_kernel); ex.tiles is filled in here.  With ex.hist1 set, launch_clear on the
+// histograms must be the call before it on the stream.
 wcc_status launch_haar_norms(const void* x, int N, int C, int H, int W, int L, wcc_dtype dt,
                              float* nrm2, float* amaxpos, const NormsExtra& ex, cudaStream_t st)
 {

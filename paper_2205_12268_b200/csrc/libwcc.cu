@@ -243,7 +243,7 @@ static FusedWs carve_fused_ws(void* ws, int N, int Cin, int Cout, int H, int W, 
     f.rank = reinterpret_cast<int32_t*>(take((size_t)N * P * 4));
     f.idx = reinterpret_cast<int32_t*>(take(M * 4));
     f.thr = reinterpret_cast<uint32_t*>(take((size_t)N * 16));
-    // the 16-bit histogram sits right before the select scratch, whose zeroed part comes first: one memset clears both
+    // the 16-bit histogram sits right before the select scratch, whose zeroed part comes first: one launch clears both
     f.fine_bytes = align_up((size_t)N * FINE_BINS * 4, 256);
     f.fine = reinterpret_cast<uint32_t*>(take(f.fine_bytes));
     f.sel_bytes = select_ws_bytes(N, (int)P);
@@ -295,7 +295,7 @@ static WideWs carve_wide_ws(void* ws, int N, int Cin, int Cout, int H, int W, in
     f.rank = reinterpret_cast<int32_t*>(take((size_t)N * P * 4));
     f.idx = reinterpret_cast<int32_t*>(take(M * 4));
     f.thr = reinterpret_cast<uint32_t*>(take((size_t)N * 16));
-    f.fine_bytes = align_up((size_t)N * FINE_BINS * 4, 256);       // right before the select scratch: one memset clears both
+    f.fine_bytes = align_up((size_t)N * FINE_BINS * 4, 256);       // right before the select scratch: one launch clears both
     f.fine = reinterpret_cast<uint32_t*>(take(f.fine_bytes));
     f.sel_bytes = select_ws_bytes(N, (int)P);
     f.sel = take(f.sel_bytes);
@@ -334,7 +334,7 @@ static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int 
     wcc_status s;
     if ((s = profile_mark(0, st)) != WCC_OK) return s;
     const SelectWs sw = carve_select_ws(f.sel, N, P);
-    WCC_CUDA_TRY(cudaMemsetAsync(f.fine, 0, f.fine_bytes + sw.zero_bytes, st));       // histograms, max |kept|, barrier counters
+    if ((s = launch_clear(f.fine, f.fine_bytes + sw.zero_bytes, st)) != WCC_OK) return s;      // histograms, max |kept|, barrier counters
     NormsExtra ex = {};
     ex.hist1 = sw.hist;
     ex.fine = f.fine;
@@ -411,7 +411,7 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     // coefficient map is written only when a test asks for it).  The same launch fills round 1 of the select's
     // histogram and quantizes the weights in a few extra CTAs.
     const SelectWs sw = carve_select_ws(f.sel, N, P);
-    WCC_CUDA_TRY(cudaMemsetAsync(f.fine, 0, f.fine_bytes + sw.zero_bytes, st));       // histograms, max |kept|, barrier counters
+    if ((s = launch_clear(f.fine, f.fine_bytes + sw.zero_bytes, st)) != WCC_OK) return s;      // histograms, max |kept|, barrier counters
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
     NormsExtra ex = {};
     ex.coef = taps ? taps->coef : nullptr;

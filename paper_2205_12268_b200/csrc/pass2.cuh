@@ -121,6 +121,7 @@ pass2_kernel(const Params pr)
     const PatchOff off = patch_off<T>(lp, pr.W);
     const uint64_t xb = reinterpret_cast<uint64_t>(pr.x) + (uint64_t)n * pr.Cin * plane;
 
+    pdl_launch();
     Raw<T> raw[NB];
     const int ureal = (pr.Cin + 7) >> 3;               // units that hold real channels
     auto preload = [&](int u) {
@@ -149,17 +150,15 @@ pass2_kernel(const Params pr)
     };
     if (pr.b_resident) load_b(o_lo, o_cnt, 0, 2 * ksteps);
     // kept or dropped: from the rank map when the select wrote one (thr[n][2] != 0), else by the threshold key
-    float mul[8];
+    float nv[8], mul[8];
     int rk[8];
 #pragma unroll
-    for (int s = 0; s < 8; ++s) { mul[s] = 0.0f; rk[s] = -1; }
+    for (int s = 0; s < 8; ++s) nv[s] = (live && slot_ok<L>(lp, s)) ? pr.nrm2[(size_t)n * P + lp.pos[s]] : 0.0f;
+    pdl_wait();                                        // what follows reads the selection's results
     float amax = 0.0f;
     if (I8) amax = (CLAMP && pr.alpha > 0.0f) ? pr.alpha : *pr.amax_kept;
-    if (live) {
+    {
         const uint4 th = *reinterpret_cast<const uint4*>(pr.thr + n * 4);      // {threshold key, ties kept, use-rank flag, -}
-        float nv[8];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) nv[s] = slot_ok<L>(lp, s) ? pr.nrm2[(size_t)n * P + lp.pos[s]] : 0.0f;
         float inv = 1.0f;
         if (I8) inv = (amax > 0.0f) ? __fdiv_rn(pr.qmax, amax) : 0.0f;
         // the transform runs without its halvings: they go into the per-slot factor (exact, a power of two)
@@ -167,7 +166,8 @@ pass2_kernel(const Params pr)
         slot_scales<L>(lane, false, sc);
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
-            if (slot_ok<L>(lp, s)) {
+            rk[s] = -1;
+            if (live && slot_ok<L>(lp, s)) {
                 if (th.z) rk[s] = pr.rank[(size_t)n * P + lp.pos[s]];
                 else rk[s] = (float_key(nv[s]) >= th.x) ? 0 : -1;
             }
@@ -463,9 +463,7 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     const unsigned ctas = (unsigned)pr.split_from + (groups - (unsigned)pr.split_from) * (unsigned)pr.parts;
     auto launch = [&](auto kern) -> wcc_status {
         WCC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        kern<<<ctas, p2::TILES * plan.wpt * 32, plan.smem, st>>>(pr);
-        WCC_LAUNCH_CHECK();
-        return WCC_OK;
+        return launch_overlapped(kern, dim3(ctas), dim3(p2::TILES * plan.wpt * 32), plan.smem, st, true, 1, pr);
     };
     const bool clampv = i8 && fx.alpha > 0.0f, tap = xq_tap || acc_tap;
     const int want = (fx.relu ? 1 : 0) | (tap ? 2 : 0) | (clampv ? 4 : 0) | (fx.residual ? 8 : 0);

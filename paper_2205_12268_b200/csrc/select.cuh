@@ -600,6 +600,11 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
     const int base = (crank * (int)blockDim.x + (int)threadIdx.x) * kpt;  // kpt consecutive keys per thread
     const int lane = threadIdx.x & 31;
 
+    for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
+    if (threadIdx.x == 0) { sm.amax = 0u; sm.ncand = 0u; sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u; }   // thr: keep nothing
+                                                       // unless a candidate is found (histograms that do not match the keys)
+    pdl_wait();
+    pdl_launch();
     uint32_t key[MAXKPT];
 #pragma unroll
     for (int i = 0; i < MAXKPT; ++i) key[i] = (i < kpt && base + i < P) ? float_key(v[base + i]) : 0u;
@@ -613,9 +618,6 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
         for (int i = 0; i < MAXKPT; ++i) pre[PRE ? i : 0] = (amaxpos && valid(i)) ? amaxpos[(size_t)n * P + base + i] : 0.0f;
     }
 
-    for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
-    if (threadIdx.x == 0) { sm.amax = 0u; sm.ncand = 0u; sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u; }   // thr: keep nothing
-                                                       // unless a candidate is found (histograms that do not match the keys)
     __syncthreads();
 
     uint32_t tkey = 0, need_eq = 0, total_eq = 0, ranked = 0;    // ranked: candidates counted through (diagnostic)
@@ -875,28 +877,13 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         const int kpt = ceil_div(P, cs * threads);
         if (amax_kept && !hist1_ready) WCC_CUDA_TRY(cudaMemsetAsync(amax_kept, 0, sizeof(float), st));
         const uint32_t* hist1 = hist1_ready ? s.hist : nullptr;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cs, N);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cs;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
         const uint32_t* fine_use = hist1_ready ? fine : (const uint32_t*)nullptr;
         const int wr = (want_rank || !thr) ? 1 : 0;
         if (kpt <= 4)                                  // few keys per thread: the instantiation with four key registers
-            WCC_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_cluster_kernel<4>, nrm2, P, k, kpt, idx, tau, rank, amaxpos, amax_kept, hist1,
-                                            fine_use, thr, wr));
-        else
-            WCC_CUDA_TRY(cudaLaunchKernelEx(&cfg, select_cluster_kernel<CL_MAXKPT>, nrm2, P, k, kpt, idx, tau, rank, amaxpos, amax_kept,
-                                            hist1, fine_use, thr, wr));
-        WCC_LAUNCH_CHECK();
-        return WCC_OK;
+            return launch_overlapped(select_cluster_kernel<4>, dim3(cs, N), dim3(threads), 0, st, hist1_ready, cs, nrm2, P, k, kpt, idx, tau,
+                                     rank, amaxpos, amax_kept, hist1, fine_use, thr, wr);
+        return launch_overlapped(select_cluster_kernel<CL_MAXKPT>, dim3(cs, N), dim3(threads), 0, st, hist1_ready, cs, nrm2, P, k, kpt, idx,
+                                 tau, rank, amaxpos, amax_kept, hist1, fine_use, thr, wr);
     }
     if (thr) {                                        // these paths always write idx and the rank map
         thr_use_rank_kernel<<<ceil_div(N, 128), 128, 0, st>>>(thr, N);
