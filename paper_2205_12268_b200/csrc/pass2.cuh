@@ -75,7 +75,8 @@ __device__ __forceinline__ void relu_patch(float (&p)[2][4])
 // MODE is a set of compiled-in features: 1 = ReLU on the way out, 2 = taps for tests, 4 = a given clipping parameter (codes
 // are clamped), 8 = residual add.  A compiled-in feature is still switched by its run-time argument; a feature that is not
 // compiled in costs nothing (as run-time branches in one kernel the options cost the plain layer 7-18 %).
-// Instantiated: 0 (plain), 1, 13 and 15 (everything); a request runs on the smallest variant that contains it.
+// Instantiated: 0 (plain), 1, 13 and 15 (everything); a request runs on the smallest variant that contains it.  Taps run with
+// WPT = 4 only, and so do maps with W = 4m + 2, plain or with everything.
 template <typename T, int L, bool I8, int WPT, bool VEC, int MODE>
 __global__ void __launch_bounds__(TILES * WPT * 32, WPT == 2 ? 2 : 1)
 pass2_kernel(const Params pr)
@@ -441,7 +442,8 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     int dev = 0, sms = 0;
     WCC_CUDA_TRY(cudaGetDevice(&dev));
     WCC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const P2Plan plan = p2_plan(Cout, krow, i8, L, groups, sms);
+    const bool tap = xq_tap || acc_tap;
+    const P2Plan plan = (tap || !VEC) ? p2_plan_of(4, Cout, krow, i8, L) : p2_plan(Cout, krow, i8, L, groups, sms);
     if (!plan.ok) return WCC_ERR_SHAPE;
     p2::Params pr = {};
     pr.x = x; pr.Wq = static_cast<const uint8_t*>(Wq); pr.rank = rank; pr.nrm2 = nrm2; pr.thr = thr; pr.amax_kept = amax_kept;
@@ -465,14 +467,23 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
         WCC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         return launch_overlapped(kern, dim3(ctas), dim3(p2::TILES * plan.wpt * 32), plan.smem, st, true, 1, pr);
     };
-    const bool clampv = i8 && fx.alpha > 0.0f, tap = xq_tap || acc_tap;
+    const bool clampv = i8 && fx.alpha > 0.0f;
     const int want = (fx.relu ? 1 : 0) | (tap ? 2 : 0) | (clampv ? 4 : 0) | (fx.residual ? 8 : 0);
     const int mode = want == 0 ? 0 : want == 1 ? 1 : (want & 2) == 0 ? 13 : 15;
 #define WCC_P2(I8V, WPTV, MODEV) return launch(p2::pass2_kernel<T, L, I8V, WPTV, VEC, MODEV>)
-#define WCC_P2M(I8V, WPTV) do { if (mode == 0) WCC_P2(I8V, WPTV, 0); if (mode == 1) WCC_P2(I8V, WPTV, 1); if (mode == 13) WCC_P2(I8V, WPTV, 13); WCC_P2(I8V, WPTV, 15); } while (0)
-    if (i8) { if (plan.wpt == 2) WCC_P2M(true, 2); WCC_P2M(true, 4); }
-    if (plan.wpt == 2) WCC_P2M(false, 2);
-    WCC_P2M(false, 4);
+#define WCC_P2M(I8V, WPTV) do { if (mode == 0) WCC_P2(I8V, WPTV, 0); if (mode == 1) WCC_P2(I8V, WPTV, 1); WCC_P2(I8V, WPTV, 13); } while (0)
+    if constexpr (VEC) {
+        if (mode != 15) {
+            if (i8) { if (plan.wpt == 2) WCC_P2M(true, 2); WCC_P2M(true, 4); }
+            if (plan.wpt == 2) WCC_P2M(false, 2);
+            WCC_P2M(false, 4);
+        }
+    } else if (mode == 0) {
+        if (i8) WCC_P2(true, 4, 0);
+        WCC_P2(false, 4, 0);
+    }
+    if (i8) WCC_P2(true, 4, 15);
+    WCC_P2(false, 4, 15);
 #undef WCC_P2M
 #undef WCC_P2
 }

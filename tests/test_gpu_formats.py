@@ -65,3 +65,19 @@ def test_padded_layer(wcc, cfg):
         assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
     else:
         assert np.abs(got - want).max() <= 2e-2 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 3, 1, 1), (3, 5, 2, 9, 31), (2, 3, 3, 15, 8), (1, 2, 1, 7, 513)], ids=str)
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("levels", [1, 2, 3])
+def test_padded_layer_keeps_rows_apart(wcc, shape, dtype, levels):
+    """Everything kept, integers in: the padded layer without quantization is the dense product, exactly, at row ends, at
+    the last element and for one-row and one-column maps (integers below 2^8 are exact in bf16 and in every partial sum)."""
+    N, Cin, Cout, H, W = shape
+    unit = 1 << levels
+    g = torch.Generator(device="cuda").manual_seed(H * W + levels)
+    x = torch.randint(-3, 4, (N, Cin, H, W), device="cuda", generator=g).to(dtype) * 8
+    Wt = torch.randint(-2, 3, (Cout, Cin), device="cuda", generator=g).float()
+    y = wcc.forward_padded(x, Wt, levels, (-(-H // unit) * unit) * (-(-W // unit) * unit), 0)
+    assert wcc.last_status() == 0
+    assert torch.equal(y.float(), torch.einsum("oc,nchw->nohw", Wt, x.float()))
