@@ -4,6 +4,7 @@
 #include "common.cuh"
 #include "gather.cuh"
 #include "haar.cuh"
+#include "pass1.cuh"
 #include "regather.cuh"
 #include "select.cuh"
 #include "contract.cuh"
@@ -336,16 +337,18 @@ static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int 
     wcc_status s;
     if ((s = profile_mark(0, st)) != WCC_OK) return s;
     const SelectWs sw = carve_select_ws(f.sel, N, P);
+    // the per-position maxima are only built where the activation scale comes from them
+    float* const amaxpos = (bits >= 2 && !(opt && opt->alpha > 0.0f)) ? f.amaxpos : nullptr;
     if ((s = launch_clear(f.fine, f.fine_bytes + sw.zero_bytes, st)) != WCC_OK) return s;      // histograms, max |kept|, barrier counters
     NormsExtra ex = {};
     ex.hist1 = sw.hist;
     ex.fine = f.fine;
     const int wbits = (opt && opt->weight_bits && bits) ? opt->weight_bits : bits;
     ex.Wt = Wt; ex.Wq = f.Wq; ex.scale_w = f.scale_w; ex.Cout = Cout; ex.kpad = f.kpad; ex.bits = wbits;
-    s = launch_haar_norms(x, N, Cin, H, W, L, dt, f.nrm2, f.amaxpos, ex, st);
+    s = launch_pass1(x, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
-    s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, f.amaxpos, true, f.sel, f.sel_bytes, st, true, f.fine, f.thr, true);
+    s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, amaxpos, true, f.sel, f.sel_bytes, st, true, f.fine, f.thr, true);
     if (s != WCC_OK) return s;
     if (opt && opt->alpha > 0.0f && bits >= 2) {        // a given clipping parameter replaces the largest kept magnitude
         set_word_kernel<<<1, 1, 0, st>>>(f.amax_kept, opt->alpha);
@@ -413,10 +416,12 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     // coefficient map is written only when a test asks for it).  The same launch fills round 1 of the select's
     // histogram and quantizes the weights in a few extra CTAs.
     const SelectWs sw = carve_select_ws(f.sel, N, P);
+    if (taps && taps->coef && (s = launch_haar_fwd(x, N, Cin, H, W, L, dt, taps->coef, nullptr, nullptr, st)) != WCC_OK) return s;
+    // the per-position maxima are only built where the activation scale comes from them
+    float* const amaxpos = (bits >= 2 && !(opt && opt->alpha > 0.0f)) ? f.amaxpos : nullptr;
     if ((s = launch_clear(f.fine, f.fine_bytes + sw.zero_bytes, st)) != WCC_OK) return s;      // histograms, max |kept|, barrier counters
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
     NormsExtra ex = {};
-    ex.coef = taps ? taps->coef : nullptr;
     ex.hist1 = sw.hist;
     ex.fine = f.fine;
     const int wbits = (opt && opt->weight_bits && bits) ? opt->weight_bits : bits;
@@ -424,11 +429,11 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     const void* Wq_use = own_codes ? static_cast<const void*>(opt->Wq) : f.Wq;
     const float* scale_w_use = own_codes ? opt->scale_w : f.scale_w;
     const FusedExtra fx = {opt ? opt->alpha : 0.0f, opt ? opt->relu : 0, opt ? opt->residual : nullptr};
-    s = launch_haar_norms(x, N, Cin, H, W, L, dt, f.nrm2, f.amaxpos, ex, st);
+    s = launch_pass1(x, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(2, st)) != WCC_OK) return s;
     // joint shrinkage: index list, rank map, max |kept|
-    s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, f.amaxpos, true, f.sel, f.sel_bytes, st, true,
+    s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, amaxpos, true, f.sel, f.sel_bytes, st, true,
                       f.fine, f.thr, taps != nullptr);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(3, st)) != WCC_OK) return s;

@@ -1,0 +1,266 @@
+// First pass of the fused layer, and the forward transform on its own (steps A and B-norms of the WCC workflow; Eq. 3-6,
+// Alg. 1): transform x in registers, build the channel norms, the per-position max |coefficient| and the selection's
+// histograms; on request store the coefficients.
+//
+// One CTA of NW warps per (image, tile).  The warps take the boxes of NB channels in turn (box r goes to warp r % NW), loading
+// the next box of theirs straight into registers while the current one is worked on.  Only the chain of fused multiply-adds
+// that builds the norms (one per position, ascending channel order) runs in sequence: the eight partial sums of every lane
+// travel from the warp of box r to the warp of box r + 1 through shared memory (a "token", signalled on an mbarrier), so the
+// sums are the chains a single thread would build.  A slot belongs to the receiving warp; it is free again when it is
+// written next, because the chain has passed through its owner since.  The transform runs without its halvings; one exact
+// factor per slot at the end.  The last step (maxima over the warps, stores, histograms) is shared by the warps.
+//
+// Measured (B200, whole layer before -> after; the pass it replaced fed TMA rings in shared memory): 144 -> 24 bf16 37.3 -> 34.4
+// us, 384 -> 512 bf16 59.4 -> 56.2, six-layer chain 393 -> 377, 24 images of C4 131 -> 125; transform, selection and inverse of
+// 4 x 64 x 192 x 320 fp32 80 -> 70 (the norms no longer take a pass over the stored coefficients).
+#pragma once
+
+#include "common.cuh"
+#include "gather.cuh"
+#include "patch.cuh"
+
+namespace wcc {
+
+struct NormsExtra {
+    uint32_t* hist1;      // [N][3][2048] (round 1 first), cleared by launch_clear in the launch before, or NULL
+    uint32_t* fine;       // [N][65536]: histogram of the 16 bits below the sign of every norm, cleared with hist1
+    const float* Wt;      // weights to prepare in extra CTAs, or NULL
+    void* Wq;
+    float* scale_w;
+    int Cout, kpad, bits;
+};
+
+// What a launch produces besides the norms: per-position maxima (unless no scale is taken from them), coefficients.
+enum { P1_NORMS = 0, P1_MAX = 1, P1_COEF = 2 };
+
+template <typename T, int L, bool VEC, int NW, int KIND>
+__global__ void __launch_bounds__(NW * 32, 16 / NW)
+pass1_kernel(const T* __restrict__ x, int C, int H, int W, int weight_ctas, float* __restrict__ coef, float* __restrict__ nrm2,
+             float* __restrict__ amaxpos, const NormsExtra ex, int* __restrict__ status)
+{
+    constexpr int NB = (sizeof(T) == 2) ? 8 : 4;       // channels of a box: 32 registers
+    constexpr int S = 8 / ((NW < 4) ? NW : 4);         // slots a warp finishes at the end
+    constexpr bool MAXV = KIND != P1_NORMS;
+    using TT = HaarTile<L>;
+    __shared__ float4 token[(NW > 1) ? NW : 1][2][32];          // eight sums per lane, per receiving warp
+    __shared__ float fin[(NW > 1) ? NW + 1 : 1][8][32];         // maxima per warp, norms
+    __shared__ uint64_t tok_bars[NW];
+    pdl_launch();
+    const int warp = (NW > 1) ? __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0) : 0, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x < weight_ctas) {
+        const int o = (int)blockIdx.x * NW + warp;
+        if (o < ex.Cout) weight_prep_row(ex.Wt, o, C, ex.kpad, ex.bits, ex.Wq, ex.scale_w);
+        return;
+    }
+    const int tiles_x = (W + TT::TW - 1) / TT::TW, tiles_y = H / TT::TH;
+    int n, ty, tx;
+    tile_coords((int)blockIdx.x - weight_ctas, tiles_x, tiles_y, n, ty, tx);
+    const LanePos lp = lane_positions<L>(H, W, ty, tx, lane);
+    const size_t P = (size_t)H * W, plane = P * sizeof(T);
+    const PatchOff off = patch_off<T>(lp, W);
+    const uint64_t xb = reinterpret_cast<uint64_t>(x) + (uint64_t)n * C * plane;
+    const int rounds = (C + NB - 1) / NB;
+    Raw<T> raw[NB];
+    if (warp < rounds) ldg_group<T, VEC, true, true, NB>(xb, plane, off, warp * NB, C, raw);
+    if (NW > 1) {
+        if (threadIdx.x < NW) tc::mbar_init(tc::smem_u32(&tok_bars[threadIdx.x]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        __syncthreads();
+    }
+    float sc[8], amax[8];
+    slot_scales<L>(lane, false, sc);
+#pragma unroll
+    for (int s = 0; s < 8; ++s) amax[s] = 0.0f;
+    float2 acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.0f, 0.0f);
+    bool ok = true;
+    uint32_t parity = 0;
+    for (int r = warp; r < rounds; r += NW) {
+        float o[NB][8];
+#pragma unroll
+        for (int g = 0; g < NB; g += 4) fwd_group<T, L, 4>(raw + g, *reinterpret_cast<float(*)[4][8]>(&o[g]), lane);
+        if (r + NW < rounds) {                         // the words of this box are consumed: the next box goes into their registers
+            if ((r + NW) * NB + NB <= C) ldg_group<T, VEC, true, false, NB>(xb, plane, off, (r + NW) * NB, C, raw);
+            else ldg_group<T, VEC, true, true, NB>(xb, plane, off, (r + NW) * NB, C, raw);
+        }
+        if (r == rounds - 1) {                         // channels beyond the last one repeat it: they count nothing
+#pragma unroll
+            for (int d = 1; d < NB; ++d)
+                if (r * NB + d >= C) {
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) o[d][s] = 0.0f;
+                }
+        }
+        if (KIND == P1_COEF) {
+#pragma unroll
+            for (int d = 0; d < NB; ++d) {
+                if (r * NB + d < C) {
+                    float oc[8];
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) oc[s] = __fmul_rn(o[d][s], sc[s]);
+                    store_slots<L, VEC>(coef + ((size_t)n * C + r * NB + d) * P, lp, oc);
+                }
+            }
+        }
+        if (MAXV) {
+#pragma unroll
+            for (int d = 0; d < NB; ++d)
+#pragma unroll
+                for (int s = 0; s < 8; ++s) amax[s] = fmaxf(amax[s], fabsf(o[d][s]));
+        }
+        if (NW > 1 && r > 0) {                         // the token: partial sums of the boxes before this one
+            ok = ok && tc::mbar_wait(tc::smem_u32(&tok_bars[warp]), parity);
+            parity ^= 1u;
+            const float4 t0 = token[warp][0][lane], t1 = token[warp][1][lane];
+            acc[0] = make_float2(t0.x, t0.y); acc[1] = make_float2(t0.z, t0.w);
+            acc[2] = make_float2(t1.x, t1.y); acc[3] = make_float2(t1.z, t1.w);
+        }
+#pragma unroll
+        for (int d = 0; d < NB; ++d)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 v = make_float2(o[d][2 * i], o[d][2 * i + 1]);
+                acc[i] = __ffma2_rn(v, v, acc[i]);
+            }
+        if (NW > 1 && r + 1 < rounds) {
+            const int to = (warp + 1 == NW) ? 0 : warp + 1;
+            token[to][0][lane] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+            token[to][1][lane] = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(tc::smem_u32(&tok_bars[to]));
+        }
+    }
+    if (KIND == P1_COEF && !nrm2 && !amaxpos) return;
+    // ---- the norms and maxima of the tile -------------------------------------------------------------
+    float nacc[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { nacc[2 * i] = acc[i].x; nacc[2 * i + 1] = acc[i].y; }
+    if (NW > 1) {
+        if (warp == (rounds - 1) % NW) {
+#pragma unroll
+            for (int s = 0; s < 8; ++s) fin[NW][s][lane] = nacc[s];
+        }
+        if (MAXV) {
+#pragma unroll
+            for (int s = 0; s < 8; ++s) fin[warp][s][lane] = amax[s];
+        }
+        __syncthreads();
+    }
+    pdl_wait();                                        // the histograms are cleared
+    float* nr = nrm2 + (size_t)n * P;
+    float* am = amaxpos + (size_t)n * P;
+    auto finish = [&](int s0, auto first) {            // slots first .. first + S - 1
+        constexpr int F = decltype(first)::value;
+        if (s0 != F) return;
+        float v[S], m[S];
+#pragma unroll
+        for (int i = 0; i < S; ++i) {
+            const int s = F + i;
+            v[i] = __fmul_rn((NW > 1) ? fin[NW][s][lane] : nacc[s], __fmul_rn(sc[s], sc[s]));
+            if (MAXV) {
+                m[i] = (NW > 1) ? fin[0][s][lane] : amax[s];
+#pragma unroll
+                for (int w = 1; w < NW; ++w) m[i] = fmaxf(m[i], fin[w][s][lane]);
+                m[i] = __fmul_rn(m[i], sc[s]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < S; i += 2) {
+            const int s = F + i;
+            if (VEC && (L == 1 || s < 6)) {            // adjacent, 8-byte aligned positions
+                if (lp.ok0) {
+                    if (KIND != P1_COEF || nrm2) *reinterpret_cast<float2*>(nr + lp.pos[s]) = make_float2(v[i], v[i + 1]);
+                    if (MAXV && amaxpos) *reinterpret_cast<float2*>(am + lp.pos[s]) = make_float2(m[i], m[i + 1]);
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (slot_ok<L>(lp, s + j)) {
+                        if (KIND != P1_COEF || nrm2) nr[lp.pos[s + j]] = v[i + j];
+                        if (MAXV && amaxpos) am[lp.pos[s + j]] = m[i + j];
+                    }
+                }
+            }
+        }
+        // Norms that are exactly zero are not counted: after a ReLU whole regions of a map are zero, and their positions
+        // would all hit one bin (thousands of atomics on one address).  The selection knows the number of positions, so
+        // the zeros are what the bins leave out; they rank below everything else.
+        if (KIND != P1_COEF && ex.hist1) {             // norms are >= +0: the digits are the bits below the sign
+            uint32_t* h = ex.hist1 + (size_t)n * 3 * 2048;
+            uint32_t* f = ex.fine + (size_t)n * 65536;
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+                const bool count = slot_ok<L>(lp, F + i) && v[i] != 0.0f;
+                hist_add(h, norm_digit11(v[i]), count);
+                if (count) atomicAdd(&f[norm_digit16(v[i])], 1u);      // spread out: plain atomics
+            }
+        }
+    };
+    const int s0 = warp * S;
+    finish(s0, std::integral_constant<int, 0>{});
+    if constexpr (NW >= 2) finish(s0, std::integral_constant<int, S>{});
+    if constexpr (NW >= 4) {
+        finish(s0, std::integral_constant<int, 2 * S>{});
+        finish(s0, std::integral_constant<int, 3 * S>{});
+    }
+    if (NW > 1 && !__all_sync(0xFFFFFFFFu, ok ? 1 : 0) && lane == 0) atomicExch(status, (int)WCC_ERR_TIMEOUT);
+}
+
+// Warps per tile: one where the tiles alone fill the sixteen warps of every SM about once (no hand-over), up to eight where
+// they are few; four where one warp per tile would leave a long second wave.  us per layer with 1 / 2 / 4 / 8 warps: 512 tiles
+// (144 -> 24 bf16) 47.9 / 37.6 / 34.3 / 37.3; 128 tiles (384 -> 512 bf16) 101 / 73 / 61 / 56; 1024 tiles (32 -> 192 chain)
+// 405 / 377 / 387 / 414; 1440 tiles (C4) 68.7 / 71.4 / 69.8 / 72.7; 2880 tiles 130.0 / 125.8 / 125.1 / 132.5.
+template <typename T, int L, bool VEC, int KIND>
+static wcc_status pass1_launch(const void* x, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
+                               cudaStream_t st)
+{
+    using TT = HaarTile<L>;
+    const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
+    if (tiles > 0x3FFFFFFFLL) return WCC_ERR_SHAPE;
+    int dev = 0, sms = 0;
+    WCC_CUDA_TRY(cudaGetDevice(&dev));
+    WCC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int* status = nullptr;
+    WCC_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&status), g_status));
+    const long long warps = 16LL * sms;
+    const int nw = tiles > warps ? 4 : tiles * 2 > warps ? 1 : tiles * 4 > warps ? 2 : tiles * 8 > warps ? 4 : 8;
+    auto go = [&](auto kern, int w) -> wcc_status {
+        const int wctas = ex.Wt ? ceil_div(ex.Cout, w) : 0;
+        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), 0, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), C, H, W,
+                                 wctas, coef, nrm2, amaxpos, ex, status);
+    };
+    if (nw == 1) return go(pass1_kernel<T, L, VEC, 1, KIND>, 1);
+    if (nw == 2) return go(pass1_kernel<T, L, VEC, 2, KIND>, 2);
+    if (nw == 4) return go(pass1_kernel<T, L, VEC, 4, KIND>, 4);
+    return go(pass1_kernel<T, L, VEC, 8, KIND>, 8);
+}
+
+template <typename T, int L, bool VEC>
+static wcc_status pass1_dispatch(const void* x, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
+                                 cudaStream_t st)
+{
+    if (coef) return pass1_launch<T, L, VEC, P1_COEF>(x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    if (amaxpos) return pass1_launch<T, L, VEC, P1_MAX>(x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    return pass1_launch<T, L, VEC, P1_NORMS>(x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+}
+
+// First pass of the fused layer.  With ex.hist1 set, launch_clear on the histograms must be the call before it on the stream.
+static wcc_status launch_pass1(const void* x, int N, int C, int H, int W, int L, wcc_dtype dt, float* nrm2, float* amaxpos, const NormsExtra& ex,
+                               cudaStream_t st)
+{
+    const bool vec = (W % 4) == 0;
+    float* coef = nullptr;
+    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+}
+
+// Forward transform with stored coefficients; nrm2 and amaxpos may be NULL.
+wcc_status launch_haar_fwd(const void* x, int N, int C, int H, int W, int L, wcc_dtype dt, float* coef, float* nrm2, float* amaxpos,
+                           cudaStream_t st)
+{
+    const bool vec = (W % 4) == 0;                     // always true for L >= 2
+    const NormsExtra ex = {};
+    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+}
+
+}  // namespace wcc

@@ -98,7 +98,7 @@ __device__ __forceinline__ void ldg_group(uint64_t xb, size_t plane, const Patch
     }
 }
 
-// haar_fwd_lanes_raw from the loaded words.  fp32: the first step is scalar, because packing (quad 0, quad 1) pairs out of
+// Forward transform (sums and differences only, see slot_scales) from the loaded words.  fp32: the first step is scalar, because packing (quad 0, quad 1) pairs out of
 // vector loads would take a register move per word (45 instead of 35 instructions per patch); bf16 words are unpacked
 // anyway, straight into the pairs.
 template <typename T, int L, int U>

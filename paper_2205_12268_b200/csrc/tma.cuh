@@ -68,14 +68,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     return false;
 }
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-        : "memory");
-}
-
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -93,26 +85,6 @@ inline EncodeTiledFn encode_fn()
     return fn;
 }
 
-
-// Activation tensor x[N][C][H][W] (element size es = 2: bf16, 4: fp32) as a 4-D map, box = box_w columns x box_h rows
-// x box_c channels of one image, dense in shared memory ([channel][row][column]), zero fill outside the tensor
-// (ragged last tile in W, channels beyond C).  Needs W * es and the base address to be multiples of 16 bytes.
-inline bool make_map_x(CUtensorMap* tm, const void* x, int es, int N, int C, int H, int W, int box_w, int box_h, int box_c)
-{
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[4] = {(cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)C, (cuuint64_t)N};
-    cuuint64_t strides[3] = {(cuuint64_t)W * es, (cuuint64_t)H * W * es, (cuuint64_t)C * H * W * es};
-    cuuint32_t box[4] = {(cuuint32_t)box_w, (cuuint32_t)box_h, (cuuint32_t)box_c, 1u};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    return fn(tm, es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(x), dims,
-              strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-inline bool tma_ok_x(const void* x, int es, int W)
-{
-    return (reinterpret_cast<uintptr_t>(x) % 16) == 0 && ((size_t)W * es) % 16 == 0;
-}
 
 }  // namespace tc
 }  // namespace wcc
