@@ -446,8 +446,8 @@ select_coop_kernel(const float* __restrict__ nrm2, int P, int k, uint32_t* __res
 constexpr int CL_THREADS = 1024;
 constexpr int CL_MAXKPT = 16;
 constexpr int CL_MAXCS = 16;          // 8 is the portable cluster size; 16 needs the non-portable opt-in
-constexpr int CL_CAND_CTA = 512;     // candidate slots per CTA
-constexpr int CL_CAND_MAX = 1024;    // most candidates ranked by brute force; beyond that: histogram rounds
+constexpr int CL_CAND_CTA = 1024;    // candidate slots per CTA
+constexpr int CL_CAND_MAX = 2048;    // most candidates gathered by every CTA; beyond that: another round over the cluster
 constexpr int FINE_BINS = 65536;     // histogram of the 16 bits below the sign of every norm, filled by the producer of the norms
 
 struct ClusterSmem {
@@ -459,10 +459,11 @@ struct ClusterSmem {
     uint32_t res[3];                // found bin, keys above it, keys in it
     uint32_t tot[CL_MAXCS];
     uint32_t amax;
-    uint32_t ncand;                 // candidates of this CTA (keys in the 16-bit bin that holds the threshold)
+    uint32_t ncand[5];              // candidates of this CTA, per gather (a neighbour may still read an earlier count)
     uint32_t cand[CL_CAND_CTA];
     __align__(16) uint32_t all[CL_CAND_MAX];      // candidates of the whole cluster
     uint32_t thr[3];                // threshold key, ties to keep, ties in total
+    __align__(16) uint32_t range[4];              // positive keys, zeros, smallest positive key, largest key
 };
 
 // exclusive scan over the threads of the block (256, 512 or 1024); every thread also gets the total
@@ -550,6 +551,106 @@ __device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, Clu
 }
 
 
+// Shift that maps a span of keys onto at most 2048 bins.
+__device__ __forceinline__ int span_shift(uint32_t span) { return max(0, 32 - __clz(span) - 11); }
+
+// Gathers the keys in [lo, hi] of the whole cluster into sm.all of every CTA; returns how many there are (0xFFFFFFFF: too many).
+// One cluster barrier.
+template <int MAXKPT, typename Valid>
+__device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, ClusterSmem& sm, int cs, const uint32_t (&key)[MAXKPT], int kpt,
+                                                   Valid valid, uint32_t lo, uint32_t hi, int lane, int gather)
+{
+#pragma unroll
+    for (int i = 0; i < MAXKPT; ++i) {
+        if (i >= kpt) break;
+        const bool c = valid(i) && key[i] >= lo && key[i] <= hi;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, c);
+        if (m) {
+            uint32_t off = 0;
+            if (lane == 0) off = atomicAdd(&sm.ncand[gather], (uint32_t)__popc(m));
+            off = __shfl_sync(0xFFFFFFFFu, off, 0);
+            const uint32_t slot = off + (uint32_t)__popc(m & ((1u << lane) - 1u));
+            if (c && slot < CL_CAND_CTA) sm.cand[slot] = key[i];
+        }
+    }
+    cluster.sync();
+    if (threadIdx.x < cs) sm.tot[threadIdx.x] = *cluster.map_shared_rank(&sm.ncand[gather], threadIdx.x);
+    __syncthreads();
+    uint32_t M = 0;
+    bool overflow = false;
+    for (int r = 0; r < cs; ++r) { overflow = overflow || sm.tot[r] > CL_CAND_CTA; M += sm.tot[r]; }
+    if (overflow || M > CL_CAND_MAX) return 0xFFFFFFFFu;
+    // one remote load per thread, all in flight together (rank after rank would expose every rank's latency)
+    for (uint32_t g = threadIdx.x; g < M; g += blockDim.x) {
+        uint32_t pre = 0;
+        int r = 0;
+        while (g >= pre + sm.tot[r]) { pre += sm.tot[r]; ++r; }
+        sm.all[g] = cluster.map_shared_rank(sm.cand, r)[g - pre];
+    }
+    __syncthreads();
+    return M;
+}
+
+// The krem-th largest of the M candidates in sm.all, all of them in [lo, hi] -> sm.thr = {key, equal keys to keep, equal keys}.
+// Few are ranked by counting (one barrier; 2 us for 340 candidates), many by histogram rounds inside the block, eleven bits of
+// the span each (3 us for two rounds, whatever their number).
+__device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t krem, uint32_t lo, uint32_t hi)
+{
+    if (M <= 512) {
+        const uint4* all4 = reinterpret_cast<const uint4*>(sm.all);
+        for (uint32_t i = threadIdx.x; i < M; i += blockDim.x) {
+            const uint32_t ci = sm.all[i];
+            uint32_t g = 0, e = 0;
+            for (uint32_t j4 = 0; j4 < M / 4; ++j4) {            // four candidates per shared-memory load
+                const uint4 c = all4[j4];
+                g += (c.x > ci) + (c.y > ci) + (c.z > ci) + (c.w > ci);
+                e += (c.x == ci) + (c.y == ci) + (c.z == ci) + (c.w == ci);
+            }
+            for (uint32_t j = M & ~3u; j < M; ++j) { const uint32_t cj = sm.all[j]; g += cj > ci; e += cj == ci; }
+            if (g < krem && krem <= g + e) { sm.thr[0] = ci; sm.thr[1] = krem - g; sm.thr[2] = e; }      // equal keys write equal values
+        }
+        __syncthreads();
+        return;
+    }
+    for (;;) {
+        const int sh = span_shift(hi - lo);
+        for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
+        __syncthreads();
+        for (uint32_t g = threadIdx.x; g < M; g += blockDim.x) {
+            const uint32_t c = sm.all[g];
+            if (c >= lo && c <= hi) atomicAdd(&sm.hist[(c - lo) >> sh], 1u);
+        }
+        __syncthreads();
+        const int per = SEL_BINS / (int)blockDim.x, top = SEL_BINS - 1 - (int)threadIdx.x * per;
+        uint32_t c[8], mysum = 0, tot;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            c[i] = (i < per) ? sm.hist[top - i] : 0u;
+            mysum += c[i];
+        }
+        const uint32_t before = block_scan_1024(mysum, sm.warp_sums, &tot);
+        if (before < krem && krem <= before + mysum) {
+            uint32_t a = before;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (a < krem && krem <= a + c[i]) { sm.res[0] = (uint32_t)(top - i); sm.res[1] = a; sm.res[2] = c[i]; }
+                a += c[i];
+            }
+        }
+        __syncthreads();
+        const uint32_t b = sm.res[0], above = sm.res[1], cnt = sm.res[2];
+        __syncthreads();
+        krem -= above;
+        lo += b << sh;
+        if (sh == 0) {
+            if (threadIdx.x == 0) { sm.thr[0] = lo; sm.thr[1] = krem; sm.thr[2] = cnt; }
+            __syncthreads();
+            return;
+        }
+        hi = min(hi, lo + ((1u << sh) - 1u));
+    }
+}
+
 // Find the bin of a complete 2048-bin histogram in global memory that holds the krem-th key from the top; block of
 // 256, 512 or 1024 threads, every thread returns the same values.
 __device__ __forceinline__ void block_find_bin_2048(const uint32_t* __restrict__ h, uint32_t krem, ClusterSmem& sm,
@@ -578,6 +679,9 @@ __device__ __forceinline__ void block_find_bin_2048(const uint32_t* __restrict__
     __syncthreads();
 }
 
+// Measured (us): without histograms, 4 images of 61440 positions 22.7 -> 15.5 (three rounds on fixed 11 + 11 + 10 bit digits
+// before); with them, 24 images of 30720 positions as 4 instead of 8 CTAs each: one wave, layer 125.1 -> 122.2.
+//
 // hist1 ([N][3][2048], round 1 first) and fine ([N][65536]) are optional histograms of the 11 and 16 bits below the sign
 // of every norm (norm_digit11 / norm_digit16: norms are never negative) that the producer of the norms filled; with both, the threshold is usually found without any histogram round:
 // the 16-bit bin that holds the k-th key contains few keys, which the cluster gathers and ranks directly.
@@ -585,7 +689,8 @@ __device__ __forceinline__ void block_find_bin_2048(const uint32_t* __restrict__
 // (then the order of positions matters); otherwise consumers compare keys with thr[n] = {threshold key, ties
 // kept, use_rank flag, number of candidate keys that were ranked (diagnostic)}.
 // MAXKPT: key registers per thread (16, or 4 for the launches that spread an image over enough threads).
-template <int MAXKPT>
+// HIST: the histograms are supplied.
+template <int MAXKPT, bool HIST>
 __global__ void __launch_bounds__(CL_THREADS, 1)
 select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int32_t* __restrict__ idx, float* __restrict__ tau,
                       int32_t* __restrict__ rank, const float* __restrict__ amaxpos, float* __restrict__ amax_kept,
@@ -601,7 +706,9 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
     const int lane = threadIdx.x & 31;
 
     for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
-    if (threadIdx.x == 0) { sm.amax = 0u; sm.ncand = 0u; sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u; }   // thr: keep nothing
+    if (threadIdx.x < 5) sm.ncand[threadIdx.x] = 0u;
+    if (threadIdx.x < 4) sm.range[threadIdx.x] = threadIdx.x == 2 ? 0xFFFFFFFFu : 0u;
+    if (threadIdx.x == 0) { sm.amax = 0u; sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u; }   // thr: keep nothing
                                                        // unless a candidate is found (histograms that do not match the keys)
     pdl_wait();
     pdl_launch();
@@ -621,12 +728,14 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
     __syncthreads();
 
     uint32_t tkey = 0, need_eq = 0, total_eq = 0, ranked = 0;    // ranked: candidates counted through (diagnostic)
+    int gathers = 0;
+    uint32_t lo = 0, hi = 0, krem = 0;                 // the threshold is the krem-th largest key in [lo, hi]
     bool found = false;
     // The supplied histograms count the non-zero norms only; the zeros are the positions they leave out and rank
     // below everything else.  More kept positions than non-zero norms: the threshold is zero.
     bool zero_thr = false;
     uint32_t b1h = 0, aboveh = 0;
-    if (hist1 && fine) {
+    if (HIST) {
         // the 11-bit bin of the threshold
         uint32_t nonzero;
         if (threadIdx.x == 0) { sm.res[0] = 0u; sm.res[1] = 0u; sm.res[2] = 0u; }      // (a barrier follows inside)
@@ -639,7 +748,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
             found = true;
         }
     }
-    if (hist1 && fine && !zero_thr) {
+    if (HIST && !zero_thr) {
         // the 16-bit bin inside the 11-bit bin (32 fine bins, one per lane of warp 0, top bin in lane 0)
         const uint32_t b1 = b1h, above = aboveh;
         const uint32_t k1 = (uint32_t)k - above;
@@ -657,100 +766,85 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
         __syncthreads();
         const uint32_t prefix16 = sm.res[0], k16 = k1 - sm.res[1];
         __syncthreads();
-        // collect this CTA's candidates
-#pragma unroll
-        for (int i = 0; i < MAXKPT; ++i) {
-            if (i >= kpt) break;
-            const bool c = valid(i) && ((key[i] >> 15) & 0xFFFFu) == prefix16;
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, c);
-            if (m) {
-                uint32_t off = 0;
-                if (lane == 0) off = atomicAdd(&sm.ncand, (uint32_t)__popc(m));
-                off = __shfl_sync(0xFFFFFFFFu, off, 0);
-                const uint32_t slot = off + (uint32_t)__popc(m & ((1u << lane) - 1u));
-                if (c && slot < CL_CAND_CTA) sm.cand[slot] = key[i];
-            }
-        }
-        cluster.sync();
-        if (threadIdx.x < cs) sm.tot[threadIdx.x] = *cluster.map_shared_rank(&sm.ncand, threadIdx.x);
-        __syncthreads();
-        uint32_t M = 0;
-        bool overflow = false;
-        for (int r = 0; r < cs; ++r) { overflow = overflow || sm.tot[r] > CL_CAND_CTA; M += sm.tot[r]; }
-        overflow = overflow || M > CL_CAND_MAX;
-        if (!overflow) {
-            // one remote load per thread, all in flight together (rank after rank would expose every rank's latency)
-            for (uint32_t g = threadIdx.x; g < M; g += blockDim.x) {
-                uint32_t pre = 0;
-                int r = 0;
-                while (g >= pre + sm.tot[r]) { pre += sm.tot[r]; ++r; }
-                sm.all[g] = cluster.map_shared_rank(sm.cand, r)[g - pre];
-            }
-            __syncthreads();
-            // the k16-th largest candidate, by counting (M is small)
-            for (uint32_t i = threadIdx.x; i < M; i += blockDim.x) {
-                const uint32_t ci = sm.all[i];
-                uint32_t g = 0, e = 0;
-                const uint4* all4 = reinterpret_cast<const uint4*>(sm.all);
-                for (uint32_t j4 = 0; j4 < M / 4; ++j4) {        // four candidates per shared-memory load
-                    const uint4 c = all4[j4];
-                    g += (c.x > ci) + (c.y > ci) + (c.z > ci) + (c.w > ci);
-                    e += (c.x == ci) + (c.y == ci) + (c.z == ci) + (c.w == ci);
-                }
-                for (uint32_t j = M & ~3u; j < M; ++j) { const uint32_t cj = sm.all[j]; g += cj > ci; e += cj == ci; }
-                if (g < k16 && k16 <= g + e) { sm.thr[0] = ci; sm.thr[1] = k16 - g; sm.thr[2] = e; }   // equal keys write equal values
-            }
-            __syncthreads();
+        lo = 0x80000000u | (prefix16 << 15);
+        hi = lo | 0x7FFFu;
+        krem = k16;
+        const uint32_t M = cluster_gather<MAXKPT>(cluster, sm, cs, key, kpt, valid, lo, hi, lane, gathers++);
+        if (M != 0xFFFFFFFFu) {
+            if (M >= krem) block_rank(sm, M, krem, lo, hi);              // (fewer: histograms that do not match the keys, keep nothing)
             tkey = sm.thr[0]; need_eq = sm.thr[1]; total_eq = sm.thr[2];
             ranked = M;
             found = true;
         }
     }
-    if (!found) {
-        // round 1: top 11 bits (only the bin search when the producer of the norms histogrammed them).  The producer's
-        // digits start below the sign bit (norm_digit11), so with its histogram the rounds run on the keys shifted left
-        // by one: 11 + 11 + 9 bits and a zero; the threshold is shifted back at the end.
-        uint32_t b1, above;
-        const bool shifted = hist1 != nullptr;
-        if (shifted) {
+    if (!HIST) {
+        // No histograms: the range of the positive keys, and how many keys are positive or zero.  (Zeros would stretch the range
+        // by hundreds of octaves; there can be many after a ReLU.)
+        uint32_t np = 0, nz = 0, mn = 0xFFFFFFFFu, mx = 0u;
 #pragma unroll
-            for (int i = 0; i < MAXKPT; ++i) key[i] <<= 1;
+        for (int i = 0; i < MAXKPT; ++i) {
+            if (!valid(i)) continue;
+            const bool pos = key[i] > 0x80000000u;
+            np += pos;
+            nz += key[i] == 0x80000000u;
+            mn = min(mn, pos ? key[i] : 0xFFFFFFFFu);
+            mx = max(mx, key[i]);
         }
-        if (hist1) {
-            uint32_t nonzero;
-            block_find_bin_2048(hist1 + (size_t)n * 3 * SEL_BINS, (uint32_t)k, sm, b1, above, nonzero);
-        } else {
-#pragma unroll
-            for (int i = 0; i < MAXKPT; ++i)
-                if (i < kpt) hist_add(sm.hist, key[i] >> 21, valid(i));
-            cluster_find_bin(cluster, sm, cs, crank, SEL_BINS, (uint32_t)k, b1, above);
+        np = __reduce_add_sync(0xFFFFFFFFu, np);
+        nz = __reduce_add_sync(0xFFFFFFFFu, nz);
+        mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+        if (lane == 0) { atomicAdd(&sm.range[0], np); atomicAdd(&sm.range[1], nz); atomicMin(&sm.range[2], mn); atomicMax(&sm.range[3], mx); }
+        cluster.sync();
+        if (threadIdx.x < 32) {
+            uint32_t q[4] = {0u, 0u, 0xFFFFFFFFu, 0u};
+            if (lane < cs) {
+                const uint4 v = *reinterpret_cast<const uint4*>(cluster.map_shared_rank(sm.range, lane));
+                q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
+            }
+            q[0] = __reduce_add_sync(0xFFFFFFFFu, q[0]);
+            q[1] = __reduce_add_sync(0xFFFFFFFFu, q[1]);
+            q[2] = __reduce_min_sync(0xFFFFFFFFu, q[2]);
+            q[3] = __reduce_max_sync(0xFFFFFFFFu, q[3]);
+            if (lane < 4) sm.tot[lane] = lane == 0 ? q[0] : lane == 1 ? q[1] : lane == 2 ? q[2] : q[3];
+        }
+        __syncthreads();
+        np = sm.tot[0]; nz = sm.tot[1];
+        if ((uint32_t)k <= np) { lo = sm.tot[2]; hi = sm.tot[3]; krem = (uint32_t)k; }
+        else if ((uint32_t)k <= np + nz) { tkey = 0x80000000u; need_eq = (uint32_t)k - np; total_eq = nz; found = true; }
+        else { lo = 0u; hi = 0x7FFFFFFFu; krem = (uint32_t)k - np - nz; }
+        __syncthreads();
+    }
+    // Narrow [lo, hi] until its keys fit the gather: 2048 bins a round over the keys' own range.  For norms (10 to 20 octaves,
+    // most keys within two) the first round leaves tens to hundreds of keys; fixed leading digits left thousands, and most
+    // counts went to a few bins.
+    for (bool first = true; !found; first = false) {
+        const int sh = span_shift(hi - lo);
+        if (!first) {                                  // (all neighbours have read this CTA's bins)
             for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
             __syncthreads();
         }
-        const uint32_t k1 = (uint32_t)k - above;
-        // round 2: next 11 bits of the keys that match
 #pragma unroll
-        for (int i = 0; i < MAXKPT; ++i)     // plain atomics: these digits are mantissa bits, spread over the bins
-            if (valid(i) && (key[i] >> 21) == b1) atomicAdd(&sm.hist[(key[i] >> 10) & 0x7FFu], 1u);
-        uint32_t b2;
-        cluster_find_bin(cluster, sm, cs, crank, SEL_BINS, k1, b2, above);
-        const uint32_t k2 = k1 - above;
-        const uint32_t prefix = (b1 << 11) | b2;
-        // round 3: last 10 bits
-        for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < MAXKPT; ++i)
-            if (valid(i) && (key[i] >> 10) == prefix) atomicAdd(&sm.hist[key[i] & 0x3FFu], 1u);
-        uint32_t b3;
-        cluster_find_bin(cluster, sm, cs, crank, 1024, k2, b3, above);
-        tkey = (prefix << 10) | b3;
-        need_eq = k2 - above;
-        total_eq = sm.res[2];
-        if (shifted) {                                 // back to whole keys (every norm has the sign bit of +0 and above)
-            tkey = (tkey >> 1) | 0x80000000u;
-#pragma unroll
-            for (int i = 0; i < MAXKPT; ++i) key[i] = (key[i] >> 1) | 0x80000000u;
+        for (int i = 0; i < MAXKPT; ++i) {
+            const bool in = valid(i) && key[i] >= lo && key[i] <= hi;
+            const uint32_t b = (key[i] - lo) >> sh;
+            if (in) atomicAdd(&sm.hist[b], 1u);
+        }
+        uint32_t b, above;
+        cluster_find_bin(cluster, sm, cs, crank, SEL_BINS, krem, b, above);
+        const uint32_t cnt = sm.res[2];
+        krem -= above;
+        lo += b << sh;
+        if (sh == 0) { tkey = lo; need_eq = krem; total_eq = cnt; break; }
+        hi = min(hi, lo + ((1u << sh) - 1u));
+        if (cnt <= CL_CAND_MAX) {
+            const uint32_t M = cluster_gather<MAXKPT>(cluster, sm, cs, key, kpt, valid, lo, hi, lane, gathers++);
+            if (M != 0xFFFFFFFFu) {
+                block_rank(sm, M, krem, lo, hi);
+                tkey = sm.thr[0]; need_eq = sm.thr[1]; total_eq = sm.thr[2];
+                ranked = M;
+                break;
+            }
         }
     }
     if (tau && crank == 0 && threadIdx.x == 0) tau[n] = key_float(tkey);
@@ -850,8 +944,11 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
     WCC_CUDA_TRY(cudaGetDevice(&devc));
     if (devc >= 0 && devc < 64 && max_cs[devc] == 0) {
         max_cs[devc] = 8;
-        if (cudaFuncSetAttribute(select_cluster_kernel<CL_MAXKPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaFuncSetAttribute(select_cluster_kernel<4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        bool all = true;
+        auto allow16 = [&](auto kern) { all = all && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess; };
+        allow16(select_cluster_kernel<CL_MAXKPT, true>); allow16(select_cluster_kernel<CL_MAXKPT, false>);
+        allow16(select_cluster_kernel<4, true>); allow16(select_cluster_kernel<4, false>);
+        if (all) {
             cudaLaunchConfig_t q = {};
             q.gridDim = dim3(16, 1);
             q.blockDim = dim3(CL_THREADS);
@@ -860,7 +957,7 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
             qa[0].val.clusterDim.x = 16; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
             q.attrs = qa; q.numAttrs = 1;
             int nclusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&nclusters, select_cluster_kernel<CL_MAXKPT>, &q) == cudaSuccess && nclusters > 0) max_cs[devc] = 16;
+            if (cudaOccupancyMaxActiveClusters(&nclusters, select_cluster_kernel<CL_MAXKPT, true>, &q) == cudaSuccess && nclusters > 0) max_cs[devc] = 16;
         }
         (void)cudaGetLastError();
     }
@@ -871,6 +968,7 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         int cs = 1;
         while (cs < 8 && cs * 512 < P) cs <<= 1;
         if (cs == 8 && cs_cap == 16 && P > 65536) cs = 16;
+        while (cs > 1 && (long long)N * cs > 148 && P <= cs / 2 * CL_THREADS * CL_MAXKPT) cs >>= 1;      // all images in one wave
         int threads = 256;
         const int kpt_goal = hist1_ready ? 4 : CL_MAXKPT;               // few keys per thread when no scans are needed
         while (threads < CL_THREADS && (long long)cs * threads * kpt_goal < P) threads <<= 1;
@@ -879,11 +977,13 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         const uint32_t* hist1 = hist1_ready ? s.hist : nullptr;
         const uint32_t* fine_use = hist1_ready ? fine : (const uint32_t*)nullptr;
         const int wr = (want_rank || !thr) ? 1 : 0;
-        if (kpt <= 4)                                  // few keys per thread: the instantiation with four key registers
-            return launch_overlapped(select_cluster_kernel<4>, dim3(cs, N), dim3(threads), 0, st, hist1_ready, cs, nrm2, P, k, kpt, idx, tau,
-                                     rank, amaxpos, amax_kept, hist1, fine_use, thr, wr);
-        return launch_overlapped(select_cluster_kernel<CL_MAXKPT>, dim3(cs, N), dim3(threads), 0, st, hist1_ready, cs, nrm2, P, k, kpt, idx,
-                                 tau, rank, amaxpos, amax_kept, hist1, fine_use, thr, wr);
+        auto go = [&](auto kern) -> wcc_status {
+            return launch_overlapped(kern, dim3(cs, N), dim3(threads), 0, st, hist1_ready, cs, nrm2, P, k, kpt, idx, tau, rank, amaxpos, amax_kept,
+                                     hist1, fine_use, thr, wr);
+        };
+        // few keys per thread: the instantiation with four key registers
+        if (hist1_ready && fine) return kpt <= 4 ? go(select_cluster_kernel<4, true>) : go(select_cluster_kernel<CL_MAXKPT, true>);
+        return kpt <= 4 ? go(select_cluster_kernel<4, false>) : go(select_cluster_kernel<CL_MAXKPT, false>);
     }
     if (thr) {                                        // these paths always write idx and the rank map
         thr_use_rank_kernel<<<ceil_div(N, 128), 128, 0, st>>>(thr, N);
