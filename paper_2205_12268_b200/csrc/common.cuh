@@ -136,7 +136,7 @@ struct Geom {
 
 // ---- stage launchers (each enqueues on `st`, returns a wcc_status) ---------------------------
 // Forward Haar + norms (+ per-position max |coef| over channels when amaxpos != NULL).
-wcc_status launch_haar_fwd(const void* x, int N, int C, int H, int W, int L, wcc_dtype dt,
+wcc_status launch_haar_fwd(const void* x, const float* taps, int N, int C, int H, int W, int L, wcc_dtype dt,
                            float* coef, float* nrm2, float* amaxpos, cudaStream_t st);
 // Plain inverse Haar.
 wcc_status launch_haar_inv(const float* coef, int N, int C, int H, int W, int L, wcc_dtype dt,

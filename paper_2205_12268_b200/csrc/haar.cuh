@@ -1,6 +1,5 @@
-// Haar kernels: depthwise convolution + forward transform, channel norms of a stored map, plain inverse, and the fused
-// dequantize + scatter + inverse (steps A, B-norms, D, E of the WCC workflow; Eq. 3-6, Alg. 1).  The forward transform of
-// a feature map is in pass1.cuh.
+// Haar kernels: channel norms of a stored map, plain inverse, and the fused dequantize + scatter + inverse (steps B-norms, D, E
+// of the WCC workflow; Eq. 3-6, Alg. 1).  The forward transform of a feature map is in pass1.cuh.
 //
 // Work decomposition (all three kernels).  One warp owns a tile of 2^L rows x TW columns of one image,
 // TW = 4 * CG, CG = 32 / 2^(L-1).  Lane (rp, cg) = (lane / CG, lane % CG) holds the 2 x 4 patch at rows
@@ -397,161 +396,6 @@ __device__ __forceinline__ void tile_coords(int warp, int tiles_x, int tiles_y, 
     n = t / tiles_y;
 }
 
-// ---- depthwise 3x3 convolution fused with the forward transform ------------------------------------------
-// The input of the block's second pointwise layer is a depthwise convolution of the expanded map (Eq. 13); both are
-// separable per channel, so the convolution's output never goes to memory: every lane computes the convolution at the
-// eight pixels of its patch (from a 4 x 6 neighbourhood of the input, zeros outside the map) and transforms them right
-// away.  Per output pixel: one fused multiply-add per tap, row-major tap order, starting from +0 (taps outside the map
-// contribute nothing).  Same work decomposition (channel chunks included) and outputs as haar_fwd_kernel; w is fp32
-// [C][3][3].
-
-// One channel's input of the convolution as loaded: rows r0-1 .. r0+2, columns c0-1 .. c0+4 of the lane's patch (zeros
-// outside the map), and the channel's nine taps.  With W % 4 == 0 the four middle columns are one aligned vector; bf16
-// rows then stay packed (two words of middle columns, one word holding the left and the right neighbour).
-template <typename T, bool VEC>
-struct DwRaw {
-    static constexpr bool PACKED = VEC && sizeof(T) == 2;
-    static constexpr int RW = PACKED ? 3 : 6;
-    uint32_t v[4][RW];
-    float k[9];
-};
-
-// ER / EC: the tile touches the top or bottom / the left or right border of the map (or hangs over it), so rows / columns
-// of the neighbourhood can fall outside; tiles in the interior load without any bounds test.
-template <typename T, bool VEC, bool ER = true, bool EC = true>
-__device__ __forceinline__ void dwconv_load(const T* __restrict__ plane, const float* __restrict__ w9, const LanePos& lp,
-                                            int H, int W, DwRaw<T, VEC>& r)
-{
-#pragma unroll
-    for (int i = 0; i < 9; ++i) r.k[i] = __ldg(w9 + i);
-    auto load1 = [&](int rr, int cc) -> uint32_t {         // one element as fp32 bits (bf16: the upper half)
-        if (sizeof(T) == 4) return __ldg(reinterpret_cast<const uint32_t*>(plane) + (size_t)rr * W + cc);
-        return (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(plane) + (size_t)rr * W + cc) << 16;
-    };
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int rr = lp.r0 + a - 1;
-        const bool row_in = !ER || (rr >= 0 && rr < H);
-        if constexpr (VEC) {
-            const uint32_t left = (row_in && (!EC || (lp.c0 > 0 && lp.c0 - 1 < W))) ? load1(rr, lp.c0 - 1) : 0u;
-            const uint32_t right = (row_in && (!EC || lp.c0 + 4 < W)) ? load1(rr, lp.c0 + 4) : 0u;
-            if constexpr (sizeof(T) == 4) {
-                uint4 m = make_uint4(0u, 0u, 0u, 0u);
-                if (row_in && (!EC || lp.ok0)) m = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint32_t*>(plane) + (size_t)rr * W + lp.c0));
-                r.v[a][0] = left; r.v[a][1] = m.x; r.v[a][2] = m.y; r.v[a][3] = m.z; r.v[a][4] = m.w; r.v[a][5] = right;
-            } else {
-                uint2 m = make_uint2(0u, 0u);
-                if (row_in && (!EC || lp.ok0)) m = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const unsigned short*>(plane) + (size_t)rr * W + lp.c0));
-                r.v[a][0] = m.x; r.v[a][1] = m.y; r.v[a][2] = (left >> 16) | right;
-            }
-        } else {
-#pragma unroll
-            for (int b = 0; b < 6; ++b) {
-                const int cc = lp.c0 + b - 1;
-                r.v[a][b] = (row_in && cc >= 0 && cc < W) ? load1(rr, cc) : 0u;
-            }
-        }
-    }
-}
-
-// The convolution at the eight pixels of the lane's patch: one fused multiply-add per tap, row-major tap order, from +0.
-template <typename T, bool VEC>
-__device__ __forceinline__ void dwconv_compute(const DwRaw<T, VEC>& r, float (&p)[2][4])
-{
-    float in[4][6];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        if constexpr (DwRaw<T, VEC>::PACKED) {
-            in[a][0] = bf16lo(r.v[a][2]);
-            in[a][1] = bf16lo(r.v[a][0]); in[a][2] = bf16hi(r.v[a][0]);
-            in[a][3] = bf16lo(r.v[a][1]); in[a][4] = bf16hi(r.v[a][1]);
-            in[a][5] = bf16hi(r.v[a][2]);
-        } else {
-#pragma unroll
-            for (int b = 0; b < 6; ++b) in[a][b] = __uint_as_float(r.v[a][b]);
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) acc = __fmaf_rn(r.k[i * 3 + j], in[a + i][b + j], acc);
-            p[a][b] = acc;
-        }
-}
-
-// Channels [c_lo, c_hi) of one tile, two at a time: while one channel is convolved and transformed the next one's input
-// is in flight (two register buffers that swap roles).
-template <typename T, int L, bool VEC, bool NORMS, bool ER, bool EC>
-__device__ __forceinline__ void dwconv_channels(const T* __restrict__ uin, const float* __restrict__ w, float* __restrict__ cout,
-                                                int c_lo, int c_hi, const LanePos& lp, int lane, int n, int H, int W,
-                                                float* __restrict__ nrm2, float* __restrict__ amaxpos)
-{
-    const size_t P = (size_t)H * W;
-    float nacc[8], amax[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) { nacc[s] = 0.0f; amax[s] = 0.0f; }
-    auto finish = [&](const DwRaw<T, VEC>& r, int c) {
-        float p[2][4], o[8];
-        dwconv_compute<T, VEC>(r, p);
-        haar_fwd_lane<L>(p, o, lane);
-        if (cout) store_slots<L, VEC>(cout + (size_t)c * P, lp, o);
-        if (NORMS) {
-#pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                nacc[s] = __fmaf_rn(o[s], o[s], nacc[s]);
-                amax[s] = fmaxf(amax[s], fabsf(o[s]));
-            }
-        }
-    };
-    DwRaw<T, VEC> a, b;
-    if (c_lo < c_hi) dwconv_load<T, VEC, ER, EC>(uin + (size_t)c_lo * P, w + (size_t)c_lo * 9, lp, H, W, a);
-    for (int c = c_lo; c < c_hi; c += 2) {
-        if (c + 1 < c_hi) dwconv_load<T, VEC, ER, EC>(uin + (size_t)(c + 1) * P, w + (size_t)(c + 1) * 9, lp, H, W, b);
-        finish(a, c);
-        if (c + 1 < c_hi) {
-            if (c + 2 < c_hi) dwconv_load<T, VEC, ER, EC>(uin + (size_t)(c + 2) * P, w + (size_t)(c + 2) * 9, lp, H, W, a);
-            finish(b, c + 1);
-        }
-    }
-    if (NORMS) {
-        if (nrm2) store_slots<L, VEC>(nrm2 + (size_t)n * P, lp, nacc);
-        if (amaxpos) store_slots<L, VEC>(amaxpos + (size_t)n * P, lp, amax);
-    }
-}
-
-// NORMS = false: a chunk of the channels (blockIdx.y), coefficients only.
-template <typename T, int L, bool VEC, bool NORMS>
-__global__ void __launch_bounds__(128)
-dwconv_haar_fwd_kernel(const T* __restrict__ u, const float* __restrict__ w, int N, int C, int H, int W, int cpc,
-                       float* __restrict__ coef, float* __restrict__ nrm2, float* __restrict__ amaxpos)
-{
-    using TT = HaarTile<L>;
-    const int tiles_x = (W + TT::TW - 1) / TT::TW, tiles_y = H / TT::TH;
-    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (warp >= N * tiles_x * tiles_y) return;
-    const int lane = threadIdx.x & 31;
-    int n, ty, tx;
-    tile_coords(warp, tiles_x, tiles_y, n, ty, tx);
-    const LanePos lp = lane_positions<L>(H, W, ty, tx, lane);
-    const size_t P = (size_t)H * W;
-    const T* uin = u + (size_t)n * C * P;
-    float* cout = coef ? coef + (size_t)n * C * P : nullptr;
-    const int c_lo = (int)blockIdx.y * cpc, c_hi = min(C, c_lo + cpc);
-
-    // border tests only where the tile needs them
-    const int ty0 = ty * TT::TH, tx0 = tx * TT::TW;
-    const bool er = !(ty0 >= 1 && ty0 + TT::TH < H), ec = !(tx0 >= 1 && tx0 + TT::TW < W);
-    if (!VEC || (er && ec)) dwconv_channels<T, L, VEC, NORMS, true, true>(uin, w, cout, c_lo, c_hi, lp, lane, n, H, W, nrm2, amaxpos);
-    else if (er) dwconv_channels<T, L, VEC, NORMS, true, false>(uin, w, cout, c_lo, c_hi, lp, lane, n, H, W, nrm2, amaxpos);
-    else if (ec) dwconv_channels<T, L, VEC, NORMS, false, true>(uin, w, cout, c_lo, c_hi, lp, lane, n, H, W, nrm2, amaxpos);
-    else dwconv_channels<T, L, VEC, NORMS, false, false>(uin, w, cout, c_lo, c_hi, lp, lane, n, H, W, nrm2, amaxpos);
-}
-
 // Channel norms of a stored coefficient map: one thread per position builds the chain of fused multiply-adds over the
 // channels in ascending order, from +0, and max |coef|.  Thirty-two channels of loads in flight per thread.
 __global__ void __launch_bounds__(256)
@@ -581,18 +425,6 @@ coef_norms_kernel(const float* __restrict__ coef, int N, int C, long long P, flo
     }
     if (nrm2) nrm2[id] = acc;
     if (amaxpos) amaxpos[id] = am;
-}
-
-// Channels per chunk of the forward kernels: one chunk (norms in the same pass) when the tiles alone fill the GPU or no
-// coefficient map is stored; otherwise chunks of a multiple of `unit` channels, about 64 warps for each of the 148 SMs.
-static int forward_chunk_channels(long long tile_warps, int C, int unit, bool has_coef)
-{
-    constexpr long long want = 148 * 64;              // measured on the block's shapes: 24 to 96 warps per SM tried
-    if (!has_coef || tile_warps >= want || C <= 2 * unit) return C;
-    const long long chunks = std::min<long long>((C + unit - 1) / unit, (want + tile_warps - 1) / tile_warps);
-    int cpc = (int)((C + chunks - 1) / chunks);
-    cpc = (cpc + unit - 1) / unit * unit;
-    return std::min(cpc, C);
 }
 
 static wcc_status launch_coef_norms(const float* coef, int N, int C, long long P, float* nrm2, float* amaxpos, cudaStream_t st)
@@ -733,32 +565,6 @@ scatter_inv_kernel(const int32_t* __restrict__ acc, int ldc, const int32_t* __re
             return FN<__nv_bfloat16, 3, true>(__VA_ARGS__);                                          \
         }                                                                                            \
     } while (0)
-
-template <typename T, int L, bool VEC>
-static wcc_status dwconv_haar_dispatch(const void* u, const float* w, int N, int C, int H, int W, float* coef, float* nrm2,
-                                       float* amaxpos, cudaStream_t st)
-{
-    using TT = HaarTile<L>;
-    const long long warps = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
-    const int blocks = (int)((warps + 3) / 4);
-    const int cpc = forward_chunk_channels(warps, C, 8, coef != nullptr);
-    const dim3 grid(blocks, ceil_div(C, cpc));
-    if (grid.y > 1)
-        dwconv_haar_fwd_kernel<T, L, VEC, false><<<grid, 128, 0, st>>>(static_cast<const T*>(u), w, N, C, H, W, cpc, coef, nullptr, nullptr);
-    else
-        dwconv_haar_fwd_kernel<T, L, VEC, true><<<grid, 128, 0, st>>>(static_cast<const T*>(u), w, N, C, H, W, cpc, coef, nrm2, amaxpos);
-    WCC_LAUNCH_CHECK();
-    if (grid.y > 1) return launch_coef_norms(coef, N, C, (long long)H * W, nrm2, amaxpos, st);
-    return WCC_OK;
-}
-
-// Depthwise 3x3 convolution + forward Haar + norms (+ per-position max |coef|) in one pass over u.
-wcc_status launch_dwconv_haar_fwd(const void* u, const float* w, int N, int C, int H, int W, int L, wcc_dtype dt,
-                                  float* coef, float* nrm2, float* amaxpos, cudaStream_t st)
-{
-    const bool vec = (W % 4) == 0;
-    WCC_DISPATCH_TLV(dwconv_haar_dispatch, dt, L, vec, u, w, N, C, H, W, coef, nrm2, amaxpos, st);
-}
 
 template <typename T, int L, bool VEC>
 static wcc_status haar_inv_dispatch(const float* coef, int planes, int H, int W, void* out, cudaStream_t st)

@@ -173,8 +173,7 @@ static wcc_status staged_impl(const void* x, const float* Wt, int N, int Cin, in
 
     if ((s = profile_mark(0, st)) != WCC_OK) return s;
     // A: Haar transform + channel norms (and the per-position max |coef| the activation scale is taken from)
-    s = dwk ? launch_dwconv_haar_fwd(x, dwk, N, Cin, H, W, L, dt, f.coef, f.nrm2, f.amaxpos, st)
-            : launch_haar_fwd(x, N, Cin, H, W, L, dt, f.coef, f.nrm2, f.amaxpos, st);
+    s = launch_haar_fwd(x, dwk, N, Cin, H, W, L, dt, f.coef, f.nrm2, f.amaxpos, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
     // B: joint shrinkage: kept index list, rank map, max |kept|
@@ -345,7 +344,7 @@ static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int 
     ex.fine = f.fine;
     const int wbits = (opt && opt->weight_bits && bits) ? opt->weight_bits : bits;
     ex.Wt = Wt; ex.Wq = f.Wq; ex.scale_w = f.scale_w; ex.Cout = Cout; ex.kpad = f.kpad; ex.bits = wbits;
-    s = launch_pass1(x, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
+    s = launch_pass1(x, nullptr, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
     s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, amaxpos, true, f.sel, f.sel_bytes, st, true, f.fine, f.thr, true);
@@ -416,7 +415,7 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     // coefficient map is written only when a test asks for it).  The same launch fills round 1 of the select's
     // histogram and quantizes the weights in a few extra CTAs.
     const SelectWs sw = carve_select_ws(f.sel, N, P);
-    if (taps && taps->coef && (s = launch_haar_fwd(x, N, Cin, H, W, L, dt, taps->coef, nullptr, nullptr, st)) != WCC_OK) return s;
+    if (taps && taps->coef && (s = launch_haar_fwd(x, nullptr, N, Cin, H, W, L, dt, taps->coef, nullptr, nullptr, st)) != WCC_OK) return s;
     // the per-position maxima are only built where the activation scale comes from them
     float* const amaxpos = (bits >= 2 && !(opt && opt->alpha > 0.0f)) ? f.amaxpos : nullptr;
     if ((s = launch_clear(f.fine, f.fine_bytes + sw.zero_bytes, st)) != WCC_OK) return s;      // histograms, max |kept|, barrier counters
@@ -429,7 +428,7 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     const void* Wq_use = own_codes ? static_cast<const void*>(opt->Wq) : f.Wq;
     const float* scale_w_use = own_codes ? opt->scale_w : f.scale_w;
     const FusedExtra fx = {opt ? opt->alpha : 0.0f, opt ? opt->relu : 0, opt ? opt->residual : nullptr};
-    s = launch_pass1(x, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
+    s = launch_pass1(x, nullptr, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(2, st)) != WCC_OK) return s;
     // joint shrinkage: index list, rank map, max |kept|
@@ -719,7 +718,7 @@ wcc_status wcc_haar_fwd(const void* x, int N, int C, int H, int Wd, int levels, 
     wcc_status s = check_plane_args(N, C, H, Wd, levels, dt);
     if (s != WCC_OK) return s;
     if (!aligned16(x) || !aligned16(coef) || !aligned16(nrm2)) return WCC_ERR_ALIGN;
-    return launch_haar_fwd(x, N, C, H, Wd, levels, dt, coef, nrm2, nullptr, static_cast<cudaStream_t>(stream));
+    return launch_haar_fwd(x, nullptr, N, C, H, Wd, levels, dt, coef, nrm2, nullptr, static_cast<cudaStream_t>(stream));
 }
 
 wcc_status wcc_haar_inv(const float* coef, int N, int C, int H, int Wd, int levels, wcc_dtype dt,
@@ -781,7 +780,7 @@ wcc_status wcc_dwconv_haar_fwd(const void* u, const float* Wdw, int N, int C, in
     wcc_status s = check_plane_args(N, C, H, Wd, levels, dt);
     if (s != WCC_OK) return s;
     if (!aligned16(u) || !aligned16(Wdw) || !aligned16(coef) || !aligned16(nrm2)) return WCC_ERR_ALIGN;
-    return launch_dwconv_haar_fwd(u, Wdw, N, C, H, Wd, levels, dt, coef, nrm2, nullptr, static_cast<cudaStream_t>(stream));
+    return launch_haar_fwd(u, Wdw, N, C, H, Wd, levels, dt, coef, nrm2, nullptr, static_cast<cudaStream_t>(stream));
 }
 
 size_t wcc_block_workspace_bytes(int N, int C, int E, int H, int Wd, int levels, int k, int bits, wcc_dtype dt)

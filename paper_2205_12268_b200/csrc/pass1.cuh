@@ -33,18 +33,22 @@ struct NormsExtra {
 // What a launch produces besides the norms: per-position maxima (unless no scale is taken from them), coefficients.
 enum { P1_NORMS = 0, P1_MAX = 1, P1_COEF = 2 };
 
-template <typename T, int L, bool VEC, int NW, int KIND>
-__global__ void __launch_bounds__(NW * 32, NW == 1 ? 12 : 16 / NW)
-pass1_kernel(const T* __restrict__ x, int C, int H, int W, int weight_ctas, float* __restrict__ coef, float* __restrict__ nrm2,
+// DW: a depthwise 3x3 convolution (taps fp32 [C][3][3]) is applied to x first; its output never goes to memory (App. H, "a kernel
+// for a fused depthwise convolution and Haar transform").
+template <typename T, int L, bool VEC, int NW, int KIND, bool DW>
+__global__ void __launch_bounds__(NW * 32, ((DW && NW < 8) || NW == 1) ? 12 / NW : 16 / NW)
+pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int H, int W, int weight_ctas, float* __restrict__ coef, float* __restrict__ nrm2,
              float* __restrict__ amaxpos, const NormsExtra ex, int* __restrict__ status)
 {
-    constexpr int NB = (sizeof(T) == 2) ? 8 : 4;       // channels of a box: 32 registers
+    constexpr int NB = (sizeof(T) == 2 && !DW) ? 8 : 4;       // channels of a box (32 registers of input; a convolution's input
+                                                       // is loaded channel by channel, one ahead)
     constexpr int S = 8 / ((NW < 4) ? NW : 4);         // slots a warp finishes at the end
     constexpr bool MAXV = KIND != P1_NORMS;
     using TT = HaarTile<L>;
     __shared__ float4 token[(NW > 1) ? NW : 1][2][32];          // eight sums per lane, per receiving warp
     __shared__ float fin[(NW > 1) ? NW + 1 : 1][8][32];         // maxima per warp, norms
     __shared__ uint64_t tok_bars[NW];
+    __shared__ __align__(16) float2 tap_sm[DW ? NW : 1][NB * 10];
     pdl_launch();
     const int warp = (NW > 1) ? __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0) : 0, lane = threadIdx.x & 31;
     if ((int)blockIdx.x < weight_ctas) {
@@ -60,8 +64,14 @@ pass1_kernel(const T* __restrict__ x, int C, int H, int W, int weight_ctas, floa
     const PatchOff off = patch_off<T>(lp, W);
     const uint64_t xb = reinterpret_cast<uint64_t>(x) + (uint64_t)n * C * plane;
     const int rounds = (C + NB - 1) / NB;
-    constexpr int D = (NW == 1) ? 2 : 1;               // boxes ahead: a lone warp per tile has registers for two (C4 22.4 against 23.5 us)
-    Raw<T> raw[D][NB];
+    constexpr int D = (NW == 1 && !DW) ? 2 : 1;               // boxes ahead: a lone warp per tile has registers for two (C4 22.4 against 23.5 us)
+    Raw<T> raw[DW ? 1 : D][DW ? 1 : NB];
+    DwIn<T> in[DW ? 2 : 1];
+    DwOff dwo;
+    if constexpr (DW) {
+        dwo = dw_off<T, L, VEC>(lp, H, W, ty, tx);
+        if (warp < rounds) dw_load<T, VEC>(xb + (uint64_t)min(warp * NB, C - 1) * plane, dwo, in[0]);
+    } else
 #pragma unroll
     for (int b = 0; b < D; ++b)
         if (warp + b * NW < rounds) ldg_group<T, VEC, true, true, NB>(xb, plane, off, (warp + b * NW) * NB, C, raw[b]);
@@ -85,11 +95,28 @@ pass1_kernel(const T* __restrict__ x, int C, int H, int W, int weight_ctas, floa
         const int r = rb + b * NW;
         if (r >= rounds) break;
         float o[NB][8];
+        if constexpr (DW) {
+            __syncwarp();                              // the taps of the box before have been read
+            dw_stage_taps(taps, r * NB, NB, C, tap_sm[warp], lane);
+            __syncwarp();
+            float2 ll[NB];
+#pragma unroll
+            for (int d = 0; d < NB; ++d) {
+                const int cn = (d + 1 < NB) ? r * NB + d + 1 : (r + NW) * NB;          // the channel after this one
+                if (d + 1 < NB || r + NW < rounds) dw_load<T, VEC>(xb + (uint64_t)min(cn, C - 1) * plane, dwo, in[(d + 1) & 1]);
+                float2 k[10];
+                dw_read_taps(&tap_sm[warp][d * 10], k);
+                dw_conv<T>(in[d & 1], k, ll[d], o[d]);
+                if (L == 1) { o[d][6] = ll[d].x; o[d][7] = ll[d].y; }
+            }
+            fwd_levels<L, NB>(ll, o, lane);
+        } else {
 #pragma unroll
         for (int g = 0; g < NB; g += 4) fwd_group<T, L, 4>(raw[b] + g, *reinterpret_cast<float(*)[4][8]>(&o[g]), lane);
         if (r + NW * D < rounds) {                     // the words of this box are consumed: the next box goes into their registers
             if ((r + NW * D) * NB + NB <= C) ldg_group<T, VEC, true, false, NB>(xb, plane, off, (r + NW * D) * NB, C, raw[b]);
             else ldg_group<T, VEC, true, true, NB>(xb, plane, off, (r + NW * D) * NB, C, raw[b]);
+        }
         }
         if (r == rounds - 1) {                         // channels beyond the last one repeat it: they count nothing
 #pragma unroll
@@ -218,8 +245,8 @@ pass1_kernel(const T* __restrict__ x, int C, int H, int W, int weight_ctas, floa
 // they are few; four where one warp per tile would leave a long second wave.  us per layer with 1 / 2 / 4 / 8 warps: 512 tiles
 // (144 -> 24 bf16) 47.9 / 37.6 / 34.3 / 37.3; 128 tiles (384 -> 512 bf16) 101 / 73 / 61 / 56; 1024 tiles (32 -> 192 chain)
 // 405 / 377 / 387 / 414; 1440 tiles (C4) 68.7 / 71.4 / 69.8 / 72.7; 2880 tiles 130.0 / 125.8 / 125.1 / 132.5.
-template <typename T, int L, bool VEC, int KIND>
-static wcc_status pass1_launch(const void* x, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
+template <typename T, int L, bool VEC, int KIND, bool DW>
+static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
                                cudaStream_t st)
 {
     using TT = HaarTile<L>;
@@ -234,40 +261,47 @@ static wcc_status pass1_launch(const void* x, int N, int C, int H, int W, float*
     const int nw = tiles > warps ? 4 : tiles * 2 > warps ? 1 : tiles * 4 > warps ? 2 : tiles * 8 > warps ? 4 : 8;
     auto go = [&](auto kern, int w) -> wcc_status {
         const int wctas = ex.Wt ? ceil_div(ex.Cout, w) : 0;
-        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), 0, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), C, H, W,
+        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), 0, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), taps, C, H, W,
                                  wctas, coef, nrm2, amaxpos, ex, status);
     };
-    if (nw == 1) return go(pass1_kernel<T, L, VEC, 1, KIND>, 1);
-    if (nw == 2) return go(pass1_kernel<T, L, VEC, 2, KIND>, 2);
-    if (nw == 4) return go(pass1_kernel<T, L, VEC, 4, KIND>, 4);
-    return go(pass1_kernel<T, L, VEC, 8, KIND>, 8);
+    if constexpr (!DW) {
+        if (nw == 1) return go(pass1_kernel<T, L, VEC, 1, KIND, DW>, 1);
+        if (nw == 2) return go(pass1_kernel<T, L, VEC, 2, KIND, DW>, 2);
+    }
+    if (nw <= 4) return go(pass1_kernel<T, L, VEC, 4, KIND, DW>, 4);
+    return go(pass1_kernel<T, L, VEC, 8, KIND, DW>, 8);
 }
 
 template <typename T, int L, bool VEC>
-static wcc_status pass1_dispatch(const void* x, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
-                                 cudaStream_t st)
+static wcc_status pass1_dispatch(const void* x, const float* taps, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos,
+                                 const NormsExtra& ex, cudaStream_t st)
 {
-    if (coef) return pass1_launch<T, L, VEC, P1_COEF>(x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
-    if (amaxpos) return pass1_launch<T, L, VEC, P1_MAX>(x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
-    return pass1_launch<T, L, VEC, P1_NORMS>(x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    if (taps) {
+        if (coef) return pass1_launch<T, L, VEC, P1_COEF, true>(x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+        return pass1_launch<T, L, VEC, P1_MAX, true>(x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    }
+    if (coef) return pass1_launch<T, L, VEC, P1_COEF, false>(x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    if (amaxpos) return pass1_launch<T, L, VEC, P1_MAX, false>(x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    return pass1_launch<T, L, VEC, P1_NORMS, false>(x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
 }
 
-// First pass of the fused layer.  With ex.hist1 set, launch_clear on the histograms must be the call before it on the stream.
-static wcc_status launch_pass1(const void* x, int N, int C, int H, int W, int L, wcc_dtype dt, float* nrm2, float* amaxpos, const NormsExtra& ex,
-                               cudaStream_t st)
+// First pass of the fused layer; taps: NULL, or a depthwise convolution in front.  With ex.hist1 set, launch_clear on the
+// histograms must be the call before it on the stream.
+static wcc_status launch_pass1(const void* x, const float* taps, int N, int C, int H, int W, int L, wcc_dtype dt, float* nrm2, float* amaxpos,
+                               const NormsExtra& ex, cudaStream_t st)
 {
     const bool vec = (W % 4) == 0;
     float* coef = nullptr;
-    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
 }
 
-// Forward transform with stored coefficients; nrm2 and amaxpos may be NULL.
-wcc_status launch_haar_fwd(const void* x, int N, int C, int H, int W, int L, wcc_dtype dt, float* coef, float* nrm2, float* amaxpos,
-                           cudaStream_t st)
+// Forward transform with stored coefficients, after the depthwise convolution if taps are given; nrm2 and amaxpos may be NULL.
+wcc_status launch_haar_fwd(const void* x, const float* taps, int N, int C, int H, int W, int L, wcc_dtype dt, float* coef, float* nrm2,
+                           float* amaxpos, cudaStream_t st)
 {
     const bool vec = (W % 4) == 0;                     // always true for L >= 2
     const NormsExtra ex = {};
-    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
 }
 
 }  // namespace wcc

@@ -98,35 +98,11 @@ __device__ __forceinline__ void ldg_group(uint64_t xb, size_t plane, const Patch
     }
 }
 
-// Forward transform (sums and differences only, see slot_scales) from the loaded words.  fp32: the first step is scalar, because packing (quad 0, quad 1) pairs out of
-// vector loads would take a register move per word (45 instead of 35 instructions per patch); bf16 words are unpacked
-// anyway, straight into the pairs.
-template <typename T, int L, int U>
-__device__ __forceinline__ void fwd_group(const Raw<T>* raw, float (&o)[U][8], int lane)
+// Levels 2 and 3 of the forward transform: ll holds the level-1 sums of both quads of the lane, slots 6 and 7 come out.
+template <int L, int U>
+__device__ __forceinline__ void fwd_levels(const float2 (&ll)[U], float (&o)[U][8], int lane)
 {
     using TT = HaarTile<L>;
-    float2 ll[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        float2 s0, d0, s1, d1;
-        if constexpr (sizeof(T) == 4) {
-            float a[4], c[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { a[i] = __uint_as_float(raw[u].w[0][i]); c[i] = __uint_as_float(raw[u].w[1][i]); }
-            s0 = make_float2(__fadd_rn(a[0], a[1]), __fadd_rn(a[2], a[3]));
-            d0 = make_float2(__fsub_rn(a[0], a[1]), __fsub_rn(a[2], a[3]));
-            s1 = make_float2(__fadd_rn(c[0], c[1]), __fadd_rn(c[2], c[3]));
-            d1 = make_float2(__fsub_rn(c[0], c[1]), __fsub_rn(c[2], c[3]));
-        } else {
-            const float2 a = make_float2(bf16lo(raw[u].w[0][0]), bf16lo(raw[u].w[0][1])), b = make_float2(bf16hi(raw[u].w[0][0]), bf16hi(raw[u].w[0][1]));
-            const float2 c = make_float2(bf16lo(raw[u].w[1][0]), bf16lo(raw[u].w[1][1])), d = make_float2(bf16hi(raw[u].w[1][0]), bf16hi(raw[u].w[1][1]));
-            s0 = add2(a, b); d0 = diff2(a, b); s1 = add2(c, d); d1 = diff2(c, d);
-        }
-        ll[u] = add2(s0, s1);
-        const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
-        o[u][0] = y2.x; o[u][1] = y2.y; o[u][2] = y3.x; o[u][3] = y3.y; o[u][4] = y4.x; o[u][5] = y4.y;
-        if (L == 1) { o[u][6] = ll[u].x; o[u][7] = ll[u].y; }
-    }
     if (L == 1) return;
     const int rp = lane / TT::CG, cg = lane % TT::CG;
     const bool even = (rp & 1) == 0;
@@ -160,6 +136,37 @@ __device__ __forceinline__ void fwd_group(const Raw<T>* raw, float (&o)[U][8], i
             if (even) o[u][6] = r;
         }
     }
+}
+
+// Forward transform (sums and differences only, see slot_scales) from the loaded words.  fp32: the first step is scalar,
+// because packing (quad 0, quad 1) pairs out of vector loads would take a register move per word (45 instead of 35
+// instructions per patch); bf16 words are unpacked anyway, straight into the pairs.
+template <typename T, int L, int U>
+__device__ __forceinline__ void fwd_group(const Raw<T>* raw, float (&o)[U][8], int lane)
+{
+    float2 ll[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        float2 s0, d0, s1, d1;
+        if constexpr (sizeof(T) == 4) {
+            float a[4], c[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { a[i] = __uint_as_float(raw[u].w[0][i]); c[i] = __uint_as_float(raw[u].w[1][i]); }
+            s0 = make_float2(__fadd_rn(a[0], a[1]), __fadd_rn(a[2], a[3]));
+            d0 = make_float2(__fsub_rn(a[0], a[1]), __fsub_rn(a[2], a[3]));
+            s1 = make_float2(__fadd_rn(c[0], c[1]), __fadd_rn(c[2], c[3]));
+            d1 = make_float2(__fsub_rn(c[0], c[1]), __fsub_rn(c[2], c[3]));
+        } else {
+            const float2 a = make_float2(bf16lo(raw[u].w[0][0]), bf16lo(raw[u].w[0][1])), b = make_float2(bf16hi(raw[u].w[0][0]), bf16hi(raw[u].w[0][1]));
+            const float2 c = make_float2(bf16lo(raw[u].w[1][0]), bf16lo(raw[u].w[1][1])), d = make_float2(bf16hi(raw[u].w[1][0]), bf16hi(raw[u].w[1][1]));
+            s0 = add2(a, b); d0 = diff2(a, b); s1 = add2(c, d); d1 = diff2(c, d);
+        }
+        ll[u] = add2(s0, s1);
+        const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
+        o[u][0] = y2.x; o[u][1] = y2.y; o[u][2] = y3.x; o[u][3] = y3.y; o[u][4] = y4.x; o[u][5] = y4.y;
+        if (L == 1) { o[u][6] = ll[u].x; o[u][7] = ll[u].y; }
+    }
+    fwd_levels<L, U>(ll, o, lane);
 }
 
 // Inverse of slots already multiplied by slot_scales.  fp32: the last step is scalar (the four values of a row leave as one
@@ -245,6 +252,134 @@ __device__ __forceinline__ void store_rows(uint64_t b, const PatchOff& f, bool o
             }
         }
     }
+}
+
+// ---- depthwise 3x3 convolution in front of the transform (stride 1, zero padding 1, cross-correlation) -----------------
+// One channel's input for the lane's patch: rows r0-1 .. r0+2 of columns c0 .. c0+3 (m), the element to the left (bf16: the word
+// that ends with it) and to the right (bf16: the word that starts with it); zeros outside the map.
+template <typename T> struct DwIn { uint32_t m[4][sizeof(T)], l[4], r[4]; };
+
+struct DwOff {
+    uint32_t o[4];            // byte offsets of the rows at column c0
+    uint32_t rows;            // bit a: row a lies in the map
+    bool left, mid0, mid1, right;
+    bool edge;                // the tile touches a border or hangs over it (the same for the whole warp)
+};
+template <typename T, int L, bool VEC>
+__device__ __forceinline__ DwOff dw_off(const LanePos& lp, int H, int W, int ty, int tx)
+{
+    using TT = HaarTile<L>;
+    DwOff f;
+    f.rows = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const int r = lp.r0 + a - 1;
+        f.o[a] = (uint32_t)(((long long)r * W + lp.c0) * (long long)sizeof(T));
+        if (r >= 0 && r < H) f.rows |= 1u << a;
+    }
+    f.left = lp.c0 > 0 && lp.c0 - 1 < W;
+    f.mid0 = lp.ok0;
+    f.mid1 = lp.ok1;
+    f.right = lp.c0 + 4 < W;
+    const int y0 = ty * TT::TH, x0 = tx * TT::TW;
+    f.edge = !VEC || y0 == 0 || y0 + TT::TH >= H || x0 == 0 || x0 + TT::TW >= W;
+    return f;
+}
+
+template <typename T, bool VEC, bool EDGE>
+__device__ __forceinline__ void dw_load_rows(uint64_t b, const DwOff& f, DwIn<T>& in)
+{
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const bool row = !EDGE || ((f.rows >> a) & 1u);
+        const uint64_t p = b + f.o[a];
+        in.l[a] = 0u; in.r[a] = 0u;
+        if (row && (!EDGE || f.left)) in.l[a] = __ldg(reinterpret_cast<const uint32_t*>(p - 4));
+        if (row && (!EDGE || f.right)) in.r[a] = __ldg(reinterpret_cast<const uint32_t*>(p + 4 * sizeof(T)));
+#pragma unroll
+        for (int i = 0; i < (int)sizeof(T); ++i) in.m[a][i] = 0u;
+        if constexpr (VEC) {
+            if (row && (!EDGE || f.mid0)) {
+                if constexpr (sizeof(T) == 4) {
+                    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+                    in.m[a][0] = v.x; in.m[a][1] = v.y; in.m[a][2] = v.z; in.m[a][3] = v.w;
+                } else {
+                    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+                    in.m[a][0] = v.x; in.m[a][1] = v.y;
+                }
+            }
+        } else if constexpr (sizeof(T) == 4) {
+            if (row && f.mid0) { const uint2 v = __ldg(reinterpret_cast<const uint2*>(p)); in.m[a][0] = v.x; in.m[a][1] = v.y; }
+            if (row && f.mid1) { const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + 8)); in.m[a][2] = v.x; in.m[a][3] = v.y; }
+        } else {
+            if (row && f.mid0) in.m[a][0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+            if (row && f.mid1) in.m[a][1] = __ldg(reinterpret_cast<const uint32_t*>(p + 4));
+        }
+    }
+}
+template <typename T, bool VEC>
+__device__ __forceinline__ void dw_load(uint64_t b, const DwOff& f, DwIn<T>& in)
+{
+    if (f.edge) dw_load_rows<T, VEC, true>(b, f, in);
+    else dw_load_rows<T, VEC, false>(b, f, in);
+}
+
+// The convolution at the eight pixels of the patch, in pairs (columns 0 and 2; 1 and 3), and its first transform level: per
+// pixel one fused multiply-add per tap, row-major tap order, from +0.  k: taps, each duplicated.
+template <typename T>
+__device__ __forceinline__ void dw_conv(const DwIn<T>& in, const float2* k, float2& ll, float (&o)[8])
+{
+    float2 e[2], d[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) { e[i] = make_float2(0.0f, 0.0f); d[i] = make_float2(0.0f, 0.0f); }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        float x[6];
+        if constexpr (sizeof(T) == 2) {
+            x[0] = bf16hi(in.l[a]);
+            x[1] = bf16lo(in.m[a][0]); x[2] = bf16hi(in.m[a][0]);
+            x[3] = bf16lo(in.m[a][1]); x[4] = bf16hi(in.m[a][1]);
+            x[5] = bf16lo(in.r[a]);
+        } else {
+            x[0] = __uint_as_float(in.l[a]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[1 + i] = __uint_as_float(in.m[a][i]);
+            x[5] = __uint_as_float(in.r[a]);
+        }
+        const float2 p0 = make_float2(x[0], x[2]), p1 = make_float2(x[1], x[3]), p2 = make_float2(x[2], x[4]), p3 = make_float2(x[3], x[5]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {                  // output row q takes tap row a - q
+            const int i = a - q;
+            if (i < 0 || i > 2) continue;
+            e[q] = __ffma2_rn(k[3 * i], p0, e[q]);
+            d[q] = __ffma2_rn(k[3 * i], p1, d[q]);
+            e[q] = __ffma2_rn(k[3 * i + 1], p1, e[q]);
+            d[q] = __ffma2_rn(k[3 * i + 1], p2, d[q]);
+            e[q] = __ffma2_rn(k[3 * i + 2], p2, e[q]);
+            d[q] = __ffma2_rn(k[3 * i + 2], p3, d[q]);
+        }
+    }
+    const float2 s0 = add2(e[0], d[0]), d0 = diff2(e[0], d[0]), s1 = add2(e[1], d[1]), d1 = diff2(e[1], d[1]);
+    ll = add2(s0, s1);
+    const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
+    o[0] = y2.x; o[1] = y2.y; o[2] = y3.x; o[3] = y3.y; o[4] = y4.x; o[5] = y4.y;
+}
+
+// Taps of n consecutive channels from c0 on (n * 9 floats, clipped at the last channel) into shared memory, duplicated, ten
+// pairs per channel (80 bytes: rows of sixteen-byte pairs of pairs).
+__device__ __forceinline__ void dw_stage_taps(const float* __restrict__ w, int c0, int n, int C, float2* dst, int lane)
+{
+    for (int e = lane; e < n * 9; e += 32) {
+        const int ch = e / 9, t = e - ch * 9;
+        const float v = (c0 + ch < C) ? __ldg(w + (size_t)(c0 + ch) * 9 + t) : 0.0f;
+        dst[ch * 10 + t] = make_float2(v, v);
+    }
+}
+__device__ __forceinline__ void dw_read_taps(const float2* src, float2 (&k)[10])
+{
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) { const float4 v = s4[i]; k[2 * i] = make_float2(v.x, v.y); k[2 * i + 1] = make_float2(v.z, v.w); }
 }
 
 }  // namespace wcc
