@@ -310,6 +310,7 @@ static WideWs carve_wide_ws(void* ws, int N, int Cin, int Cout, int H, int W, in
     return f;
 }
 
+// dwk: NULL, or depthwise 3x3 kernels fp32 [Cin][3][3] applied to x in front of both of its transforms.
 // One cluster per image in the selection (it reads the first pass's histograms), vector loads of whole patches.
 static bool wide_fits(int Cin, int Cout, int H, int W, int bits)
 {
@@ -328,7 +329,7 @@ static bool fused_fits(int N, int Cin, int Cout, int H, int W, int L, int bits)
 
 static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int Cout, int H, int W,
                             int L, int k, int bits, void* y, wcc_dtype dt, void* ws, size_t ws_bytes,
-                            cudaStream_t st, const wcc_taps* taps, const wcc_options* opt)
+                            cudaStream_t st, const wcc_taps* taps, const wcc_options* opt, const float* dwk = nullptr)
 {
     const WideWs f = carve_wide_ws(ws, N, Cin, Cout, H, W, k, bits);
     if (ws_bytes < f.total) return WCC_ERR_WORKSPACE;
@@ -344,7 +345,7 @@ static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int 
     ex.fine = f.fine;
     const int wbits = (opt && opt->weight_bits && bits) ? opt->weight_bits : bits;
     ex.Wt = Wt; ex.Wq = f.Wq; ex.scale_w = f.scale_w; ex.Cout = Cout; ex.kpad = f.kpad; ex.bits = wbits;
-    s = launch_pass1(x, nullptr, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
+    s = launch_pass1(x, dwk, N, Cin, H, W, L, dt, f.nrm2, amaxpos, ex, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(1, st)) != WCC_OK) return s;
     s = launch_select(f.nrm2, N, P, k, f.idx, nullptr, f.rank, amaxpos, true, f.sel, f.sel_bytes, st, true, f.fine, f.thr, true);
@@ -355,7 +356,7 @@ static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int 
     }
     for (int i = 2; i <= 3; ++i)
         if ((s = profile_mark(i, st)) != WCC_OK) return s;
-    s = launch_regather_quant(x, f.rank, f.amax_kept, N, Cin, H, W, L, k, f.kpad, bits, dt, f.Xq, st);
+    s = launch_regather_quant(x, dwk, f.rank, f.amax_kept, N, Cin, H, W, L, k, f.kpad, bits, opt && opt->alpha > 0.0f, dt, f.Xq, st);
     if (s != WCC_OK) return s;
     if ((s = profile_mark(4, st)) != WCC_OK) return s;
     s = launch_contract(f.Xq, f.Wq, M, Cout, f.kpad, bits, f.acc, f.ldc, st);
@@ -627,7 +628,8 @@ static BlockWs carve_block_ws(void* ws, int N, int C, int E, int H, int W, int L
     BlockWs b = {};
     const size_t es = (dt == WCC_BF16) ? 2 : 4;
     const size_t w1 = wcc_workspace_bytes(N, C, E, H, W, L, k, bits, dt);
-    const size_t w3 = wcc_staged_workspace_bytes(N, E, C, H, W, L, k, bits, dt);
+    const size_t w3 = wide_fits(E, C, H, W, bits) ? carve_wide_ws(nullptr, N, E, C, H, W, k, bits).total
+                                                  : wcc_staged_workspace_bytes(N, E, C, H, W, L, k, bits, dt);
     if (w1 == 0 || w3 == 0) return b;
     char* base = static_cast<char*>(ws);
     size_t off = 0;
@@ -806,9 +808,13 @@ wcc_status wcc_block_forward(const void* x, const float* W1, const float* Wdw, c
     // u = WCC(W1, x): C -> E channels
     s = forward_impl(x, W1, N, C, E, H, Wd, levels, k, bits, b.u, dt, b.layer_ws, b.layer_ws_bytes, st, nullptr);
     if (s != WCC_OK) return s;
-    // y = x + WCC(W3, dw3x3(u)): the depthwise convolution is fused with the second layer's transform
+    // y = x + WCC(W3, dw3x3(u)): the depthwise convolution is fused with the second layer's transform.  Convolving and
+    // transforming u again for the kept columns is cheaper than keeping the coefficients (4 bytes each, written once, gathered
+    // over nearly all of their sectors).
     wcc_options o = {};
     o.residual = x;
+    if (wide_fits(E, C, H, Wd, bits))
+        return wide_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, b.layer_ws_bytes, st, nullptr, &o, Wdw);
     return staged_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, b.layer_ws_bytes, st, nullptr, &o, Wdw);
 }
 

@@ -48,7 +48,9 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
     __shared__ float4 token[(NW > 1) ? NW : 1][2][32];          // eight sums per lane, per receiving warp
     __shared__ float fin[(NW > 1) ? NW + 1 : 1][8][32];         // maxima per warp, norms
     __shared__ uint64_t tok_bars[NW];
-    __shared__ __align__(16) float2 tap_sm[DW ? NW : 1][NB * 10];
+    using Dw = DwTile<T, L, VEC>;
+    __shared__ __align__(16) float2 tap_sm[DW ? NW : 1][2][NB * 10];
+    extern __shared__ __align__(16) uint8_t dw_sm[];            // DW: [NW][Dw::BYTES]
     pdl_launch();
     const int warp = (NW > 1) ? __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0) : 0, lane = threadIdx.x & 31;
     if ((int)blockIdx.x < weight_ctas) {
@@ -66,11 +68,22 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
     const int rounds = (C + NB - 1) / NB;
     constexpr int D = (NW == 1 && !DW) ? 2 : 1;               // boxes ahead: a lone warp per tile has registers for two (C4 22.4 against 23.5 us)
     Raw<T> raw[DW ? 1 : D][DW ? 1 : NB];
-    DwIn<T> in[DW ? 2 : 1];
-    DwOff dwo;
+    uint32_t piece[DW ? Dw::CHS : 1][DW ? Dw::IT : 1][DW ? Dw::PW : 1];
+    Dw dw;
+    float tapv[2] = {0.0f, 0.0f};
+    auto fetch_taps = [&](int r) {                     // this lane's two of the 36 taps of box r
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int e = lane + 32 * i, g = r * NB * 9 + e;
+            tapv[i] = (e < NB * 9 && g < C * 9) ? __ldg(taps + g) : 0.0f;
+        }
+    };
     if constexpr (DW) {
-        dwo = dw_off<T, L, VEC>(lp, H, W, ty, tx);
-        if (warp < rounds) dw_load<T, VEC>(xb + (uint64_t)min(warp * NB, C - 1) * plane, dwo, in[0]);
+        dw.init(dw_sm + warp * Dw::BYTES, H, W, ty, tx, lane);
+        if (warp < rounds) {
+            dw.load(xb, plane, warp * NB, C, piece);
+            fetch_taps(warp);
+        }
     } else
 #pragma unroll
     for (int b = 0; b < D; ++b)
@@ -96,18 +109,27 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
         if (r >= rounds) break;
         float o[NB][8];
         if constexpr (DW) {
-            __syncwarp();                              // the taps of the box before have been read
-            dw_stage_taps(taps, r * NB, NB, C, tap_sm[warp], lane);
-            __syncwarp();
             float2 ll[NB];
+            float2* tp = tap_sm[warp][((r - warp) / NW) & 1];
 #pragma unroll
-            for (int d = 0; d < NB; ++d) {
-                const int cn = (d + 1 < NB) ? r * NB + d + 1 : (r + NW) * NB;          // the channel after this one
-                if (d + 1 < NB || r + NW < rounds) dw_load<T, VEC>(xb + (uint64_t)min(cn, C - 1) * plane, dwo, in[(d + 1) & 1]);
-                float2 k[10];
-                dw_read_taps(&tap_sm[warp][d * 10], k);
-                dw_conv<T>(in[d & 1], k, ll[d], o[d]);
-                if (L == 1) { o[d][6] = ll[d].x; o[d][7] = ll[d].y; }
+            for (int i = 0; i < 2; ++i) {
+                const int e = lane + 32 * i;
+                if (e < NB * 9) tp[(e / 9) * 10 + e % 9] = make_float2(tapv[i], tapv[i]);
+            }
+            if (r + NW < rounds) fetch_taps(r + NW);
+#pragma unroll
+            for (int st = 0; st < NB / Dw::CHS; ++st) {
+                dw.store(st & 1, piece);
+                __syncwarp();
+                const int cn = (st + 1 < NB / Dw::CHS) ? r * NB + (st + 1) * Dw::CHS : (r + NW) * NB;      // the channels after these
+                if (st + 1 < NB / Dw::CHS || r + NW < rounds) dw.load(xb, plane, cn, C, piece);
+#pragma unroll
+                for (int ch = 0; ch < Dw::CHS; ++ch) {
+                    const int d = st * Dw::CHS + ch;
+                    float2 k[10];
+                    dw_read_taps(tp + d * 10, k);
+                    dw.conv(st & 1, ch, k, ll[d], o[d]);
+                }
             }
             fwd_levels<L, NB>(ll, o, lane);
         } else {
@@ -261,7 +283,9 @@ static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, i
     const int nw = tiles > warps ? 4 : tiles * 2 > warps ? 1 : tiles * 4 > warps ? 2 : tiles * 8 > warps ? 4 : 8;
     auto go = [&](auto kern, int w) -> wcc_status {
         const int wctas = ex.Wt ? ceil_div(ex.Cout, w) : 0;
-        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), 0, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), taps, C, H, W,
+        const size_t smem = DW ? (size_t)w * DwTile<T, L, VEC>::BYTES : 0;
+        if (DW) WCC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), smem, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), taps, C, H, W,
                                  wctas, coef, nrm2, amaxpos, ex, status);
     };
     if constexpr (!DW) {

@@ -255,115 +255,132 @@ __device__ __forceinline__ void store_rows(uint64_t b, const PatchOff& f, bool o
 }
 
 // ---- depthwise 3x3 convolution in front of the transform (stride 1, zero padding 1, cross-correlation) -----------------
-// One channel's input for the lane's patch: rows r0-1 .. r0+2 of columns c0 .. c0+3 (m), the element to the left (bf16: the word
-// that ends with it) and to the right (bf16: the word that starts with it); zeros outside the map.
-template <typename T> struct DwIn { uint32_t m[4][sizeof(T)], l[4], r[4]; };
-
-struct DwOff {
-    uint32_t o[4];            // byte offsets of the rows at column c0
-    uint32_t rows;            // bit a: row a lies in the map
-    bool left, mid0, mid1, right;
-    bool edge;                // the tile touches a border or hangs over it (the same for the whole warp)
-};
+// A warp tile with a border of one row and one piece, staged through shared memory by the warp that uses it: a lane needs a
+// 4 x 6 neighbourhood of its patch, and out of global memory that was twelve loads with as many 64-bit addresses, their border
+// tests or masks on top (202 to 262 instructions per patch); here a lane moves four or five pieces of four elements per
+// channel (zeros outside the map) and then reads at constant offsets (181 per patch).  Bound by the shared-memory pipe (70 %
+// of its wavefronts) and issue: 1024 channels of 4 x 128 x 128 bf16 convolved, transformed and normed in 96 us.
 template <typename T, int L, bool VEC>
-__device__ __forceinline__ DwOff dw_off(const LanePos& lp, int H, int W, int ty, int tx)
-{
+struct DwTile {
     using TT = HaarTile<L>;
-    DwOff f;
-    f.rows = 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int r = lp.r0 + a - 1;
-        f.o[a] = (uint32_t)(((long long)r * W + lp.c0) * (long long)sizeof(T));
-        if (r >= 0 && r < H) f.rows |= 1u << a;
-    }
-    f.left = lp.c0 > 0 && lp.c0 - 1 < W;
-    f.mid0 = lp.ok0;
-    f.mid1 = lp.ok1;
-    f.right = lp.c0 + 4 < W;
-    const int y0 = ty * TT::TH, x0 = tx * TT::TW;
-    f.edge = !VEC || y0 == 0 || y0 + TT::TH >= H || x0 == 0 || x0 + TT::TW >= W;
-    return f;
-}
+    static constexpr int ES = (int)sizeof(T);
+    static constexpr int PE = VEC ? 4 : 2;             // elements of a piece (rows of 4m + 2 elements: two)
+    static constexpr int PW = PE * ES / 4;             // its words
+    static constexpr int PR = TT::TW / PE + 2, ROWS = TT::TH + 2, PIECES = PR * ROWS, IT = (PIECES + 31) / 32;
+    // bf16, L = 3: two rows of lanes read in one go; this pitch keeps their banks apart
+    static constexpr int PITCH = (L == 3 && ES == 2) ? 96 : (TT::TW + 8) * ES;
+    static constexpr int CH_BYTES = ROWS * PITCH + 16; // (sixteen bytes take what the last, partial round of pieces writes)
+    static constexpr int CHS = 2;                      // channels per stage
+    static constexpr int BYTES = 2 * CHS * CH_BYTES;   // two stages
 
-template <typename T, bool VEC, bool EDGE>
-__device__ __forceinline__ void dw_load_rows(uint64_t b, const DwOff& f, DwIn<T>& in)
-{
+    uint32_t off[IT], dst[IT], valid;
+    bool edge;                                         // some piece lies outside the map
+    const uint8_t* rd;                                 // this lane's patch in stage 0: row -1, column 0
+    uint8_t* wr;
+
+    __device__ __forceinline__ void init(uint8_t* sm, int H, int W, int ty, int tx, int lane)
+    {
+        valid = 0u;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const bool row = !EDGE || ((f.rows >> a) & 1u);
-        const uint64_t p = b + f.o[a];
-        in.l[a] = 0u; in.r[a] = 0u;
-        if (row && (!EDGE || f.left)) in.l[a] = __ldg(reinterpret_cast<const uint32_t*>(p - 4));
-        if (row && (!EDGE || f.right)) in.r[a] = __ldg(reinterpret_cast<const uint32_t*>(p + 4 * sizeof(T)));
+        for (int it = 0; it < IT; ++it) {
+            const int i = lane + 32 * it, row = i / PR, col = i - row * PR;
+            const int gr = ty * TT::TH + row - 1, gc = tx * TT::TW + (col - 1) * PE;
+            const bool ok = i < PIECES && gr >= 0 && gr < H && gc >= 0 && gc < W;
+            off[it] = ok ? (uint32_t)(((long long)gr * W + gc) * ES) : 0u;
+            dst[it] = i < PIECES ? (uint32_t)(row * PITCH + (4 + (col - 1) * PE) * ES) : (uint32_t)(ROWS * PITCH);
+            valid |= ok ? 1u << it : 0u;
+        }
+        edge = !__all_sync(0xFFFFFFFFu, valid == (1u << IT) - 1u);
+        const int rp = lane / TT::CG, cg = lane % TT::CG;
+        rd = sm + 2 * rp * PITCH + (4 + 4 * cg) * ES;
+        wr = sm;
+    }
+    // channels [c, c + CHS), clipped at the last one
+    __device__ __forceinline__ void load(uint64_t xb, size_t plane, int c, int C, uint32_t (&w)[CHS][IT][PW]) const
+    {
 #pragma unroll
-        for (int i = 0; i < (int)sizeof(T); ++i) in.m[a][i] = 0u;
-        if constexpr (VEC) {
-            if (row && (!EDGE || f.mid0)) {
-                if constexpr (sizeof(T) == 4) {
+        for (int ch = 0; ch < CHS; ++ch) {
+            const uint64_t b = xb + (uint64_t)min(c + ch, C - 1) * plane;
+#pragma unroll
+            for (int it = 0; it < IT; ++it) {
+                const uint64_t p = b + off[it];
+                if constexpr (PW == 4) {
                     const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-                    in.m[a][0] = v.x; in.m[a][1] = v.y; in.m[a][2] = v.z; in.m[a][3] = v.w;
-                } else {
+                    w[ch][it][0] = v.x; w[ch][it][1] = v.y; w[ch][it][2] = v.z; w[ch][it][3] = v.w;
+                } else if constexpr (PW == 2) {
                     const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-                    in.m[a][0] = v.x; in.m[a][1] = v.y;
+                    w[ch][it][0] = v.x; w[ch][it][1] = v.y;
+                } else {
+                    w[ch][it][0] = __ldg(reinterpret_cast<const uint32_t*>(p));
                 }
             }
-        } else if constexpr (sizeof(T) == 4) {
-            if (row && f.mid0) { const uint2 v = __ldg(reinterpret_cast<const uint2*>(p)); in.m[a][0] = v.x; in.m[a][1] = v.y; }
-            if (row && f.mid1) { const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + 8)); in.m[a][2] = v.x; in.m[a][3] = v.y; }
-        } else {
-            if (row && f.mid0) in.m[a][0] = __ldg(reinterpret_cast<const uint32_t*>(p));
-            if (row && f.mid1) in.m[a][1] = __ldg(reinterpret_cast<const uint32_t*>(p + 4));
         }
     }
-}
-template <typename T, bool VEC>
-__device__ __forceinline__ void dw_load(uint64_t b, const DwOff& f, DwIn<T>& in)
-{
-    if (f.edge) dw_load_rows<T, VEC, true>(b, f, in);
-    else dw_load_rows<T, VEC, false>(b, f, in);
-}
-
-// The convolution at the eight pixels of the patch, in pairs (columns 0 and 2; 1 and 3), and its first transform level: per
-// pixel one fused multiply-add per tap, row-major tap order, from +0.  k: taps, each duplicated.
-template <typename T>
-__device__ __forceinline__ void dw_conv(const DwIn<T>& in, const float2* k, float2& ll, float (&o)[8])
-{
-    float2 e[2], d[2];
+    // A __syncwarp has to follow before the stage is read; one between two uses of a stage is enough for its reuse.
+    __device__ __forceinline__ void store(int stage, uint32_t (&w)[CHS][IT][PW]) const
+    {
+        if (edge) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) { e[i] = make_float2(0.0f, 0.0f); d[i] = make_float2(0.0f, 0.0f); }
+            for (int it = 0; it < IT; ++it) {
+                const uint32_t m = ((valid >> it) & 1u) ? 0xFFFFFFFFu : 0u;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        float x[6];
-        if constexpr (sizeof(T) == 2) {
-            x[0] = bf16hi(in.l[a]);
-            x[1] = bf16lo(in.m[a][0]); x[2] = bf16hi(in.m[a][0]);
-            x[3] = bf16lo(in.m[a][1]); x[4] = bf16hi(in.m[a][1]);
-            x[5] = bf16lo(in.r[a]);
-        } else {
-            x[0] = __uint_as_float(in.l[a]);
+                for (int ch = 0; ch < CHS; ++ch)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[1 + i] = __uint_as_float(in.m[a][i]);
-            x[5] = __uint_as_float(in.r[a]);
+                    for (int i = 0; i < PW; ++i) w[ch][it][i] &= m;
+            }
         }
-        const float2 p0 = make_float2(x[0], x[2]), p1 = make_float2(x[1], x[3]), p2 = make_float2(x[2], x[4]), p3 = make_float2(x[3], x[5]);
+        uint8_t* sp = wr + stage * (CHS * CH_BYTES);
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {                  // output row q takes tap row a - q
-            const int i = a - q;
-            if (i < 0 || i > 2) continue;
-            e[q] = __ffma2_rn(k[3 * i], p0, e[q]);
-            d[q] = __ffma2_rn(k[3 * i], p1, d[q]);
-            e[q] = __ffma2_rn(k[3 * i + 1], p1, e[q]);
-            d[q] = __ffma2_rn(k[3 * i + 1], p2, d[q]);
-            e[q] = __ffma2_rn(k[3 * i + 2], p2, e[q]);
-            d[q] = __ffma2_rn(k[3 * i + 2], p3, d[q]);
-        }
+        for (int ch = 0; ch < CHS; ++ch)
+#pragma unroll
+            for (int it = 0; it < IT; ++it) {
+                uint8_t* d = sp + ch * CH_BYTES + dst[it];
+                if constexpr (PW == 4) *reinterpret_cast<uint4*>(d) = make_uint4(w[ch][it][0], w[ch][it][1], w[ch][it][2], w[ch][it][3]);
+                else if constexpr (PW == 2) *reinterpret_cast<uint2*>(d) = make_uint2(w[ch][it][0], w[ch][it][1]);
+                else *reinterpret_cast<uint32_t*>(d) = w[ch][it][0];
+            }
     }
-    const float2 s0 = add2(e[0], d[0]), d0 = diff2(e[0], d[0]), s1 = add2(e[1], d[1]), d1 = diff2(e[1], d[1]);
-    ll = add2(s0, s1);
-    const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
-    o[0] = y2.x; o[1] = y2.y; o[2] = y3.x; o[3] = y3.y; o[4] = y4.x; o[5] = y4.y;
-}
+    // The convolution at the eight pixels of the patch, in pairs (columns 0 and 2; 1 and 3), and its first transform level: per
+    // pixel one fused multiply-add per tap, row-major tap order, from +0 (taps outside the map meet zeros).  k: taps, duplicated.
+    __device__ __forceinline__ void conv(int stage, int ch, const float2* k, float2& ll, float (&o)[8]) const
+    {
+        const uint8_t* p = rd + stage * (CHS * CH_BYTES) + ch * CH_BYTES;
+        float2 e[2], d[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) { e[i] = make_float2(0.0f, 0.0f); d[i] = make_float2(0.0f, 0.0f); }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            float x[6];
+            const uint32_t lw = *reinterpret_cast<const uint32_t*>(p + a * PITCH - 4), rw = *reinterpret_cast<const uint32_t*>(p + a * PITCH + 4 * ES);
+            if constexpr (ES == 2) {
+                const uint2 m = *reinterpret_cast<const uint2*>(p + a * PITCH);
+                x[0] = bf16hi(lw);
+                x[1] = bf16lo(m.x); x[2] = bf16hi(m.x); x[3] = bf16lo(m.y); x[4] = bf16hi(m.y);
+                x[5] = bf16lo(rw);
+            } else {
+                const float4 m = *reinterpret_cast<const float4*>(p + a * PITCH);
+                x[0] = __uint_as_float(lw); x[1] = m.x; x[2] = m.y; x[3] = m.z; x[4] = m.w; x[5] = __uint_as_float(rw);
+            }
+            const float2 p0 = make_float2(x[0], x[2]), p1 = make_float2(x[1], x[3]), p2 = make_float2(x[2], x[4]), p3 = make_float2(x[3], x[5]);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {              // output row q takes tap row a - q
+                const int i = a - q;
+                if (i < 0 || i > 2) continue;
+                e[q] = __ffma2_rn(k[3 * i], p0, e[q]);
+                d[q] = __ffma2_rn(k[3 * i], p1, d[q]);
+                e[q] = __ffma2_rn(k[3 * i + 1], p1, e[q]);
+                d[q] = __ffma2_rn(k[3 * i + 1], p2, d[q]);
+                e[q] = __ffma2_rn(k[3 * i + 2], p2, e[q]);
+                d[q] = __ffma2_rn(k[3 * i + 2], p3, d[q]);
+            }
+        }
+        const float2 s0 = add2(e[0], d[0]), d0 = diff2(e[0], d[0]), s1 = add2(e[1], d[1]), d1 = diff2(e[1], d[1]);
+        ll = add2(s0, s1);
+        const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
+        o[0] = y2.x; o[1] = y2.y; o[2] = y3.x; o[3] = y3.y; o[4] = y4.x; o[5] = y4.y;
+        if (L == 1) { o[6] = ll.x; o[7] = ll.y; }
+    }
+};
 
 // Taps of n consecutive channels from c0 on (n * 9 floats, clipped at the last channel) into shared memory, duplicated, ten
 // pairs per channel (80 bytes: rows of sixteen-byte pairs of pairs).
