@@ -27,7 +27,7 @@ if ROOT not in sys.path:
 METRIC = "WCC layer output Gpix/s"
 UNIT = "Gpix/s"
 FLUSH_BYTES = 256 << 20          # > 126 MB of L2
-STAGE_FILES = ("haar.cuh", "pass1.cuh", "select.cuh", "gather.cuh", "regather.cuh", "contract.cuh", "patch.cuh", "pass2.cuh", "tma.cuh",
+STAGE_FILES = ("haar.cuh", "pass1.cuh", "select.cuh", "gather.cuh", "regather.cuh", "scatter.cuh", "contract.cuh", "patch.cuh", "pass2.cuh", "tma.cuh",
                "libwcc.cu", "common.cuh")
 
 # DRAM bytes per launch of the dominant kernel from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum),

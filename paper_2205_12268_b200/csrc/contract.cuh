@@ -111,6 +111,8 @@ contract_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     bool failed = false;
+    pdl_wait();                                          // set up; the operands come from the kernels before
+    pdl_launch();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -270,12 +272,8 @@ wcc_status launch_contract(const void* Xq, const void* Wq, int M, int Cout, int 
     WCC_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&status), g_status));
     const long long items = (long long)ceil_div(M, TILE_M) * ceil_div(npad, TILE_N);
     const int grid = (int)(items < sm_count[dev] ? items : sm_count[dev]);
-    if (i8)
-        contract_kernel<true><<<grid, 192, smem, st>>>(tmA, tmB, M, npad, krow_bytes, acc, ldc, status);
-    else
-        contract_kernel<false><<<grid, 192, smem, st>>>(tmA, tmB, M, npad, krow_bytes, acc, ldc, status);
-    WCC_LAUNCH_CHECK();
-    return WCC_OK;
+    return launch_overlapped(i8 ? contract_kernel<true> : contract_kernel<false>, dim3((unsigned)grid), dim3(192), smem, st, true, 1, tmA, tmB, M, npad,
+                             krow_bytes, acc, ldc, status);
 }
 
 }  // namespace wcc

@@ -1,5 +1,5 @@
-// Haar kernels: channel norms of a stored map, plain inverse, and the fused dequantize + scatter + inverse (steps B-norms, D, E
-// of the WCC workflow; Eq. 3-6, Alg. 1).  The forward transform of a feature map is in pass1.cuh.
+// Haar kernels: channel norms of a stored map and the plain inverse (Eq. 3-6, Alg. 1), and the tile geometry all transforms share.
+// The forward transform of a feature map is in pass1.cuh, dequantize + scatter + inverse in scatter.cuh.
 //
 // Work decomposition (all three kernels).  One warp owns a tile of 2^L rows x TW columns of one image,
 // TW = 4 * CG, CG = 32 / 2^(L-1).  Lane (rp, cg) = (lane / CG, lane % CG) holds the 2 x 4 patch at rows
@@ -209,60 +209,6 @@ __device__ __forceinline__ void slot_scales(int lane, bool swapped, float (&sc)[
     }
 }
 
-// Inverse on slots that the caller has already multiplied by slot_scales (not swapped): sums and differences only.
-template <int L, int U>
-__device__ __forceinline__ void haar_inv_lanes_raw(const float (&o)[U][8], float (&p)[U][2][4], int lane)
-{
-    using T = HaarTile<L>;
-    float2 ll[U];
-    if (L == 1) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) ll[u] = make_float2(o[u][6], o[u][7]);
-    } else {
-        const int rp = lane / T::CG, cg = lane % T::CG;
-        const float sg = (rp & 1) == 0 ? 1.0f : -1.0f;
-        float m0[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) m0[u] = o[u][6];
-        if (L == 3) {
-            const float sgh = (cg & 1) == 0 ? 1.0f : -1.0f;
-            const float sgv = (rp & 2) == 0 ? 1.0f : -1.0f;
-            float pv[U], w[U], q[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) pv[u] = __shfl_xor_sync(0xFFFFFFFFu, m0[u], 2 * T::CG);
-#pragma unroll
-            for (int u = 0; u < U; ++u) w[u] = __fmaf_rn(m0[u], sgv, pv[u]);
-#pragma unroll
-            for (int u = 0; u < U; ++u) q[u] = __shfl_xor_sync(0xFFFFFFFFu, w[u], 1);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const float r = __fmaf_rn(w[u], sgh, q[u]);
-                if ((rp & 1) == 0) m0[u] = r;
-            }
-        }
-        float p0[U], p1[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            p0[u] = __shfl_xor_sync(0xFFFFFFFFu, m0[u], T::CG);
-            p1[u] = __shfl_xor_sync(0xFFFFFFFFu, o[u][7], T::CG);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const float2 tu = __ffma2_rn(make_float2(m0[u], o[u][7]), make_float2(sg, sg), make_float2(p0[u], p1[u]));
-            ll[u] = make_float2(__fadd_rn(tu.x, tu.y), __fsub_rn(tu.x, tu.y));
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const float2 y2 = make_float2(o[u][0], o[u][1]), y3 = make_float2(o[u][2], o[u][3]), y4 = make_float2(o[u][4], o[u][5]);
-        const float2 t0 = add2(ll[u], y3), t1 = sub2(ll[u], y3), u0 = add2(y2, y4), u1 = sub2(y2, y4);
-        const float2 a = add2(t0, u0), b = sub2(t0, u0);
-        const float2 c = add2(t1, u1), d = sub2(t1, u1);
-        p[u][0][0] = a.x; p[u][0][1] = b.x; p[u][0][2] = a.y; p[u][0][3] = b.y;
-        p[u][1][0] = c.x; p[u][1][1] = d.x; p[u][1][2] = c.y; p[u][1][3] = d.y;
-    }
-}
-
 // ---- patch load / store ------------------------------------------------------------------------
 struct RawPatch { uint32_t w[8]; };   // fp32: 2 rows x 4 words; bf16: 2 rows x 2 words (w[0..1], w[4..5])
 
@@ -456,102 +402,6 @@ haar_inv_kernel(const float* __restrict__ coef, int planes, int H, int W, T* __r
     store_patch<T, VEC>(out + (size_t)pl * P, W, lp, p);
 }
 
-// ---- fused dequantize + scatter + inverse ----------------------------------------------------
-// One warp per (image, tile, group of ocw output channels; ocw a multiple of 4).  rank[n][p] is the row of position p
-// in the compressed matrix (or -1 when p was dropped: the zero map).  acc row r = n*k + rank holds the int32
-// accumulators (or fp32 products when ACCF) of all output channels, pitch ldc (multiple of 4).  The accumulators of
-// the next four channels are gathered while the current four are transformed.
-template <typename T, int L, bool VEC, bool ACCF>
-__global__ void __launch_bounds__(128, 5)
-scatter_inv_kernel(const int32_t* __restrict__ acc, int ldc, const int32_t* __restrict__ rank,
-                   const float* __restrict__ amax_kept, float qmax, const float* __restrict__ scale_w,
-                   int N, int Cout, int ocw, int H, int W, int k, T* __restrict__ y, const T* __restrict__ residual, int relu)
-{
-    using TT = HaarTile<L>;
-    const int tiles_x = (W + TT::TW - 1) / TT::TW, tiles_y = H / TT::TH;
-    const int groups = (Cout + ocw - 1) / ocw;
-    const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (gw >= (long long)N * tiles_x * tiles_y * groups) return;
-    const int lane = threadIdx.x & 31;
-    const int g = (int)(gw % groups);
-    int n, ty, tx;
-    tile_coords((int)(gw / groups), tiles_x, tiles_y, n, ty, tx);
-    const LanePos lp = lane_positions<L>(H, W, ty, tx, lane);
-    const size_t P = (size_t)H * W;
-
-    const int32_t* rk = rank + (size_t)n * P;
-    const int32_t* rowp[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-        int r = -1;
-        if (slot_ok<L>(lp, s)) r = rk[lp.pos[s]];
-        rowp[s] = (r >= 0) ? acc + ((size_t)n * k + r) * ldc : nullptr;
-    }
-    float scale_a = 1.0f;
-    if (!ACCF) scale_a = __fdiv_rn(*amax_kept, qmax);
-
-    // Four channels at a time: dequantize straight into the pre-scaled slots of haar_inv_lanes_raw, acc * (scale * 2^-level)
-    // (the halvings of the inverse transform are exact powers of two and commute with every rounding).
-    const bool coarse6 = L == 3 && ((lane / TT::CG) & 1) == 0;         // slot 6 holds a level-3 coefficient
-    const int o_end = min(Cout, (g + 1) * ocw);
-    int4 v[8], vn[8];
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-        v[s] = rowp[s] ? __ldg(reinterpret_cast<const int4*>(rowp[s] + g * ocw)) : make_int4(0, 0, 0, 0);
-        vn[s] = v[s];
-    }
-    for (int o0 = g * ocw; o0 < o_end; o0 += 4) {
-        if (o0 + 4 < o_end) {
-#pragma unroll
-            for (int s = 0; s < 8; ++s)
-                vn[s] = rowp[s] ? __ldg(reinterpret_cast<const int4*>(rowp[s] + o0 + 4)) : make_int4(0, 0, 0, 0);
-        }
-        float sl[4][8], p[4][2][4];
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-            const int o = o0 + d;
-            float sc = 1.0f;
-            if (!ACCF) sc = (o < o_end) ? __fmul_rn(scale_a, scale_w[o]) : 0.0f;
-            const float s1 = __fmul_rn(sc, 0.5f), s2 = __fmul_rn(sc, 0.25f);
-            const float s6 = (L == 1) ? s1 : (coarse6 ? __fmul_rn(sc, 0.125f) : s2), s7 = (L == 1) ? s1 : s2;
-#pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                const int a = (d == 0) ? v[s].x : (d == 1) ? v[s].y : (d == 2) ? v[s].z : v[s].w;
-                const float f = ACCF ? __int_as_float(a) : __int2float_rn(a);
-                sl[d][s] = __fmul_rn(f, s < 6 ? s1 : (s == 6 ? s6 : s7));
-            }
-        }
-        haar_inv_lanes_raw<L, 4>(sl, p, lane);
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-            const int o = o0 + d;
-            if (o < o_end) {      // warp-uniform
-                if (residual) {                        // the skip connection (Eq. 13): one fp32 addition per element
-                    RawPatch rr;
-                    float rp[2][4];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) rr.w[i] = 0u;
-                    load_patch<T, VEC>(residual + ((size_t)n * Cout + o) * P, W, lp, rr);
-                    unpack_patch<T>(rr, rp);
-#pragma unroll
-                    for (int a = 0; a < 2; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) p[d][a][b] = __fadd_rn(p[d][a][b], rp[a][b]);
-                }
-                if (relu) {
-#pragma unroll
-                    for (int a = 0; a < 2; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) p[d][a][b] = fmaxf(p[d][a][b], 0.0f);
-                }
-                store_patch<T, VEC>(y + ((size_t)n * Cout + o) * P, W, lp, p[d]);
-            }
-        }
-#pragma unroll
-        for (int s = 0; s < 8; ++s) v[s] = vn[s];
-    }
-}
-
 // ---- launchers -------------------------------------------------------------------------------
 #define WCC_DISPATCH_TLV(FN, dt, L, vec, ...)                                                        \
     do {                                                                                             \
@@ -582,42 +432,6 @@ wcc_status launch_haar_inv(const float* coef, int N, int C, int H, int W, int L,
 {
     const bool vec = (W % 4) == 0;
     WCC_DISPATCH_TLV(haar_inv_dispatch, dt, L, vec, coef, N * C, H, W, out, st);
-}
-
-template <typename T, int L, bool VEC>
-static wcc_status scatter_inv_dispatch(const int32_t* acc, int ldc, bool accf, const int32_t* rank,
-                                       const float* amax_kept, float qmax, const float* scale_w,
-                                       int N, int Cout, int H, int W, int k, void* y, const void* residual, int relu,
-                                       cudaStream_t st)
-{
-    using TT = HaarTile<L>;
-    // channels per warp: as many as still leave about 32 warps for each of the 148 SMs (8 to 64)
-    const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
-    int ocw = 64;
-    while (ocw > 8 && tiles * ceil_div(Cout, ocw) < 148 * 32) ocw >>= 1;
-    const long long warps = tiles * ceil_div(Cout, ocw);
-    const int blocks = (int)((warps + 3) / 4);
-    if (accf)
-        scatter_inv_kernel<T, L, VEC, true><<<blocks, 128, 0, st>>>(acc, ldc, rank, amax_kept, qmax, scale_w,
-                                                                     N, Cout, ocw, H, W, k, static_cast<T*>(y),
-                                                                     static_cast<const T*>(residual), relu);
-    else
-        scatter_inv_kernel<T, L, VEC, false><<<blocks, 128, 0, st>>>(acc, ldc, rank, amax_kept, qmax, scale_w,
-                                                                      N, Cout, ocw, H, W, k, static_cast<T*>(y),
-                                                                      static_cast<const T*>(residual), relu);
-    WCC_LAUNCH_CHECK();
-    return WCC_OK;
-}
-
-wcc_status launch_scatter_inv(const int32_t* acc, int ldc, bool acc_is_float, const int32_t* rank,
-                              const float* amax_kept, int bits, const float* scale_w,
-                              int N, int Cout, int H, int W, int L, int k, wcc_dtype dt, void* y, cudaStream_t st,
-                              const void* residual, int relu)
-{
-    const bool vec = (W % 4) == 0;
-    const float qmax = (bits >= 2) ? (float)((1 << (bits - 1)) - 1) : 1.0f;
-    WCC_DISPATCH_TLV(scatter_inv_dispatch, dt, L, vec, acc, ldc, acc_is_float, rank, amax_kept, qmax, scale_w,
-                     N, Cout, H, W, k, y, residual, relu, st);
 }
 
 }  // namespace wcc

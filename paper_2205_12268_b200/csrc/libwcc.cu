@@ -6,6 +6,7 @@
 #include "haar.cuh"
 #include "pass1.cuh"
 #include "regather.cuh"
+#include "scatter.cuh"
 #include "select.cuh"
 #include "contract.cuh"
 #include "pass2.cuh"

@@ -64,14 +64,6 @@ __device__ __forceinline__ void tmem_ld4_nowait(uint32_t taddr, uint32_t (&r)[4]
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
 }
 
-__device__ __forceinline__ void relu_patch(float (&p)[2][4])
-{
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) p[a][b] = fmaxf(p[a][b], 0.0f);
-}
-
 // MODE is a set of compiled-in features: 1 = ReLU on the way out, 2 = taps for tests, 4 = a given clipping parameter (codes
 // are clamped), 8 = residual add.  A compiled-in feature is still switched by its run-time argument; a feature that is not
 // compiled in costs nothing (as run-time branches in one kernel the options cost the plain layer 7-18 %).

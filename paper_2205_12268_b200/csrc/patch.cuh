@@ -254,6 +254,14 @@ __device__ __forceinline__ void store_rows(uint64_t b, const PatchOff& f, bool o
     }
 }
 
+__device__ __forceinline__ void relu_patch(float (&p)[2][4])
+{
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) p[a][b] = fmaxf(p[a][b], 0.0f);
+}
+
 // ---- depthwise 3x3 convolution in front of the transform (stride 1, zero padding 1, cross-correlation) -----------------
 // A warp tile with a border of one row and one piece, staged through shared memory by the warp that uses it: a lane needs a
 // 4 x 6 neighbourhood of its patch, and out of global memory that was twelve loads with as many 64-bit addresses, their border
