@@ -7,6 +7,8 @@
 #include <stdint.h>
 #include <stdlib.h>
 
+#include <atomic>
+
 #include "wcc.h"
 
 namespace wcc {
@@ -48,6 +50,37 @@ static unsigned long long g_launches = 0;
 //  - A kernel that reads anything early has such a kernel as its predecessor (never the caller's own kernels).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// What launches need to know about the current device, looked up once per device: each of these calls costs a few hundred
+// nanoseconds, and a small layer is over in 16 us.
+constexpr int MAX_DEVICES = 64;
+struct DeviceInfo { int dev, sms; int* status; };
+static wcc_status device_info(DeviceInfo& d)
+{
+    static std::atomic<int> sms[MAX_DEVICES];
+    static std::atomic<int*> status[MAX_DEVICES];
+    WCC_CUDA_TRY(cudaGetDevice(&d.dev));
+    if (d.dev < 0 || d.dev >= MAX_DEVICES) return WCC_ERR_CUDA;
+    d.sms = sms[d.dev].load(std::memory_order_relaxed);
+    d.status = status[d.dev].load(std::memory_order_relaxed);
+    if (!d.sms || !d.status) {
+        WCC_CUDA_TRY(cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, d.dev));
+        WCC_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&d.status), g_status));
+        sms[d.dev].store(d.sms, std::memory_order_relaxed);
+        status[d.dev].store(d.status, std::memory_order_relaxed);
+    }
+    return WCC_OK;
+}
+// Allows kernel K up to `smem` bytes of dynamic shared memory, once per device.
+template <auto K>
+static wcc_status allow_smem(int dev, int smem)
+{
+    static std::atomic<int> allowed[MAX_DEVICES];
+    if (allowed[dev].load(std::memory_order_relaxed) >= smem) return WCC_OK;
+    WCC_CUDA_TRY(cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    allowed[dev].store(smem, std::memory_order_relaxed);
+    return WCC_OK;
+}
 
 // `overlap` false: an ordinary launch.  cluster > 1: cluster size along x.
 template <typename... KArgs, typename... Args>

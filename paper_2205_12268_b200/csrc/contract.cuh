@@ -257,23 +257,14 @@ wcc_status launch_contract(const void* Xq, const void* Wq, int M, int Cout, int 
     if (!make_map(&tmB, Wq, i8, (uint64_t)kpad, (uint64_t)Cout, TILE_N)) return WCC_ERR_CUDA;   // rows beyond Cout arrive as zeros
 
     const size_t smem = 1024 + (size_t)STAGES * STAGE_BYTES + sizeof(SmemCtl) + 16;
-    static int sm_count[64] = {0};
-    static bool attr_set[64][2] = {{false}};
-    int dev = 0;
-    WCC_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return WCC_ERR_CUDA;
-    if (!sm_count[dev]) WCC_CUDA_TRY(cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev));
-    if (!attr_set[dev][i8]) {
-        if (i8) WCC_CUDA_TRY(cudaFuncSetAttribute(contract_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        else WCC_CUDA_TRY(cudaFuncSetAttribute(contract_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr_set[dev][i8] = true;
-    }
-    int* status = nullptr;
-    WCC_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&status), g_status));
+    DeviceInfo di;
+    wcc_status s = device_info(di);
+    if (s != WCC_OK) return s;
+    if ((s = i8 ? allow_smem<contract_kernel<true>>(di.dev, (int)smem) : allow_smem<contract_kernel<false>>(di.dev, (int)smem)) != WCC_OK) return s;
     const long long items = (long long)ceil_div(M, TILE_M) * ceil_div(npad, TILE_N);
-    const int grid = (int)(items < sm_count[dev] ? items : sm_count[dev]);
+    const int grid = (int)(items < di.sms ? items : di.sms);
     return launch_overlapped(i8 ? contract_kernel<true> : contract_kernel<false>, dim3((unsigned)grid), dim3(192), smem, st, true, 1, tmA, tmB, M, npad,
-                             krow_bytes, acc, ldc, status);
+                             krow_bytes, acc, ldc, di.status);
 }
 
 }  // namespace wcc

@@ -274,26 +274,26 @@ static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, i
     using TT = HaarTile<L>;
     const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
     if (tiles > 0x3FFFFFFFLL) return WCC_ERR_SHAPE;
-    int dev = 0, sms = 0;
-    WCC_CUDA_TRY(cudaGetDevice(&dev));
-    WCC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    int* status = nullptr;
-    WCC_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&status), g_status));
-    const long long warps = 16LL * sms;
+    DeviceInfo di;
+    wcc_status s = device_info(di);
+    if (s != WCC_OK) return s;
+    const long long warps = 16LL * di.sms;
     const int nw = tiles > warps ? 4 : tiles * 2 > warps ? 1 : tiles * 4 > warps ? 2 : tiles * 8 > warps ? 4 : 8;
-    auto go = [&](auto kern, int w) -> wcc_status {
+    auto go = [&](auto nwc) -> wcc_status {
+        constexpr int w = decltype(nwc)::value;
+        constexpr auto kern = pass1_kernel<T, L, VEC, w, KIND, DW>;
+        constexpr int smem = DW ? w * DwTile<T, L, VEC>::BYTES : 0;
         const int wctas = ex.Wt ? ceil_div(ex.Cout, w) : 0;
-        const size_t smem = DW ? (size_t)w * DwTile<T, L, VEC>::BYTES : 0;
-        if (DW) WCC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), smem, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), taps, C, H, W,
-                                 wctas, coef, nrm2, amaxpos, ex, status);
+        if (DW && (s = allow_smem<kern>(di.dev, smem)) != WCC_OK) return s;
+        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), smem, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), taps, C,
+                                 H, W, wctas, coef, nrm2, amaxpos, ex, di.status);
     };
     if constexpr (!DW) {
-        if (nw == 1) return go(pass1_kernel<T, L, VEC, 1, KIND, DW>, 1);
-        if (nw == 2) return go(pass1_kernel<T, L, VEC, 2, KIND, DW>, 2);
+        if (nw == 1) return go(std::integral_constant<int, 1>{});
+        if (nw == 2) return go(std::integral_constant<int, 2>{});
     }
-    if (nw <= 4) return go(pass1_kernel<T, L, VEC, 4, KIND, DW>, 4);
-    return go(pass1_kernel<T, L, VEC, 8, KIND, DW>, 8);
+    if (nw <= 4) return go(std::integral_constant<int, 4>{});
+    return go(std::integral_constant<int, 8>{});
 }
 
 template <typename T, int L, bool VEC>

@@ -431,9 +431,10 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
     if (tiles > 0x7FFFFFFFLL) return WCC_ERR_SHAPE;
     const unsigned groups = (unsigned)((tiles + p2::TILES - 1) / p2::TILES);
-    int dev = 0, sms = 0;
-    WCC_CUDA_TRY(cudaGetDevice(&dev));
-    WCC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    DeviceInfo di;
+    wcc_status s = device_info(di);
+    if (s != WCC_OK) return s;
+    const int sms = di.sms;
     const bool tap = xq_tap || acc_tap;
     const P2Plan plan = (tap || !VEC) ? p2_plan_of(4, Cout, krow, i8, L) : p2_plan(Cout, krow, i8, L, groups, sms);
     if (!plan.ok) return WCC_ERR_SHAPE;
@@ -445,7 +446,7 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     pr.npad = plan.npad; pr.nchunk = plan.nchunk; pr.ksteps_part = plan.ksteps_part; pr.b_resident = plan.b_resident;
     pr.tmem_cols = plan.tmem_cols;
     pr.y = y; pr.xq_tap = static_cast<uint8_t*>(xq_tap); pr.acc_tap = acc_tap;
-    WCC_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&pr.status), g_status));
+    pr.status = di.status;
     // The groups of a last, partial wave are shared 4 or 2 ways by output channels when that still fits one wave (the SMs
     // would idle otherwise).
     const unsigned rem = sms > 0 ? groups % (unsigned)sms : 0u;
@@ -455,14 +456,15 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
             if (rem * (unsigned)parts <= (unsigned)sms && plan.npad % (16 * parts) == 0) { pr.parts = parts; break; }
     pr.split_from = (pr.parts > 1) ? (int)(groups - rem) : (int)groups;
     const unsigned ctas = (unsigned)pr.split_from + (groups - (unsigned)pr.split_from) * (unsigned)pr.parts;
-    auto launch = [&](auto kern) -> wcc_status {
-        WCC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        return launch_overlapped(kern, dim3(ctas), dim3(p2::TILES * plan.wpt * 32), plan.smem, st, true, 1, pr);
-    };
     const bool clampv = i8 && fx.alpha > 0.0f;
     const int want = (fx.relu ? 1 : 0) | (tap ? 2 : 0) | (clampv ? 4 : 0) | (fx.residual ? 8 : 0);
     const int mode = want == 0 ? 0 : want == 1 ? 1 : (want & 2) == 0 ? 13 : 15;
-#define WCC_P2(I8V, WPTV, MODEV) return launch(p2::pass2_kernel<T, L, I8V, WPTV, VEC, MODEV>)
+#define WCC_P2(I8V, WPTV, MODEV)                                                                                     \
+    do {                                                                                                            \
+        constexpr auto kern = p2::pass2_kernel<T, L, I8V, WPTV, VEC, MODEV>;                                        \
+        if ((s = allow_smem<kern>(di.dev, 227 * 1024)) != WCC_OK) return s;                                         \
+        return launch_overlapped(kern, dim3(ctas), dim3(p2::TILES * WPTV * 32), plan.smem, st, true, 1, pr);        \
+    } while (0)
 #define WCC_P2M(I8V, WPTV) do { if (mode == 0) WCC_P2(I8V, WPTV, 0); if (mode == 1) WCC_P2(I8V, WPTV, 1); WCC_P2(I8V, WPTV, 13); } while (0)
     if constexpr (VEC) {
         if (mode != 15) {
