@@ -77,7 +77,10 @@ pass2_kernel(const Params pr)
     constexpr int THREADS = TILES * WPT * 32;
     constexpr int ES = I8 ? 1 : 2;                     // bytes of an operand element
     constexpr int UPK = 32 / (8 * ES);                 // units of eight channels per K step
-    constexpr int U = 2;                               // channels transformed at a time
+    // Channels transformed at a time on the way in (more shuffles of a stage in flight; four fit the registers of the quantized
+    // path: six-layer bf16 chain 380 -> 361 us, unquantized 46.3 -> 46.7) and on the way out (four only pay where the residual's
+    // loads are to be covered: 39.8 -> 39.1, chain 361 -> 368).
+    constexpr int U = I8 ? 4 : 2, U3 = RES ? 4 : 2;
     // Channels loaded ahead, as one batch: all loads of a batch are issued together and waited for together, a batch later.
     // (Refilled two channels at a time the loads shared scoreboards with younger ones: 39 % of the stalls on bf16.)
     constexpr int NB = (sizeof(T) == 2 && I8) ? 8 : 4;
@@ -221,11 +224,10 @@ pass2_kernel(const Params pr)
                     }
 #pragma unroll
                     for (int s = 0; s < 8; ++s) {
-                        if (I8) {
-                            const uint32_t w = __byte_perm(code[0][s], code[1][s], 0x0040);
-                            packed[s][i >> 1] = (i & 1) ? __byte_perm(packed[s][i >> 1], w, 0x5410) : w;
+                        if constexpr (I8) {
+                            packed[s][i] = __byte_perm(__byte_perm(code[0][s], code[1][s], 0x0040), __byte_perm(code[2][s], code[3][s], 0x0040), 0x5410);
                         } else {
-                            packed[s][i * (ES - 1)] = pack_bf16x2(__uint_as_float(code[0][s]), __uint_as_float(code[1][s]));
+                            packed[s][i] = pack_bf16x2(__uint_as_float(code[0][s]), __uint_as_float(code[1][s]));
                         }
                     }
                 }
@@ -320,10 +322,10 @@ pass2_kernel(const Params pr)
             }
             uint64_t yo = yb + (uint64_t)o0 * plane;
 #pragma unroll
-            for (int h = 0; h < 4; h += U) {
-                float sl[U][8], p[U][2][4];
+            for (int h = 0; h < 4; h += U3) {
+                float sl[U3][8], p[U3][2][4];
 #pragma unroll
-                for (int d = 0; d < U; ++d) {
+                for (int d = 0; d < U3; ++d) {
                     // dequantize straight into the pre-scaled slots of the inverse: acc * (scale * 2^-level)
                     float4 f;
                     if (I8) f = dq[(o0 + h + d) * DQ];
@@ -338,9 +340,9 @@ pass2_kernel(const Params pr)
                         sl[d][s + 1] = __fmul_rn(a.y, s < 6 ? f.y : f.w);
                     }
                 }
-                inv_group<T, L, U>(sl, p, lane);
+                inv_group<T, L, U3>(sl, p, lane);
 #pragma unroll
-                for (int d = 0; d < U; ++d) {
+                for (int d = 0; d < U3; ++d) {
                     if (RES && pr.residual) {          // y = WCC(x) + residual: one fp32 addition per element (Eq. 13)
 #pragma unroll
                         for (int row = 0; row < 2; ++row) {
