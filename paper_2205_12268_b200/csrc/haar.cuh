@@ -387,6 +387,8 @@ template <typename T, int L, bool VEC>
 __global__ void __launch_bounds__(128)
 haar_inv_kernel(const float* __restrict__ coef, int planes, int H, int W, T* __restrict__ out)
 {
+    pdl_wait();
+    pdl_launch();
     using TT = HaarTile<L>;
     const int tiles_x = (W + TT::TW - 1) / TT::TW, tiles_y = H / TT::TH;
     const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -422,9 +424,7 @@ static wcc_status haar_inv_dispatch(const float* coef, int planes, int H, int W,
     using TT = HaarTile<L>;
     const long long warps = (long long)planes * ceil_div(W, TT::TW) * (H / TT::TH);
     const int blocks = (int)((warps + 3) / 4);
-    haar_inv_kernel<T, L, VEC><<<blocks, 128, 0, st>>>(coef, planes, H, W, static_cast<T*>(out));
-    WCC_LAUNCH_CHECK();
-    return WCC_OK;
+    return launch_overlapped(haar_inv_kernel<T, L, VEC>, dim3(blocks), dim3(128), 0, st, true, 1, coef, planes, H, W, static_cast<T*>(out));
 }
 
 wcc_status launch_haar_inv(const float* coef, int N, int C, int H, int W, int L, wcc_dtype dt,

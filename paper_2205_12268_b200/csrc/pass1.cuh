@@ -51,6 +51,7 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
     using Dw = DwTile<T, L, VEC>;
     __shared__ __align__(16) float2 tap_sm[DW ? NW : 1][2][NB * 10];
     extern __shared__ __align__(16) uint8_t dw_sm[];            // DW: [NW][Dw::BYTES]
+    if (KIND == P1_COEF) pdl_wait();                   // its predecessor can be anything: nothing may be read early
     pdl_launch();
     const int warp = (NW > 1) ? __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0) : 0, lane = threadIdx.x & 31;
     if ((int)blockIdx.x < weight_ctas) {
@@ -285,7 +286,7 @@ static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, i
         constexpr int smem = DW ? w * DwTile<T, L, VEC>::BYTES : 0;
         const int wctas = ex.Wt ? ceil_div(ex.Cout, w) : 0;
         if (DW && (s = allow_smem<kern>(di.dev, smem)) != WCC_OK) return s;
-        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), smem, st, ex.hist1 != nullptr, 1, static_cast<const T*>(x), taps, C,
+        return launch_overlapped(kern, dim3((unsigned)(tiles + wctas)), dim3(w * 32), smem, st, KIND == P1_COEF || ex.hist1, 1, static_cast<const T*>(x), taps, C,
                                  H, W, wctas, coef, nrm2, amaxpos, ex, di.status);
     };
     if constexpr (!DW) {

@@ -978,7 +978,7 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         const uint32_t* fine_use = hist1_ready ? fine : (const uint32_t*)nullptr;
         const int wr = (want_rank || !thr) ? 1 : 0;
         auto go = [&](auto kern) -> wcc_status {
-            return launch_overlapped(kern, dim3(cs, N), dim3(threads), 0, st, hist1_ready, cs, nrm2, P, k, kpt, idx, tau, rank, amaxpos, amax_kept,
+            return launch_overlapped(kern, dim3(cs, N), dim3(threads), 0, st, true, cs, nrm2, P, k, kpt, idx, tau, rank, amaxpos, amax_kept,
                                      hist1, fine_use, thr, wr);
         };
         // few keys per thread: the instantiation with four key registers
