@@ -67,7 +67,9 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
     const PatchOff off = patch_off<T>(lp, W);
     const uint64_t xb = reinterpret_cast<uint64_t>(x) + (uint64_t)n * C * plane;
     const int rounds = (C + NB - 1) / NB;
-    constexpr int D = (NW == 1 && !DW) ? 2 : 1;               // boxes ahead: a lone warp per tile has registers for two (C4 22.4 against 23.5 us)
+    // Boxes ahead: two where the registers allow it (a lone warp per tile: C4 22.4 against 23.5 us; fp32: 24 images of C4 119.8
+    // against 122.2 us a layer, but with coefficients to store 69.5 against 61.4 for the transform case of pass1's header).
+    constexpr int D = (!DW && (NW == 1 || (sizeof(T) == 4 && KIND != P1_COEF))) ? 2 : 1;
     Raw<T> raw[DW ? 1 : D][DW ? 1 : NB];
     uint32_t piece[DW ? Dw::CHS : 1][DW ? Dw::IT : 1][DW ? Dw::PW : 1];
     Dw dw;
