@@ -266,10 +266,12 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
     if (NW > 1 && !__all_sync(0xFFFFFFFFu, ok ? 1 : 0) && lane == 0) atomicExch(status, (int)WCC_ERR_TIMEOUT);
 }
 
-// Warps per tile: one where the tiles alone fill the sixteen warps of every SM about once (no hand-over), up to eight where
-// they are few; four where one warp per tile would leave a long second wave.  us per layer with 1 / 2 / 4 / 8 warps: 512 tiles
-// (144 -> 24 bf16) 47.9 / 37.6 / 34.3 / 37.3; 128 tiles (384 -> 512 bf16) 101 / 73 / 61 / 56; 1024 tiles (32 -> 192 chain)
-// 405 / 377 / 387 / 414; 1440 tiles (C4) 68.7 / 71.4 / 69.8 / 72.7; 2880 tiles 130.0 / 125.8 / 125.1 / 132.5.
+// Warps per tile: one where the tiles alone fill the resident warps of every SM about once, or several times over (no hand-over),
+// up to eight where they are few, two or four where one warp per tile would leave a long second wave.  us per layer with
+// 1 / 2 / 4 / 8 warps: 128 tiles (384 -> 512 bf16) 101 / 73 / 61 / 56; 512 tiles (144 -> 24 bf16) 47.9 / 37.6 / 34.3 / 37.3;
+// 1024 tiles (32 -> 192 chain) 405 / 377 / 387 / 414; 1440 tiles (C4) 67.9 / 71.1 / 70.4; 1664 tiles (144 -> 24 bf16)
+// 105.6 / 98.9 / 101.3; 2048 tiles 117.5 / 109.0 / 111.9, fp32 1920 tiles 93.9 / 87.6 / 87.9; 2880 tiles fp32 130.0 / 125.8 /
+// 125.1; 3072 tiles (100 -> 24 bf16) 105.6 / 107.2 / 111.4; 4800 tiles 117.7 / 120.4 / 123.1.
 template <typename T, int L, bool VEC, int KIND, bool DW>
 static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
                                cudaStream_t st)
@@ -281,7 +283,8 @@ static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, i
     wcc_status s = device_info(di);
     if (s != WCC_OK) return s;
     const long long warps = 16LL * di.sms;
-    const int nw = tiles > warps ? 4 : tiles * 2 > warps ? 1 : tiles * 4 > warps ? 2 : tiles * 8 > warps ? 4 : 8;
+    const int nw = tiles * 4 > warps * 5 ? 1 : tiles > warps ? (sizeof(T) == 4 ? 4 : 2) : tiles * 3 > warps * 2 ? 2 : tiles * 2 > warps ? 1
+                   : tiles * 4 > warps ? 2 : tiles * 8 > warps ? 4 : 8;
     auto go = [&](auto nwc) -> wcc_status {
         constexpr int w = decltype(nwc)::value;
         constexpr auto kern = pass1_kernel<T, L, VEC, w, KIND, DW>;

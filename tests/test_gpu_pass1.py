@@ -15,7 +15,9 @@ SHAPES = [  # N, C, H, W, levels  (tiles of 256 positions)
     (3, 17, 128, 256, 3), (5, 8, 96, 150, 1),                                         # four
     (6, 33, 128, 256, 2),                                                             # two
     (10, 5, 128, 264, 3),                                                             # one
-    (19, 12, 128, 256, 3),                                                            # four again: more than one wave
+    (14, 9, 128, 256, 2),                                                             # two again: more than one wave
+    (19, 12, 128, 256, 3),                                                            # two (bf16), four (fp32)
+    (24, 9, 128, 256, 1),                                                             # one again: several waves
 ]
 
 
