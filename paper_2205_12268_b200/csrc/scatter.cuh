@@ -32,25 +32,27 @@ scatter_inv_kernel(const int32_t* __restrict__ acc, int ldc, const int32_t* __re
     const size_t P = (size_t)H * W, plane = P * sizeof(T);
     pdl_wait();
     pdl_launch();
-    // rows as offsets in units of sixteen bytes
+    // Rows count inside the image; its first row is a 64-bit address and an access one 32 x 32 -> 64 bit multiply-add (an offset
+    // into the whole matrix would not fit 32 bits: 17 images of 131072 kept positions x 8192 channels are 68 GiB).
     uint32_t row[8], kept = 0u;
-    const uint32_t pitch4 = (uint32_t)(ldc / 4);
+    const uint32_t pitch = (uint32_t)ldc * 4u;
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
         const int r = slot_ok<L>(lp, s) ? rank[(size_t)n * P + lp.pos[s]] : -1;
-        row[s] = (uint32_t)((size_t)n * k + max(r, 0)) * pitch4 + (uint32_t)(o_lo >> 2);
+        row[s] = (uint32_t)max(r, 0);
         kept |= r >= 0 ? 1u << s : 0u;
     }
-    const uint4* acc4 = reinterpret_cast<const uint4*>(acc);
+    uint64_t ab = reinterpret_cast<uint64_t>(acc) + ((uint64_t)n * k * ldc + o_lo) * 4;
     uint4 v[8];
-    auto gather = [&](uint32_t g) {
+    auto gather = [&]() {                              // the next four channels
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
             v[s] = make_uint4(0u, 0u, 0u, 0u);
-            if (kept & (1u << s)) v[s] = __ldg(acc4 + row[s] + g);
+            if (kept & (1u << s)) v[s] = __ldg(reinterpret_cast<const uint4*>(ab + (uint64_t)row[s] * pitch));
         }
+        ab += 16;
     };
-    gather(0u);
+    gather();
     float scale_a = 1.0f;
     if (!ACCF) scale_a = __fdiv_rn(*amax_kept, qmax);
     const bool coarse6 = L == 3 && ((lane / TT::CG) & 1) == 0;         // slot 6 holds a level-3 coefficient
@@ -75,7 +77,7 @@ scatter_inv_kernel(const int32_t* __restrict__ acc, int ldc, const int32_t* __re
                 sl[d][s] = __fmul_rn(f, s < 6 ? s1 : (s == 6 ? s6 : s7));
             }
         }
-        if (o0 + 4 < o_end) gather((uint32_t)(o0 + 4 - o_lo) >> 2);
+        if (o0 + 4 < o_end) gather();
 #pragma unroll
         for (int h = 0; h < 4; h += U) {
             float p[U][2][4];
