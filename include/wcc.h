@@ -54,7 +54,8 @@ typedef enum {
 typedef enum { WCC_F32 = 0, WCC_BF16 = 1 } wcc_dtype;   /* element type of activations x and y */
 #define WCC_MAX_CHANNELS 8192
 
-/* Scratch bytes wcc_forward / wcc_forward_debug need for these arguments (0 on invalid arguments). */
+/* Scratch bytes with which wcc_forward / wcc_forward_debug run these arguments fastest (0 on invalid arguments).  A workspace of
+ * this size also serves smaller batches, maps and kept counts of the same layer, if not always by the fastest pipeline. */
 size_t wcc_workspace_bytes(int N, int Cin, int Cout, int H, int Wd, int levels, int k, int bits, wcc_dtype dt);
 /* Scratch bytes wcc_forward_staged needs (it materialises the coefficient map, the compressed matrix and the accumulators). */
 size_t wcc_staged_workspace_bytes(int N, int Cin, int Cout, int H, int Wd, int levels, int k, int bits, wcc_dtype dt);

@@ -328,6 +328,26 @@ static bool fused_fits(int N, int Cin, int Cout, int H, int W, int L, int bits)
     return !wide_fits(Cin, Cout, H, W, bits) && krow <= 256 && p2_plan_of(4, Cout, krow, i8, L).ok;
 }
 
+// The pipeline that a call of wcc_forward runs.  Which of them is fastest depends on the batch and the map, and the fused kernels
+// need far less scratch than the other two.  So that a workspace sized for the largest batch or map of a layer serves the
+// smaller ones too, a workspace that is too small for the faster pipeline but holds the fused one is used with that.
+enum class Path { FUSED, WIDE, STAGED };
+static Path layer_path(int N, int Cin, int Cout, int H, int W, int L, int k, int bits, bool own_codes, bool coef_tap, size_t ws_bytes)
+{
+    if (own_codes || fused_fits(N, Cin, Cout, H, W, L, bits)) return Path::FUSED;      // (codes only enter the fused kernels)
+    const bool wide = wide_fits(Cin, Cout, H, W, bits) && !coef_tap;
+    const size_t need = wide ? carve_wide_ws(nullptr, N, Cin, Cout, H, W, k, bits).total : carve_forward_ws(nullptr, N, Cin, Cout, H, W, k, bits).total;
+    if (ws_bytes < need && p2_plan_of(4, Cout, wcc_kpad(Cin, bits) * (bits >= 2 ? 1 : 2), bits >= 2, L).ok) return Path::FUSED;
+    return wide ? Path::WIDE : Path::STAGED;
+}
+
+// The least scratch with which wcc_forward runs the layer; `most` (wcc_workspace_bytes) is what its fastest pipeline takes.
+static size_t least_workspace_bytes(size_t most, int N, int Cin, int Cout, int H, int W, int L, int k, int bits)
+{
+    if (most == 0 || !p2_plan_of(4, Cout, wcc_kpad(Cin, bits) * (bits >= 2 ? 1 : 2), bits >= 2, L).ok) return most;
+    return carve_fused_ws(nullptr, N, Cin, Cout, H, W, k, bits).total;
+}
+
 static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int Cout, int H, int W,
                             int L, int k, int bits, void* y, wcc_dtype dt, void* ws, size_t ws_bytes,
                             cudaStream_t st, const wcc_taps* taps, const wcc_options* opt, const float* dwk = nullptr)
@@ -400,13 +420,11 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     if (!aligned16(x) || !aligned16(Wt) || !aligned16(y) || (reinterpret_cast<uintptr_t>(ws) & 255u)) return WCC_ERR_ALIGN;
     if (taps && (!aligned16(taps->coef) || !aligned16(taps->Xq) || !aligned16(taps->Xb) || !aligned16(taps->acc)))
         return WCC_ERR_ALIGN;
-    if (own_codes) {                                   // codes only enter the fused kernels
-        const int krow = wcc_kpad(Cin, bits);
-        if (!p2_plan_of(4, Cout, krow, true, L).ok) return WCC_ERR_SHAPE;
-    } else if (!fused_fits(N, Cin, Cout, H, W, L, bits)) {                     // decided before anything is launched
-        if (wide_fits(Cin, Cout, H, W, bits) && !(taps && taps->coef))
-            return wide_impl(x, Wt, N, Cin, Cout, H, W, L, k, bits, y, dt, ws, ws_bytes, st, taps, opt);
-        return staged_impl(x, Wt, N, Cin, Cout, H, W, L, k, bits, y, dt, ws, ws_bytes, st, taps, opt);
+    if (own_codes && !p2_plan_of(4, Cout, wcc_kpad(Cin, bits), true, L).ok) return WCC_ERR_SHAPE;
+    switch (layer_path(N, Cin, Cout, H, W, L, k, bits, own_codes, taps && taps->coef, ws_bytes)) {      // decided before anything is launched
+        case Path::WIDE: return wide_impl(x, Wt, N, Cin, Cout, H, W, L, k, bits, y, dt, ws, ws_bytes, st, taps, opt);
+        case Path::STAGED: return staged_impl(x, Wt, N, Cin, Cout, H, W, L, k, bits, y, dt, ws, ws_bytes, st, taps, opt);
+        case Path::FUSED: break;
     }
     const FusedWs f = carve_fused_ws(ws, N, Cin, Cout, H, W, k, bits);
     if (ws_bytes < f.total) return WCC_ERR_WORKSPACE;
@@ -576,7 +594,8 @@ static wcc_status launch_crop(const void* src, long long planes, int H, int W, i
                              Wp, static_cast<E*>(dst));
 }
 
-struct PaddedWs { void* xp; void* yp; void* inner; size_t inner_bytes; size_t total; int Hp, Wp; };
+// `least`: the smallest workspace that works; the layer's own scratch comes last and takes whatever there is beyond `inner_off`.
+struct PaddedWs { void* xp; void* yp; void* inner; size_t inner_off; size_t least, total; int Hp, Wp; };
 
 static PaddedWs carve_padded_ws(void* ws, int N, int Cin, int Cout, int H, int W, int L, int k, int bits, wcc_dtype dt)
 {
@@ -590,9 +609,11 @@ static PaddedWs carve_padded_ws(void* ws, int N, int Cin, int Cout, int H, int W
     auto take = [&](size_t bytes) { char* q = base ? base + off : nullptr; off += align_up(bytes, 256); return q; };
     p.xp = take((size_t)N * Cin * p.Hp * p.Wp * es);
     p.yp = take((size_t)N * Cout * p.Hp * p.Wp * es);
-    p.inner_bytes = wcc_workspace_bytes(N, Cin, Cout, p.Hp, p.Wp, L, k, bits, dt);
-    p.inner = take(p.inner_bytes);
-    p.total = p.inner_bytes ? off : 0;
+    const size_t inner_bytes = wcc_workspace_bytes(N, Cin, Cout, p.Hp, p.Wp, L, k, bits, dt);
+    p.inner_off = off;
+    p.least = off + least_workspace_bytes(inner_bytes, N, Cin, Cout, p.Hp, p.Wp, L, k, bits);
+    p.inner = take(inner_bytes);
+    p.total = inner_bytes ? off : 0;
     return p;
 }
 
@@ -622,7 +643,7 @@ static WaveletWs carve_wavelet_ws(void* ws, int N, int Cin, int Cout, int H, int
 }
 
 // ---- inverted residual block -------------------------------------------------------------------------
-struct BlockWs { void* u; void* layer_ws; size_t layer_ws_bytes; size_t total; };
+struct BlockWs { void* u; void* layer_ws; size_t layer_off; size_t least, total; };
 
 static BlockWs carve_block_ws(void* ws, int N, int C, int E, int H, int W, int L, int k, int bits, wcc_dtype dt)
 {
@@ -636,14 +657,16 @@ static BlockWs carve_block_ws(void* ws, int N, int C, int E, int H, int W, int L
     size_t off = 0;
     auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align_up(bytes, 256); return p; };
     b.u = take((size_t)N * E * H * W * es);
-    b.layer_ws_bytes = w1 > w3 ? w1 : w3;
-    b.layer_ws = take(b.layer_ws_bytes);
+    b.layer_off = off;
+    const size_t l1 = least_workspace_bytes(w1, N, C, E, H, W, L, k, bits);
+    b.least = off + (l1 > w3 ? l1 : w3);
+    b.layer_ws = take(w1 > w3 ? w1 : w3);
     b.total = off;
     return b;
 }
 
 // ---- chain of layers -------------------------------------------------------------------------------
-struct ChainWs { void* act[2]; void* layer_ws; size_t layer_ws_bytes; size_t total; };
+struct ChainWs { void* act[2]; void* layer_ws; size_t layer_off; size_t least, total; };
 
 static wcc_status chain_shapes_ok(const wcc_chain_layer* layers, int n_layers)
 {
@@ -659,19 +682,22 @@ static ChainWs carve_chain_ws(void* ws, const wcc_chain_layer* layers, int n_lay
 {
     ChainWs c = {};
     const size_t es = (dt == WCC_BF16) ? 2 : 4, P = (size_t)H * W;
-    size_t act = 0, lw = 0;
+    size_t act = 0, lw = 0, least = 0;
     for (int i = 0; i < n_layers; ++i) {
         if (i + 1 < n_layers) { const size_t b = (size_t)N * layers[i].Cout * P * es; if (b > act) act = b; }
         const size_t b = wcc_workspace_bytes(N, layers[i].Cin, layers[i].Cout, H, W, L, k, bits, dt);
         if (b == 0) { c.total = 0; return c; }
         if (b > lw) lw = b;
+        const size_t a = least_workspace_bytes(b, N, layers[i].Cin, layers[i].Cout, H, W, L, k, bits);
+        if (a > least) least = a;
     }
     char* b = static_cast<char*>(ws);
     size_t off = 0;
     auto take = [&](size_t bytes) { char* p = b ? b + off : nullptr; off += align_up(bytes, 256); return p; };
     c.act[0] = take(act);
     c.act[1] = take(act);
-    c.layer_ws_bytes = lw;
+    c.layer_off = off;
+    c.least = off + least;
     c.layer_ws = take(lw);
     c.total = off;
     return c;
@@ -804,10 +830,11 @@ wcc_status wcc_block_forward(const void* x, const float* W1, const float* Wdw, c
         (reinterpret_cast<uintptr_t>(ws) & 255u)) return WCC_ERR_ALIGN;
     const BlockWs b = carve_block_ws(ws, N, C, E, H, Wd, levels, k, bits, dt);
     if (b.total == 0) return WCC_ERR_SHAPE;
-    if (ws_bytes < b.total) return WCC_ERR_WORKSPACE;
+    if (ws_bytes < b.least) return WCC_ERR_WORKSPACE;
+    const size_t layer_ws_bytes = ws_bytes - b.layer_off;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // u = WCC(W1, x): C -> E channels
-    s = forward_impl(x, W1, N, C, E, H, Wd, levels, k, bits, b.u, dt, b.layer_ws, b.layer_ws_bytes, st, nullptr);
+    s = forward_impl(x, W1, N, C, E, H, Wd, levels, k, bits, b.u, dt, b.layer_ws, layer_ws_bytes, st, nullptr);
     if (s != WCC_OK) return s;
     // y = x + WCC(W3, dw3x3(u)): the depthwise convolution is fused with the second layer's transform.  Convolving and
     // transforming u again for the kept columns is cheaper than keeping the coefficients (4 bytes each, written once, gathered
@@ -815,8 +842,8 @@ wcc_status wcc_block_forward(const void* x, const float* W1, const float* Wdw, c
     wcc_options o = {};
     o.residual = x;
     if (wide_fits(E, C, H, Wd, bits))
-        return wide_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, b.layer_ws_bytes, st, nullptr, &o, Wdw);
-    return staged_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, b.layer_ws_bytes, st, nullptr, &o, Wdw);
+        return wide_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, layer_ws_bytes, st, nullptr, &o, Wdw);
+    return staged_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, layer_ws_bytes, st, nullptr, &o, Wdw);
 }
 
 wcc_status wcc_dwt_fwd(const void* x, int N, int C, int H, int Wd, int levels, wcc_dtype dt,
@@ -960,15 +987,16 @@ wcc_status wcc_forward_padded(const void* x, const float* Wt, int N, int Cin, in
     wcc_status s = check_forward_args(N, Cin, Cout, p.Hp, p.Wp, levels, k, bits, dt);       // k counts padded positions
     if (s != WCC_OK) return s;
     if (p.total == 0) return WCC_ERR_SHAPE;
-    if (ws_bytes < p.total) return WCC_ERR_WORKSPACE;
+    if (ws_bytes < p.least) return WCC_ERR_WORKSPACE;
+    const size_t inner_bytes = ws_bytes - p.inner_off;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (p.Hp == H && p.Wp == Wd)                       // nothing to pad: the plain layer
-        return forward_impl(x, Wt, N, Cin, Cout, H, Wd, levels, k, bits, y, dt, p.inner, p.inner_bytes, st, nullptr);
+        return forward_impl(x, Wt, N, Cin, Cout, H, Wd, levels, k, bits, y, dt, p.inner, inner_bytes, st, nullptr);
     const long long in_planes = (long long)N * Cin, out_planes = (long long)N * Cout;
     s = dt == WCC_BF16 ? launch_pad<uint16_t>(x, in_planes, H, Wd, p.Hp, p.Wp, p.xp, st)
                        : launch_pad<uint32_t>(x, in_planes, H, Wd, p.Hp, p.Wp, p.xp, st);
     if (s != WCC_OK) return s;
-    s = forward_impl(p.xp, Wt, N, Cin, Cout, p.Hp, p.Wp, levels, k, bits, p.yp, dt, p.inner, p.inner_bytes, st, nullptr);
+    s = forward_impl(p.xp, Wt, N, Cin, Cout, p.Hp, p.Wp, levels, k, bits, p.yp, dt, p.inner, inner_bytes, st, nullptr);
     if (s != WCC_OK) return s;
     return dt == WCC_BF16 ? launch_crop<uint16_t>(p.yp, out_planes, H, Wd, p.Hp, p.Wp, y, st)
                           : launch_crop<uint32_t>(p.yp, out_planes, H, Wd, p.Hp, p.Wp, y, st);
@@ -997,7 +1025,7 @@ wcc_status wcc_chain_forward(const void* x, const wcc_chain_layer* layers, int n
     }
     const ChainWs c = carve_chain_ws(ws, layers, n_layers, N, H, Wd, levels, k, bits, dt);
     if (c.total == 0) return WCC_ERR_SHAPE;
-    if (ws_bytes < c.total) return WCC_ERR_WORKSPACE;
+    if (ws_bytes < c.least) return WCC_ERR_WORKSPACE;
     const void* in = x;
     for (int i = 0; i < n_layers; ++i) {
         void* out = (i + 1 == n_layers) ? y : c.act[i & 1];
@@ -1005,7 +1033,7 @@ wcc_status wcc_chain_forward(const void* x, const wcc_chain_layer* layers, int n
         o.alpha = layers[i].alpha;
         o.relu = layers[i].relu;
         s = forward_impl(in, layers[i].Wt, N, layers[i].Cin, layers[i].Cout, H, Wd, levels, k, bits, out, dt, c.layer_ws,
-                         c.layer_ws_bytes, static_cast<cudaStream_t>(stream), nullptr, &o);
+                         ws_bytes - c.layer_off, static_cast<cudaStream_t>(stream), nullptr, &o);
         if (s != WCC_OK) return s;
         in = out;
     }
