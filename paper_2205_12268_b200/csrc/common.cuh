@@ -102,8 +102,11 @@ static wcc_status launch_overlapped(void (*kern)(KArgs...), dim3 grid, dim3 bloc
         ++na;
     }
     cfg.attrs = attr; cfg.numAttrs = (unsigned)na;
-    WCC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...));
-    WCC_LAUNCH_CHECK();
+    if (cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...) != cudaSuccess) {
+        (void)cudaGetLastError();                      // a rejected launch is this call's error, not the next one's
+        return WCC_ERR_CUDA;
+    }
+    ++g_launches;
     return WCC_OK;
 }
 
