@@ -388,7 +388,10 @@ struct FusedExtra { float alpha; int relu; const void* residual; };
 // weights stay in shared memory.  Pure arithmetic: callers decide before anything is launched.
 struct P2Plan { int wpt, npad, nchunk, ksteps_part, b_resident, tmem_cols; size_t smem; bool ok; };
 
-static P2Plan p2_plan_of(int wpt, int Cout, int krow, bool i8, int L)
+// Loads in flight live in what the operands leave of an SM's 256 KB to the L1: two CTAs of three K steps each, or one of six,
+// leave about 28 KB, and phase 1 then waits on its loads (182 -> 38 channels fp32 on 9 x 176 x 120, second pass alone: 82 us with
+// the six steps at once, 53 in two parts).  Two CTAs therefore hold two steps each; see p2_plan for one CTA.
+static P2Plan p2_plan_of(int wpt, int Cout, int krow, bool i8, int L, int most_ksteps = 0)
 {
     P2Plan p = {};
     p.wpt = wpt;
@@ -398,9 +401,10 @@ static P2Plan p2_plan_of(int wpt, int Cout, int krow, bool i8, int L)
     p.tmem_cols = 32;
     while (p.tmem_cols < 8 * p.nchunk) p.tmem_cols <<= 1;
     const int ksteps = krow / 32;
+    if (!most_ksteps) most_ksteps = (wpt == 2) ? 2 : ksteps;
     const size_t budget = (wpt == 2) ? 113 * 1024 : 227 * 1024;
     const size_t fixed = 128 + (i8 ? (size_t)p.npad * 16 * (L == 3 ? 2 : 1) : 0) + sizeof(p2::Ctl);
-    for (int parts = 1; ; ++parts) {                   // fewest K parts that fit
+    for (int parts = ceil_div(ksteps, most_ksteps); ; ++parts) {                  // fewest K parts that fit
         p.ksteps_part = ceil_div(ksteps, parts);
         const size_t a = (size_t)p.ksteps_part * p2::ROWS * 32;
         const size_t b_all = (size_t)krow * p.npad, b_chunk = (size_t)p.ksteps_part * 32 * p.nchunk;
@@ -414,12 +418,22 @@ static P2Plan p2_plan_of(int wpt, int Cout, int krow, bool i8, int L)
 // Two CTAs of eight warps on an SM while there are enough tile groups for it (and the operand does not have to be rebuilt for
 // every chunk of output channels): what one CTA waits for, the other covers.  One CTA of sixteen warps otherwise.
 // C4 (360 groups) 36.5 against 38.4 us, 24 -> 144 channels on 2 x 256 x 512 (256 groups) 22.8 against 29.5 us; with 128
-// groups the sixteen warps win: 96 -> 96 channels on 4 x 128 x 256 23.3 against 32.3 us.
-static P2Plan p2_plan(int Cout, int krow, bool i8, int L, long long groups, int sms)
+// groups the sixteen warps win: 96 -> 96 channels on 4 x 128 x 256 23.3 against 32.3 us.  With K in parts of two steps and one
+// chunk, two CTAs are 1.0 to 1.4 times as fast from four K steps on (whole layers; 152 -> 10 fp32 on 14 x 76 x 156 52.5 against
+// 56.5 us); with two or more chunks and three K steps one CTA is (82 -> 54 fp32 on 2 x 248 x 392 58.6 against 69.4).
+// One CTA with one chunk takes K in parts of at most five steps where its loads are what it waits for: six steps in two parts
+// from half a wave of groups on (189 -> 45 bf16 on 7 x 296 x 184 159 -> 103 us; below it the second part's first loads cost
+// what the L1 gives, +-3 %), more steps from a full wave on (190 -> 42 unquantized fp32 on 6 x 124 x 496 186 -> 148; 247 -> 10
+// with 88 groups 37.3 -> 39.2).  Several chunks keep K whole: they would rebuild the operand (192 -> 96 on 4 x 128 x 256 49.7
+// against 57.4).
+static P2Plan p2_plan(bool two_ctas, int Cout, int krow, bool i8, int L, long long groups, int sms)
 {
-    const P2Plan two = p2_plan_of(2, Cout, krow, i8, L);
-    const bool whole_k = two.ksteps_part == krow / 32 || two.npad <= two.nchunk;
-    return (two.ok && whole_k && groups > sms) ? two : p2_plan_of(4, Cout, krow, i8, L);
+    const int ksteps = krow / 32;
+    const P2Plan two = p2_plan_of(2, Cout, krow, i8, L), one = p2_plan_of(4, Cout, krow, i8, L);
+    const bool whole_k = two.ksteps_part == ksteps || two.npad <= two.nchunk;
+    if (two_ctas && two.ok && whole_k && groups > sms) return two;
+    if (one.npad <= one.nchunk && ksteps > 5 && (ksteps == 6 ? groups * 2 : groups) > sms) return p2_plan_of(4, Cout, krow, i8, L, 5);
+    return one;
 }
 
 template <typename T, int L, bool VEC>
@@ -438,7 +452,7 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     if (s != WCC_OK) return s;
     const int sms = di.sms;
     const bool tap = xq_tap || acc_tap;
-    const P2Plan plan = (tap || !VEC) ? p2_plan_of(4, Cout, krow, i8, L) : p2_plan(Cout, krow, i8, L, groups, sms);
+    const P2Plan plan = p2_plan(VEC && !tap, Cout, krow, i8, L, groups, sms);
     if (!plan.ok) return WCC_ERR_SHAPE;
     p2::Params pr = {};
     pr.x = x; pr.Wq = static_cast<const uint8_t*>(Wq); pr.rank = rank; pr.nrm2 = nrm2; pr.thr = thr; pr.amax_kept = amax_kept;
