@@ -53,6 +53,7 @@ __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.laun
 
 // What launches need to know about the current device, looked up once per device: each of these calls costs a few hundred
 // nanoseconds, and a small layer is over in 16 us.
+constexpr int B200_SMS = 148;           // where a decision is made without a device (sizes of workspaces)
 constexpr int MAX_DEVICES = 64;
 struct DeviceInfo { int dev, sms; int* status; };
 static wcc_status device_info(DeviceInfo& d)

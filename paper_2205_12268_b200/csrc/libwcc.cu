@@ -38,21 +38,28 @@ static wcc_status check_forward_args(int N, int Cin, int Cout, int H, int W, int
     return WCC_OK;
 }
 
-// Run the second pass as one kernel, or gather the kept columns and contract only those (wide_impl)?  One kernel, unless its
-// operand has to be rebuilt for many chunks of output channels, or the channel loop of a few CTAs gets long (bf16 input,
-// one kernel / gathered, us): 256 -> 256 on 2 x 128 x 256 81 / 83, 320 -> 64 there 56 / 69, 128 -> 1024 on 2 x 64 x 128
-// 54 / 65, 180 -> 512 on 2 x 64 x 64 48 / 50; the other way 256 -> 320 on 2 x 64 x 128 65 / 57, 192 -> 1024 there 89 / 65,
-// 512 -> 64 there 69 / 59, 384 -> 384 on 2 x 64 x 64 80 / 55.
-static bool one_kernel(int N, int Cin, int Cout, int H, int W, int L, int bits)
+// Run the second pass as one kernel, or gather the kept columns and contract only those (wide_impl)?
+//  - K in one piece: one kernel up to 72 K steps over all chunks of output channels (bf16 input, one kernel / gathered, us:
+//    128 -> 1024 on 2 x 64 x 128 54 / 65, 180 -> 512 on 2 x 64 x 64 48 / 50; the other way 192 -> 1024 on 2 x 64 x 128 89 / 65).
+//  - K in parts, and no CTA rebuilds its operand for a further chunk (all channels fit one, or the CTAs that share a tile group
+//    take one each): one kernel up to ten K steps (256 -> 64 on 8 x 64 x 128 40 / 49, 256 -> 256 on 2 x 64 x 128 37 / 39), up
+//    to sixteen from 64 tile groups on (384 -> 64 on 8 x 64 x 128 58 / 60; with 28 groups 31 / 26).
+//  - K in parts and rebuilt: gathered (256 -> 288 on 2 x 64 x 128 76 / 42, 246 -> 205 on 2 x 164 x 32 81 / 34, 256 -> 256 on
+//    4 x 128 x 256 144 / 102), unless at least half of the positions are kept, so that gathering saves little, of 64 tile groups
+//    or more (223 -> 114 with 321 groups 124 / 180, 237 -> 234 with 137 groups 122 / 158; with 44 groups 60 / 38).
+// A workspace query has no device: the plan is that of a B200's 148 SMs.
+static bool one_kernel(int N, int Cin, int Cout, int H, int W, int L, int k, int bits)
 {
     const bool i8 = bits >= 2;
     const int krow = wcc_kpad(Cin, bits) * (i8 ? 1 : 2), ksteps = krow / 32;
     const P2Plan p = p2_plan_of(4, Cout, krow, i8, L);
     if (!p.ok) return false;
-    const int chunks = ceil_div(p.npad, p.nchunk);
-    if (p.ksteps_part == ksteps) return chunks * ksteps <= 72;
-    if (ksteps <= 10) return chunks * ksteps <= 40;
-    return chunks == 1 && ksteps <= 16 && (long long)N * H * W >= 64 * p2::ROWS;
+    const int chunks = ceil_div(p.npad, p.nchunk), parts = ceil_div(ksteps, p.ksteps_part);
+    if (parts == 1) return chunks * ksteps <= 72;
+    const long long groups = ((long long)N * ceil_div(W, 128 >> (L - 1)) * (H >> L) + p2::TILES - 1) / p2::TILES;
+    const int share = groups > B200_SMS ? 1 : p2_shares(groups, B200_SMS, p.npad);
+    if (ceil_div(p.npad / share, p.nchunk) == 1) return ksteps <= 10 || (ksteps <= 16 && groups >= 64);
+    return parts == 2 && ksteps <= 8 && chunks <= 4 && 2LL * k >= (long long)H * W && groups >= 64;
 }
 
 // Can the staged contraction kernel run it?  (Mirrors launch_contract: K is a loop and N is tiled, so only the
@@ -311,18 +318,17 @@ static WideWs carve_wide_ws(void* ws, int N, int Cin, int Cout, int H, int W, in
     return f;
 }
 
-// dwk: NULL, or depthwise 3x3 kernels fp32 [Cin][3][3] applied to x in front of both of its transforms.
-// One cluster per image in the selection (it reads the first pass's histograms), vector loads of whole patches.
+// One cluster per image in the selection (it reads the first pass's histograms).
 static bool wide_fits(int Cin, int Cout, int H, int W, int bits)
 {
-    return staged_fits(Cin, Cout, bits) && select_in_cluster(H * W) && (W % 4) == 0;
+    return staged_fits(Cin, Cout, bits) && select_in_cluster(H * W);
 }
 
 // Does wcc_forward run the fused kernels?  Where the gathered pipeline cannot run, they also take the layers that it would
 // be faster for (up to eight K steps; beyond, stage by stage).
-static bool fused_fits(int N, int Cin, int Cout, int H, int W, int L, int bits)
+static bool fused_fits(int N, int Cin, int Cout, int H, int W, int L, int k, int bits)
 {
-    if (one_kernel(N, Cin, Cout, H, W, L, bits)) return true;
+    if (one_kernel(N, Cin, Cout, H, W, L, k, bits)) return true;
     const bool i8 = bits >= 2;
     const int krow = wcc_kpad(Cin, bits) * (i8 ? 1 : 2);
     return !wide_fits(Cin, Cout, H, W, bits) && krow <= 256 && p2_plan_of(4, Cout, krow, i8, L).ok;
@@ -334,7 +340,7 @@ static bool fused_fits(int N, int Cin, int Cout, int H, int W, int L, int bits)
 enum class Path { FUSED, WIDE, STAGED };
 static Path layer_path(int N, int Cin, int Cout, int H, int W, int L, int k, int bits, bool own_codes, bool coef_tap, size_t ws_bytes)
 {
-    if (own_codes || fused_fits(N, Cin, Cout, H, W, L, bits)) return Path::FUSED;      // (codes only enter the fused kernels)
+    if (own_codes || fused_fits(N, Cin, Cout, H, W, L, k, bits)) return Path::FUSED;      // (codes only enter the fused kernels)
     const bool wide = wide_fits(Cin, Cout, H, W, bits) && !coef_tap;
     const size_t need = wide ? carve_wide_ws(nullptr, N, Cin, Cout, H, W, k, bits).total : carve_forward_ws(nullptr, N, Cin, Cout, H, W, k, bits).total;
     if (ws_bytes < need && p2_plan_of(4, Cout, wcc_kpad(Cin, bits) * (bits >= 2 ? 1 : 2), bits >= 2, L).ok) return Path::FUSED;
@@ -348,6 +354,7 @@ static size_t least_workspace_bytes(size_t most, int N, int Cin, int Cout, int H
     return carve_fused_ws(nullptr, N, Cin, Cout, H, W, k, bits).total;
 }
 
+// dwk: NULL, or depthwise 3x3 kernels fp32 [Cin][3][3] applied to x in front of both of its transforms.
 static wcc_status wide_impl(const void* x, const float* Wt, int N, int Cin, int Cout, int H, int W,
                             int L, int k, int bits, void* y, wcc_dtype dt, void* ws, size_t ws_bytes,
                             cudaStream_t st, const wcc_taps* taps, const wcc_options* opt, const float* dwk = nullptr)
@@ -718,7 +725,7 @@ int wcc_kpad(int Cin, int bits)
 size_t wcc_workspace_bytes(int N, int Cin, int Cout, int H, int Wd, int levels, int k, int bits, wcc_dtype dt)
 {
     if (check_forward_args(N, Cin, Cout, H, Wd, levels, k, bits, dt) != WCC_OK) return 0;
-    if (!fused_fits(N, Cin, Cout, H, Wd, levels, bits)) {                      // these shapes run around the tiled contraction
+    if (!fused_fits(N, Cin, Cout, H, Wd, levels, k, bits)) {                      // these shapes run around the tiled contraction
         if (!staged_fits(Cin, Cout, bits)) return 0;
         const size_t a = carve_forward_ws(nullptr, N, Cin, Cout, H, Wd, k, bits).total;
         const size_t b = carve_wide_ws(nullptr, N, Cin, Cout, H, Wd, k, bits).total;

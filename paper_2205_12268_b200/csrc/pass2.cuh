@@ -408,7 +408,7 @@ static P2Plan p2_plan_of(int wpt, int Cout, int krow, bool i8, int L, int most_k
         p.ksteps_part = ceil_div(ksteps, parts);
         const size_t a = (size_t)p.ksteps_part * p2::ROWS * 32;
         const size_t b_all = (size_t)krow * p.npad, b_chunk = (size_t)p.ksteps_part * 32 * p.nchunk;
-        p.b_resident = fixed + a + b_all <= budget;
+        p.b_resident = fixed + a + b_all <= (wpt == 2 ? budget : 195 * 1024);     // (shared memory beyond 196 KB comes out of the L1's last 60)
         p.smem = fixed + a + (p.b_resident ? b_all : b_chunk);
         p.ok = p.smem <= budget;
         if (p.ok || p.ksteps_part == 1) return p;
@@ -434,6 +434,14 @@ static P2Plan p2_plan(bool two_ctas, int Cout, int krow, bool i8, int L, long lo
     if (two_ctas && two.ok && whole_k && groups > sms) return two;
     if (one.npad <= one.nchunk && ksteps > 5 && (ksteps == 6 ? groups * 2 : groups) > sms) return p2_plan_of(4, Cout, krow, i8, L, 5);
     return one;
+}
+
+// CTAs that share each of `groups` tile groups by output channels, where they would not fill the SMs otherwise.
+static int p2_shares(long long groups, int sms, int npad)
+{
+    for (int parts = 4; parts >= 2; parts >>= 1)
+        if (groups * parts <= sms && npad % (16 * parts) == 0) return parts;
+    return 1;
 }
 
 template <typename T, int L, bool VEC>
@@ -466,10 +474,7 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     // The groups of a last, partial wave are shared 4 or 2 ways by output channels when that still fits one wave (the SMs
     // would idle otherwise).
     const unsigned rem = sms > 0 ? groups % (unsigned)sms : 0u;
-    pr.parts = 1;
-    if (rem > 0)
-        for (int parts = 4; parts >= 2; parts >>= 1)
-            if (rem * (unsigned)parts <= (unsigned)sms && plan.npad % (16 * parts) == 0) { pr.parts = parts; break; }
+    pr.parts = rem > 0 ? p2_shares(rem, sms, plan.npad) : 1;
     pr.split_from = (pr.parts > 1) ? (int)(groups - rem) : (int)groups;
     const unsigned ctas = (unsigned)pr.split_from + (groups - (unsigned)pr.split_from) * (unsigned)pr.parts;
     const bool clampv = i8 && fx.alpha > 0.0f;
