@@ -143,7 +143,9 @@ wcc_status wcc_select_topk_static(const float* nrm2, int N, int P, int k, int32_
  * also quantizes the weights); the selection finds the threshold norm, max|kept| and, only if ties at the threshold
  * are kept in part, the rank of every position; pass 2 transforms x again, zeroes the dropped positions, quantizes
  * into shared memory, runs the contraction on tensor cores, dequantizes, applies the inverse transform and stores y.
- * The results are those of the step-by-step definition above (same integers, same fp32 operation order).
+ * The results are those of the step-by-step definition above (same integers, same fp32 operation order), as long as no norm
+ * exceeds 2^128 / 4^levels and no coefficient 2^128 / 2^levels, and neither coefficients nor their squares are subnormal: the
+ * halvings of the transform are applied as one factor of 2^-level at its end.
  */
 wcc_status wcc_forward(const void* x, const float* Wt, int N, int Cin, int Cout, int H, int Wd,
                        int levels, int k, int bits, void* y, wcc_dtype dt,

@@ -191,8 +191,9 @@ __device__ __forceinline__ void haar_inv_lane(const float (&o)[8], float (&p)[2]
 // Multiplying by a power of two commutes with every rounding (barring overflow and subnormal results), so the forward
 // transform can run on sums and differences alone and leave one exact multiplication per slot to the consumer:
 // true coefficient of slot s = raw value * slot_scale[s], where |slot_scale| = 2^-level.  The same holds for squares
-// (norm = raw norm * scale^2) and maxima.  Results are bit-identical to haar_fwd_lane for inputs whose partial sums stay
-// below 2^125 and above the subnormal range.
+// (norm = raw norm * scale^2) and maxima.  Results are bit-identical to the transform with its halvings while the raw sums of
+// squares (up to 4^levels times a norm) stay below 2^128, the raw values below 2^128, and neither squares nor values fall into
+// the subnormal range.  Kernels that store coefficients halve at every level and have the whole range.
 // `swapped`: the lane passes its two patch rows in exchanged order (a shared-memory bank trick of the TMA rings); the sums
 // over rows are unchanged and the differences over rows (y3, y4 of level 1) change sign, which goes into the scale.
 template <int L>

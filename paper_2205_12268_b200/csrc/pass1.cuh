@@ -7,8 +7,8 @@
 // that builds the norms (one per position, ascending channel order) runs in sequence: the eight partial sums of every lane
 // travel from the warp of box r to the warp of box r + 1 through shared memory (a "token", signalled on an mbarrier), so the
 // sums are the chains a single thread would build.  A slot belongs to the receiving warp; it is free again when it is
-// written next, because the chain has passed through its owner since.  The transform runs without its halvings; one exact
-// factor per slot at the end.  The last step (maxima over the warps, stores, histograms) is shared by the warps.
+// written next, because the chain has passed through its owner since.  Where only norms and maxima are built, the transform
+// runs without its halvings; one exact factor per slot at the end.  The last step (maxima over the warps, stores, histograms) is shared by the warps.
 //
 // Measured (B200, whole layer before -> after; the pass it replaced fed TMA rings in shared memory): 144 -> 24 bf16 37.3 -> 34.4
 // us, 384 -> 512 bf16 59.4 -> 56.2, six-layer chain 393 -> 377, 24 images of C4 131 -> 125; transform, selection and inverse of
@@ -44,6 +44,8 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
                                                        // is loaded channel by channel, one ahead)
     constexpr int S = 8 / ((NW < 4) ? NW : 4);         // slots a warp finishes at the end
     constexpr bool MAXV = KIND != P1_NORMS;
+    // Coefficients that are stored, and all behind a convolution (bound by other things), are transformed with the halvings.
+    constexpr bool HALVE = KIND == P1_COEF || DW;
     using TT = HaarTile<L>;
     __shared__ float4 token[(NW > 1) ? NW : 1][2][32];          // eight sums per lane, per receiving warp
     __shared__ float fin[(NW > 1) ? NW + 1 : 1][8][32];         // maxima per warp, norms
@@ -134,10 +136,10 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
                     dw.conv(st & 1, ch, k, ll[d], o[d]);
                 }
             }
-            fwd_levels<L, NB>(ll, o, lane);
+            fwd_levels<L, NB, HALVE>(ll, o, lane);
         } else {
 #pragma unroll
-        for (int g = 0; g < NB; g += 4) fwd_group<T, L, 4>(raw[b] + g, *reinterpret_cast<float(*)[4][8]>(&o[g]), lane);
+        for (int g = 0; g < NB; g += 4) fwd_group<T, L, 4, HALVE>(raw[b] + g, *reinterpret_cast<float(*)[4][8]>(&o[g]), lane);
         if (r + NW * D < rounds) {                     // the words of this box are consumed: the next box goes into their registers
             if ((r + NW * D) * NB + NB <= C) ldg_group<T, VEC, true, false, NB>(xb, plane, off, (r + NW * D) * NB, C, raw[b]);
             else ldg_group<T, VEC, true, true, NB>(xb, plane, off, (r + NW * D) * NB, C, raw[b]);
@@ -154,12 +156,7 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
         if (KIND == P1_COEF) {
 #pragma unroll
             for (int d = 0; d < NB; ++d) {
-                if (r * NB + d < C) {
-                    float oc[8];
-#pragma unroll
-                    for (int s = 0; s < 8; ++s) oc[s] = __fmul_rn(o[d][s], sc[s]);
-                    store_slots<L, VEC>(coef + ((size_t)n * C + r * NB + d) * P, lp, oc);
-                }
+                if (r * NB + d < C) store_slots<L, VEC>(coef + ((size_t)n * C + r * NB + d) * P, lp, o[d]);
             }
         }
         if (MAXV) {
@@ -216,12 +213,13 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
 #pragma unroll
         for (int i = 0; i < S; ++i) {
             const int s = F + i;
-            v[i] = __fmul_rn((NW > 1) ? fin[NW][s][lane] : nacc[s], __fmul_rn(sc[s], sc[s]));
+            v[i] = (NW > 1) ? fin[NW][s][lane] : nacc[s];
+            if (!HALVE) v[i] = __fmul_rn(v[i], __fmul_rn(sc[s], sc[s]));
             if (MAXV) {
                 m[i] = (NW > 1) ? fin[0][s][lane] : amax[s];
 #pragma unroll
                 for (int w = 1; w < NW; ++w) m[i] = fmaxf(m[i], fin[w][s][lane]);
-                m[i] = __fmul_rn(m[i], sc[s]);
+                if (!HALVE) m[i] = __fmul_rn(m[i], sc[s]);
             }
         }
 #pragma unroll

@@ -99,7 +99,8 @@ __device__ __forceinline__ void ldg_group(uint64_t xb, size_t plane, const Patch
 }
 
 // Levels 2 and 3 of the forward transform: ll holds the level-1 sums of both quads of the lane, slots 6 and 7 come out.
-template <int L, int U>
+// HALVE: with the halvings of Eq. 3 (true coefficients); without, sums and differences (see slot_scales).
+template <int L, int U, bool HALVE = false>
 __device__ __forceinline__ void fwd_levels(const float2 (&ll)[U], float (&o)[U][8], int lane)
 {
     using TT = HaarTile<L>;
@@ -119,6 +120,7 @@ __device__ __forceinline__ void fwd_levels(const float2 (&ll)[U], float (&o)[U][
     for (int u = 0; u < U; ++u) {
         o[u][6] = __fmaf_rn(s[u], sg, ps[u]);
         o[u][7] = __fmaf_rn(dd[u], sg, pd[u]);
+        if (HALVE) { o[u][6] = __fmul_rn(o[u][6], 0.5f); o[u][7] = __fmul_rn(o[u][7], 0.5f); }
     }
     if (L == 3) {
         const float sgh = (cg & 1) == 0 ? 1.0f : -1.0f;
@@ -132,16 +134,28 @@ __device__ __forceinline__ void fwd_levels(const float2 (&ll)[U], float (&o)[U][
         for (int u = 0; u < U; ++u) q[u] = __shfl_xor_sync(0xFFFFFFFFu, t[u], 2 * TT::CG);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const float r = __fmaf_rn(t[u], sgv, q[u]);
+            float r = __fmaf_rn(t[u], sgv, q[u]);
+            if (HALVE) r = __fmul_rn(r, 0.5f);
             if (even) o[u][6] = r;
         }
     }
 }
 
-// Forward transform (sums and differences only, see slot_scales) from the loaded words.  fp32: the first step is scalar,
+// The first level from the sums and differences of both rows: low-pass values out, slots 0 to 5 (one level: all) written.
+template <int L, bool HALVE>
+__device__ __forceinline__ void fwd_first(float2 s0, float2 d0, float2 s1, float2 d1, float2& ll, float (&o)[8])
+{
+    ll = add2(s0, s1);
+    float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
+    if (HALVE) { ll = half2x(ll); y2 = half2x(y2); y3 = half2x(y3); y4 = half2x(y4); }
+    o[0] = y2.x; o[1] = y2.y; o[2] = y3.x; o[3] = y3.y; o[4] = y4.x; o[5] = y4.y;
+    if (L == 1) { o[6] = ll.x; o[7] = ll.y; }
+}
+
+// Forward transform from the loaded words.  fp32: the first step is scalar,
 // because packing (quad 0, quad 1) pairs out of vector loads would take a register move per word (45 instead of 35
 // instructions per patch); bf16 words are unpacked anyway, straight into the pairs.
-template <typename T, int L, int U>
+template <typename T, int L, int U, bool HALVE = false>
 __device__ __forceinline__ void fwd_group(const Raw<T>* raw, float (&o)[U][8], int lane)
 {
     float2 ll[U];
@@ -161,12 +175,9 @@ __device__ __forceinline__ void fwd_group(const Raw<T>* raw, float (&o)[U][8], i
             const float2 c = make_float2(bf16lo(raw[u].w[1][0]), bf16lo(raw[u].w[1][1])), d = make_float2(bf16hi(raw[u].w[1][0]), bf16hi(raw[u].w[1][1]));
             s0 = add2(a, b); d0 = diff2(a, b); s1 = add2(c, d); d1 = diff2(c, d);
         }
-        ll[u] = add2(s0, s1);
-        const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
-        o[u][0] = y2.x; o[u][1] = y2.y; o[u][2] = y3.x; o[u][3] = y3.y; o[u][4] = y4.x; o[u][5] = y4.y;
-        if (L == 1) { o[u][6] = ll[u].x; o[u][7] = ll[u].y; }
+        fwd_first<L, HALVE>(s0, d0, s1, d1, ll[u], o[u]);
     }
-    fwd_levels<L, U>(ll, o, lane);
+    fwd_levels<L, U, HALVE>(ll, o, lane);
 }
 
 // Inverse of slots already multiplied by slot_scales.  fp32: the last step is scalar (the four values of a row leave as one
@@ -382,11 +393,7 @@ struct DwTile {
                 d[q] = __ffma2_rn(k[3 * i + 2], p3, d[q]);
             }
         }
-        const float2 s0 = add2(e[0], d[0]), d0 = diff2(e[0], d[0]), s1 = add2(e[1], d[1]), d1 = diff2(e[1], d[1]);
-        ll = add2(s0, s1);
-        const float2 y2 = add2(d0, d1), y3 = diff2(s0, s1), y4 = diff2(d0, d1);
-        o[0] = y2.x; o[1] = y2.y; o[2] = y3.x; o[3] = y3.y; o[4] = y4.x; o[5] = y4.y;
-        if (L == 1) { o[6] = ll.x; o[7] = ll.y; }
+        fwd_first<L, true>(add2(e[0], d[0]), diff2(e[0], d[0]), add2(e[1], d[1]), diff2(e[1], d[1]), ll, o);
     }
 };
 

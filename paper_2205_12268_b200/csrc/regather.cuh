@@ -59,6 +59,10 @@ regather_quant_kernel(const T* __restrict__ x, const float* __restrict__ taps, c
     if (!__any_sync(0xFFFFFFFFu, any ? 1 : 0)) return;                // nothing kept in this tile
     float mul[8];
     slot_scales<L>(lane, false, mul);                  // the halvings of the transform and the quantizer's factor in one
+    if (DW) {                                          // (behind a convolution the transform halves, as in the first pass)
+#pragma unroll
+        for (int s = 0; s < 8; ++s) mul[s] = 1.0f;
+    }
     if (QUANT) {
         const float amax = *amax_kept;
         const float inv = (amax > 0.0f) ? __fdiv_rn(qmax, amax) : 0.0f;
@@ -84,7 +88,7 @@ regather_quant_kernel(const T* __restrict__ x, const float* __restrict__ taps, c
                     dw.conv(st & 1, ch, kk, ll[st * Dw::CHS + ch], o[st * Dw::CHS + ch]);
                 }
             }
-            fwd_levels<L, 4>(ll, o, lane);
+            fwd_levels<L, 4, true>(ll, o, lane);
         } else {
             fwd_group<T, L, 4>(raw + (g * 4) % NB, o, lane);
             if ((g * 4 + 4) % NB == 0 && g * 4 + 4 < CH) ldg_group<T, VEC, true, true, NB>(xb, plane, off, c0 + g * 4 + 4, C, raw);
