@@ -286,8 +286,9 @@ __device__ __forceinline__ void store_patch(T* __restrict__ plane, int W, const 
     }
 }
 
-// Store the eight slots of a lane into a quadrant-layout fp32 plane.
-template <int L, bool VEC>
+// Store the eight slots of a lane into a quadrant-layout fp32 plane.  PAIRS: rows of 4m + 2 store the pairs of the left half, whose
+// positions are even, as one (coef_kernel; pass1_kernel is faster without: 12 against 16 us on 293 channels of 4 x 60 x 106 fp32).
+template <int L, bool VEC, bool PAIRS = false>
 __device__ __forceinline__ void store_slots(float* __restrict__ plane, const LanePos& lp, const float (&o)[8])
 {
     if (VEC) {   // W % 4 == 0: both quads valid together and the pairs are 8-byte aligned
@@ -304,8 +305,13 @@ __device__ __forceinline__ void store_slots(float* __restrict__ plane, const Lan
         }
     } else {
 #pragma unroll
-        for (int s = 0; s < 8; ++s)
-            if (slot_ok<L>(lp, s)) plane[lp.pos[s]] = o[s];
+        for (int s = 0; s < 8; s += 2) {
+            if (PAIRS && (s & 2) && lp.ok1) *reinterpret_cast<float2*>(plane + lp.pos[s]) = make_float2(o[s], o[s + 1]);
+            else {
+                if (slot_ok<L>(lp, s)) plane[lp.pos[s]] = o[s];
+                if (slot_ok<L>(lp, s + 1)) plane[lp.pos[s + 1]] = o[s + 1];
+            }
+        }
     }
 }
 
@@ -383,9 +389,9 @@ static wcc_status launch_coef_norms(const float* coef, int N, int C, long long P
 }
 
 // ---- plain inverse -------------------------------------------------------------------------------
-// One warp per (plane, tile).
+// One warp per (plane, tile), four or sixteen to a block.
 template <typename T, int L, bool VEC>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(512)
 haar_inv_kernel(const float* __restrict__ coef, int planes, int H, int W, T* __restrict__ out)
 {
     pdl_wait();
@@ -424,8 +430,12 @@ static wcc_status haar_inv_dispatch(const float* coef, int planes, int H, int W,
 {
     using TT = HaarTile<L>;
     const long long warps = (long long)planes * ceil_div(W, TT::TW) * (H / TT::TH);
-    const int blocks = (int)((warps + 3) / 4);
-    return launch_overlapped(haar_inv_kernel<T, L, VEC>, dim3(blocks), dim3(128), 0, st, true, 1, coef, planes, H, W, static_cast<T*>(out));
+    // Blocks that wait for the launch before them come and go at one a nanosecond at most.  Four warps move up to 6 or 8 KB, as much
+    // as memory does in that time, where the tiles are full; tiles that are not take sixteen warps a block (148 x 14 planes of
+    // 346 x 16 bf16 92 -> 66 us; 64 x 180 x 360, full, 3 images of it as blocks of sixteen 62.7 instead of 56.1 for the case).
+    const int wpb = (long long)W * (4 + (int)sizeof(T)) * 2 >= 11LL * ceil_div(W, TT::TW) * TT::TW ? 4 : 16;
+    const int blocks = (int)((warps + wpb - 1) / wpb);
+    return launch_overlapped(haar_inv_kernel<T, L, VEC>, dim3(blocks), dim3(32 * wpb), 0, st, true, 1, coef, planes, H, W, static_cast<T*>(out));
 }
 
 wcc_status launch_haar_inv(const float* coef, int N, int C, int H, int W, int L, wcc_dtype dt,

@@ -15,6 +15,8 @@
 // 4 x 64 x 192 x 320 fp32 80 -> 70 (the norms no longer take a pass over the stored coefficients).
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "gather.cuh"
 #include "patch.cuh"
@@ -323,13 +325,167 @@ static wcc_status launch_pass1(const void* x, const float* taps, int N, int C, i
     WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
 }
 
+// ---- coefficients alone ----------------------------------------------------------------------------
+// One warp per (tile, `cpc` channels), four channels at a time, the next four in flight.  NORMS: the warp has all channels and
+// builds norms and maxima as well; otherwise they are built afterwards from the stored map: free of the norms' chain, the
+// channels of a few tiles spread over the whole chip.
+template <typename T, int L, bool VEC, bool DW, bool NORMS>
+__global__ void __launch_bounds__(128)
+coef_kernel(const T* __restrict__ x, const float* __restrict__ taps, int N, int C, int H, int W, int cpc, float* __restrict__ coef,
+            float* __restrict__ nrm2, float* __restrict__ amaxpos)
+{
+    using TT = HaarTile<L>;
+    using Dw = DwTile<T, L, VEC>;
+    __shared__ __align__(16) float2 tap_sm[DW ? 4 : 1][4 * 10];
+    __shared__ __align__(16) uint8_t dw_sm[DW ? 4 : 1][DW ? Dw::BYTES : 16];
+    pdl_wait();
+    pdl_launch();
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int tiles_x = (W + TT::TW - 1) / TT::TW, tiles_y = H / TT::TH;
+    const long long gw = (long long)blockIdx.x * 4 + warp;
+    if (gw >= (long long)N * tiles_x * tiles_y) return;
+    const int c_lo = (int)blockIdx.y * cpc, c_hi = min(C, c_lo + cpc);
+    int n, ty, tx;
+    tile_coords((int)gw, tiles_x, tiles_y, n, ty, tx);
+    const LanePos lp = lane_positions<L>(H, W, ty, tx, lane);
+    const size_t P = (size_t)H * W, plane = P * sizeof(T);
+    const uint64_t xb = reinterpret_cast<uint64_t>(x) + (uint64_t)n * C * plane;
+    float* out = coef + ((size_t)n * C + c_lo) * P;
+    const PatchOff off = patch_off<T>(lp, W);
+    Raw<T> raw[DW ? 1 : 4];
+    uint32_t piece[DW ? Dw::CHS : 1][DW ? Dw::IT : 1][DW ? Dw::PW : 1];
+    Dw dw;
+    if constexpr (DW) {
+        dw.init(dw_sm[warp], H, W, ty, tx, lane);
+        dw.load(xb, plane, c_lo, C, piece);
+    } else {
+        ldg_group<T, VEC, true, true, 4>(xb, plane, off, c_lo, C, raw);
+    }
+    float nacc[8], amax[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) { nacc[s] = 0.0f; amax[s] = 0.0f; }
+    for (int c = c_lo; c < c_hi; c += 4) {
+        float o[4][8];
+        if constexpr (DW) {
+            float2 ll[4];
+            __syncwarp();                              // the taps of the group before are read
+            dw_stage_taps(taps, c, 4, C, tap_sm[warp], lane);
+#pragma unroll
+            for (int st = 0; st < 4 / Dw::CHS; ++st) {
+                dw.store(st & 1, piece);
+                __syncwarp();
+                const int cn = c + (st + 1) * Dw::CHS;
+                if (cn < c_hi) dw.load(xb, plane, cn, C, piece);
+#pragma unroll
+                for (int ch = 0; ch < Dw::CHS; ++ch) {
+                    const int d = st * Dw::CHS + ch;
+                    float2 k[10];
+                    dw_read_taps(tap_sm[warp] + d * 10, k);
+                    dw.conv(st & 1, ch, k, ll[d], o[d]);
+                }
+            }
+            fwd_levels<L, 4, true>(ll, o, lane);
+        } else {
+            fwd_group<T, L, 4, true>(raw, o, lane);
+            if (c + 4 < c_hi) {
+                if (c + 8 <= C) ldg_group<T, VEC, true, false, 4>(xb, plane, off, c + 4, C, raw);
+                else ldg_group<T, VEC, true, true, 4>(xb, plane, off, c + 4, C, raw);
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            if (c + d < c_hi) {
+                store_slots<L, VEC, true>(out, lp, o[d]);
+                if (NORMS) {
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) {
+                        nacc[s] = __fmaf_rn(o[d][s], o[d][s], nacc[s]);
+                        amax[s] = fmaxf(amax[s], fabsf(o[d][s]));
+                    }
+                }
+            }
+            out += P;
+        }
+    }
+    if (NORMS) {
+        if (nrm2) store_slots<L, VEC>(nrm2 + (size_t)n * P, lp, nacc);
+        if (amaxpos) store_slots<L, VEC>(amaxpos + (size_t)n * P, lp, amax);
+    }
+}
+
+// How wcc_haar_fwd and its depthwise form split the channels of a tile.  0: pass1_kernel; 1: coefficients, norms and maxima by one
+// warp; more: that many chunks, about 64 warps per SM, and the norms from the stored map.  Measured on some 500 drawn shapes
+// (geometric means of pass1_kernel's time over the other's; `sparse`: the map's rows fill less than 5/8 of its tiles):
+//  - rows of vectors: chunks 0.6 to 0.9, but 1.3 (fp32) and 1.6 (bf16) from four tiles per SM on with 257 channels, 1.1 and 1.7
+//    from eight on with 97; one warp 1.5 up to eight channels from eight tiles per SM on;
+//  - rows of 4m + 2: fp32 0.6 to 0.9 for chunks (1.2 to 1.3 from four tiles per SM and 97 channels on where the tiles are less
+//    than 5/8 full) and at most 1.1 for one warp; bf16, where the element-wise accesses and the norms
+//    together keep a warp busy, one warp 1.2 to 1.8 up to 16 channels, 1.05 to 1.8 up to 32 from one tile per SM on and 1.15 to
+//    1.7 up to 96 from two on, chunks 1.2 to 2.3 from 97 channels on (145 channels of 17 x 36 x 146: 60 against 24 us);
+//  - behind a convolution, where few warps per SM cost more, rows of vectors: one warp 1.2 to 1.4 up to 32 channels from eight
+//    tiles per SM on; chunks 1.1 to 1.9 below half a tile per SM from 97 channels on in fp32 and 1.04 to 1.4 from 257 on in bf16,
+//    1.05 to 1.2 with 257 from one per SM and with 97 from four per SM on.  Rows of 4m + 2: fp32 one warp 1.2 up to 32 channels
+//    from eight tiles per SM on, chunks 1.0 to 2.3 from 97 channels on; bf16 chunks 1.2 to 2.6 from 97 channels on below two
+//    tiles per SM (0.9 above).
+template <typename T, bool VEC>
+static int channel_chunks(bool dw, long long tiles, bool sparse, int C, int sms)
+{
+    const bool b16 = sizeof(T) == 2, many = tiles >= 4 * sms, most = tiles >= 8 * sms;
+    bool one = false, split = false;
+    if (dw) {
+        one = most && C <= 32 && (VEC || !b16);
+        if (!VEC) split = C >= 97 && (!b16 || tiles < 2 * sms);
+        else if (many) split = C >= 97;
+        else if (tiles * 2 < sms) split = C >= (b16 ? 257 : 97);
+        else split = tiles >= sms && C >= 257;
+    } else if (VEC) {
+        one = most && C <= 8;
+        split = (many && C >= 257) || (most && C >= 97);
+    } else if (b16) {
+        one = C <= 16 || (C <= 32 && tiles >= sms) || (C <= 96 && tiles >= 2 * sms);
+        split = C >= 97;
+    } else {
+        split = sparse && many && C >= 97;
+    }
+    if (one) return 1;
+    return split ? (int)std::min<long long>(ceil_div(C, 4), (64LL * sms + tiles - 1) / tiles) : 0;
+}
+
+template <typename T, int L, bool VEC, bool DW>
+static wcc_status coef_launch(const void* x, const float* taps, int N, int C, int H, int W, long long tiles, int chunks, float* coef, float* nrm2, float* amaxpos,
+                              cudaStream_t st)
+{
+    const int cpc = ceil_div(ceil_div(C, chunks), 4) * 4;
+    auto go = [&](auto kern) {
+        return launch_overlapped(kern, dim3((unsigned)((tiles + 3) / 4), (unsigned)ceil_div(C, cpc)), dim3(128), 0, st, true, 1, static_cast<const T*>(x), taps, N,
+                                 C, H, W, cpc, coef, nrm2, amaxpos);
+    };
+    if (chunks == 1) return go(coef_kernel<T, L, VEC, DW, true>);
+    const wcc_status s = go(coef_kernel<T, L, VEC, DW, false>);
+    return s != WCC_OK ? s : launch_coef_norms(coef, N, C, (long long)H * W, nrm2, amaxpos, st);
+}
+
+template <typename T, int L, bool VEC>
+static wcc_status haar_fwd_dispatch(const void* x, const float* taps, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, cudaStream_t st)
+{
+    using TT = HaarTile<L>;
+    const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
+    if (tiles > 0x7FFFFFFFLL) return WCC_ERR_SHAPE;
+    DeviceInfo di;
+    wcc_status s = device_info(di);
+    if (s != WCC_OK) return s;
+    const int chunks = channel_chunks<T, VEC>(taps != nullptr, tiles, W * 8LL < 5LL * ceil_div(W, TT::TW) * TT::TW, C, di.sms);
+    if (!chunks) return pass1_dispatch<T, L, VEC>(x, taps, N, C, H, W, coef, nrm2, amaxpos, NormsExtra{}, st);
+    return taps ? coef_launch<T, L, VEC, true>(x, taps, N, C, H, W, tiles, chunks, coef, nrm2, amaxpos, st)
+                : coef_launch<T, L, VEC, false>(x, taps, N, C, H, W, tiles, chunks, coef, nrm2, amaxpos, st);
+}
+
 // Forward transform with stored coefficients, after the depthwise convolution if taps are given; nrm2 and amaxpos may be NULL.
 wcc_status launch_haar_fwd(const void* x, const float* taps, int N, int C, int H, int W, int L, wcc_dtype dt, float* coef, float* nrm2,
                            float* amaxpos, cudaStream_t st)
 {
     const bool vec = (W % 4) == 0;                     // always true for L >= 2
-    const NormsExtra ex = {};
-    WCC_DISPATCH_TLV(pass1_dispatch, dt, L, vec, x, taps, N, C, H, W, coef, nrm2, amaxpos, ex, st);
+    WCC_DISPATCH_TLV(haar_fwd_dispatch, dt, L, vec, x, taps, N, C, H, W, coef, nrm2, amaxpos, st);
 }
 
 }  // namespace wcc
