@@ -40,7 +40,8 @@ static wcc_status check_forward_args(int N, int Cin, int Cout, int H, int W, int
 
 // Run the second pass as one kernel, or gather the kept columns and contract only those (wide_impl)?
 //  - K in one piece: one kernel up to 72 K steps over all chunks of output channels (bf16 input, one kernel / gathered, us:
-//    128 -> 1024 on 2 x 64 x 128 54 / 65, 180 -> 512 on 2 x 64 x 64 48 / 50; the other way 192 -> 1024 on 2 x 64 x 128 89 / 65).
+//    128 -> 1024 on 2 x 64 x 128 54 / 65; the other way 192 -> 1024 there 89 / 65), but below 40 tile groups gathered where a CTA
+//    goes through sixteen and more (173 -> 289 on 2 x 16 x 412 53 / 32, 148 -> 201 with 39 groups 39 / 37).
 //  - K in parts, and no CTA rebuilds its operand for a further chunk (all channels fit one, or the CTAs that share a tile group
 //    take one each): one kernel up to ten K steps (256 -> 64 on 8 x 64 x 128 40 / 49, 256 -> 256 on 2 x 64 x 128 37 / 39), up
 //    to sixteen from 64 tile groups on (384 -> 64 on 8 x 64 x 128 58 / 60; with 28 groups 31 / 26).
@@ -55,10 +56,11 @@ static bool one_kernel(int N, int Cin, int Cout, int H, int W, int L, int k, int
     const P2Plan p = p2_plan_of(4, Cout, krow, i8, L);
     if (!p.ok) return false;
     const int chunks = ceil_div(p.npad, p.nchunk), parts = ceil_div(ksteps, p.ksteps_part);
-    if (parts == 1) return chunks * ksteps <= 72;
     const long long groups = ((long long)N * ceil_div(W, 128 >> (L - 1)) * (H >> L) + p2::TILES - 1) / p2::TILES;
     const int share = groups > B200_SMS ? 1 : p2_shares(groups, B200_SMS, p.npad);
-    if (ceil_div(p.npad / share, p.nchunk) == 1) return ksteps <= 10 || (ksteps <= 16 && groups >= 64);
+    const int cta_chunks = ceil_div(p.npad / share, p.nchunk);
+    if (parts == 1) return chunks * ksteps <= 72 && (cta_chunks * ksteps < 16 || groups >= 40);
+    if (cta_chunks == 1) return ksteps <= 10 || (ksteps <= 16 && groups >= 64);
     return parts == 2 && ksteps <= 8 && chunks <= 4 && 2LL * k >= (long long)H * W && groups >= 64;
 }
 
