@@ -652,23 +652,34 @@ static WaveletWs carve_wavelet_ws(void* ws, int N, int Cin, int Cout, int H, int
 }
 
 // ---- inverted residual block -------------------------------------------------------------------------
-struct BlockWs { void* u; void* layer_ws; size_t layer_off; size_t least, total; };
+// Does the second layer of a block store its coefficients?  That convolves once instead of twice, for a coefficient written and
+// gathered.  Measured with at least 600 channels: fp32 1.06 to 1.3 times as fast (1422 channels of 6 x 32 x 124 364 / 276 us), bf16 1.1 to 1.5 from 320 tiles on (1698 channels of 15 x 132 x 16
+// 877 / 573) and within 5 % below (1024 channels of 4 x 128 x 128 370 / 361); with fewer channels 0.8 to 1.1.
+static bool block_stores_coefficients(int N, int E, int H, int W, int L, wcc_dtype dt)
+{
+    const long long tiles = (long long)N * ceil_div(W, 128 >> (L - 1)) * (H >> L);
+    return E >= 600 && (dt == WCC_F32 || tiles >= 320);
+}
+
+struct BlockWs { void* u; void* layer_ws; size_t layer_off, stored_bytes, gathered_bytes; size_t least, total; };      // gathered_bytes: 0 if not possible
 
 static BlockWs carve_block_ws(void* ws, int N, int C, int E, int H, int W, int L, int k, int bits, wcc_dtype dt)
 {
     BlockWs b = {};
     const size_t es = (dt == WCC_BF16) ? 2 : 4;
     const size_t w1 = wcc_workspace_bytes(N, C, E, H, W, L, k, bits, dt);
-    const size_t w3 = wide_fits(E, C, H, W, bits) ? carve_wide_ws(nullptr, N, E, C, H, W, k, bits).total
-                                                  : wcc_staged_workspace_bytes(N, E, C, H, W, L, k, bits, dt);
-    if (w1 == 0 || w3 == 0) return b;
+    b.stored_bytes = wcc_staged_workspace_bytes(N, E, C, H, W, L, k, bits, dt);
+    b.gathered_bytes = wide_fits(E, C, H, W, bits) ? carve_wide_ws(nullptr, N, E, C, H, W, k, bits).total : 0;
+    const size_t w3 = b.gathered_bytes && !block_stores_coefficients(N, E, H, W, L, dt) ? b.gathered_bytes : b.stored_bytes;
+    if (w1 == 0 || b.stored_bytes == 0) return b;
     char* base = static_cast<char*>(ws);
     size_t off = 0;
     auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align_up(bytes, 256); return p; };
     b.u = take((size_t)N * E * H * W * es);
     b.layer_off = off;
     const size_t l1 = least_workspace_bytes(w1, N, C, E, H, W, L, k, bits);
-    b.least = off + (l1 > w3 ? l1 : w3);
+    const size_t l3 = b.gathered_bytes && b.gathered_bytes < b.stored_bytes ? b.gathered_bytes : b.stored_bytes;
+    b.least = off + (l1 > l3 ? l1 : l3);
     b.layer_ws = take(w1 > w3 ? w1 : w3);
     b.total = off;
     return b;
@@ -845,12 +856,12 @@ wcc_status wcc_block_forward(const void* x, const float* W1, const float* Wdw, c
     // u = WCC(W1, x): C -> E channels
     s = forward_impl(x, W1, N, C, E, H, Wd, levels, k, bits, b.u, dt, b.layer_ws, layer_ws_bytes, st, nullptr);
     if (s != WCC_OK) return s;
-    // y = x + WCC(W3, dw3x3(u)): the depthwise convolution is fused with the second layer's transform.  Convolving and
-    // transforming u again for the kept columns is cheaper than keeping the coefficients (4 bytes each, written once, gathered
-    // over nearly all of their sectors).
+    // y = x + WCC(W3, dw3x3(u)): the depthwise convolution is fused with the second layer's transform, once with its coefficients
+    // stored or twice, the second time for the kept columns only
     wcc_options o = {};
     o.residual = x;
-    if (wide_fits(E, C, H, Wd, bits))
+    const bool prefer_stored = block_stores_coefficients(N, E, H, Wd, levels, dt);
+    if (b.gathered_bytes && layer_ws_bytes >= b.gathered_bytes && !(prefer_stored && layer_ws_bytes >= b.stored_bytes))
         return wide_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, layer_ws_bytes, st, nullptr, &o, Wdw);
     return staged_impl(b.u, W3, N, E, C, H, Wd, levels, k, bits, y, dt, b.layer_ws, layer_ws_bytes, st, nullptr, &o, Wdw);
 }

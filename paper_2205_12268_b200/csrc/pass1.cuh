@@ -424,7 +424,8 @@ coef_kernel(const T* __restrict__ x, const float* __restrict__ taps, int N, int 
 //    1.7 up to 96 from two on, chunks 1.2 to 2.3 from 97 channels on (145 channels of 17 x 36 x 146: 60 against 24 us);
 //  - behind a convolution, where few warps per SM cost more, rows of vectors: one warp 1.2 to 1.4 up to 32 channels from eight
 //    tiles per SM on; chunks 1.1 to 1.9 below half a tile per SM from 97 channels on in fp32 and 1.04 to 1.4 from 257 on in bf16,
-//    1.05 to 1.2 with 257 from one per SM and with 97 from four per SM on.  Rows of 4m + 2: fp32 one warp 1.2 up to 32 channels
+//    1.05 to 1.2 with 257 from one per SM and with 97 from four per SM on; fp32 with 600 everywhere, for the second layer of a
+//    block (1422 channels of 6 x 32 x 124 there 223 against about 130 us).  Rows of 4m + 2: fp32 one warp 1.2 up to 32 channels
 //    from eight tiles per SM on, chunks 1.0 to 2.3 from 97 channels on; bf16 chunks 1.2 to 2.6 from 97 channels on below two
 //    tiles per SM (0.9 above).
 template <typename T, bool VEC>
@@ -437,7 +438,7 @@ static int channel_chunks(bool dw, long long tiles, bool sparse, int C, int sms)
         if (!VEC) split = C >= 97 && (!b16 || tiles < 2 * sms);
         else if (many) split = C >= 97;
         else if (tiles * 2 < sms) split = C >= (b16 ? 257 : 97);
-        else split = tiles >= sms && C >= 257;
+        else split = (tiles >= sms && C >= 257) || (!b16 && C >= 600);
     } else if (VEC) {
         one = most && C <= 8;
         split = (many && C >= 257) || (most && C >= 97);
