@@ -1,4 +1,5 @@
 // libwcc: C-ABI entry points (see include/wcc.h).  One translation unit: the kernels live in the *.cuh files.
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -581,12 +582,17 @@ crop_planes_kernel(const E* __restrict__ src, uint64_t total, int H, int W, int 
 template <typename E>
 static wcc_status launch_pad(const void* src, long long planes, int H, int W, int Hp, int Wp, void* dst, cudaStream_t st)
 {
-    const long long rows = planes * Hp;
-    if (rows > 0xFFFFFFF0LL) return WCC_ERR_SHAPE;
+    const long long most = 0xFFFFFFF0LL / Hp;          // planes whose rows a launch can number in 32 bits (Hp is at most 2^30)
     auto go = [&](auto vec) -> wcc_status {
         constexpr int V = decltype(vec)::value;
-        return launch_overlapped(pad_planes_kernel<E, V>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, true, 1, static_cast<const E*>(src),
-                                 (uint32_t)rows, H, W, Hp, (uint32_t)(Wp / V), static_cast<E*>(dst));
+        for (long long p0 = 0; p0 < planes; p0 += most) {
+            const long long rows = std::min(planes - p0, most) * Hp;
+            const wcc_status s = launch_overlapped(pad_planes_kernel<E, V>, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, st, true, 1,
+                                                   static_cast<const E*>(src) + p0 * H * W, (uint32_t)rows, H, W, Hp, (uint32_t)(Wp / V),
+                                                   static_cast<E*>(dst) + p0 * Hp * Wp);
+            if (s != WCC_OK) return s;
+        }
+        return WCC_OK;
     };
     if (sizeof(E) == 2 && Wp % 8 == 0) return go(std::integral_constant<int, 16 / sizeof(E)>{});
     if (Wp % 4 == 0) return go(std::integral_constant<int, 4>{});

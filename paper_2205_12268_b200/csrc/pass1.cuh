@@ -278,7 +278,7 @@ static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, i
 {
     using TT = HaarTile<L>;
     const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
-    if (tiles > 0x3FFFFFFFLL) return WCC_ERR_SHAPE;
+    if (tiles > 0x7FFFFFFFLL - WCC_MAX_CHANNELS) return WCC_ERR_SHAPE;        // (blocks of a grid, those of the weights among them)
     DeviceInfo di;
     wcc_status s = device_info(di);
     if (s != WCC_OK) return s;
