@@ -144,9 +144,14 @@ def _dt(t: torch.Tensor) -> int:
     raise TypeError("activations must be float32 or bfloat16, got %s" % t.dtype)
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
-    """Handle of the current stream (without the Stream object that torch.cuda.current_stream() builds around it)."""
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    """Handle of the current stream, where torch has a call for it without the Stream object of current_stream()."""
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t):
