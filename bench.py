@@ -33,12 +33,8 @@ STAGE_FILES = ("haar.cuh", "pass1.cuh", "select.cuh", "gather.cuh", "regather.cu
 # DRAM bytes per launch of the dominant kernel from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum),
 # keyed by (workload, stage); valid only while the kernel sources still hash to `src`.
 NCU_TRAFFIC = {
-    # dram__bytes_read.sum + dram__bytes_write.sum of one launch, from the ncu captures summarised under profiles/.
-    # C4 was captured with N=24 images (x = 189 MB > L2) and is divided by 2, C2 with N=16 and divided by 4: every stage
-    # is per image, so traffic grows in proportion to the batch.
-    ("C4", "fused_pass2"): {"bytes": (191.8e6 + 131.6e6) / 2, "src": "56e867d58c48"},
-    ("C4", "haar_norms"): {"bytes": (189.2e6 + 5.2e6) / 2, "src": "56e867d58c48"},
-    ("C2", "fused_pass2"): {"bytes": (153.2e6 + 8.4e6) / 4, "src": "56e867d58c48"},
+    # (workload, stage): {"bytes": dram__bytes_read.sum + dram__bytes_write.sum per launch, "src": _source_hash()}.  None for the
+    # present sources: what an earlier capture wrote to DRAM left out the part of y that the L2 still held when the launch ended.
 }
 
 

@@ -22,9 +22,9 @@
  *    along the width) top-right, y3 (difference along the height) bottom-left, y4 bottom-right.
  *    A "position" p = row * Wd + col indexes this layout; P = H * Wd.
  *  - levels is 1, 2 or 3 (the paper uses 3); H and Wd must be multiples of 2^levels.
- *  - Cin, Cout <= WCC_MAX_CHANNELS.  wcc_forward runs its fused two-pass kernels while the operands of one tile group
- *    fit one SM's shared memory and tensor memory (up to 256 channels on the quantized path) and otherwise the
- *    stage-by-stage pipeline of wcc_forward_staged, whose contraction tiles K and N; wcc_workspace_bytes accounts for it.
+ *  - Cin, Cout <= WCC_MAX_CHANNELS.  wcc_forward runs its fused two-pass kernels while the operands of one tile group need not
+ *    be rebuilt for every chunk of output channels, and otherwise two passes around a contraction of the kept columns that
+ *    tiles K and N (maps beyond 131072 positions: the stage-by-stage pipeline); wcc_workspace_bytes accounts for it.
  *  - There is no CPU fallback: the library is built for sm_100a only.
  */
 #ifndef WCC_H_
@@ -206,7 +206,8 @@ wcc_status wcc_forward_padded(const void* x, const float* Wt, int N, int Cin, in
  *                connection of the inverted residual block (Eq. 13); one fp32 addition per element.  May be y itself.
  *   Wq, scale_w  NULL, or the weights already quantized (DEVICE): int8 [Cout][wcc_kpad(Cin, bits)], rows zero padded,
  *                and fp32 [Cout] scales (what taps Wq / scale_w return).  Static weights need quantizing only once;
- *                Wt is then not read and may be NULL.  Only with bits >= 2.
+ *                Wt is then not read and may be NULL.  Only with bits >= 2.  Such layers always run the fused kernels
+ *                (with K in parts where the channels need it; Cout up to about 6000).
  */
 typedef struct wcc_options {
     float alpha;
@@ -313,7 +314,8 @@ const char* wcc_status_str(wcc_status s);
 
 /*
  * Test hooks for the device-side timeout contract (no counterpart in the paper).  Every wait inside a kernel (on an
- * mbarrier of a TMA ring, of the tensor-core pipeline, on the arrival counter of the cooperative select) polls a
+ * mbarrier of the tensor-core pipeline, of its TMA ring or of the hand-over between the warps of a tile, on the arrival counter
+ * of the cooperative select) polls a
  * bounded number of times, then the kernel records WCC_ERR_TIMEOUT, lets its copies in flight land, frees its TMEM
  * and returns; nothing traps or faults.
  *   wcc_debug_set_wait_limit  sets the number of polls (each suspends for up to about a microsecond) on the current

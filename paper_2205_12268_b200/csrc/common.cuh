@@ -53,7 +53,7 @@ __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.laun
 
 // What launches need to know about the current device, looked up once per device: each of these calls costs a few hundred
 // nanoseconds, and a small layer is over in 16 us.
-constexpr int B200_SMS = 148;           // where a decision is made without a device (sizes of workspaces)
+constexpr int B200_SMS = 148;           // for decisions that need no device (sizes of workspaces), or only its size
 constexpr int MAX_DEVICES = 64;
 struct DeviceInfo { int dev, sms; int* status; };
 static wcc_status device_info(DeviceInfo& d)
@@ -164,12 +164,6 @@ __device__ __forceinline__ void hist_add(uint32_t* h, uint32_t bin, bool pred)
         if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&h[bin], (uint32_t)__popc(peers));
     }
 }
-
-// ---- geometry of one call -------------------------------------------------------------------
-struct Geom {
-    int N, C, H, W, L;
-    int P;          // H*W
-};
 
 // ---- stage launchers (each enqueues on `st`, returns a wcc_status) ---------------------------
 // Forward Haar + norms (+ per-position max |coef| over channels when amaxpos != NULL).

@@ -102,7 +102,7 @@ wcc_status launch_gather_quant(const float* coef, const int32_t* idx, const floa
     const int M = N * k;
     const float qmax = (bits >= 2) ? (float)((1 << (bits - 1)) - 1) : 1.0f;
     // rows alone fill the GPU from about 150 K kept positions on; below that the channels are split as well
-    const int cpc = (M >= 148 * 1024) ? kpad : 64;
+    const int cpc = (M >= B200_SMS * 1024) ? kpad : 64;
     const dim3 grid(ceil_div(M, 128), ceil_div(kpad, cpc));
     if (bits >= 2)
         gather_quant_kernel<true><<<grid, 128, 0, st>>>(coef, idx, amax_kept, M, Cin, P, k, kpad, cpc, qmax, Xq);

@@ -1,7 +1,7 @@
 // Haar kernels: channel norms of a stored map and the plain inverse (Eq. 3-6, Alg. 1), and the tile geometry all transforms share.
 // The forward transform of a feature map is in pass1.cuh, dequantize + scatter + inverse in scatter.cuh.
 //
-// Work decomposition (all three kernels).  One warp owns a tile of 2^L rows x TW columns of one image,
+// Work decomposition (all transforms).  One warp owns a tile of 2^L rows x TW columns of one image,
 // TW = 4 * CG, CG = 32 / 2^(L-1).  Lane (rp, cg) = (lane / CG, lane % CG) holds the 2 x 4 patch at rows
 // 2rp, 2rp+1 and columns 4cg..4cg+3 of the tile: level 1 is computed inside the lane, level 2 pairs the
 // lanes rp and rp^1 (lane ^ CG), level 3 combines the four lanes {rp, rp^2} x {cg, cg^1}.  After the
@@ -103,51 +103,6 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b)
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 half2x(float2 a) { return mul2(a, make_float2(0.5f, 0.5f)); }
 
-// Forward transform of the lane's patch p[row][col] into its eight slots.  The two quads of the patch are processed
-// side by side in packed pairs: (quad 0, quad 1).
-template <int L>
-__device__ __forceinline__ void haar_fwd_lane(const float (&p)[2][4], float (&o)[8], int lane)
-{
-    using T = HaarTile<L>;
-    const float2 a = make_float2(p[0][0], p[0][2]), b = make_float2(p[0][1], p[0][3]);
-    const float2 c = make_float2(p[1][0], p[1][2]), d = make_float2(p[1][1], p[1][3]);
-    const float2 s0 = add2(a, b), d0 = sub2(a, b), s1 = add2(c, d), d1 = sub2(c, d);
-    const float2 ll = half2x(add2(s0, s1));            // y1 of both quads
-    const float2 y2 = half2x(add2(d0, d1));
-    const float2 y3 = half2x(sub2(s0, s1));
-    const float2 y4 = half2x(sub2(d0, d1));
-    o[0] = y2.x; o[1] = y2.y; o[2] = y3.x; o[3] = y3.y; o[4] = y4.x; o[5] = y4.y;
-    if (L == 1) {
-        o[6] = ll.x;
-        o[7] = ll.y;
-        return;
-    }
-    // Level 2: the lane pair (rp, rp^1) holds the 2x2 block of level-1 low-pass values, one row each.  With
-    // sg = +1 on the upper (even) lane and -1 on the lower one, fma(own, sg, other) is own+other on the upper lane
-    // (s0+s1, d0+d1 -> y1, y2) and other-own on the lower lane (s0-s1, d0-d1 -> y3, y4): one rounding, as an add.
-    const int rp = lane / T::CG, cg = lane % T::CG;
-    const bool even = (rp & 1) == 0;
-    const float sg = even ? 1.0f : -1.0f;
-    const float s = __fadd_rn(ll.x, ll.y), dd = __fsub_rn(ll.x, ll.y);
-    const float ps = __shfl_xor_sync(0xFFFFFFFFu, s, T::CG);
-    const float pd = __shfl_xor_sync(0xFFFFFFFFu, dd, T::CG);
-    const float2 l2 = half2x(__ffma2_rn(make_float2(s, dd), make_float2(sg, sg), make_float2(ps, pd)));
-    o[6] = l2.x;                                       // even: y1, odd: y3
-    o[7] = l2.y;                                       // even: y2, odd: y4
-    if (L == 3) {
-        // Level 3: the four even lanes {rp, rp^2} x {cg, cg^1} hold a, b / c, d.  Horizontal step: left lane a+b (c+d),
-        // right lane a-b (c-d); vertical step: top lanes sum (y1, y2), bottom lanes difference (y3, y4).
-        const float sgh = (cg & 1) == 0 ? 1.0f : -1.0f;
-        const float sgv = (rp & 2) == 0 ? 1.0f : -1.0f;
-        const float v = o[6];
-        const float h = __shfl_xor_sync(0xFFFFFFFFu, v, 1);
-        const float t = __fmaf_rn(v, sgh, h);
-        const float q = __shfl_xor_sync(0xFFFFFFFFu, t, 2 * T::CG);
-        const float r = __fmul_rn(__fmaf_rn(t, sgv, q), 0.5f);
-        if (even) o[6] = r;
-    }
-}
-
 // Inverse transform of the lane's eight slots into its patch.
 template <int L>
 __device__ __forceinline__ void haar_inv_lane(const float (&o)[8], float (&p)[2][4], int lane)
@@ -190,77 +145,25 @@ __device__ __forceinline__ void haar_inv_lane(const float (&o)[8], float (&p)[2]
 // ---- transforms with the halvings taken out ------------------------------------------------------------
 // Multiplying by a power of two commutes with every rounding (barring overflow and subnormal results), so the forward
 // transform can run on sums and differences alone and leave one exact multiplication per slot to the consumer:
-// true coefficient of slot s = raw value * slot_scale[s], where |slot_scale| = 2^-level.  The same holds for squares
+// true coefficient of slot s = raw value * slot_scale[s], where slot_scale = 2^-level.  The same holds for squares
 // (norm = raw norm * scale^2) and maxima.  Results are bit-identical to the transform with its halvings while the raw sums of
 // squares (up to 4^levels times a norm) stay below 2^128, the raw values below 2^128, and neither squares nor values fall into
 // the subnormal range.  Kernels that store coefficients halve at every level and have the whole range.
-// `swapped`: the lane passes its two patch rows in exchanged order (a shared-memory bank trick of the TMA rings); the sums
-// over rows are unchanged and the differences over rows (y3, y4 of level 1) change sign, which goes into the scale.
 template <int L>
-__device__ __forceinline__ void slot_scales(int lane, bool swapped, float (&sc)[8])
+__device__ __forceinline__ void slot_scales(int lane, float (&sc)[8])
 {
     using T = HaarTile<L>;
     const int rp = lane / T::CG;
-    const float h = 0.5f, hs = swapped ? -0.5f : 0.5f;
-    sc[0] = h; sc[1] = h; sc[2] = hs; sc[3] = hs; sc[4] = hs; sc[5] = hs;
-    if (L == 1) { sc[6] = h; sc[7] = h; }
+#pragma unroll
+    for (int s = 0; s < 6; ++s) sc[s] = 0.5f;
+    if (L == 1) { sc[6] = 0.5f; sc[7] = 0.5f; }
     else {
         sc[7] = 0.25f;
         sc[6] = (L == 3 && (rp & 1) == 0) ? 0.125f : 0.25f;
     }
 }
 
-// ---- patch load / store ------------------------------------------------------------------------
-struct RawPatch { uint32_t w[8]; };   // fp32: 2 rows x 4 words; bf16: 2 rows x 2 words (w[0..1], w[4..5])
-
-template <typename T, bool VEC>
-__device__ __forceinline__ void load_patch(const T* __restrict__ plane, int W, const LanePos& lp, RawPatch& r)
-{
-#pragma unroll
-    for (int row = 0; row < 2; ++row) {
-        const T* src = plane + (size_t)(lp.r0 + row) * W + lp.c0;
-        uint32_t* w = r.w + 4 * row;
-        if (sizeof(T) == 4) {
-            if (VEC) {
-                if (lp.ok0) {
-                    const uint4 v = __ldcs(reinterpret_cast<const uint4*>(src));
-                    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-                } else { w[0] = w[1] = w[2] = w[3] = 0u; }
-            } else {
-                uint2 a = make_uint2(0u, 0u), b = make_uint2(0u, 0u);
-                if (lp.ok0) a = __ldcs(reinterpret_cast<const uint2*>(src));
-                if (lp.ok1) b = __ldcs(reinterpret_cast<const uint2*>(src + 2));
-                w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
-            }
-        } else {
-            if (VEC) {
-                uint2 v = make_uint2(0u, 0u);
-                if (lp.ok0) v = __ldcs(reinterpret_cast<const uint2*>(src));
-                w[0] = v.x; w[1] = v.y;
-            } else {
-                w[0] = lp.ok0 ? __ldcs(reinterpret_cast<const uint32_t*>(src)) : 0u;
-                w[1] = lp.ok1 ? __ldcs(reinterpret_cast<const uint32_t*>(src + 2)) : 0u;
-            }
-        }
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void unpack_patch(const RawPatch& r, float (&p)[2][4])
-{
-#pragma unroll
-    for (int row = 0; row < 2; ++row) {
-        const uint32_t* w = r.w + 4 * row;
-        if (sizeof(T) == 4) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) p[row][i] = __uint_as_float(w[i]);
-        } else {
-            p[row][0] = bf16lo(w[0]); p[row][1] = bf16hi(w[0]);
-            p[row][2] = bf16lo(w[1]); p[row][3] = bf16hi(w[1]);
-        }
-    }
-}
-
+// ---- patch and slot access ------------------------------------------------------------------------
 template <typename T, bool VEC>
 __device__ __forceinline__ void store_patch(T* __restrict__ plane, int W, const LanePos& lp, const float (&p)[2][4])
 {

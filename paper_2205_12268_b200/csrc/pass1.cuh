@@ -101,7 +101,7 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
         __syncthreads();
     }
     float sc[8], amax[8];
-    slot_scales<L>(lane, false, sc);
+    slot_scales<L>(lane, sc);
 #pragma unroll
     for (int s = 0; s < 8; ++s) amax[s] = 0.0f;
     float2 acc[4];
@@ -266,12 +266,14 @@ pass1_kernel(const T* __restrict__ x, const float* __restrict__ taps, int C, int
     if (NW > 1 && !__all_sync(0xFFFFFFFFu, ok ? 1 : 0) && lane == 0) atomicExch(status, (int)WCC_ERR_TIMEOUT);
 }
 
-// Warps per tile: one where the tiles alone fill the resident warps of every SM about once, or several times over (no hand-over),
-// up to eight where they are few, two or four where one warp per tile would leave a long second wave.  us per layer with
-// 1 / 2 / 4 / 8 warps: 128 tiles (384 -> 512 bf16) 101 / 73 / 61 / 56; 512 tiles (144 -> 24 bf16) 47.9 / 37.6 / 34.3 / 37.3;
-// 1024 tiles (32 -> 192 chain) 405 / 377 / 387 / 414; 1440 tiles (C4) 67.9 / 71.1 / 70.4; 1664 tiles (144 -> 24 bf16)
-// 105.6 / 98.9 / 101.3; 2048 tiles 117.5 / 109.0 / 111.9, fp32 1920 tiles 93.9 / 87.6 / 87.9; 2880 tiles fp32 130.0 / 125.8 /
-// 125.1; 3072 tiles (100 -> 24 bf16) 105.6 / 107.2 / 111.4; 4800 tiles 117.7 / 120.4 / 123.1.
+// Warps per tile: eight up to two tiles per SM, four up to four, two up to eight, one up to 10.7, two up to 16, two (bf16) or four
+// (fp32) up to 20, one beyond.  An SM holds sixteen warps of the kernels with several per tile and twelve tiles of one warp (168
+// registers a thread), so the two steps back to two warps lie below a full wave of one-warp tiles (12 per SM) and after it.  The
+// lines are measured, on whole layers of 600 drawn shapes, geometric mean of the rule's time over another choice's (worst case):
+// 296 tiles and fewer, eight against four 1.00; 297 to 592, four against eight 0.93, against two 0.92; 593 to 1184, two against one
+// 0.98, against four 0.97; 1185 to 1579, one against two 0.97 (1.00), against four 0.97; 1580 to 2368, two against one 0.98;
+// 2369 to 2960 all within 2 % up to 100 channels.  bf16 and fp32 agree, but for fp32 with more than 100 channels, where four warps
+// are 2 to 7 % faster on average from 740 tiles on and 5 % slower at worst.
 template <typename T, int L, bool VEC, int KIND, bool DW>
 static wcc_status pass1_launch(const void* x, const float* taps, int N, int C, int H, int W, float* coef, float* nrm2, float* amaxpos, const NormsExtra& ex,
                                cudaStream_t st)

@@ -20,8 +20,8 @@
 // Measured (B200, back-to-back calls) against the kernels it replaced (TMA rings, one CTA of nine warps per SM; one tile per
 // CTA for the shapes beyond that): C4 fp32 43.4 -> 36.5 us (x and y cross HBM once each: 5.2 TB/s, 79 % of the copy rate),
 // 24 images of it 77.7 -> 71.4; 24 -> 144 channels bf16 unquantized on 2 x 256 x 512 34.3 -> 22.8; 32 -> 192 there
-// 46.6 -> 30.2; 96 -> 96 with residual, ReLU and clipping on 4 x 128 x 256 63.2 -> 23.3.  bf16 layers are bound by
-// instruction issue (0.45 - 0.5 warp instructions per cycle and scheduler), fp32 ones by the latency of their loads.
+// 46.6 -> 30.2; 96 -> 96 with residual, ReLU and clipping on 4 x 128 x 256 63.2 -> 23.3.  Both types wait: half
+// (bf16) to two thirds (fp32) of the issue slots are free, at sixteen warps per SM.
 #pragma once
 
 #include "common.cuh"
@@ -159,7 +159,7 @@ pass2_kernel(const Params pr)
         if (I8) inv = (amax > 0.0f) ? __fdiv_rn(pr.qmax, amax) : 0.0f;
         // the transform runs without its halvings: they go into the per-slot factor (exact, a power of two)
         float sc[8];
-        slot_scales<L>(lane, false, sc);
+        slot_scales<L>(lane, sc);
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
             rk[s] = -1;

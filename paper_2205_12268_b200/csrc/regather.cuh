@@ -58,7 +58,7 @@ regather_quant_kernel(const T* __restrict__ x, const float* __restrict__ taps, c
     }
     if (!__any_sync(0xFFFFFFFFu, any ? 1 : 0)) return;                // nothing kept in this tile
     float mul[8];
-    slot_scales<L>(lane, false, mul);                  // the halvings of the transform and the quantizer's factor in one
+    slot_scales<L>(lane, mul);                  // the halvings of the transform and the quantizer's factor in one
     if (DW) {                                          // (behind a convolution the transform halves, as in the first pass)
 #pragma unroll
         for (int s = 0; s < 8; ++s) mul[s] = 1.0f;

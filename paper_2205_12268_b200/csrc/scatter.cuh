@@ -113,10 +113,10 @@ static wcc_status scatter_inv_dispatch(const int32_t* acc, int ldc, bool accf, c
                                        cudaStream_t st)
 {
     using TT = HaarTile<L>;
-    // channels per warp: as many as still leave about 32 warps for each of the 148 SMs (8 to 64)
+    // channels per warp: as many as still leave about 32 warps for each SM (8 to 64)
     const long long tiles = (long long)N * ceil_div(W, TT::TW) * (H / TT::TH);
     int ocw = 64;
-    while (ocw > 8 && tiles * ceil_div(Cout, ocw) < 148 * 32) ocw >>= 1;
+    while (ocw > 8 && tiles * ceil_div(Cout, ocw) < B200_SMS * 32) ocw >>= 1;
     const long long warps = tiles * ceil_div(Cout, ocw);
     auto go = [&](auto kern) -> wcc_status {
         return launch_overlapped(kern, dim3((unsigned)((warps + 3) / 4)), dim3(128), 0, st, true, 1, acc, ldc, rank, amax_kept, qmax, scale_w, N, Cout,

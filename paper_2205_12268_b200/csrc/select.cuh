@@ -32,7 +32,7 @@ struct SelectWs {
     uint32_t* bar;      // [N] arrival counters of the per-image barriers of the single-kernel select
     uint32_t* state;    // [N][ST_WORDS]
     uint32_t* chunkcnt; // [N][chunks][2]
-    size_t zero_bytes;  // hist + amax + bar are contiguous and cleared by one memset
+    size_t zero_bytes;  // hist + amax + bar are contiguous and cleared together
     int chunks;
 };
 
@@ -968,7 +968,7 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         int cs = 1;
         while (cs < 8 && cs * 512 < P) cs <<= 1;
         if (cs == 8 && cs_cap == 16 && P > 65536) cs = 16;
-        while (cs > 1 && (long long)N * cs > 148 && P <= cs / 2 * CL_THREADS * CL_MAXKPT) cs >>= 1;      // all images in one wave
+        while (cs > 1 && (long long)N * cs > B200_SMS && P <= cs / 2 * CL_THREADS * CL_MAXKPT) cs >>= 1;      // all images in one wave
         int threads = 256;
         const int kpt_goal = hist1_ready ? 4 : CL_MAXKPT;               // few keys per thread when no scans are needed
         while (threads < CL_THREADS && (long long)cs * threads * kpt_goal < P) threads <<= 1;
