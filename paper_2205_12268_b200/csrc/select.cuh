@@ -438,33 +438,53 @@ select_coop_kernel(const float* __restrict__ nrm2, int P, int k, uint32_t* __res
 }
 
 // ---- the select as one thread-block cluster per image -------------------------------------------------
-// Up to 8 CTAs of 1024 threads form one cluster per image (P <= 131072 keys, at most 16 per thread, held in
-// registers).  Each CTA histograms its keys in shared memory; the histograms are combined through distributed
-// shared memory (every CTA sums one slice of the bins over all CTAs, then all CTAs read the slice totals and the
-// slice that holds the k-th key), and the phases are separated by hardware cluster barriers: no global-memory
-// round trips, no spinning, no scratch memory.
-constexpr int CL_THREADS = 1024;
-constexpr int CL_MAXKPT = 16;
+// Up to 16 CTAs of 256 threads form one cluster per image (P <= 131072 keys, at most 32 per thread, held in registers).  What is
+// found in one CTA is pushed into the shared memory of the others (st.shared::cluster, one hardware cluster barrier) instead of
+// being read there afterwards; histograms of whole key ranges, needed where the caller supplies none, are combined slice by slice.
+// No global-memory round trips between the phases, no spinning, no scratch memory.
+constexpr int CL_THREADS = 256;
+constexpr int CL_MAXKPT = 32;
 constexpr int CL_MAXCS = 16;          // 8 is the portable cluster size; 16 needs the non-portable opt-in
-constexpr int CL_CAND_CTA = 1024;    // candidate slots per CTA
-constexpr int CL_CAND_MAX = 2048;    // most candidates gathered by every CTA; beyond that: another round over the cluster
+constexpr int CL_CAND_MAX = 1024;    // candidates a CTA has room for: CL_CAND_MAX / cs from each CTA of the cluster; beyond that: another round
+constexpr int CL_MSG = 64;           // words of the message in which a CTA sends up to CL_MSG - 1 candidates
+constexpr int CL_FEW = 256;          // candidates ranked by few_rank
 constexpr int FINE_BINS = 65536;     // histogram of the 16 bits below the sign of every norm, filled by the producer of the norms
 
 struct ClusterSmem {
-    uint32_t hist[SEL_BINS];
+    union {
+        uint32_t hist[SEL_BINS];
+        uint32_t local[CL_CAND_MAX];      // this CTA's candidates until they are sent
+    };
     uint32_t slice[SEL_BINS];       // sums over all CTAs of this CTA's slice of bins
     uint32_t warp_sums[CL_THREADS / 32 + 1];
+    uint32_t warp_eq[CL_THREADS / 32];
     uint32_t slice_total;
-    uint32_t cnt[2];                // keys above / equal to the threshold in this CTA
     uint32_t res[3];                // found bin, keys above it, keys in it
     uint32_t tot[CL_MAXCS];
     uint32_t amax;
-    uint32_t ncand[5];              // candidates of this CTA, per gather (a neighbour may still read an earlier count)
-    uint32_t cand[CL_CAND_CTA];
-    __align__(16) uint32_t all[CL_CAND_MAX];      // candidates of the whole cluster
+    uint32_t ncand;                 // candidates of this CTA in the gather at hand
+    __align__(16) uint32_t out[CL_MSG];           // this CTA's message: number of candidates, candidates, zeros
+    __align__(16) uint32_t msg[CL_MAXCS][CL_MSG];  // the messages of all CTAs of the cluster
+    uint64_t msg_bar;               // counts their bytes
+    uint32_t few[CL_FEW];           // the candidates in them without the gaps, zeros behind
+    __align__(16) uint32_t counts[2][CL_THREADS / 32];         // of a round of few_rank, per warp
+    uint32_t pushed[CL_CAND_MAX];   // candidates of every CTA of the cluster, CL_CAND_MAX / cs slots each
+    uint32_t pushed_cnt[CL_MAXCS];  // how many each has (more than its slots: none were sent)
+    uint2 kept_cnt[CL_MAXCS];       // keys above / equal to the threshold in every CTA
+    __align__(16) uint32_t all[CL_CAND_MAX];      // keys of `pushed` without the gaps
     uint32_t thr[3];                // threshold key, ties to keep, ties in total
     __align__(16) uint32_t range[4];              // positive keys, zeros, smallest positive key, largest key
 };
+
+// Store to a CTA of the cluster (addr: this CTA's address of the same variable).
+__device__ __forceinline__ void push_u32(uint32_t* addr, int rank, uint32_t v)
+{
+    asm volatile("{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n st.shared::cluster.u32 [ra], %2;\n}\n" ::"r"(tc::smem_u32(addr)), "r"(rank), "r"(v) : "memory");
+}
+__device__ __forceinline__ void push_u64(uint2* addr, int rank, uint2 v)
+{
+    asm volatile("{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n st.shared::cluster.v2.u32 [ra], {%2, %3};\n}\n" ::"r"(tc::smem_u32(addr)), "r"(rank), "r"(v.x), "r"(v.y) : "memory");
+}
 
 // exclusive scan over the threads of the block (256, 512 or 1024); every thread also gets the total
 __device__ __forceinline__ uint32_t block_scan_1024(uint32_t v, uint32_t* warp_sums, uint32_t* total)
@@ -555,59 +575,177 @@ __device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, Clu
 __device__ __forceinline__ int span_shift(uint32_t span) { return max(0, 32 - __clz(span) - 11); }
 
 // Gathers the keys in [lo, hi] of the whole cluster into sm.all of every CTA; returns how many there are (0xFFFFFFFF: too many).
-// One cluster barrier.
-template <int MAXKPT, typename Valid>
-__device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, ClusterSmem& sm, int cs, const uint32_t (&key)[MAXKPT], int kpt,
-                                                   Valid valid, uint32_t lo, uint32_t hi, int lane, int gather)
+// One cluster barrier.  sm.ncand is zero before.
+template <int KPT>
+__device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, ClusterSmem& sm, int cs, int crank, const uint32_t (&key)[KPT], uint32_t in_map,
+                                                   uint32_t lo, uint32_t hi, int lane)
 {
+    uint32_t in = 0u;
 #pragma unroll
-    for (int i = 0; i < MAXKPT; ++i) {
-        if (i >= kpt) break;
-        const bool c = valid(i) && key[i] >= lo && key[i] <= hi;
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, c);
-        if (m) {
-            uint32_t off = 0;
-            if (lane == 0) off = atomicAdd(&sm.ncand[gather], (uint32_t)__popc(m));
-            off = __shfl_sync(0xFFFFFFFFu, off, 0);
-            const uint32_t slot = off + (uint32_t)__popc(m & ((1u << lane) - 1u));
-            if (c && slot < CL_CAND_CTA) sm.cand[slot] = key[i];
-        }
+    for (int i = 0; i < KPT; ++i) in |= (key[i] >= lo && key[i] <= hi) ? 1u << i : 0u;
+    in &= in_map;
+    if (__any_sync(0xFFFFFFFFu, in != 0u)) {
+        uint32_t slot = 0;
+        if (in) slot = atomicAdd(&sm.ncand, (uint32_t)__popc(in));
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if (in & (1u << i)) {
+                if (slot < CL_CAND_MAX) sm.local[slot] = key[i];
+                ++slot;
+            }
     }
-    cluster.sync();
-    if (threadIdx.x < cs) sm.tot[threadIdx.x] = *cluster.map_shared_rank(&sm.ncand[gather], threadIdx.x);
     __syncthreads();
-    uint32_t M = 0;
-    bool overflow = false;
-    for (int r = 0; r < cs; ++r) { overflow = overflow || sm.tot[r] > CL_CAND_CTA; M += sm.tot[r]; }
-    if (overflow || M > CL_CAND_MAX) return 0xFFFFFFFFu;
-    // one remote load per thread, all in flight together (rank after rank would expose every rank's latency)
-    for (uint32_t g = threadIdx.x; g < M; g += blockDim.x) {
-        uint32_t pre = 0;
-        int r = 0;
-        while (g >= pre + sm.tot[r]) { pre += sm.tot[r]; ++r; }
-        sm.all[g] = cluster.map_shared_rank(sm.cand, r)[g - pre];
+    const uint32_t mine = sm.ncand, slots = CL_CAND_MAX / (uint32_t)cs;
+    if ((int)threadIdx.x < cs) push_u32(&sm.pushed_cnt[crank], (int)threadIdx.x, mine);
+    if (mine <= slots)
+        for (uint32_t t = threadIdx.x; t < mine * (uint32_t)cs; t += blockDim.x)
+            push_u32(&sm.pushed[(uint32_t)crank * slots + t / (uint32_t)cs], (int)(t & (uint32_t)(cs - 1)), sm.local[t / (uint32_t)cs]);
+    cluster.sync();
+    const uint32_t cnt = lane < cs ? sm.pushed_cnt[lane] : 0u, M = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    if (__any_sync(0xFFFFFFFFu, cnt > slots)) return 0xFFFFFFFFu;
+    uint32_t upto = cnt;                               // of the CTAs up to `lane`
+#pragma unroll
+    for (int d = 1; d < CL_MAXCS; d <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+        if (lane >= d) upto += t;
+    }
+#pragma unroll 1
+    for (uint32_t g = threadIdx.x; g < CL_CAND_MAX; g += blockDim.x) {        // (at least 64 slots each: r is the same in a warp)
+        const int r = (int)(g / slots);
+        const uint32_t j = g - (uint32_t)r * slots, c = __shfl_sync(0xFFFFFFFFu, cnt, r), at = __shfl_sync(0xFFFFFFFFu, upto, r) - c;
+        if (j < c) sm.all[at + j] = sm.pushed[g];
     }
     __syncthreads();
     return M;
 }
 
+// The short way of a gather: every CTA sends one message of fixed size to every CTA (st.async, counted by the receiver's mbarrier).
+// A cluster barrier would also wait for everything that its threads have under way in global memory (its release): 1.6 to 3.4
+// us for the gather and its block barriers against 0.8 to 1.3.  The candidates end up in sm.few; returns how many there are,
+// 0xFFFFFFFF if there are too many for a message or for sm.few, or 0 with the status set when the wait ran out.
+template <int KPT>
+__device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, int crank, const uint32_t (&key)[KPT], uint32_t in_map, uint32_t lo,
+                                                     uint32_t hi, int warp, int lane)
+{
+    const bool alone = cs == 1;                        // (a launch without clusters: st.async is for launches that have them)
+    uint32_t in = 0u;
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) in |= (key[i] >= lo && key[i] <= hi) ? 1u << i : 0u;
+    in &= in_map;
+    if (__any_sync(0xFFFFFFFFu, in != 0u)) {
+        uint32_t* const list = alone ? sm.few : sm.out + 1;
+        const uint32_t most = alone ? CL_FEW : CL_MSG - 1;
+        uint32_t slot = most;
+        if (in) slot = atomicAdd(&sm.ncand, (uint32_t)__popc(in));
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+            if (in & (1u << i)) {
+                if (slot < most) list[slot] = key[i];
+                ++slot;
+            }
+    }
+    __syncthreads();
+    if (alone) return sm.ncand <= CL_FEW ? sm.ncand : 0xFFFFFFFFu;
+    if ((int)threadIdx.x < cs * (CL_MSG / 4)) {        // sixteen bytes to one CTA per thread
+        const int to = (int)threadIdx.x / (CL_MSG / 4), j = (int)threadIdx.x % (CL_MSG / 4);
+        uint4 w = *reinterpret_cast<const uint4*>(&sm.out[4 * j]);
+        if (j == 0) w.x = sm.ncand;
+        asm volatile("{\n .reg .b32 ra, rb;\n mapa.shared::cluster.u32 ra, %0, %2;\n mapa.shared::cluster.u32 rb, %1, %2;\n"
+                     " st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [ra], {%3, %4, %5, %6}, [rb];\n}\n"
+                     ::"r"(tc::smem_u32(&sm.msg[crank][4 * j])), "r"(tc::smem_u32(&sm.msg_bar)), "r"(to), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w) : "memory");
+    }
+    const uint32_t bar = tc::smem_u32(&sm.msg_bar), limit = tc::c_wait_limit;
+    uint32_t ok = 0;
+    for (uint32_t it = 0; it < limit && !ok; ++it)
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(ok) : "r"(bar), "r"(1000u) : "memory");
+    if (!__syncthreads_and(ok ? 1 : 0)) {              // (the same for the whole block)
+        if (threadIdx.x == 0) atomicExch(&g_status, (int)WCC_ERR_TIMEOUT);
+        return 0u;
+    }
+    const uint32_t cnt = lane < cs ? sm.msg[lane][0] : 0u, M = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    if (__any_sync(0xFFFFFFFFu, cnt >= CL_MSG) || M > CL_FEW) return 0xFFFFFFFFu;
+    uint32_t upto = cnt;                               // of the CTAs up to `lane`
+#pragma unroll
+    for (int d = 1; d < CL_MAXCS; d <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+        if (lane >= d) upto += t;
+    }
+    for (int r = warp; r < cs; r += CL_THREADS / 32) {
+        const uint32_t c = __shfl_sync(0xFFFFFFFFu, cnt, r), at = __shfl_sync(0xFFFFFFFFu, upto, r) - c;
+        for (uint32_t j = lane; j < c; j += 32) sm.few[at + j] = sm.msg[r][1 + j];
+    }
+    __syncthreads();
+    return M;
+}
+
+// The krem-th largest of the M candidates in sm.few, which agree with `base` in all but their low 15 bits (zeros: none).  Three bits a
+// round, a threshold per warp, until one candidate is left.
+__device__ __forceinline__ void few_rank(ClusterSmem& sm, uint32_t M, uint32_t krem, uint32_t base, int warp, int lane, uint32_t& key, uint32_t& need, uint32_t& equal)
+{
+    uint32_t c[CL_FEW / 32];
+#pragma unroll
+    for (int i = 0; i < CL_FEW / 32; ++i) c[i] = sm.few[32 * i + lane];
+    uint32_t t = base, above = 0, all = M;             // the key is in [t, t + 2^bits): `all` are t or larger, `above` beyond
+    int bits = 15;
+#pragma unroll 1
+    for (int round = 0; bits > 0 && all - above > 1; ++round) {
+        bits -= 3;
+        const uint32_t mine = t + ((uint32_t)warp << bits);
+        uint32_t n = 0;
+#pragma unroll
+        for (int i = 0; i < CL_FEW / 32; ++i) n += c[i] >= mine ? 1u : 0u;
+        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        if (lane == 0) sm.counts[round & 1][warp] = n;
+        __syncthreads();
+        const uint4 a = *reinterpret_cast<const uint4*>(&sm.counts[round & 1][0]), b = *reinterpret_cast<const uint4*>(&sm.counts[round & 1][4]);
+        const uint32_t v[9] = {all, a.y, a.z, a.w, b.x, b.y, b.z, b.w, above};
+        uint32_t w = 0;
+#pragma unroll
+        for (int i = 1; i < 8; ++i)
+            if (v[i] >= krem) { w = i; all = v[i]; }
+        above = v[8];
+#pragma unroll
+        for (int i = 7; i >= 1; --i)
+            if (v[i] < krem) above = v[i];             // (counts fall with i: ends at the smallest threshold too large)
+        t += w << bits;
+    }
+    if (bits > 0) {                                    // one candidate left
+        uint32_t m = 0;
+#pragma unroll
+        for (int i = 0; i < CL_FEW / 32; ++i) m = max(m, c[i] < t + (1u << bits) ? c[i] : 0u);
+        t = __reduce_max_sync(0xFFFFFFFFu, m);
+    }
+    key = t; need = krem - above; equal = all - above;
+}
+
 // The krem-th largest of the M candidates in sm.all, all of them in [lo, hi] -> sm.thr = {key, equal keys to keep, equal keys}.
-// Few are ranked by counting (one barrier; 2 us for 340 candidates), many by histogram rounds inside the block, eleven bits of
-// the span each (3 us for two rounds, whatever their number).
+// Few are ranked by counting, as many threads to a candidate as there are (one barrier; 168 candidates by one thread each took
+// 2.4 us), many by histogram rounds inside the block, eleven bits of the span each (3 us for two rounds, whatever their number).
 __device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t krem, uint32_t lo, uint32_t hi)
 {
-    if (M <= 512) {
+    if (M <= 384) {
         const uint4* all4 = reinterpret_cast<const uint4*>(sm.all);
-        for (uint32_t i = threadIdx.x; i < M; i += blockDim.x) {
-            const uint32_t ci = sm.all[i];
+        uint32_t q = 1;                                // threads per candidate, neighbours in a warp
+        while (q < 8 && M * q * 2 <= blockDim.x) q <<= 1;
+        const uint32_t part = threadIdx.x & (q - 1);
+        for (uint32_t i0 = 0; i0 < M; i0 += blockDim.x / q) {                 // (uniform over the block: whole warps shuffle)
+            const uint32_t i = i0 + threadIdx.x / q;
+            const uint32_t ci = i < M ? sm.all[i] : 0u;
             uint32_t g = 0, e = 0;
-            for (uint32_t j4 = 0; j4 < M / 4; ++j4) {            // four candidates per shared-memory load
+#pragma unroll 4
+            for (uint32_t j4 = part; j4 < M / 4; j4 += q) {                   // four candidates per shared-memory load
                 const uint4 c = all4[j4];
                 g += (c.x > ci) + (c.y > ci) + (c.z > ci) + (c.w > ci);
                 e += (c.x == ci) + (c.y == ci) + (c.z == ci) + (c.w == ci);
             }
-            for (uint32_t j = M & ~3u; j < M; ++j) { const uint32_t cj = sm.all[j]; g += cj > ci; e += cj == ci; }
-            if (g < krem && krem <= g + e) { sm.thr[0] = ci; sm.thr[1] = krem - g; sm.thr[2] = e; }      // equal keys write equal values
+            if (part == 0)
+                for (uint32_t j = M & ~3u; j < M; ++j) { const uint32_t cj = sm.all[j]; g += cj > ci; e += cj == ci; }
+            for (uint32_t d = 1; d < q; d <<= 1) {
+                g += __shfl_xor_sync(0xFFFFFFFFu, g, d);
+                e += __shfl_xor_sync(0xFFFFFFFFu, e, d);
+            }
+            if (i < M && g < krem && krem <= g + e) { sm.thr[0] = ci; sm.thr[1] = krem - g; sm.thr[2] = e; }      // equal keys write equal values
         }
         __syncthreads();
         return;
@@ -651,48 +789,23 @@ __device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t
     }
 }
 
-// Find the bin of a complete 2048-bin histogram in global memory that holds the krem-th key from the top; block of
-// 256, 512 or 1024 threads, every thread returns the same values.
-__device__ __forceinline__ void block_find_bin_2048(const uint32_t* __restrict__ h, uint32_t krem, ClusterSmem& sm,
-                                                    uint32_t& bin, uint32_t& above, uint32_t& tot)
-{
-    const int per = SEL_BINS / (int)blockDim.x;            // 8, 4 or 2
-    const int top = SEL_BINS - 1 - (int)threadIdx.x * per;
-    uint32_t c[8], mysum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        c[i] = (i < per) ? __ldcg(&h[top - i]) : 0u;
-        mysum += c[i];
-    }
-    const uint32_t before = block_scan_1024(mysum, sm.warp_sums, &tot);
-    if (before < krem && krem <= before + mysum) {
-        uint32_t a = before;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            if (a < krem && krem <= a + c[i]) { sm.res[0] = (uint32_t)(top - i); sm.res[1] = a; sm.res[2] = c[i]; }
-            a += c[i];
-        }
-    }
-    __syncthreads();
-    bin = sm.res[0];
-    above = sm.res[1];
-    __syncthreads();
-}
-
-// Measured (us): without histograms, 4 images of 61440 positions 22.7 -> 15.5 (three rounds on fixed 11 + 11 + 10 bit digits
-// before); with them, 24 images of 30720 positions as 4 instead of 8 CTAs each: one wave, layer 125.1 -> 122.2.
-//
 // hist1 ([N][3][2048], round 1 first) and fine ([N][65536]) are optional histograms of the 11 and 16 bits below the sign
 // of every norm (norm_digit11 / norm_digit16: norms are never negative) that the producer of the norms filled; with both, the threshold is usually found without any histogram round:
 // the 16-bit bin that holds the k-th key contains few keys, which the cluster gathers and ranks directly.
 // idx and rank are written only when asked for (want_rank) or when the threshold's ties are kept only in part
 // (then the order of positions matters); otherwise consumers compare keys with thr[n] = {threshold key, ties
 // kept, use_rank flag, number of candidate keys that were ranked (diagnostic)}.
-// MAXKPT: key registers per thread (16, or 4 for the launches that spread an image over enough threads).
-// HIST: the histograms are supplied.
-template <int MAXKPT, bool HIST>
-__global__ void __launch_bounds__(CL_THREADS, 1)
-select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int32_t* __restrict__ idx, float* __restrict__ tau,
+// A warp owns 32 * KPT consecutive positions, 32 at a time: every load and store is a full line (as consecutive keys per
+// thread the loads alone took a microsecond).  The work after the first load is a chain of latencies, so each step is the one
+// with the fewest block barriers: warp sums by redux instead of block scans, the owner of the coarse bin goes on to the fine one
+// alone, the maxima of what is certainly kept are taken while the cluster barrier is pending.
+// Blocks of 256 threads: what every warp has to do besides its keys (some 500 instructions) was most of the issue slots of 1024.
+// Measured, from the end of the first pass to the start of the second's threshold (us, blocks of up to 1024 threads that read each
+// other's candidates after a cluster barrier -> this): 2 x 131072 positions 14.3 -> 8.3, 12 x 30720 7.8 -> 5.3, 4 x 32768 8.0 -> 6.2.
+// KPT: keys per thread (8, 16 or 32).  HIST: the histograms are supplied.
+template <int KPT, bool HIST>
+__global__ void __launch_bounds__(CL_THREADS, 2)
+select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __restrict__ idx, float* __restrict__ tau,
                       int32_t* __restrict__ rank, const float* __restrict__ amaxpos, float* __restrict__ amax_kept,
                       const uint32_t* __restrict__ hist1, const uint32_t* __restrict__ fine, uint32_t* __restrict__ thr,
                       int want_rank)
@@ -702,79 +815,129 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
     const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
     const int n = blockIdx.y;
     const float* v = nrm2 + (size_t)n * P;
-    const int base = (crank * (int)blockDim.x + (int)threadIdx.x) * kpt;  // kpt consecutive keys per thread
-    const int lane = threadIdx.x & 31;
+    constexpr int WARPS = CL_THREADS / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int base = (crank * WARPS + warp) * 32 * KPT + lane;            // this thread's keys: base, base + 32, ...
 
-    for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
-    if (threadIdx.x < 5) sm.ncand[threadIdx.x] = 0u;
+    if (!HIST)
+        for (int i = threadIdx.x; i < SEL_BINS; i += CL_THREADS) sm.hist[i] = 0u;
     if (threadIdx.x < 4) sm.range[threadIdx.x] = threadIdx.x == 2 ? 0xFFFFFFFFu : 0u;
-    if (threadIdx.x == 0) { sm.amax = 0u; sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u; }   // thr: keep nothing
-                                                       // unless a candidate is found (histograms that do not match the keys)
+    if (threadIdx.x < CL_MSG) sm.out[threadIdx.x] = 0u;
+    for (int i = threadIdx.x; i < CL_FEW; i += CL_THREADS) sm.few[i] = 0u;
+    if (threadIdx.x == 0) {
+        tc::mbar_init(tc::smem_u32(&sm.msg_bar), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc::mbar_expect_tx(tc::smem_u32(&sm.msg_bar), (uint32_t)(cs * CL_MSG * 4));
+        sm.amax = 0u;
+        sm.ncand = 0u;
+        sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u;          // keep nothing unless a candidate is found (histograms
+        sm.res[0] = 0u; sm.res[1] = 0u; sm.res[2] = 0u;                   // that do not match the keys)
+    }
+    cluster.barrier_arrive();                          // this CTA runs: others may write to its shared memory
     pdl_wait();
     pdl_launch();
-    uint32_t key[MAXKPT];
+    uint32_t key[KPT], in_map = 0u;                    // in_map: the keys that exist
 #pragma unroll
-    for (int i = 0; i < MAXKPT; ++i) key[i] = (i < kpt && base + i < P) ? float_key(v[base + i]) : 0u;
-    auto valid = [&](int i) { return i < kpt && base + i < P; };
-    // few keys per thread: the per-position maxima are fetched together with the keys, so that the pass over the kept
-    // positions at the end waits for no further load
-    constexpr bool PRE = MAXKPT <= 4;
-    float pre[PRE ? MAXKPT : 1];
-    if (PRE) {
+    for (int i = 0; i < KPT; ++i) key[i] = __float_as_uint(__ldcg(v + min(base + 32 * i, P - 1)));      // (no branches: all loads in flight)
+    constexpr int PER = SEL_BINS / CL_THREADS;         // coarse bins per thread
+    uint4 bins[PER / 4];
+    if (HIST) {
+        const uint32_t* h = hist1 + (size_t)n * 3 * SEL_BINS + SEL_BINS - 4 - (int)threadIdx.x * PER;
 #pragma unroll
-        for (int i = 0; i < MAXKPT; ++i) pre[PRE ? i : 0] = (amaxpos && valid(i)) ? amaxpos[(size_t)n * P + base + i] : 0.0f;
+        for (int i = 0; i < PER / 4; ++i) bins[i] = __ldcg(reinterpret_cast<const uint4*>(h - 4 * i));
     }
-
-    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < KPT; ++i) {
+        key[i] = HIST ? key[i] & 0x7FFFFFFFu : float_key(__uint_as_float(key[i]));       // (norms are never negative)
+        in_map |= base + 32 * i < P ? 1u << i : 0u;
+    }
+    auto valid = [&](int i) { return (in_map & (1u << i)) != 0u; };
+    uint32_t am[KPT];                                  // maxima at the positions that may be kept
+    auto load_amax = [&](uint32_t limit) {
+        const float* a = amaxpos + (size_t)n * P + base;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) {
+            const uint32_t take = valid(i) && key[i] >= limit ? 1u : 0u;
+            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n mov.u32 %0, 0;\n @p ld.global.cg.u32 %0, [%1];\n}\n" : "=r"(am[i]) : "l"(a + 32 * i), "r"(take));
+        }
+    };
 
     uint32_t tkey = 0, need_eq = 0, total_eq = 0, ranked = 0;    // ranked: candidates counted through (diagnostic)
-    int gathers = 0;
     uint32_t lo = 0, hi = 0, krem = 0;                 // the threshold is the krem-th largest key in [lo, hi]
-    bool found = false;
+    bool found = false, reads_remote = !HIST, amax_loaded = false;
     // The supplied histograms count the non-zero norms only; the zeros are the positions they leave out and rank
     // below everything else.  More kept positions than non-zero norms: the threshold is zero.
     bool zero_thr = false;
-    uint32_t b1h = 0, aboveh = 0;
     if (HIST) {
-        // the 11-bit bin of the threshold
-        uint32_t nonzero;
-        if (threadIdx.x == 0) { sm.res[0] = 0u; sm.res[1] = 0u; sm.res[2] = 0u; }      // (a barrier follows inside)
-        block_find_bin_2048(hist1 + (size_t)n * 3 * SEL_BINS, (uint32_t)k, sm, b1h, aboveh, nonzero);
+        // The 11-bit bin of the threshold: thread t takes the t-th group of bins from the top, the warp that finds the k-th key among
+        // its bins goes on to the 16-bit bin (32 fine bins, one per lane, top bin in lane 0).
+        uint32_t c[PER], mysum = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i += 4) {
+            const uint4 b = bins[i / 4];
+            c[i] = b.w; c[i + 1] = b.z; c[i + 2] = b.y; c[i + 3] = b.x;
+            mysum += (b.x + b.y) + (b.z + b.w);
+        }
+        const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, mysum);
+        if (lane == 0) sm.warp_sums[warp] = wsum;
+        __syncthreads();
+        const uint32_t ws = lane < WARPS ? sm.warp_sums[lane] : 0u;
+        const uint32_t nonzero = __reduce_add_sync(0xFFFFFFFFu, ws), wbefore = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? ws : 0u);
         zero_thr = (uint32_t)k > nonzero;              // the same in every CTA of the cluster
         if (zero_thr) {
-            tkey = 0x80000000u;                        // key of +0
+            tkey = 0u;                                 // +0
             need_eq = (uint32_t)k - nonzero;
             total_eq = (uint32_t)P - nonzero;
             found = true;
+        } else {
+            if (wbefore < (uint32_t)k && (uint32_t)k <= wbefore + wsum) {             // one warp
+                uint32_t inc = mysum;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                    if (lane >= d) inc += t;
+                }
+                uint32_t a = wbefore + inc - mysum, b1 = 0, above = 0;
+                bool mine = false;
+#pragma unroll
+                for (int i = 0; i < PER; ++i) {
+                    if (a < (uint32_t)k && (uint32_t)k <= a + c[i]) { mine = true; b1 = (uint32_t)(SEL_BINS - 1 - (int)threadIdx.x * PER - i); above = a; }
+                    a += c[i];
+                }
+                const int from = __ffs(__ballot_sync(0xFFFFFFFFu, mine)) - 1;
+                b1 = __shfl_sync(0xFFFFFFFFu, b1, from);
+                const uint32_t k1 = (uint32_t)k - __shfl_sync(0xFFFFFFFFu, above, from);
+                const uint32_t bin = (b1 << 5) + 31u - (uint32_t)lane;
+                const uint32_t f = __ldcg(&fine[(size_t)n * FINE_BINS + bin]);
+                inc = f;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+                    if (lane >= d) inc += t;
+                }
+                const uint32_t before = inc - f;
+                if (before < k1 && k1 <= inc) { sm.res[0] = bin; sm.res[1] = k1 - before; }
+            }
+            __syncthreads();
+            lo = max(sm.res[0] << 15, 1u);             // (zeros are not counted)
+            hi = lo | 0x7FFFu;
+            krem = sm.res[1];
         }
     }
+    cluster.barrier_wait();                            // every CTA of the cluster runs
     if (HIST && !zero_thr) {
-        // the 16-bit bin inside the 11-bit bin (32 fine bins, one per lane of warp 0, top bin in lane 0)
-        const uint32_t b1 = b1h, above = aboveh;
-        const uint32_t k1 = (uint32_t)k - above;
-        if (threadIdx.x < 32) {
-            const uint32_t f = __ldcg(&fine[(size_t)n * FINE_BINS + (b1 << 5) + 31u - (uint32_t)lane]);
-            uint32_t inc = f;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-                if (lane >= d) inc += t;
-            }
-            const uint32_t before = inc - f;
-            if (before < k1 && k1 <= inc) { sm.res[0] = (b1 << 5) + 31u - (uint32_t)lane; sm.res[1] = before; sm.res[2] = f; }
-        }
-        __syncthreads();
-        const uint32_t prefix16 = sm.res[0], k16 = k1 - sm.res[1];
-        __syncthreads();
-        lo = 0x80000000u | (prefix16 << 15);
-        hi = lo | 0x7FFFu;
-        krem = k16;
-        const uint32_t M = cluster_gather<MAXKPT>(cluster, sm, cs, key, kpt, valid, lo, hi, lane, gathers++);
+        if (amaxpos) { load_amax(lo); amax_loaded = true; }          // (on their way while the threshold is found)
+        const uint32_t M = cluster_exchange<KPT>(sm, cs, crank, key, in_map, lo, hi, warp, lane);
         if (M != 0xFFFFFFFFu) {
-            if (M >= krem) block_rank(sm, M, krem, lo, hi);              // (fewer: histograms that do not match the keys, keep nothing)
-            tkey = sm.thr[0]; need_eq = sm.thr[1]; total_eq = sm.thr[2];
+            tkey = 0xFFFFFFFFu;                        // keep nothing if there are fewer (histograms that do not match the keys)
+            if (M >= krem) few_rank(sm, M, krem, hi & ~0x7FFFu, warp, lane, tkey, need_eq, total_eq);
             ranked = M;
             found = true;
+        } else {
+            reads_remote = true;
+            if (threadIdx.x == 0) sm.ncand = 0u;
+            for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
+            __syncthreads();
         }
     }
     if (!HIST) {
@@ -782,7 +945,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
         // by hundreds of octaves; there can be many after a ReLU.)
         uint32_t np = 0, nz = 0, mn = 0xFFFFFFFFu, mx = 0u;
 #pragma unroll
-        for (int i = 0; i < MAXKPT; ++i) {
+        for (int i = 0; i < KPT; ++i) {
             if (!valid(i)) continue;
             const bool pos = key[i] > 0x80000000u;
             np += pos;
@@ -821,11 +984,12 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
     for (bool first = true; !found; first = false) {
         const int sh = span_shift(hi - lo);
         if (!first) {                                  // (all neighbours have read this CTA's bins)
+            if (threadIdx.x == 0) sm.ncand = 0u;
             for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
             __syncthreads();
         }
 #pragma unroll
-        for (int i = 0; i < MAXKPT; ++i) {
+        for (int i = 0; i < KPT; ++i) {
             const bool in = valid(i) && key[i] >= lo && key[i] <= hi;
             const uint32_t b = (key[i] - lo) >> sh;
             if (in) atomicAdd(&sm.hist[b], 1u);
@@ -838,7 +1002,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
         if (sh == 0) { tkey = lo; need_eq = krem; total_eq = cnt; break; }
         hi = min(hi, lo + ((1u << sh) - 1u));
         if (cnt <= CL_CAND_MAX) {
-            const uint32_t M = cluster_gather<MAXKPT>(cluster, sm, cs, key, kpt, valid, lo, hi, lane, gathers++);
+            const uint32_t M = cluster_gather<KPT>(cluster, sm, cs, crank, key, in_map, lo, hi, lane);
             if (M != 0xFFFFFFFFu) {
                 block_rank(sm, M, krem, lo, hi);
                 tkey = sm.thr[0]; need_eq = sm.thr[1]; total_eq = sm.thr[2];
@@ -847,73 +1011,71 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int kpt, int
             }
         }
     }
-    if (tau && crank == 0 && threadIdx.x == 0) tau[n] = key_float(tkey);
+    const uint32_t tkey_out = HIST ? tkey | 0x80000000u : tkey;               // as float_key
+    if (tau && crank == 0 && threadIdx.x == 0) tau[n] = key_float(tkey_out);
 
     // Ties kept in part need the order of positions, except ties at zero: a position whose norm is zero holds only zero
     // coefficients, so keeping more of them than asked changes nothing downstream (consumers that get the threshold
     // alone keep every position with key >= threshold).
-    const bool ordered = want_rank || (need_eq < total_eq && !zero_thr);       // uniform over the cluster
-    float amax = 0.0f;
-    // Nobody may leave while a neighbour can still read its shared memory.  When no further exchange follows, every CTA
-    // signals here that it is done reading and only waits for the others at the very end (the wait is hidden behind the
-    // pass over the kept positions).
-    if (!ordered) cluster.barrier_arrive();
-    if (!ordered) {
-        // every key >= threshold is kept; nobody needs the order
-        if (amaxpos) {
-#pragma unroll
-            for (int i = 0; i < MAXKPT; ++i)
-                if (valid(i) && key[i] >= tkey) amax = fmaxf(amax, PRE ? pre[PRE ? i : 0] : amaxpos[(size_t)n * P + base + i]);
-        }
-    } else {
-        // ordered compaction: ascending idx, rank map, ties to the lowest positions
-        uint32_t gt = 0, eq = 0;
-#pragma unroll
-        for (int i = 0; i < MAXKPT; ++i) {
-            if (!valid(i)) continue;
-            gt += key[i] > tkey;
-            eq += key[i] == tkey;
-        }
-        uint32_t tot_gt, tot_eq;
-        uint32_t gt_before = block_scan_1024(gt, sm.warp_sums, &tot_gt);
-        uint32_t eq_before = block_scan_1024(eq, sm.warp_sums, &tot_eq);
-        if (threadIdx.x == 0) { sm.cnt[0] = tot_gt; sm.cnt[1] = tot_eq; }
-        cluster.sync();
-        for (int r = 0; r < crank; ++r) {
-            const uint32_t* c = cluster.map_shared_rank(sm.cnt, r);
-            gt_before += c[0];
-            eq_before += c[1];
-        }
-#pragma unroll
-        for (int i = 0; i < MAXKPT; ++i) {
-            if (!valid(i)) continue;
-            const bool is_gt = key[i] > tkey, is_eq = key[i] == tkey;
-            const bool keep = is_gt || (is_eq && eq_before < need_eq);
-            const uint32_t pos = gt_before + min(eq_before, need_eq);
-            if (keep) {
-                if (idx) idx[(size_t)n * k + pos] = base + i;
-                if (amaxpos) amax = fmaxf(amax, PRE ? pre[PRE ? i : 0] : amaxpos[(size_t)n * P + base + i]);
-            }
-            if (rank) rank[(size_t)n * P + base + i] = keep ? (int32_t)pos : -1;
-            gt_before += is_gt;
-            eq_before += is_eq;
-        }
-    }
+    const bool split_ties = need_eq < total_eq && !zero_thr;
+    const bool ordered = want_rank || split_ties;      // uniform over the cluster
     if (thr && crank == 0 && threadIdx.x == 0) {
-        thr[n * 4 + 0] = tkey;
+        thr[n * 4 + 0] = tkey_out;
         thr[n * 4 + 1] = need_eq;
         thr[n * 4 + 2] = ordered ? 1u : 0u;
         thr[n * 4 + 3] = ranked;
     }
-    if (amax_kept) {
+    if (amaxpos && !amax_loaded) load_amax(tkey);
+    uint32_t amax = 0u;                                // (bits of a non-negative float: ordered like an integer)
+    if (!ordered) {
+        // every key >= threshold is kept; nobody needs the order
+        if (amaxpos) {
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, d));
-        if (lane == 0) atomicMax(&sm.amax, __float_as_uint(amax));
+            for (int i = 0; i < KPT; ++i)
+                if (key[i] >= tkey) amax = max(amax, am[i]);           // (what does not exist has no maximum)
+        }
+    } else {
+        // ordered compaction: ascending idx, rank map, ties to the lowest positions
+        uint32_t gt = 0, eq = 0;                       // of the warp
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) {
+            gt += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, valid(i) && key[i] > tkey));
+            eq += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, valid(i) && key[i] == tkey));
+        }
+        if (lane == 0) { sm.warp_sums[warp] = gt; sm.warp_eq[warp] = eq; }
+        __syncthreads();
+        const uint32_t wg = lane < WARPS ? sm.warp_sums[lane] : 0u, we = lane < WARPS ? sm.warp_eq[lane] : 0u;
+        uint32_t gt_before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wg : 0u), eq_before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? we : 0u);
+        const uint32_t tot_gt = __reduce_add_sync(0xFFFFFFFFu, wg), tot_eq = __reduce_add_sync(0xFFFFFFFFu, we);
+        if ((int)threadIdx.x < cs) push_u64(&sm.kept_cnt[crank], (int)threadIdx.x, make_uint2(tot_gt, tot_eq));
+        cluster.sync();
+        const uint2 before = lane < crank ? sm.kept_cnt[lane] : make_uint2(0u, 0u);
+        gt_before += __reduce_add_sync(0xFFFFFFFFu, before.x);
+        eq_before += __reduce_add_sync(0xFFFFFFFFu, before.y);
+        const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) {
+            const bool is_gt = valid(i) && key[i] > tkey, is_eq = valid(i) && key[i] == tkey;
+            const unsigned mg = __ballot_sync(0xFFFFFFFFu, is_gt), me = __ballot_sync(0xFFFFFFFFu, is_eq);
+            const uint32_t g = gt_before + (uint32_t)__popc(mg & below), e = eq_before + (uint32_t)__popc(me & below);
+            const bool keep = is_gt || (is_eq && e < need_eq);
+            const uint32_t pos = g + min(e, need_eq);
+            if (keep) {
+                if (idx) idx[(size_t)n * k + pos] = base + 32 * i;
+                if (amaxpos) amax = max(amax, am[i]);
+            }
+            if (rank && valid(i)) rank[(size_t)n * P + base + 32 * i] = keep ? (int32_t)pos : -1;
+            gt_before += (uint32_t)__popc(mg);
+            eq_before += (uint32_t)__popc(me);
+        }
+    }
+    if (amax_kept) {
+        amax = __reduce_max_sync(0xFFFFFFFFu, amax);
+        if (lane == 0 && amax) atomicMax(&sm.amax, amax);
         __syncthreads();
         if (threadIdx.x == 0 && sm.amax) atomicMax(reinterpret_cast<uint32_t*>(amax_kept), sm.amax);
     }
-    if (!ordered) cluster.barrier_wait();
-    else cluster.sync();                             // nobody leaves while a neighbour may still read its shared memory
+    if (reads_remote) cluster.sync();                  // nobody leaves while a neighbour may still read its shared memory
 }
 
 __global__ void thr_use_rank_kernel(uint32_t* thr, int N)
@@ -923,7 +1085,7 @@ __global__ void thr_use_rank_kernel(uint32_t* thr, int N)
 }
 
 // One cluster per image holds up to this many positions in registers (the path that uses a producer's histograms).
-inline bool select_in_cluster(int P) { return P <= 8 * CL_THREADS * CL_MAXKPT; }
+inline bool select_in_cluster(int P) { return P <= CL_MAXCS * CL_THREADS * CL_MAXKPT; }
 
 // hist1_ready: the caller has already cleared the zero region of the workspace (carve_select_ws(...).hist,
 // zero_bytes) and filled round 1 of the histogram (norm_digit11 of every non-zero norm) before this call.
@@ -937,8 +1099,7 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
     if (ws_bytes < select_ws_bytes(N, P)) return WCC_ERR_WORKSPACE;
     const SelectWs s = carve_select_ws(ws, N, P);
     float* amax_kept = want_amax ? s.amax : nullptr;
-    // one cluster per image while its keys fit in the registers of 8 x 1024 threads
-    // clusters of 16 CTAs (opt-in) for images beyond 64 K positions, when the device schedules them
+    // one cluster per image while its keys fit in the registers of 16 x 256 threads, when the device schedules clusters of 16 CTAs (opt-in)
     static int max_cs[64] = {0};
     int devc = 0;
     WCC_CUDA_TRY(cudaGetDevice(&devc));
@@ -946,8 +1107,8 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         max_cs[devc] = 8;
         bool all = true;
         auto allow16 = [&](auto kern) { all = all && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess; };
-        allow16(select_cluster_kernel<CL_MAXKPT, true>); allow16(select_cluster_kernel<CL_MAXKPT, false>);
-        allow16(select_cluster_kernel<4, true>); allow16(select_cluster_kernel<4, false>);
+        allow16(select_cluster_kernel<8, true>); allow16(select_cluster_kernel<16, true>); allow16(select_cluster_kernel<CL_MAXKPT, true>);
+        allow16(select_cluster_kernel<8, false>); allow16(select_cluster_kernel<16, false>); allow16(select_cluster_kernel<CL_MAXKPT, false>);
         if (all) {
             cudaLaunchConfig_t q = {};
             q.gridDim = dim3(16, 1);
@@ -962,28 +1123,23 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
         (void)cudaGetLastError();
     }
     const int cs_cap = (devc >= 0 && devc < 64) ? max_cs[devc] : 8;
-    if (select_in_cluster(P)) {
-        // as many CTAs per image as useful, then as few threads as hold the keys (<= 16 each): the per-thread cost of
-        // the scans and barriers is fixed, so fewer, busier threads finish sooner
+    if (select_in_cluster(P) && P <= cs_cap * CL_THREADS * CL_MAXKPT) {
         int cs = 1;
-        while (cs < 8 && cs * 512 < P) cs <<= 1;
-        if (cs == 8 && cs_cap == 16 && P > 65536) cs = 16;
-        while (cs > 1 && (long long)N * cs > B200_SMS && P <= cs / 2 * CL_THREADS * CL_MAXKPT) cs >>= 1;      // all images in one wave
-        int threads = 256;
-        const int kpt_goal = hist1_ready ? 4 : CL_MAXKPT;               // few keys per thread when no scans are needed
-        while (threads < CL_THREADS && (long long)cs * threads * kpt_goal < P) threads <<= 1;
-        const int kpt = ceil_div(P, cs * threads);
+        while (cs < cs_cap && cs * CL_THREADS * 8 < P) cs <<= 1;        // about eight keys per thread,
+        while (cs > 1 && (long long)N * cs > 2 * B200_SMS && P <= cs / 2 * CL_THREADS * CL_MAXKPT) cs >>= 1;      // all images in one wave
+        const int kpt = ceil_div(P, cs * CL_THREADS);
         if (amax_kept && !hist1_ready) WCC_CUDA_TRY(cudaMemsetAsync(amax_kept, 0, sizeof(float), st));
         const uint32_t* hist1 = hist1_ready ? s.hist : nullptr;
         const uint32_t* fine_use = hist1_ready ? fine : (const uint32_t*)nullptr;
         const int wr = (want_rank || !thr) ? 1 : 0;
         auto go = [&](auto kern) -> wcc_status {
-            return launch_overlapped(kern, dim3(cs, N), dim3(threads), 0, st, true, cs, nrm2, P, k, kpt, idx, tau, rank, amaxpos, amax_kept,
+            return launch_overlapped(kern, dim3(cs, N), dim3(CL_THREADS), 0, st, true, cs, nrm2, P, k, idx, tau, rank, amaxpos, amax_kept,
                                      hist1, fine_use, thr, wr);
         };
-        // few keys per thread: the instantiation with four key registers
-        if (hist1_ready && fine) return kpt <= 4 ? go(select_cluster_kernel<4, true>) : go(select_cluster_kernel<CL_MAXKPT, true>);
-        return kpt <= 4 ? go(select_cluster_kernel<4, false>) : go(select_cluster_kernel<CL_MAXKPT, false>);
+        // few keys per thread: the instantiations with fewer key registers
+        if (hist1_ready && fine)
+            return kpt <= 8 ? go(select_cluster_kernel<8, true>) : kpt <= 16 ? go(select_cluster_kernel<16, true>) : go(select_cluster_kernel<CL_MAXKPT, true>);
+        return kpt <= 8 ? go(select_cluster_kernel<8, false>) : kpt <= 16 ? go(select_cluster_kernel<16, false>) : go(select_cluster_kernel<CL_MAXKPT, false>);
     }
     if (thr) {                                        // these paths always write idx and the rank map
         thr_use_rank_kernel<<<ceil_div(N, 128), 128, 0, st>>>(thr, N);
