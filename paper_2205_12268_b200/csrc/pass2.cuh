@@ -48,7 +48,9 @@ struct Params {
     int relu;                    // non-zero: y = max(., 0)
     const void* residual;        // NULL, or [N][Cout][H][W] of the activation type, added before the ReLU
     int N, Cin, Cout, H, W, k, krow, npad, nchunk, ksteps_part, b_resident, tmem_cols, tiles_total;
-    int split_from, parts;       // CTAs from split_from on share a tile group `parts` ways by output channels
+    int grp0;                    // the launch's first tile group
+    int split_from, parts, share;    // CTAs from split_from on share a tile group `parts` ways, `share` output channels each
+    int last;                    // non-zero (WPT = 4 only): the launch for the last groups of a layer, behind one with WPT = 2 for the others
     void* y; uint8_t* xq_tap; int32_t* acc_tap; int* status;
 };
 
@@ -101,13 +103,14 @@ pass2_kernel(const Params pr)
     const int t = warp & 3, q = warp >> 2;
     // The last, partial wave of tile groups is spread over the SMs that would idle: `parts` CTAs take one group each, all of
     // them build the whole operand and each runs the contraction and the way out for its share of the output channels.
-    int grp = (int)blockIdx.x, o_lo = 0, o_cnt = pr.npad;
+    int grp = (int)blockIdx.x, o_lo = 0, o_hi = pr.npad;
     if ((int)blockIdx.x >= pr.split_from) {
         const int r = (int)blockIdx.x - pr.split_from;
         grp = pr.split_from + r / pr.parts;
-        o_cnt = pr.npad / pr.parts;
-        o_lo = (r % pr.parts) * o_cnt;
+        o_lo = (r % pr.parts) * pr.share;
+        o_hi = min(o_lo + pr.share, pr.npad);
     }
+    grp += pr.grp0;
     const bool live = grp * TILES + t < pr.tiles_total;
     const int tiles_x = (pr.W + TT::TW - 1) / TT::TW, tiles_y = pr.H / TT::TH;
     int n, ty, tx;
@@ -117,7 +120,7 @@ pass2_kernel(const Params pr)
     const PatchOff off = patch_off<T>(lp, pr.W);
     const uint64_t xb = reinterpret_cast<uint64_t>(pr.x) + (uint64_t)n * pr.Cin * plane;
 
-    pdl_launch();
+    if (WPT == 4) pdl_launch();
     Raw<T> raw[NB];
     const int ureal = (pr.Cin + 7) >> 3;               // units that hold real channels
     auto preload = [&](int u) {
@@ -144,13 +147,15 @@ pass2_kernel(const Params pr)
             *reinterpret_cast<uint4*>(sB + ((size_t)j * bpitch + row) * 16) = v;
         }
     };
-    if (pr.b_resident) load_b(o_lo, o_cnt, 0, 2 * ksteps);
+    if (pr.b_resident) load_b(o_lo, o_hi - o_lo, 0, 2 * ksteps);
     // kept or dropped: from the rank map when the select wrote one (thr[n][2] != 0), else by the threshold key
     float nv[8], mul[8];
     int rk[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s) nv[s] = (live && slot_ok<L>(lp, s)) ? pr.nrm2[(size_t)n * P + lp.pos[s]] : 0.0f;
-    pdl_wait();                                        // what follows reads the selection's results
+    if (WPT == 2 || !pr.last) pdl_wait();              // what follows reads the selection's results
+    // A launch that follows this one for the last groups does not wait for the selection, so it may not run before that is complete.
+    if (WPT == 2) pdl_launch();
     float amax = 0.0f;
     if (I8) amax = (CLAMP && pr.alpha > 0.0f) ? pr.alpha : *pr.amax_kept;
     {
@@ -260,8 +265,8 @@ pass2_kernel(const Params pr)
     bool ok = true;
     uint32_t parity = 0;
     const bool k_parts = pr.ksteps_part < ksteps;
-    for (int n0 = o_lo; n0 < o_lo + o_cnt && ok; n0 += pr.nchunk) {
-        const int cur = min(pr.nchunk, o_lo + o_cnt - n0);
+    for (int n0 = o_lo; n0 < o_hi && ok; n0 += pr.nchunk) {
+        const int cur = min(pr.nchunk, o_hi - n0);
         for (int ks0 = 0; ks0 < ksteps && ok; ks0 += pr.ksteps_part) {
             const int ks1 = min(ksteps, ks0 + pr.ksteps_part);
             if (k_parts && (ks0 > 0 || n0 > o_lo)) preload(ks0 * UPK + q);
@@ -377,6 +382,7 @@ pass2_kernel(const Params pr)
         tc::fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ctl->tmem_base), "r"((uint32_t)pr.tmem_cols) : "memory");
     }
+    if (WPT == 4 && pr.last) pdl_wait();               // complete only after the launch before it: what waits for this one waits for both
 }
 
 }  // namespace p2
@@ -436,12 +442,28 @@ static P2Plan p2_plan(bool two_ctas, int Cout, int krow, bool i8, int L, long lo
     return one;
 }
 
-// CTAs that share each of `groups` tile groups by output channels, where they would not fill the SMs otherwise.
+// CTAs that share each of `groups` tile groups by output channels, where they would not fill the SMs otherwise: the split in equal
+// parts that one_kernel (libwcc.cu) reckons with.
 static int p2_shares(long long groups, int sms, int npad)
 {
     for (int parts = 4; parts >= 2; parts >>= 1)
         if (groups * parts <= sms && npad % (16 * parts) == 0) return parts;
     return 1;
+}
+
+// The split that a launch uses: up to eight CTAs to a group, sixteen channels or more each, the last one perhaps fewer.  Equal parts
+// alone (2 or 4, where the padded channels divide) left 3 x 58 -> 70 channels of 60 x 92 bf16, 80 padded channels, to 23 CTAs:
+// layer 18.5 us, as 115 CTAs 15.5.
+struct P2Split { int parts, share; };
+static P2Split p2_split(long long groups, int sms, int npad)
+{
+    const int units = npad / 16;
+    P2Split best = {1, npad};
+    for (int parts = 2; parts <= 8 && groups * parts <= sms; ++parts) {
+        const int per = ceil_div(units, parts), real = ceil_div(units, per);
+        if (real > best.parts) best = {real, per * 16};
+    }
+    return best;
 }
 
 template <typename T, int L, bool VEC>
@@ -460,47 +482,65 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     if (s != WCC_OK) return s;
     const int sms = di.sms;
     const bool tap = xq_tap || acc_tap;
-    const P2Plan plan = p2_plan(VEC && !tap, Cout, krow, i8, L, groups, sms);
-    if (!plan.ok) return WCC_ERR_SHAPE;
+    const P2Plan first = p2_plan(VEC && !tap, Cout, krow, i8, L, groups, sms);
+    if (!first.ok) return WCC_ERR_SHAPE;
     p2::Params pr = {};
     pr.x = x; pr.Wq = static_cast<const uint8_t*>(Wq); pr.rank = rank; pr.nrm2 = nrm2; pr.thr = thr; pr.amax_kept = amax_kept;
     pr.scale_w = scale_w; pr.qmax = i8 ? (float)((1 << (bits - 1)) - 1) : 1.0f;
     pr.alpha = fx.alpha; pr.relu = fx.relu; pr.residual = fx.residual;
     pr.N = N; pr.Cin = Cin; pr.Cout = Cout; pr.H = H; pr.W = W; pr.k = k; pr.krow = krow; pr.tiles_total = (int)tiles;
-    pr.npad = plan.npad; pr.nchunk = plan.nchunk; pr.ksteps_part = plan.ksteps_part; pr.b_resident = plan.b_resident;
-    pr.tmem_cols = plan.tmem_cols;
     pr.y = y; pr.xq_tap = static_cast<uint8_t*>(xq_tap); pr.acc_tap = acc_tap;
     pr.status = di.status;
-    // The groups of a last, partial wave are shared 4 or 2 ways by output channels when that still fits one wave (the SMs
-    // would idle otherwise).
-    const unsigned rem = sms > 0 ? groups % (unsigned)sms : 0u;
-    pr.parts = rem > 0 ? p2_shares(rem, sms, plan.npad) : 1;
-    pr.split_from = (pr.parts > 1) ? (int)(groups - rem) : (int)groups;
-    const unsigned ctas = (unsigned)pr.split_from + (groups - (unsigned)pr.split_from) * (unsigned)pr.parts;
     const bool clampv = i8 && fx.alpha > 0.0f;
     const int want = (fx.relu ? 1 : 0) | (tap ? 2 : 0) | (clampv ? 4 : 0) | (fx.residual ? 8 : 0);
     const int mode = want == 0 ? 0 : want == 1 ? 1 : (want & 2) == 0 ? 13 : 15;
+    // Groups [g0, g0 + count) by one launch.  The groups of a last, partial wave are shared by output channels when that still fits
+    // one wave (the SMs would idle otherwise).
+    auto run = [&](const P2Plan& plan, unsigned g0, unsigned count) -> wcc_status {
+        pr.npad = plan.npad; pr.nchunk = plan.nchunk; pr.ksteps_part = plan.ksteps_part; pr.b_resident = plan.b_resident;
+        pr.tmem_cols = plan.tmem_cols;
+        pr.grp0 = (int)g0;
+        pr.last = g0 > 0;
+        const unsigned rem = count % (unsigned)sms;
+        const P2Split split = rem > 0 ? p2_split(rem, sms, plan.npad) : P2Split{1, plan.npad};
+        pr.parts = split.parts;
+        pr.share = split.share;
+        pr.split_from = (split.parts > 1) ? (int)(count - rem) : (int)count;
+        const unsigned ctas = (unsigned)pr.split_from + (count - (unsigned)pr.split_from) * (unsigned)split.parts;
 #define WCC_P2(I8V, WPTV, MODEV)                                                                                     \
-    do {                                                                                                            \
-        constexpr auto kern = p2::pass2_kernel<T, L, I8V, WPTV, VEC, MODEV>;                                        \
-        if ((s = allow_smem<kern>(di.dev, 227 * 1024)) != WCC_OK) return s;                                         \
-        return launch_overlapped(kern, dim3(ctas), dim3(p2::TILES * WPTV * 32), plan.smem, st, true, 1, pr);        \
-    } while (0)
+        do {                                                                                                        \
+            constexpr auto kern = p2::pass2_kernel<T, L, I8V, WPTV, VEC, MODEV>;                                    \
+            if ((s = allow_smem<kern>(di.dev, 227 * 1024)) != WCC_OK) return s;                                     \
+            return launch_overlapped(kern, dim3(ctas), dim3(p2::TILES * WPTV * 32), plan.smem, st, true, 1, pr);    \
+        } while (0)
 #define WCC_P2M(I8V, WPTV) do { if (mode == 0) WCC_P2(I8V, WPTV, 0); if (mode == 1) WCC_P2(I8V, WPTV, 1); WCC_P2(I8V, WPTV, 13); } while (0)
-    if constexpr (VEC) {
-        if (mode != 15) {
-            if (i8) { if (plan.wpt == 2) WCC_P2M(true, 2); WCC_P2M(true, 4); }
-            if (plan.wpt == 2) WCC_P2M(false, 2);
-            WCC_P2M(false, 4);
+        if constexpr (VEC) {
+            if (mode != 15) {
+                if (i8) { if (plan.wpt == 2) WCC_P2M(true, 2); WCC_P2M(true, 4); }
+                if (plan.wpt == 2) WCC_P2M(false, 2);
+                WCC_P2M(false, 4);
+            }
+        } else if (mode == 0) {
+            if (i8) WCC_P2(true, 4, 0);
+            WCC_P2(false, 4, 0);
         }
-    } else if (mode == 0) {
-        if (i8) WCC_P2(true, 4, 0);
-        WCC_P2(false, 4, 0);
-    }
-    if (i8) WCC_P2(true, 4, 15);
-    WCC_P2(false, 4, 15);
+        if (i8) WCC_P2(true, 4, 15);
+        WCC_P2(false, 4, 15);
 #undef WCC_P2M
 #undef WCC_P2
+    };
+    // Two CTAs of eight warps to an SM leave a last wave of up to one CTA per SM at half speed.  Its groups get sixteen warps each, in a
+    // launch of their own that takes the SMs as they fall free: 64 -> 64 channels fp32 on 12 x 96 x 320 (360 groups, 64 of them in
+    // the last wave) 65.3 -> 63.7 us a layer, 24 images of it (720, 128) 116.0 -> 109.6.
+    const unsigned wave = 2u * (unsigned)sms, last = groups % wave;
+    if (first.wpt == 2 && groups > wave && last > 0 && last <= (unsigned)sms) {
+        const P2Plan rest = p2_plan(false, Cout, krow, i8, L, last, sms);
+        if (rest.ok) {
+            if ((s = run(first, 0, groups - last)) != WCC_OK) return s;
+            return run(rest, groups - last, last);
+        }
+    }
+    return run(first, 0, groups);
 }
 
 // Second pass.  xq_tap ([N*k][kpad] of int8 or bf16) and acc_tap (int32 [N*k][Cout]) may be NULL.

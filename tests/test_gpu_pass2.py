@@ -1,6 +1,7 @@
 """Second pass of the fused layer at the edges of its tiling: both CTA shapes, K ranges that are built in parts, several
 chunks of output channels, ragged tiles and channel counts.  Comparison and tolerances are those of the layer tests."""
 import pytest
+import torch
 
 from paper_2205_12268_b200 import inputs
 from test_gpu_layer import _run_and_compare, wcc      # noqa: F401  (fixture)
@@ -23,3 +24,34 @@ SHAPES = [  # N, Cin, Cout, H, W, dtype, levels, gamma, bits
 def test_second_pass(wcc, cfg):                       # noqa: F811
     N, Cin, Cout, H, W, dtype, L, gamma, bits = cfg
     _run_and_compare(wcc, inputs.custom("pass2", 4, N, Cin, Cout, H, W, dtype, L, gamma, bits, n_sin=4, fmax=3.0))
+
+
+# One launch or two, and how the last groups are shared.  Plain calls against calls with taps, which take one launch of sixteen warps
+# per group and are compared with the oracle by the tests above: the same integers, so the same bits.
+SPLITS = [
+    (3, 12, 20, 400, 256, "f32", 2, 0.2),             # 300 groups: 296 by one launch, 4 by the next
+    (9, 40, 24, 132, 376, "bf16", 2, 0.3),            # 446: nearly all the SMs once more
+    (5, 10, 50, 440, 272, "bf16", 3, 0.1),            # 619: two waves and 27 groups
+    (4, 9, 12, 216, 360, "f32", 3, 0.25),             # 324 with a ragged width
+    (1, 20, 70, 60, 92, "bf16", 2, 0.25),             # 80 padded channels on few groups: shares of 16
+    (2, 33, 112, 64, 128, "f32", 3, 0.25),            # seven units of sixteen
+    (3, 24, 200, 96, 160, "bf16", 3, 0.25),           # thirteen units among three CTAs: the last one has fewer
+]
+
+
+@pytest.mark.parametrize("cfg", SPLITS, ids=lambda c: "N%d_%dto%d_%dx%d_%s_L%d_g%s" % c)
+def test_launches_and_shares(wcc, cfg):               # noqa: F811
+    N, Cin, Cout, H, W, dtype, L, gamma = cfg
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((N, Cin, H, W), device="cuda", generator=gen).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    Wt = torch.randn((Cout, Cin), device="cuda", generator=gen)
+    W2 = torch.randn((Cin, Cout), device="cuda", generator=gen)
+    k = inputs.keep_count(gamma, H * W)
+    want, _ = wcc.forward(x, Wt, L, k, 8, taps=("Xq", "acc"))
+    for _ in range(2):
+        assert torch.equal(wcc.forward(x, Wt, L, k, 8, y=torch.full_like(want, 7.0)), want)
+    # a layer behind it starts only when both launches are complete
+    relu = torch.relu(want)
+    want2, _ = wcc.forward(relu, W2, L, k, 8, taps=("Xq", "acc"))
+    assert torch.equal(wcc.Chain(x, [Wt, W2], L, k, 8)(x), want2)
+    assert wcc.last_status() == 0
