@@ -48,6 +48,8 @@ static unsigned long long g_launches = 0;
 //    that clear zeroes.  Pass 2 reads x, the quantized weights and the norms early and waits before it reads what the
 //    selection writes.
 //  - A kernel that reads anything early has such a kernel as its predecessor (never the caller's own kernels).
+//  - A layer whose second pass is two launches: the first signals only after its own wait, so the second runs only once the selection
+//    is complete and reads its results without waiting; it waits at its end, and so is complete only after the first.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

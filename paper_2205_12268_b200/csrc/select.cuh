@@ -858,7 +858,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
 #pragma unroll
         for (int i = 0; i < KPT; ++i) {
             const uint32_t take = valid(i) && key[i] >= limit ? 1u : 0u;
-            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n mov.u32 %0, 0;\n @p ld.global.cg.u32 %0, [%1];\n}\n" : "=r"(am[i]) : "l"(a + 32 * i), "r"(take));
+            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n mov.u32 %0, 0;\n @p ld.global.cg.u32 %0, [%1];\n}\n" : "=&r"(am[i]) : "l"(a + 32 * i), "r"(take));
         }
     };
 
