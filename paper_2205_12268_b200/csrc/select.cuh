@@ -935,6 +935,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
             found = true;
         } else {
             reads_remote = true;
+            __syncthreads();                           // (a lone CTA has just read its count)
             if (threadIdx.x == 0) sm.ncand = 0u;
             for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
             __syncthreads();

@@ -14,6 +14,21 @@ SIZES = [(2, 8), (32, 64), (34, 64), (64, 66), (96, 320), (256, 256), (256, 260)
 CLOSE = [1, 2, 63, 64, 256, 257, 2000]       # keys in the threshold's bin
 
 
+def _map_of(v, H, W):
+    """Map of one channel whose low-pass quadrants hold 2 v at one level ([N, H W / 4]), and its norms [N, H W]."""
+    N = v.shape[0]
+    q = v.reshape(N, H // 2, W // 2)
+    x = np.repeat(np.repeat(q, 2, 1), 2, 2)[:, None]
+    nrm = np.zeros((N, H, W), np.float32)
+    nrm[:, :H // 2, :W // 2] = (2 * q) * (2 * q)
+    return torch.from_numpy(x.copy()).cuda(), nrm.reshape(N, H * W)
+
+
+def _largest(nrm, k):
+    """The kept positions: the k largest norms of every image, the lowest positions among equal ones, ascending."""
+    return np.sort(np.argsort(-nrm, axis=1, kind="stable")[:, :k], axis=1)
+
+
 @pytest.mark.parametrize("together", [True, False])
 @pytest.mark.parametrize("close", CLOSE)
 @pytest.mark.parametrize("hw", SIZES)
@@ -25,14 +40,31 @@ def test_candidates_of_the_threshold_bin(wcc, hw, close, together):      # noqa:
     v = (4.0 + rng.integers(0, 4096, n) / 1024.0).astype(np.float32)     # norms of 64 to 256: above the bin below
     at = np.arange(close) + (n - close) // 2 if together else rng.choice(n, close, replace=False)
     v[at] = 1.0 + rng.integers(0, 512, close).astype(np.float32) / 2.0 ** 19            # norms of 4 to 4 + 2^-7: one bin, some of them equal
-    x = torch.from_numpy(np.repeat(np.repeat(v.reshape(H // 2, W // 2), 2, 0), 2, 1)[None, None].copy()).cuda()
+    x, nrm = _map_of(v[None], H, W)
     Wt = torch.ones((1, 1), device="cuda")
-    nrm = np.zeros((H, W), np.float32)
-    nrm[:H // 2, :W // 2] = ((2 * v) * (2 * v)).reshape(H // 2, W // 2)
-    order = np.argsort(-nrm.reshape(-1), kind="stable")
     for k in {n - close + 1, n - close + (close + 1) // 2, n}:
         y, t = wcc.forward(x, Wt, 1, k, 8, taps=("idx", "nrm2"))
-        assert np.array_equal(t["nrm2"].cpu().numpy().reshape(H, W), nrm)
-        assert np.array_equal(t["idx"].cpu().numpy()[0], np.sort(order[:k]))
+        assert np.array_equal(t["nrm2"].cpu().numpy().reshape(1, -1), nrm)
+        assert np.array_equal(t["idx"].cpu().numpy(), _largest(nrm, k))
         assert torch.equal(wcc.forward(x, Wt, 1, k, 8), y)               # (by the threshold alone where no ties are split)
+    assert wcc.last_status() == 0
+
+
+@pytest.mark.parametrize("hw", [(32, 64), (64, 128)])
+def test_crowded_bins_in_lone_ctas(wcc, hw):          # noqa: F811
+    """One CTA per image, on every SM at once, more close keys than it ranks directly: the count that says so is set back only
+    after all of its warps have read it."""
+    H, W = hw
+    n, N = H * W // 4, 320
+    rng = np.random.default_rng(H)
+    v = 1.0 + rng.integers(0, 512, (N, n)).astype(np.float32) / 2.0 ** 19
+    v[::3, rng.choice(n, n - 257, replace=False)] += 4.0             # every third image: one key too many, the others: all of them
+    x, nrm = _map_of(v.astype(np.float32), H, W)
+    Wt = torch.ones((1, 1), device="cuda")
+    for k in (n - 200, n - 3):
+        want = _largest(nrm, k)
+        for _ in range(3):
+            y, t = wcc.forward(x, Wt, 1, k, 8, taps=("idx",))
+            assert np.array_equal(t["idx"].cpu().numpy(), want)
+        assert torch.equal(wcc.forward(x, Wt, 1, k, 8), y)
     assert wcc.last_status() == 0
