@@ -457,7 +457,7 @@ struct ClusterSmem {
     };
     uint32_t slice[SEL_BINS];       // sums over all CTAs of this CTA's slice of bins
     uint32_t warp_sums[CL_THREADS / 32 + 1];
-    uint32_t warp_eq[CL_THREADS / 32];
+    uint32_t warp_gt[CL_THREADS / 32], warp_eq[CL_THREADS / 32];         // (not warp_sums: with a zero threshold no barrier follows its last reading)
     uint32_t slice_total;
     uint32_t res[3];                // found bin, keys above it, keys in it
     uint32_t tot[CL_MAXCS];
@@ -1043,9 +1043,9 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
             gt += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, valid(i) && key[i] > tkey));
             eq += (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, valid(i) && key[i] == tkey));
         }
-        if (lane == 0) { sm.warp_sums[warp] = gt; sm.warp_eq[warp] = eq; }
+        if (lane == 0) { sm.warp_gt[warp] = gt; sm.warp_eq[warp] = eq; }
         __syncthreads();
-        const uint32_t wg = lane < WARPS ? sm.warp_sums[lane] : 0u, we = lane < WARPS ? sm.warp_eq[lane] : 0u;
+        const uint32_t wg = lane < WARPS ? sm.warp_gt[lane] : 0u, we = lane < WARPS ? sm.warp_eq[lane] : 0u;
         uint32_t gt_before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wg : 0u), eq_before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? we : 0u);
         const uint32_t tot_gt = __reduce_add_sync(0xFFFFFFFFu, wg), tot_eq = __reduce_add_sync(0xFFFFFFFFu, we);
         if ((int)threadIdx.x < cs) push_u64(&sm.kept_cnt[crank], (int)threadIdx.x, make_uint2(tot_gt, tot_eq));

@@ -59,3 +59,36 @@ def test_relu_output_as_next_input_is_fast_path_correct(wcc):
     want = oracle.forward(w.x_f32(), w.Wt, 3, w.k, 8, out_bf16=True, relu=True)
     assert wcc.last_status() == 0
     assert np.array_equal(y.float().cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("nonzero", [0, 1, 37])
+@pytest.mark.parametrize("cfg", [(40, 300, 320, 32, 64), (12, 320, 304, 64, 128)], ids=lambda c: "N%d_%dto%d_%dx%d" % c)
+def test_ordered_with_a_zero_threshold(wcc, cfg, nonzero):
+    """Layers that gather their columns always want the order of the kept positions, here with fewer non-zero norms than kept
+    positions in every image (none at all in an all-zero map): the zeros that are kept are the lowest positions."""
+    N, Cin, Cout, H, W = cfg
+    L, k = 1, 600
+    assert wcc.workspace_bytes(N, Cin, Cout, H, W, L, k, 8, 0) > N * k * (Cin + 4 * Cout)        # gathered: compressed matrix and accumulators
+    rng = np.random.default_rng(nonzero)
+    x = np.zeros((N, Cin, H, W), np.float32)
+    at = np.zeros((N, nonzero), np.int64)
+    for n in range(N):
+        blocks = rng.choice(H * W // 4, nonzero, replace=False)
+        r, c = blocks // (W // 2), blocks % (W // 2)
+        at[n] = r * W + c
+        v = rng.integers(1, 9, (Cin, nonzero)).astype(np.float32)
+        for dr in (0, 1):
+            for dc in (0, 1):
+                x[n][:, 2 * r + dr, 2 * c + dc] = v
+    Wt = torch.ones((Cout, Cin), device="cuda")
+    want = np.stack([np.sort(np.concatenate([at[n], np.setdiff1d(np.arange(H * W), at[n])[:k - nonzero]])) for n in range(N)])
+    xd = torch.from_numpy(x).cuda()
+    for _ in range(3):
+        y, t = wcc.forward(xd, Wt, L, k, 8, taps=("idx", "acc"))
+        assert np.array_equal(t["idx"].cpu().numpy(), want)
+        assert torch.equal(wcc.forward(xd, Wt, L, k, 8), y)
+    assert wcc.last_status() == 0
+    acc = t["acc"].reshape(N, k, Cout)
+    assert int((acc[:, :, 0] != 0).sum()) == N * nonzero and torch.equal(acc, acc[:, :, :1].expand_as(acc))
+    if nonzero == 0:
+        assert not y.any()
