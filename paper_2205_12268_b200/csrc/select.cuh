@@ -486,10 +486,11 @@ __device__ __forceinline__ void push_u64(uint2* addr, int rank, uint2 v)
     asm volatile("{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n st.shared::cluster.v2.u32 [ra], {%2, %3};\n}\n" ::"r"(tc::smem_u32(addr)), "r"(rank), "r"(v.x), "r"(v.y) : "memory");
 }
 
-// exclusive scan over the threads of the block (256, 512 or 1024); every thread also gets the total
-__device__ __forceinline__ uint32_t block_scan_1024(uint32_t v, uint32_t* warp_sums, uint32_t* total)
+// Exclusive scan over the threads of a block of CL_THREADS; every thread also gets the total, which warp_sums[WARPS] carries.
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t (&warp_sums)[CL_THREADS / 32 + 1], uint32_t* total)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    constexpr int WARPS = CL_THREADS / 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t inc = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -499,19 +500,19 @@ __device__ __forceinline__ uint32_t block_scan_1024(uint32_t v, uint32_t* warp_s
     if (lane == 31) warp_sums[w] = inc;
     __syncthreads();
     if (w == 0) {
-        const uint32_t s = (lane < nw) ? warp_sums[lane] : 0u;
+        const uint32_t s = (lane < WARPS) ? warp_sums[lane] : 0u;
         uint32_t si = s;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, si, d);
             if (lane >= d) si += t;
         }
-        if (lane < nw) warp_sums[lane] = si - s;
-        if (lane == 31) warp_sums[32] = si;
+        if (lane < WARPS) warp_sums[lane] = si - s;
+        if (lane == 31) warp_sums[WARPS] = si;
     }
     __syncthreads();
     const uint32_t res = warp_sums[w] + inc - v;
-    *total = warp_sums[32];
+    *total = warp_sums[WARPS];
     __syncthreads();
     return res;
 }
@@ -531,7 +532,7 @@ __device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, Clu
         mine += sum;
     }
     uint32_t total;
-    block_scan_1024(mine, sm.warp_sums, &total);
+    block_scan(mine, sm.warp_sums, &total);
     if (threadIdx.x == 0) sm.slice_total = total;
     cluster.sync();                                  // all slices and slice totals complete
     if (threadIdx.x < cs) sm.tot[threadIdx.x] = *cluster.map_shared_rank(&sm.slice_total, threadIdx.x);
@@ -555,7 +556,7 @@ __device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, Clu
         mysum += c[i];
     }
     uint32_t tot2;
-    const uint32_t before = block_scan_1024(mysum, sm.warp_sums, &tot2);
+    const uint32_t before = block_scan(mysum, sm.warp_sums, &tot2);
     if (before < kin && kin <= before + mysum) {
         uint32_t a = before;
 #pragma unroll
@@ -766,7 +767,7 @@ __device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t
             c[i] = (i < per) ? sm.hist[top - i] : 0u;
             mysum += c[i];
         }
-        const uint32_t before = block_scan_1024(mysum, sm.warp_sums, &tot);
+        const uint32_t before = block_scan(mysum, sm.warp_sums, &tot);
         if (before < krem && krem <= before + mysum) {
             uint32_t a = before;
 #pragma unroll

@@ -90,6 +90,19 @@ def test_select_random(wcc, P):
         _check_select(wcc, nrm, k)
 
 
+@pytest.mark.parametrize("P,crowd", [(131072, 3000), (131071, 1500), (70001, 20000)])
+def test_select_rounds_over_sixteen_ctas(wcc, P, crowd):
+    """Clusters of sixteen CTAs without histograms, with so many equal norms, spread over the CTAs or all in the last ones, that the
+    range is narrowed to the end: the totals of all sixteen slices of bins are needed in every round."""
+    rng = np.random.default_rng(P)
+    nrm = (rng.random((3, P)) ** 4 * 100).astype(np.float32)
+    nrm[0, rng.choice(P, crowd, replace=False)] = 1.0
+    nrm[1, P - crowd:] = 1.0
+    nrm[2] = np.ldexp(1.0, rng.integers(-120, 120, P)).astype(np.float32)          # few values over the whole range of bins
+    for k in (1, int((nrm[0] > 1).sum()) + crowd // 2, int((nrm[1] > 1).sum()) + crowd // 2, P // 2, P - 1):
+        _check_select(wcc, nrm, k)
+
+
 @pytest.mark.parametrize("N,P", [(2, 200000), (10, 200000)])
 def test_select_large_images_other_code_paths(wcc, N, P):
     """More keys per image than one cluster holds: the cooperative single kernel (few CTAs) and the one-kernel-per-phase
