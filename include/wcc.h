@@ -327,6 +327,16 @@ wcc_status wcc_debug_set_wait_limit(unsigned polls);
 wcc_status wcc_debug_wait_selftest(void* stream);
 
 /*
+ * Test hook: the selection of one image as wcc_forward launches it, on histograms that the caller supplies.  Histograms that do not
+ * match the norms (in a layer: a workspace that something else writes to) end in a selection of at most k positions, usually none.
+ *   nrm2 in: fp32 [P], P <= 16384      hist11 in: uint32 [2048], hist16 in: uint32 [65536]: the non-zero norms by the 11 and the 16 bits
+ *   below their sign      thr out: uint32 [4]: threshold as an ordered key, ties kept, 1 if rank and idx hold the kept set, -
+ *   rank out: int32 [P] (place among the kept positions or -1), idx out: int32 [k], with want_rank or where ties are kept in part
+ */
+wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* hist11, const unsigned* hist16, int want_rank, unsigned* thr,
+                            int* rank, int* idx, void* stream);
+
+/*
  * Measurement helpers (no counterpart in the paper).  With profiling on, wcc_forward records CUDA events on its
  * stream around each stage; wcc_profile_read waits for the last recorded call and writes, to the HOST array ms, the
  * milliseconds of, for wcc_forward_staged: 0 Haar transform + norms, 1 top-k select + compaction, 2 weight

@@ -1110,6 +1110,19 @@ wcc_status wcc_debug_wait_selftest(void* stream)
     return WCC_OK;
 }
 
+wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* hist11, const unsigned* hist16, int want_rank, unsigned* thr,
+                            int* rank, int* idx, void* stream)
+{
+    if (!nrm2 || !hist11 || !hist16 || !thr || !rank || !idx) return WCC_ERR_NULL;
+    if (P < 1 || P > 8 * CL_THREADS * 8) return WCC_ERR_SHAPE;
+    if (k < 1 || k > P) return WCC_ERR_K;
+    if (!aligned16(hist11) || !aligned16(hist16) || !aligned16(thr)) return WCC_ERR_ALIGN;
+    int cs = 1;
+    while (cs * CL_THREADS * 8 < P) cs <<= 1;
+    return launch_overlapped(select_cluster_kernel<8, true>, dim3(cs, 1), dim3(CL_THREADS), 0, static_cast<cudaStream_t>(stream), true, cs, nrm2, P, k,
+                             idx, nullptr, rank, nullptr, nullptr, hist11, hist16, thr, want_rank);
+}
+
 wcc_status wcc_profile_enable(int on)
 {
     g_profile = on != 0;

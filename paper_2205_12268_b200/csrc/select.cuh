@@ -537,14 +537,16 @@ __device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, Clu
     cluster.sync();                                  // all slices and slice totals complete
     if (threadIdx.x < cs) sm.tot[threadIdx.x] = *cluster.map_shared_rank(&sm.slice_total, threadIdx.x);
     __syncthreads();
+    if (threadIdx.x == 0) sm.res[2] = 0u;            // (a barrier follows: the scan's)
     uint32_t above_slices = 0;
     int target = 0;
+    bool any = false;                                // (fewer keys than krem: histograms that do not match them)
     for (int r = cs - 1; r >= 0; --r) {              // slices from the top bins downwards
         const uint32_t t = sm.tot[r];
-        if (krem <= above_slices + t) { target = r; break; }
+        if (krem <= above_slices + t) { target = r; any = true; break; }
         above_slices += t;
     }
-    const uint32_t kin = krem - above_slices;        // rank inside the target slice, from its top bin
+    const uint32_t kin = any ? krem - above_slices : 0u;        // rank inside the target slice, from its top bin
     const uint32_t* rs = cluster.map_shared_rank(sm.slice, target);
     // thread t covers the `per` bins (B-1 - t*per) downwards of the slice (per <= 8)
     const int per = (B + (int)blockDim.x - 1) / (int)blockDim.x;
@@ -926,7 +928,8 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
         }
     }
     cluster.barrier_wait();                            // every CTA of the cluster runs
-    if (HIST && !zero_thr) {
+    if (HIST && !found && krem == 0) { tkey = 0xFFFFFFFFu; found = true; }       // no such fine bin: keep nothing, as above
+    if (HIST && !found) {
         if (amaxpos) { load_amax(lo); amax_loaded = true; }          // (on their way while the threshold is found)
         const uint32_t M = cluster_exchange<KPT>(sm, cs, crank, key, in_map, lo, hi, warp, lane);
         if (M != 0xFFFFFFFFu) {
@@ -999,6 +1002,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
         uint32_t b, above;
         cluster_find_bin(cluster, sm, cs, crank, SEL_BINS, krem, b, above);
         const uint32_t cnt = sm.res[2];
+        if (HIST && cnt == 0) { tkey = 0xFFFFFFFFu; need_eq = total_eq = 0u; break; }    // fewer keys than the histograms say: keep nothing
         krem -= above;
         lo += b << sh;
         if (sh == 0) { tkey = lo; need_eq = krem; total_eq = cnt; break; }
@@ -1060,8 +1064,8 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
             const bool is_gt = valid(i) && key[i] > tkey, is_eq = valid(i) && key[i] == tkey;
             const unsigned mg = __ballot_sync(0xFFFFFFFFu, is_gt), me = __ballot_sync(0xFFFFFFFFu, is_eq);
             const uint32_t g = gt_before + (uint32_t)__popc(mg & below), e = eq_before + (uint32_t)__popc(me & below);
-            const bool keep = is_gt || (is_eq && e < need_eq);
             const uint32_t pos = g + min(e, need_eq);
+            const bool keep = (is_gt || (is_eq && e < need_eq)) && pos < (uint32_t)k;          // (beyond k: only where the histograms do not match)
             if (keep) {
                 if (idx) idx[(size_t)n * k + pos] = base + 32 * i;
                 if (amaxpos) amax = max(amax, am[i]);

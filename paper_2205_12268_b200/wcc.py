@@ -21,7 +21,7 @@ _STATUS = {0: "ok", 1: "null pointer", 2: "bad shape", 3: "k out of range", 4: "
 EXPORTS = ("wcc_staged_workspace_bytes", "wcc_forward_staged", "wcc_workspace_bytes", "wcc_select_workspace_bytes", "wcc_haar_fwd", "wcc_haar_inv", "wcc_select_topk",
            "wcc_forward", "wcc_forward_debug", "wcc_kpad", "wcc_last_status", "wcc_status_str",
            "wcc_profile_enable", "wcc_profile_read", "wcc_kernel_launches", "wcc_select_topk_static",
-           "wcc_debug_set_wait_limit", "wcc_debug_wait_selftest", "wcc_forward_ex", "wcc_chain_workspace_bytes",
+           "wcc_debug_set_wait_limit", "wcc_debug_wait_selftest", "wcc_debug_select", "wcc_forward_ex", "wcc_chain_workspace_bytes",
            "wcc_chain_forward", "wcc_select_bitmap_workspace_bytes", "wcc_select_topk_bitmap",
            "wcc_padded_workspace_bytes", "wcc_forward_padded", "wcc_dwconv_haar_fwd", "wcc_block_workspace_bytes",
            "wcc_block_forward", "wcc_dwt_fwd", "wcc_dwt_inv", "wcc_wavelet_workspace_bytes", "wcc_forward_wavelet")
@@ -125,6 +125,8 @@ def lib() -> C.CDLL:
         L.wcc_debug_set_wait_limit.argtypes = [C.c_uint]
         L.wcc_debug_wait_selftest.restype = i
         L.wcc_debug_wait_selftest.argtypes = [vp]
+        L.wcc_debug_select.restype = i
+        L.wcc_debug_select.argtypes = [vp, i, i, vp, vp, i, vp, vp, vp, vp]
         L.wcc_status_str.restype = C.c_char_p
         L.wcc_status_str.argtypes = [i]
         _lib = L
@@ -489,6 +491,12 @@ def debug_set_wait_limit(polls: int):
 def debug_wait_selftest():
     """Enqueues one warp that waits on a barrier nobody arrives on (it gives up after the wait limit)."""
     _check(lib().wcc_debug_wait_selftest(_stream()), "wcc_debug_wait_selftest")
+
+
+def debug_select(nrm2, k: int, hist11, hist16, want_rank: bool, thr, rank, idx):
+    """The selection inside a layer on one image's norms and the caller's histograms of them (wcc_debug_select)."""
+    _check(lib().wcc_debug_select(nrm2.data_ptr(), nrm2.numel(), k, hist11.data_ptr(), hist16.data_ptr(), int(want_rank), thr.data_ptr(),
+                                  rank.data_ptr(), idx.data_ptr(), _stream()), "wcc_debug_select")
 
 
 def profile_enable(on: bool):
