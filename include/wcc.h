@@ -331,9 +331,11 @@ wcc_status wcc_debug_wait_selftest(void* stream);
  * match the norms (in a layer: a workspace that something else writes to) end in a selection of at most k positions, usually none.
  *   nrm2 in: fp32 [P], P <= 16384      hist11 in: uint32 [2048], hist16 in: uint32 [65536]: the non-zero norms by the 11 and the 16 bits
  *   below their sign      thr out: uint32 [4]: threshold as an ordered key, ties kept, 1 if rank and idx hold the kept set, -
+ *   late: non-zero: where several blocks share the image, one waits for more than the others send.  Its bounded wait runs out (set a small
+ *   limit), the status word says so, and nothing is kept there, nor by those that would need to hear from it.
  *   rank out: int32 [P] (place among the kept positions or -1), idx out: int32 [k], with want_rank or where ties are kept in part
  */
-wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* hist11, const unsigned* hist16, int want_rank, unsigned* thr,
+wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* hist11, const unsigned* hist16, int want_rank, int late, unsigned* thr,
                             int* rank, int* idx, void* stream);
 
 /*

@@ -1110,7 +1110,7 @@ wcc_status wcc_debug_wait_selftest(void* stream)
     return WCC_OK;
 }
 
-wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* hist11, const unsigned* hist16, int want_rank, unsigned* thr,
+wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* hist11, const unsigned* hist16, int want_rank, int late, unsigned* thr,
                             int* rank, int* idx, void* stream)
 {
     if (!nrm2 || !hist11 || !hist16 || !thr || !rank || !idx) return WCC_ERR_NULL;
@@ -1119,8 +1119,8 @@ wcc_status wcc_debug_select(const float* nrm2, int P, int k, const unsigned* his
     if (!aligned16(hist11) || !aligned16(hist16) || !aligned16(thr)) return WCC_ERR_ALIGN;
     int cs = 1;
     while (cs * CL_THREADS * 8 < P) cs <<= 1;
-    return launch_overlapped(select_cluster_kernel<8, true>, dim3(cs, 1), dim3(CL_THREADS), 0, static_cast<cudaStream_t>(stream), true, cs, nrm2, P, k,
-                             idx, nullptr, rank, nullptr, nullptr, hist11, hist16, thr, want_rank);
+    return launch_overlapped(late ? select_cluster_kernel<8, true, true> : select_cluster_kernel<8, true>, dim3(cs, 1), dim3(CL_THREADS), 0,
+                             static_cast<cudaStream_t>(stream), true, cs, nrm2, P, k, idx, nullptr, rank, nullptr, nullptr, hist11, hist16, thr, want_rank);
 }
 
 wcc_status wcc_profile_enable(int on)

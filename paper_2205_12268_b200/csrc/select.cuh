@@ -448,6 +448,7 @@ constexpr int CL_MAXCS = 16;          // 8 is the portable cluster size; 16 need
 constexpr int CL_CAND_MAX = 1024;    // candidates a CTA has room for: CL_CAND_MAX / cs from each CTA of the cluster; beyond that: another round
 constexpr int CL_MSG = 64;           // words of the message in which a CTA sends up to CL_MSG - 1 candidates
 constexpr int CL_FEW = 256;          // candidates ranked by few_rank
+constexpr uint32_t TOO_MANY = 0xFFFFFFFFu, GAVE_UP = 0xFFFFFFFEu;      // instead of a number of candidates (GAVE_UP: or of kept keys)
 constexpr int FINE_BINS = 65536;     // histogram of the 16 bits below the sign of every norm, filled by the producer of the norms
 
 struct ClusterSmem {
@@ -470,7 +471,8 @@ struct ClusterSmem {
     __align__(16) uint32_t counts[2][CL_THREADS / 32];         // of a round of few_rank, per warp
     uint32_t pushed[CL_CAND_MAX];   // candidates of every CTA of the cluster, CL_CAND_MAX / cs slots each
     uint32_t pushed_cnt[CL_MAXCS];  // how many each has (more than its slots: none were sent)
-    uint2 kept_cnt[CL_MAXCS];       // keys above / equal to the threshold in every CTA
+    uint2 kept_cnt[CL_MAXCS];       // keys above / equal to the threshold in every CTA; GAVE_UP until it has sent them
+    uint32_t narrowing[CL_MAXCS];   // non-zero: the CTA goes on to the histogram rounds
     __align__(16) uint32_t all[CL_CAND_MAX];      // keys of `pushed` without the gaps
     uint32_t thr[3];                // threshold key, ties to keep, ties in total
     __align__(16) uint32_t range[4];              // positive keys, zeros, smallest positive key, largest key
@@ -518,12 +520,15 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t (&warp_sums)
 }
 
 // After every CTA has filled sm.hist: find the bin holding the krem-th key from the top over the whole cluster.
-// nbins = 2048 or 1024.  Contains two cluster barriers.  Every thread of every CTA returns the same (bin, above).
-__device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, ClusterSmem& sm, int cs, int crank, int nbins,
+// nbins = 2048 or 1024.  Contains two cluster barriers.  Every thread of every CTA returns the same (bin, above), or false after
+// the first barrier if a CTA of the cluster has given up (HIST: see cluster_exchange).
+template <bool HIST>
+__device__ __forceinline__ bool cluster_find_bin(cg::cluster_group& cluster, ClusterSmem& sm, int cs, int crank, int nbins,
                                                  uint32_t krem, uint32_t& bin, uint32_t& above)
 {
     const int B = nbins / cs;                        // bins per slice: 128 .. 2048
     cluster.sync();                                  // all local histograms complete
+    if (HIST && __any_sync(0xFFFFFFFFu, (int)(threadIdx.x & 31) < cs && sm.narrowing[threadIdx.x & (CL_MAXCS - 1)] == 0u)) return false;
     uint32_t mine = 0;
     for (int t = threadIdx.x; t < B; t += blockDim.x) {
         uint32_t sum = 0;
@@ -571,13 +576,14 @@ __device__ __forceinline__ void cluster_find_bin(cg::cluster_group& cluster, Clu
     bin = sm.res[0];
     above = sm.res[1];
     __syncthreads();
+    return true;
 }
 
 
 // Shift that maps a span of keys onto at most 2048 bins.
 __device__ __forceinline__ int span_shift(uint32_t span) { return max(0, 32 - __clz(span) - 11); }
 
-// Gathers the keys in [lo, hi] of the whole cluster into sm.all of every CTA; returns how many there are (0xFFFFFFFF: too many).
+// Gathers the keys in [lo, hi] of the whole cluster into sm.all of every CTA; returns how many there are or TOO_MANY.
 // One cluster barrier.  sm.ncand is zero before.
 template <int KPT>
 __device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, ClusterSmem& sm, int cs, int crank, const uint32_t (&key)[KPT], uint32_t in_map,
@@ -605,7 +611,7 @@ __device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, C
             push_u32(&sm.pushed[(uint32_t)crank * slots + t / (uint32_t)cs], (int)(t & (uint32_t)(cs - 1)), sm.local[t / (uint32_t)cs]);
     cluster.sync();
     const uint32_t cnt = lane < cs ? sm.pushed_cnt[lane] : 0u, M = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    if (__any_sync(0xFFFFFFFFu, cnt > slots)) return 0xFFFFFFFFu;
+    if (__any_sync(0xFFFFFFFFu, cnt > slots)) return TOO_MANY;
     uint32_t upto = cnt;                               // of the CTAs up to `lane`
 #pragma unroll
     for (int d = 1; d < CL_MAXCS; d <<= 1) {
@@ -622,15 +628,39 @@ __device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, C
     return M;
 }
 
+// Waits for the messages of all CTAs of the cluster, at most so long.
+__device__ __forceinline__ bool cluster_listen(ClusterSmem& sm)
+{
+    const uint32_t bar = tc::smem_u32(&sm.msg_bar), limit = tc::c_wait_limit;
+    uint32_t ok = 0;
+    for (uint32_t it = 0; it < limit && !ok; ++it)
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(ok) : "r"(bar), "r"(1000u) : "memory");
+    return ok != 0u;
+}
+
+// A CTA whose wait ran out may not leave at once: messages are still on their way to it, and neighbours that heard everything may go
+// on to a cluster barrier (histogram rounds, ordered compaction).  It joins one barrier, which ends when every neighbour has left or come
+// to its first one, and listens a little longer.  Behind that barrier neighbours look whether all have sent what is sent in
+// front of it, and otherwise give up too, without a further barrier.
+__device__ __forceinline__ void cluster_give_up(ClusterSmem& sm)
+{
+    if (threadIdx.x == 0) atomicExch(&g_status, (int)WCC_ERR_TIMEOUT);
+    cg::this_cluster().sync();
+    cluster_listen(sm);
+}
+
 // The short way of a gather: every CTA sends one message of fixed size to every CTA (st.async, counted by the receiver's mbarrier).
 // A cluster barrier would also wait for everything that its threads have under way in global memory (its release): 1.6 to 3.4
 // us for the gather and its block barriers against 0.8 to 1.3.  The candidates end up in sm.few; returns how many there are,
-// 0xFFFFFFFF if there are too many for a message or for sm.few, or 0 with the status set when the wait ran out.
+// or TOO_MANY for a message or for sm.few, or GAVE_UP with the status set when the wait ran out.
+// st.async is left to launches with the cluster attribute (a lone CTA keeps its candidates): in a launch without it the store faulted
+// once, although st.shared::cluster to the own CTA works there.  Nothing documented says why.
 template <int KPT>
 __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, int crank, const uint32_t (&key)[KPT], uint32_t in_map, uint32_t lo,
                                                      uint32_t hi, int warp, int lane)
 {
-    const bool alone = cs == 1;                        // (a launch without clusters: st.async is for launches that have them)
+    const bool alone = cs == 1;                        // (a launch without clusters)
     uint32_t in = 0u;
 #pragma unroll
     for (int i = 0; i < KPT; ++i) in |= (key[i] >= lo && key[i] <= hi) ? 1u << i : 0u;
@@ -648,7 +678,7 @@ __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, in
             }
     }
     __syncthreads();
-    if (alone) return sm.ncand <= CL_FEW ? sm.ncand : 0xFFFFFFFFu;
+    if (alone) return sm.ncand <= CL_FEW ? sm.ncand : TOO_MANY;
     if ((int)threadIdx.x < cs * (CL_MSG / 4)) {        // sixteen bytes to one CTA per thread
         const int to = (int)threadIdx.x / (CL_MSG / 4), j = (int)threadIdx.x % (CL_MSG / 4);
         uint4 w = *reinterpret_cast<const uint4*>(&sm.out[4 * j]);
@@ -657,17 +687,12 @@ __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, in
                      " st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [ra], {%3, %4, %5, %6}, [rb];\n}\n"
                      ::"r"(tc::smem_u32(&sm.msg[crank][4 * j])), "r"(tc::smem_u32(&sm.msg_bar)), "r"(to), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w) : "memory");
     }
-    const uint32_t bar = tc::smem_u32(&sm.msg_bar), limit = tc::c_wait_limit;
-    uint32_t ok = 0;
-    for (uint32_t it = 0; it < limit && !ok; ++it)
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(ok) : "r"(bar), "r"(1000u) : "memory");
-    if (!__syncthreads_and(ok ? 1 : 0)) {              // (the same for the whole block)
-        if (threadIdx.x == 0) atomicExch(&g_status, (int)WCC_ERR_TIMEOUT);
-        return 0u;
+    if (!__syncthreads_and(cluster_listen(sm) ? 1 : 0)) {        // (the same for the whole block)
+        cluster_give_up(sm);
+        return GAVE_UP;
     }
     const uint32_t cnt = lane < cs ? sm.msg[lane][0] : 0u, M = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    if (__any_sync(0xFFFFFFFFu, cnt >= CL_MSG) || M > CL_FEW) return 0xFFFFFFFFu;
+    if (__any_sync(0xFFFFFFFFu, cnt >= CL_MSG) || M > CL_FEW) return TOO_MANY;
     uint32_t upto = cnt;                               // of the CTAs up to `lane`
 #pragma unroll
     for (int d = 1; d < CL_MAXCS; d <<= 1) {
@@ -805,15 +830,15 @@ __device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t
 // Blocks of 256 threads: what every warp has to do besides its keys (some 500 instructions) was most of the issue slots of 1024.
 // Measured, from the end of the first pass to the start of the second's threshold (us, blocks of up to 1024 threads that read each
 // other's candidates after a cluster barrier -> this): 2 x 131072 positions 14.3 -> 8.3, 12 x 30720 7.8 -> 5.3, 4 x 32768 8.0 -> 6.2.
-// KPT: keys per thread (8, 16 or 32).  HIST: the histograms are supplied.
-template <int KPT, bool HIST>
-__global__ void __launch_bounds__(CL_THREADS, 2)
-select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __restrict__ idx, float* __restrict__ tau,
-                      int32_t* __restrict__ rank, const float* __restrict__ amaxpos, float* __restrict__ amax_kept,
-                      const uint32_t* __restrict__ hist1, const uint32_t* __restrict__ fine, uint32_t* __restrict__ thr,
-                      int want_rank)
+// KPT: keys per thread (8, 16 or 32).  HIST: the histograms are supplied.  LATE (a test's): the second CTA expects more than is sent to
+// it, so its wait runs out.
+// False: this CTA has given up, or has not heard from one that has.
+template <int KPT, bool HIST, bool LATE>
+__device__ __forceinline__ bool cluster_select(ClusterSmem& sm, const float* __restrict__ nrm2, int P, int k, int32_t* __restrict__ idx,
+                                               float* __restrict__ tau, int32_t* __restrict__ rank, const float* __restrict__ amaxpos,
+                                               float* __restrict__ amax_kept, const uint32_t* __restrict__ hist1, const uint32_t* __restrict__ fine,
+                                               uint32_t* __restrict__ thr, int want_rank)
 {
-    __shared__ ClusterSmem sm;
     cg::cluster_group cluster = cg::this_cluster();
     const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
     const int n = blockIdx.y;
@@ -827,10 +852,11 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
     if (threadIdx.x < 4) sm.range[threadIdx.x] = threadIdx.x == 2 ? 0xFFFFFFFFu : 0u;
     if (threadIdx.x < CL_MSG) sm.out[threadIdx.x] = 0u;
     for (int i = threadIdx.x; i < CL_FEW; i += CL_THREADS) sm.few[i] = 0u;
+    if (HIST && threadIdx.x < CL_MAXCS) { sm.kept_cnt[threadIdx.x].x = GAVE_UP; sm.narrowing[threadIdx.x] = 0u; }
     if (threadIdx.x == 0) {
         tc::mbar_init(tc::smem_u32(&sm.msg_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tc::mbar_expect_tx(tc::smem_u32(&sm.msg_bar), (uint32_t)(cs * CL_MSG * 4));
+        tc::mbar_expect_tx(tc::smem_u32(&sm.msg_bar), (uint32_t)(cs * CL_MSG * 4 + (LATE && crank == 1 ? 16 : 0)));
         sm.amax = 0u;
         sm.ncand = 0u;
         sm.thr[0] = 0xFFFFFFFFu; sm.thr[1] = 0u; sm.thr[2] = 0u;          // keep nothing unless a candidate is found (histograms
@@ -932,7 +958,8 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
     if (HIST && !found) {
         if (amaxpos) { load_amax(lo); amax_loaded = true; }          // (on their way while the threshold is found)
         const uint32_t M = cluster_exchange<KPT>(sm, cs, crank, key, in_map, lo, hi, warp, lane);
-        if (M != 0xFFFFFFFFu) {
+        if (HIST && M == GAVE_UP) { return false; }
+        if (M != TOO_MANY) {
             tkey = 0xFFFFFFFFu;                        // keep nothing if there are fewer (histograms that do not match the keys)
             if (M >= krem) few_rank(sm, M, krem, hi & ~0x7FFFu, warp, lane, tkey, need_eq, total_eq);
             ranked = M;
@@ -940,6 +967,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
         } else {
             reads_remote = true;
             __syncthreads();                           // (a lone CTA has just read its count)
+            if ((int)threadIdx.x < cs) push_u32(&sm.narrowing[crank], (int)threadIdx.x, 1u);
             if (threadIdx.x == 0) sm.ncand = 0u;
             for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
             __syncthreads();
@@ -1000,7 +1028,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
             if (in) atomicAdd(&sm.hist[b], 1u);
         }
         uint32_t b, above;
-        cluster_find_bin(cluster, sm, cs, crank, SEL_BINS, krem, b, above);
+        if (!cluster_find_bin<HIST>(cluster, sm, cs, crank, SEL_BINS, krem, b, above)) { return false; }
         const uint32_t cnt = sm.res[2];
         if (HIST && cnt == 0) { tkey = 0xFFFFFFFFu; need_eq = total_eq = 0u; break; }    // fewer keys than the histograms say: keep nothing
         krem -= above;
@@ -1009,7 +1037,7 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
         hi = min(hi, lo + ((1u << sh) - 1u));
         if (cnt <= CL_CAND_MAX) {
             const uint32_t M = cluster_gather<KPT>(cluster, sm, cs, crank, key, in_map, lo, hi, lane);
-            if (M != 0xFFFFFFFFu) {
+            if (M != TOO_MANY) {
                 block_rank(sm, M, krem, lo, hi);
                 tkey = sm.thr[0]; need_eq = sm.thr[1]; total_eq = sm.thr[2];
                 ranked = M;
@@ -1055,9 +1083,10 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
         const uint32_t tot_gt = __reduce_add_sync(0xFFFFFFFFu, wg), tot_eq = __reduce_add_sync(0xFFFFFFFFu, we);
         if ((int)threadIdx.x < cs) push_u64(&sm.kept_cnt[crank], (int)threadIdx.x, make_uint2(tot_gt, tot_eq));
         cluster.sync();
-        const uint2 before = lane < crank ? sm.kept_cnt[lane] : make_uint2(0u, 0u);
-        gt_before += __reduce_add_sync(0xFFFFFFFFu, before.x);
-        eq_before += __reduce_add_sync(0xFFFFFFFFu, before.y);
+        const uint2 sent = lane < cs ? sm.kept_cnt[lane] : make_uint2(0u, 0u);
+        if (HIST && __any_sync(0xFFFFFFFFu, sent.x == GAVE_UP)) { return false; }
+        gt_before += __reduce_add_sync(0xFFFFFFFFu, lane < crank ? sent.x : 0u);
+        eq_before += __reduce_add_sync(0xFFFFFFFFu, lane < crank ? sent.y : 0u);
         const unsigned below = (1u << lane) - 1u;
 #pragma unroll
         for (int i = 0; i < KPT; ++i) {
@@ -1082,6 +1111,23 @@ select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __r
         if (threadIdx.x == 0 && sm.amax) atomicMax(reinterpret_cast<uint32_t*>(amax_kept), sm.amax);
     }
     if (reads_remote) cluster.sync();                  // nobody leaves while a neighbour may still read its shared memory
+    return true;
+}
+
+template <int KPT, bool HIST, bool LATE = false>
+__global__ void __launch_bounds__(CL_THREADS, 2)
+select_cluster_kernel(const float* __restrict__ nrm2, int P, int k, int32_t* __restrict__ idx, float* __restrict__ tau,
+                      int32_t* __restrict__ rank, const float* __restrict__ amaxpos, float* __restrict__ amax_kept,
+                      const uint32_t* __restrict__ hist1, const uint32_t* __restrict__ fine, uint32_t* __restrict__ thr,
+                      int want_rank)
+{
+    __shared__ ClusterSmem sm;
+    if (cluster_select<KPT, HIST, LATE>(sm, nrm2, P, k, idx, tau, rank, amaxpos, amax_kept, hist1, fine, thr, want_rank)) return;
+    // none of this CTA's positions is kept
+    const int from = (int)blockIdx.x * CL_THREADS * KPT, n = blockIdx.y;
+    if (rank)
+        for (int p = from + (int)threadIdx.x; p < min(from + CL_THREADS * KPT, P); p += CL_THREADS) rank[(size_t)n * P + p] = -1;
+    if (thr && blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<uint4*>(thr + n * 4) = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
 }
 
 __global__ void thr_use_rank_kernel(uint32_t* thr, int N)

@@ -126,7 +126,7 @@ def lib() -> C.CDLL:
         L.wcc_debug_wait_selftest.restype = i
         L.wcc_debug_wait_selftest.argtypes = [vp]
         L.wcc_debug_select.restype = i
-        L.wcc_debug_select.argtypes = [vp, i, i, vp, vp, i, vp, vp, vp, vp]
+        L.wcc_debug_select.argtypes = [vp, i, i, vp, vp, i, i, vp, vp, vp, vp]
         L.wcc_status_str.restype = C.c_char_p
         L.wcc_status_str.argtypes = [i]
         _lib = L
@@ -493,9 +493,9 @@ def debug_wait_selftest():
     _check(lib().wcc_debug_wait_selftest(_stream()), "wcc_debug_wait_selftest")
 
 
-def debug_select(nrm2, k: int, hist11, hist16, want_rank: bool, thr, rank, idx):
+def debug_select(nrm2, k: int, hist11, hist16, want_rank: bool, thr, rank, idx, late: bool = False):
     """The selection inside a layer on one image's norms and the caller's histograms of them (wcc_debug_select)."""
-    _check(lib().wcc_debug_select(nrm2.data_ptr(), nrm2.numel(), k, hist11.data_ptr(), hist16.data_ptr(), int(want_rank), thr.data_ptr(),
+    _check(lib().wcc_debug_select(nrm2.data_ptr(), nrm2.numel(), k, hist11.data_ptr(), hist16.data_ptr(), int(want_rank), int(late), thr.data_ptr(),
                                   rank.data_ptr(), idx.data_ptr(), _stream()), "wcc_debug_select")
 
 

@@ -10,6 +10,7 @@ from test_gpu_stages import wcc      # noqa: F401  (module fixture)
 pytestmark = pytest.mark.gpu
 
 GUARD = 4096
+WCC_ERR_TIMEOUT = 9
 
 
 def _histograms(nrm):
@@ -18,20 +19,21 @@ def _histograms(nrm):
     return np.bincount(b >> 20, minlength=2048)[:2048], np.bincount(b >> 15, minlength=65536)[:65536]
 
 
-def _select(wcc, nrm, k, h11, h16, want_rank):        # noqa: F811
+def _select(wcc, nrm, k, h11, h16, want_rank, late=False):        # noqa: F811
     P = nrm.size
     dev = [torch.from_numpy(np.ascontiguousarray(a).astype(np.int32)).cuda() for a in (h11, h16)]
     thr = torch.zeros(4, dtype=torch.int32, device="cuda")
     rank = torch.full((P,), -2, dtype=torch.int32, device="cuda")
     idx = torch.full((k + GUARD + P,), -3, dtype=torch.int32, device="cuda")       # (room for all: an overrun is seen, not made)
-    wcc.debug_select(torch.from_numpy(nrm).cuda(), k, *dev, want_rank, thr, rank, idx)
-    assert wcc.last_status() == 0
+    wcc.debug_select(torch.from_numpy(nrm).cuda(), k, *dev, want_rank, thr, rank, idx, late)
+    assert wcc.last_status() == (WCC_ERR_TIMEOUT if late else 0)
     assert bool((idx[k:] == -3).all()), "wrote beyond its list"
     thr, rank, idx = thr.cpu().numpy().view(np.uint32), rank.cpu().numpy(), idx[:k].cpu().numpy()
     keys = np.where(nrm.view(np.uint32) == 0, np.uint32(0x80000000), nrm.view(np.uint32) | np.uint32(0x80000000))
     kept = (rank >= 0) if thr[2] else (keys >= thr[0])
     if thr[2]:
         assert rank.min() >= -1 and rank.max() < k
+    if thr[2] and not late:
         assert np.array_equal(idx[rank[kept]], np.flatnonzero(kept))
     return np.flatnonzero(kept)
 
@@ -72,3 +74,25 @@ def test_histograms_of_something_else(wcc, P, want_rank):      # noqa: F811
         h = rng.integers(0, 4, 2048) * rng.integers(0, P, 2048), rng.integers(0, 3, 65536) * rng.integers(0, P, 65536)
         assert _select(wcc, nrm, k, *h, True).size <= k
         _select(wcc, nrm, k, *h, False)
+
+
+@pytest.mark.parametrize("want_rank", [False, True])
+@pytest.mark.parametrize("P", [4096, 8192, 16384])     # clusters of two, four and eight
+def test_a_wait_that_runs_out(wcc, P, want_rank):      # noqa: F811
+    """One CTA of the cluster gives up its wait for candidates.  It stays until its neighbours, which heard everything, have left or need
+    to hear from it: at the end of the threshold alone, in front of an ordered compaction (asked for, or ties kept in part), and in front
+    of the histogram rounds (more candidates than a message holds)."""
+    plain = _norms(P, P)
+    ties = plain.copy()
+    ties[:: P // 50] = 7.0                             # few enough for the messages
+    crowd = (1.0 + np.arange(P) / 2.0 ** 23).astype(np.float32)
+    wcc.debug_set_wait_limit(300)
+    try:
+        for nrm, k in ((plain, P // 4), (ties, int((ties > 7).sum()) + 20), (crowd, P // 2)):
+            h = _histograms(nrm)
+            got = _select(wcc, nrm, k, *h, want_rank, late=True)
+            right = np.sort(np.argsort(-nrm, kind="stable")[:k])
+            assert got.size == 0 or (not want_rank and nrm is plain and np.array_equal(got, right))
+    finally:
+        wcc.debug_set_wait_limit(0)
+    assert np.array_equal(_select(wcc, plain, P // 4, *_histograms(plain), want_rank), np.sort(np.argsort(-plain, kind="stable")[: P // 4]))
