@@ -49,7 +49,8 @@ static unsigned long long g_launches = 0;
 //    selection writes.
 //  - A kernel that reads anything early has such a kernel as its predecessor (never the caller's own kernels).
 //  - A layer whose second pass is two launches: the first signals only after its own wait, so the second runs only once the selection
-//    is complete and reads its results without waiting; it waits at its end, and so is complete only after the first.
+//    is complete; it reads the selection's results behind an acquire of a word that the first released after that wait (and
+//    waits itself if it does not see it).  It waits at its end, and so is complete only after the first.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

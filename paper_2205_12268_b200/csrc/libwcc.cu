@@ -468,8 +468,8 @@ static wcc_status forward_impl(const void* x, const float* Wt, int N, int Cin, i
     if ((s = profile_mark(3, st)) != WCC_OK) return s;
     // second pass over x: transform, mask + quantize, tensor-core contraction, dequantize, inverse, store
     void* xq_tap = taps ? (bits >= 2 ? static_cast<void*>(taps->Xq) : taps->Xb) : nullptr;
-    s = launch_pass2(x, Wq_use, f.rank, f.nrm2, f.thr, f.amax_kept, bits, scale_w_use, N, Cin, Cout, H, W, L, k, f.kpad, dt, y,
-                     xq_tap, taps ? taps->acc : nullptr, fx, st);
+    s = launch_pass2(x, Wq_use, f.rank, f.nrm2, f.thr, f.amax_kept, bits, scale_w_use, N, Cin, Cout, H, W, L, k, f.kpad, dt, sw.selected,
+                     y, xq_tap, taps ? taps->acc : nullptr, fx, st);
     if (s != WCC_OK) return s;
     for (int i = 4; i <= WCC_NUM_STAGES; ++i)
         if ((s = profile_mark(i, st)) != WCC_OK) return s;

@@ -50,7 +50,9 @@ struct Params {
     int N, Cin, Cout, H, W, k, krow, npad, nchunk, ksteps_part, b_resident, tmem_cols, tiles_total;
     int grp0;                    // the launch's first tile group
     int split_from, parts, share;    // CTAs from split_from on share a tile group `parts` ways, `share` output channels each
-    int last;                    // non-zero (WPT = 4 only): the launch for the last groups of a layer, behind one with WPT = 2 for the others
+    int followed;                // non-zero (WPT = 2 only): a launch for the last groups of the layer comes behind this one
+    int last;                    // non-zero (WPT = 4 only): that launch
+    uint32_t* selected;          // zero until a CTA of a launch with `followed` has waited for the selection
     void* y; uint8_t* xq_tap; int32_t* acc_tap; int* status;
 };
 
@@ -153,9 +155,23 @@ pass2_kernel(const Params pr)
     int rk[8];
 #pragma unroll
     for (int s = 0; s < 8; ++s) nv[s] = (live && slot_ok<L>(lp, s)) ? pr.nrm2[(size_t)n * P + lp.pos[s]] : 0.0f;
+    if (WPT == 4 && pr.last) {
+        // The launch for the last groups starts when every CTA of the one before it has waited for the selection.  That orders the two in
+        // time; what makes the selection's results visible here is the word that the other launch released after its wait.
+        // Not seen, although written long ago: wait for that launch as a whole.  Measured against reading on without either: 24 images of
+        // 64 -> 64 channels fp32 on 96 x 320 110.5 -> 111.1 us, 12 of them 63.2 -> 63.3.
+        uint32_t seen = 1u;
+        if (lane == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(pr.selected) : "memory");
+        __syncwarp();
+        if (__any_sync(0xFFFFFFFFu, seen == 0u)) pdl_wait();
+    }
     if (WPT == 2 || !pr.last) pdl_wait();              // what follows reads the selection's results
     // A launch that follows this one for the last groups does not wait for the selection, so it may not run before that is complete.
-    if (WPT == 2) pdl_launch();
+    if (WPT == 2) {
+        if (pr.followed && blockIdx.x == 0 && threadIdx.x == 0)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(pr.selected), "r"(1u) : "memory");
+        pdl_launch();
+    }
     float amax = 0.0f;
     if (I8) amax = (CLAMP && pr.alpha > 0.0f) ? pr.alpha : *pr.amax_kept;
     {
@@ -469,7 +485,8 @@ static P2Split p2_split(long long groups, int sms, int npad)
 template <typename T, int L, bool VEC>
 static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* rank, const float* nrm2, const uint32_t* thr,
                                  const float* amax_kept, int bits, const float* scale_w, int N, int Cin, int Cout, int H, int W,
-                                 int k, int kpad, void* y, void* xq_tap, int32_t* acc_tap, const FusedExtra& fx, cudaStream_t st)
+                                 int k, int kpad, uint32_t* selected, void* y, void* xq_tap, int32_t* acc_tap, const FusedExtra& fx,
+                                 cudaStream_t st)
 {
     using TT = HaarTile<L>;
     const bool i8 = bits >= 2;
@@ -489,6 +506,7 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     pr.scale_w = scale_w; pr.qmax = i8 ? (float)((1 << (bits - 1)) - 1) : 1.0f;
     pr.alpha = fx.alpha; pr.relu = fx.relu; pr.residual = fx.residual;
     pr.N = N; pr.Cin = Cin; pr.Cout = Cout; pr.H = H; pr.W = W; pr.k = k; pr.krow = krow; pr.tiles_total = (int)tiles;
+    pr.selected = selected;
     pr.y = y; pr.xq_tap = static_cast<uint8_t*>(xq_tap); pr.acc_tap = acc_tap;
     pr.status = di.status;
     const bool clampv = i8 && fx.alpha > 0.0f;
@@ -501,6 +519,7 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
         pr.tmem_cols = plan.tmem_cols;
         pr.grp0 = (int)g0;
         pr.last = g0 > 0;
+        pr.followed = g0 + count < groups;
         const unsigned rem = count % (unsigned)sms;
         const P2Split split = rem > 0 ? p2_split(rem, sms, plan.npad) : P2Split{1, plan.npad};
         pr.parts = split.parts;
@@ -543,13 +562,13 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     return run(first, 0, groups);
 }
 
-// Second pass.  xq_tap ([N*k][kpad] of int8 or bf16) and acc_tap (int32 [N*k][Cout]) may be NULL.
+// Second pass.  xq_tap ([N*k][kpad] of int8 or bf16) and acc_tap (int32 [N*k][Cout]) may be NULL.  *selected is zero.
 static wcc_status launch_pass2(const void* x, const void* Wq, const int32_t* rank, const float* nrm2, const uint32_t* thr,
                                const float* amax_kept, int bits, const float* scale_w, int N, int Cin, int Cout, int H, int W,
-                               int L, int k, int kpad, wcc_dtype dt, void* y, void* xq_tap, int32_t* acc_tap, const FusedExtra& fx,
-                               cudaStream_t st)
+                               int L, int k, int kpad, wcc_dtype dt, uint32_t* selected, void* y, void* xq_tap, int32_t* acc_tap,
+                               const FusedExtra& fx, cudaStream_t st)
 {
-#define WCC_P2D(TY, LL, VV) return pass2_dispatch<TY, LL, VV>(x, Wq, rank, nrm2, thr, amax_kept, bits, scale_w, N, Cin, Cout, H, W, k, kpad, y, xq_tap, acc_tap, fx, st)
+#define WCC_P2D(TY, LL, VV) return pass2_dispatch<TY, LL, VV>(x, Wq, rank, nrm2, thr, amax_kept, bits, scale_w, N, Cin, Cout, H, W, k, kpad, selected, y, xq_tap, acc_tap, fx, st)
     const bool vec = (W % 4) == 0;                     // always with two or three levels
     if (dt == WCC_F32) {
         if (L == 3) WCC_P2D(float, 3, true);

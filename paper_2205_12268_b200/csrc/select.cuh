@@ -29,10 +29,11 @@ enum { ST_B1 = 0, ST_K1 = 1, ST_B2 = 2, ST_K2 = 3, ST_TAU = 4, ST_NEED_EQ = 5, S
 struct SelectWs {
     uint32_t* hist;     // [N][3][SEL_BINS]
     float* amax;        // [1] largest |coef| over the kept positions (float bits, merged by integer atomicMax)
+    uint32_t* selected; // [1] non-zero once a second pass of two launches has waited for the selection
     uint32_t* bar;      // [N] arrival counters of the per-image barriers of the single-kernel select
     uint32_t* state;    // [N][ST_WORDS]
     uint32_t* chunkcnt; // [N][chunks][2]
-    size_t zero_bytes;  // hist + amax + bar are contiguous and cleared together
+    size_t zero_bytes;  // hist + amax + selected + bar are contiguous and cleared together
     int chunks;
 };
 
@@ -51,6 +52,7 @@ inline SelectWs carve_select_ws(void* ws, int N, int P)
     s.hist = reinterpret_cast<uint32_t*>(p);
     p += align_up((size_t)N * 3 * SEL_BINS * 4, 256);
     s.amax = reinterpret_cast<float*>(p);
+    s.selected = reinterpret_cast<uint32_t*>(p + 32);
     s.bar = reinterpret_cast<uint32_t*>(p + 64);
     p += align_up(64 + (size_t)N * 4, 256);
     s.zero_bytes = (size_t)(p - static_cast<char*>(ws));

@@ -55,3 +55,34 @@ def test_launches_and_shares(wcc, cfg):               # noqa: F811
     want2, _ = wcc.forward(relu, W2, L, k, 8, taps=("Xq", "acc"))
     assert torch.equal(wcc.Chain(x, [Wt, W2], L, k, 8)(x), want2)
     assert wcc.last_status() == 0
+
+
+def _map_of_groups(groups):
+    """N, H, W of a batch that the second pass runs as this many groups at two levels (tiles of 4 x 64, four to a group)."""
+    for N in range(5, 25):
+        for w in range(8, 1, -1):
+            for h in range(90, 8, -1):
+                if -(-N * w * h // 4) == groups and 4 * h * 64 * w <= 131072:
+                    return N, 4 * h, 64 * w
+    raise AssertionError(groups)
+
+
+@pytest.mark.parametrize("opts", ["plain", "residual", "alpha", "bits0"])
+@pytest.mark.parametrize("last", [lambda sms: 1, lambda sms: 100, lambda sms: sms - 1, lambda sms: sms, lambda sms: sms + 1],
+                         ids=["1", "100", "sms-1", "sms", "sms+1"])
+def test_last_groups(wcc, last, opts):                # noqa: F811
+    """Last waves up to the size that is a launch of its own (one group per SM) and one beyond, shared among SMs and not, with every kind
+    of option; the call with taps is one launch.  Sixteen input channels: one K step, so unquantized sums have one order too."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    N, H, W = _map_of_groups(2 * sms + last(sms))
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((N, 16, H, W), device="cuda", generator=gen).to(torch.bfloat16)
+    Wt = torch.randn((36, 16), device="cuda", generator=gen)
+    kw = dict(plain={}, residual=dict(residual=torch.randn((N, 36, H, W), device="cuda", generator=gen).to(torch.bfloat16), relu=True),
+              alpha=dict(alpha=2.0), bits0={})[opts]
+    k, bits = inputs.keep_count(0.25, H * W), 0 if opts == "bits0" else 8
+    want, _ = wcc.forward(x, Wt, 2, k, bits, taps=("Xb" if bits == 0 else "Xq", "acc"), **kw)
+    ws = wcc.Workspace.for_problem(x, 36, 2, k, bits)
+    for i in range(3):                                 # the workspace of the calls before holds their words
+        assert torch.equal(wcc.forward(x, Wt, 2, k, bits, y=torch.full_like(want, 7.0), ws=ws, **kw), want)
+    assert wcc.last_status() == 0
