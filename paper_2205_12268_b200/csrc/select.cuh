@@ -1154,11 +1154,13 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
     const SelectWs s = carve_select_ws(ws, N, P);
     float* amax_kept = want_amax ? s.amax : nullptr;
     // one cluster per image while its keys fit in the registers of 16 x 256 threads, when the device schedules clusters of 16 CTAs (opt-in)
-    static int max_cs[64] = {0};
+    static std::atomic<int> max_cs[MAX_DEVICES];       // 0: not asked yet (threads that ask at the same time find the same)
     int devc = 0;
     WCC_CUDA_TRY(cudaGetDevice(&devc));
-    if (devc >= 0 && devc < 64 && max_cs[devc] == 0) {
-        max_cs[devc] = 8;
+    const bool known = devc >= 0 && devc < MAX_DEVICES;
+    int cs_cap = known ? max_cs[devc].load(std::memory_order_relaxed) : 8;
+    if (cs_cap == 0) {
+        cs_cap = 8;
         bool all = true;
         auto allow16 = [&](auto kern) { all = all && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess; };
         allow16(select_cluster_kernel<8, true>); allow16(select_cluster_kernel<16, true>); allow16(select_cluster_kernel<CL_MAXKPT, true>);
@@ -1172,11 +1174,11 @@ wcc_status launch_select(const float* nrm2, int N, int P, int k, int32_t* idx, f
             qa[0].val.clusterDim.x = 16; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
             q.attrs = qa; q.numAttrs = 1;
             int nclusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&nclusters, select_cluster_kernel<CL_MAXKPT, true>, &q) == cudaSuccess && nclusters > 0) max_cs[devc] = 16;
+            if (cudaOccupancyMaxActiveClusters(&nclusters, select_cluster_kernel<CL_MAXKPT, true>, &q) == cudaSuccess && nclusters > 0) cs_cap = 16;
         }
         (void)cudaGetLastError();
+        max_cs[devc].store(cs_cap, std::memory_order_relaxed);
     }
-    const int cs_cap = (devc >= 0 && devc < 64) ? max_cs[devc] : 8;
     if (select_in_cluster(P) && P <= cs_cap * CL_THREADS * CL_MAXKPT) {
         int cs = 1;
         while (cs < cs_cap && cs * CL_THREADS * 8 < P) cs <<= 1;        // about eight keys per thread,
