@@ -522,13 +522,13 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t (&warp_sums)
 }
 
 // After every CTA has filled sm.hist: find the bin holding the krem-th key from the top over the whole cluster.
-// nbins = 2048 or 1024.  Contains two cluster barriers.  Every thread of every CTA returns the same (bin, above), or false after
+// Contains two cluster barriers.  Every thread of every CTA returns the same (bin, above), or false after
 // the first barrier if a CTA of the cluster has given up (HIST: see cluster_exchange).
 template <bool HIST>
-__device__ __forceinline__ bool cluster_find_bin(cg::cluster_group& cluster, ClusterSmem& sm, int cs, int crank, int nbins,
-                                                 uint32_t krem, uint32_t& bin, uint32_t& above)
+__device__ __forceinline__ bool cluster_find_bin(cg::cluster_group& cluster, ClusterSmem& sm, int cs, int crank, uint32_t krem,
+                                                 uint32_t& bin, uint32_t& above)
 {
-    const int B = nbins / cs;                        // bins per slice: 128 .. 2048
+    const int B = SEL_BINS / cs;                     // bins per slice: 128 .. 2048
     cluster.sync();                                  // all local histograms complete
     if (HIST && __any_sync(0xFFFFFFFFu, (int)(threadIdx.x & 31) < cs && sm.narrowing[threadIdx.x & (CL_MAXCS - 1)] == 0u)) return false;
     uint32_t mine = 0;
@@ -789,18 +789,19 @@ __device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t
             if (c >= lo && c <= hi) atomicAdd(&sm.hist[(c - lo) >> sh], 1u);
         }
         __syncthreads();
-        const int per = SEL_BINS / (int)blockDim.x, top = SEL_BINS - 1 - (int)threadIdx.x * per;
-        uint32_t c[8], mysum = 0, tot;
+        constexpr int PER = SEL_BINS / CL_THREADS;
+        const int top = SEL_BINS - 1 - (int)threadIdx.x * PER;
+        uint32_t c[PER], mysum = 0, tot;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            c[i] = (i < per) ? sm.hist[top - i] : 0u;
+        for (int i = 0; i < PER; ++i) {
+            c[i] = sm.hist[top - i];
             mysum += c[i];
         }
         const uint32_t before = block_scan(mysum, sm.warp_sums, &tot);
         if (before < krem && krem <= before + mysum) {
             uint32_t a = before;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < PER; ++i) {
                 if (a < krem && krem <= a + c[i]) { sm.res[0] = (uint32_t)(top - i); sm.res[1] = a; sm.res[2] = c[i]; }
                 a += c[i];
             }
@@ -1030,7 +1031,7 @@ __device__ __forceinline__ bool cluster_select(ClusterSmem& sm, const float* __r
             if (in) atomicAdd(&sm.hist[b], 1u);
         }
         uint32_t b, above;
-        if (!cluster_find_bin<HIST>(cluster, sm, cs, crank, SEL_BINS, krem, b, above)) { return false; }
+        if (!cluster_find_bin<HIST>(cluster, sm, cs, crank, krem, b, above)) { return false; }
         const uint32_t cnt = sm.res[2];
         if (HIST && cnt == 0) { tkey = 0xFFFFFFFFu; need_eq = total_eq = 0u; break; }    // fewer keys than the histograms say: keep nothing
         krem -= above;
