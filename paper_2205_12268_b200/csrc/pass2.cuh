@@ -105,12 +105,12 @@ pass2_kernel(const Params pr)
     const int t = warp & 3, q = warp >> 2;
     // The last, partial wave of tile groups is spread over the SMs that would idle: `parts` CTAs take one group each, all of
     // them build the whole operand and each runs the contraction and the way out for its share of the output channels.
-    int grp = (int)blockIdx.x, o_lo = 0, o_cnt = pr.npad;
+    int grp = (int)blockIdx.x, o_lo = 0, o_hi = pr.npad;
     if ((int)blockIdx.x >= pr.split_from) {
         const int r = (int)blockIdx.x - pr.split_from;
         grp = pr.split_from + r / pr.parts;
         o_lo = (r % pr.parts) * pr.share;
-        o_cnt = min(pr.share, pr.npad - o_lo);
+        o_hi = min(o_lo + pr.share, pr.npad);
     }
     grp += pr.grp0;
     const bool live = grp * TILES + t < pr.tiles_total;
@@ -149,7 +149,7 @@ pass2_kernel(const Params pr)
             *reinterpret_cast<uint4*>(sB + ((size_t)j * bpitch + row) * 16) = v;
         }
     };
-    if (pr.b_resident) load_b(o_lo, o_cnt, 0, 2 * ksteps);
+    if (pr.b_resident) load_b(o_lo, o_hi - o_lo, 0, 2 * ksteps);
     // kept or dropped: from the rank map when the select wrote one (thr[n][2] != 0), else by the threshold key
     float nv[8], mul[8];
     int rk[8];
@@ -281,8 +281,8 @@ pass2_kernel(const Params pr)
     bool ok = true;
     uint32_t parity = 0;
     const bool k_parts = pr.ksteps_part < ksteps;
-    for (int n0 = o_lo; n0 < o_lo + o_cnt && ok; n0 += pr.nchunk) {
-        const int cur = min(pr.nchunk, o_lo + o_cnt - n0);
+    for (int n0 = o_lo; n0 < o_hi && ok; n0 += pr.nchunk) {
+        const int cur = min(pr.nchunk, o_hi - n0);
         for (int ks0 = 0; ks0 < ksteps && ok; ks0 += pr.ksteps_part) {
             const int ks1 = min(ksteps, ks0 + pr.ksteps_part);
             if (k_parts && (ks0 > 0 || n0 > o_lo)) preload(ks0 * UPK + q);
