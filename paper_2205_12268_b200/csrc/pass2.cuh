@@ -105,6 +105,8 @@ pass2_kernel(const Params pr)
     const int t = warp & 3, q = warp >> 2;
     // The last, partial wave of tile groups is spread over the SMs that would idle: `parts` CTAs take one group each, all of
     // them build the whole operand and each runs the contraction and the way out for its share of the output channels.
+    // (The end of the share costs 25 instantiations a spilled word more than its size would; with the size they took the same time or up
+    // to 0.6 % less, but bf16 with three levels and options 1.7 % more: deployed layer of 12 x 64 -> 64 on 96 x 320 59.8 -> 60.9 us.)
     int grp = (int)blockIdx.x, o_lo = 0, o_hi = pr.npad;
     if ((int)blockIdx.x >= pr.split_from) {
         const int r = (int)blockIdx.x - pr.split_from;
@@ -459,7 +461,9 @@ static P2Plan p2_plan(bool two_ctas, int Cout, int krow, bool i8, int L, long lo
 }
 
 // CTAs that share each of `groups` tile groups by output channels, where they would not fill the SMs otherwise: the split in equal
-// parts that one_kernel (libwcc.cu) reckons with.
+// parts that one_kernel (libwcc.cu) reckons with, because its lines were measured with it.  Launches use p2_split, which shares more, so
+// some layers that are gathered would be faster as one kernel (192 -> 144 bf16 with 36 groups 33.3 gathered, 28.6 as one), but its
+// shares alone do not draw the line (256 -> 144 with 24 groups 27.7 and 30.4).
 static int p2_shares(long long groups, int sms, int npad)
 {
     for (int parts = 4; parts >= 2; parts >>= 1)
@@ -469,7 +473,11 @@ static int p2_shares(long long groups, int sms, int npad)
 
 // The split that a launch uses: up to eight CTAs to a group, sixteen channels or more each, the last one perhaps fewer.  Equal parts
 // alone (2 or 4, where the padded channels divide) left 3 x 58 -> 70 channels of 60 x 92 bf16, 80 padded channels, to 23 CTAs:
-// layer 18.5 us, as 115 CTAs 15.5.
+// layer 18.5 us, as 115 CTAs 15.5.  Why as many as there are: of 165 layers with 5 to 72 groups, 1 to 8 K steps and 32 to 256 channels out
+// none gained more from fewer than two runs of one split differ (5 %); against equal parts 0.91 of the time (geometric
+// mean).  128 -> 256 fp32 with 5 groups, by 1, 2, 4 and 8 CTAs each: 42.2, 30.1, 24.5, 22.1 us; 256 -> 144 bf16 with 24 by 1, 2, 3: 64.1,
+// 46.2, 30.7.  Many K steps for few channels out neither gain nor lose (192 -> 64 with 72 groups by 1 and 2: 31.9, 31.7): the SMs that
+// build the operand again would idle.
 struct P2Split { int parts, share; };
 static P2Split p2_split(long long groups, int sms, int npad)
 {
