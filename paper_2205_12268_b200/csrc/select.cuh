@@ -447,9 +447,9 @@ select_coop_kernel(const float* __restrict__ nrm2, int P, int k, uint32_t* __res
 constexpr int CL_THREADS = 256;
 constexpr int CL_MAXKPT = 32;
 constexpr int CL_MAXCS = 16;          // 8 is the portable cluster size; 16 needs the non-portable opt-in
-constexpr int CL_CAND_MAX = 1024;    // candidates a CTA has room for: CL_CAND_MAX / cs from each CTA of the cluster; beyond that: another round
+constexpr int CL_CAND_MAX = 2048;    // candidates a CTA has room for (of a gather: CL_CAND_MAX / cs from each CTA); beyond that: another round
 constexpr int CL_MSG = 64;           // words of the message in which a CTA sends up to CL_MSG - 1 candidates
-constexpr int CL_FEW = 256;          // candidates ranked by few_rank
+constexpr int CL_FEW = 256;          // candidates exchanged by messages
 constexpr uint32_t TOO_MANY = 0xFFFFFFFFu, GAVE_UP = 0xFFFFFFFEu;      // instead of a number of candidates (GAVE_UP: or of kept keys)
 constexpr int FINE_BINS = 65536;     // histogram of the 16 bits below the sign of every norm, filled by the producer of the norms
 
@@ -466,16 +466,17 @@ struct ClusterSmem {
     uint32_t tot[CL_MAXCS];
     uint32_t amax;
     uint32_t ncand;                 // candidates of this CTA in the gather at hand
-    __align__(16) uint32_t out[CL_MSG];           // this CTA's message: number of candidates, candidates, zeros
+    union {
+        __align__(16) uint32_t out[1 + CL_CAND_MAX];      // number of this CTA's candidates, candidates; the first CL_MSG words are its message
+        uint32_t pushed[CL_CAND_MAX];     // (of a gather) candidates of every CTA of the cluster, CL_CAND_MAX / cs slots each
+    };
     __align__(16) uint32_t msg[CL_MAXCS][CL_MSG];  // the messages of all CTAs of the cluster
     uint64_t msg_bar;               // counts their bytes
-    uint32_t few[CL_FEW];           // the candidates in them without the gaps, zeros behind
-    __align__(16) uint32_t counts[2][CL_THREADS / 32];         // of a round of few_rank, per warp
-    uint32_t pushed[CL_CAND_MAX];   // candidates of every CTA of the cluster, CL_CAND_MAX / cs slots each
+    __align__(16) uint32_t counts[2][CL_THREADS / 32];         // of a round of rank_by_bits, per warp
     uint32_t pushed_cnt[CL_MAXCS];  // how many each has (more than its slots: none were sent)
     uint2 kept_cnt[CL_MAXCS];       // keys above / equal to the threshold in every CTA; GAVE_UP until it has sent them
-    uint32_t narrowing[CL_MAXCS];   // non-zero: the CTA goes on to the histogram rounds
-    __align__(16) uint32_t all[CL_CAND_MAX];      // keys of `pushed` without the gaps
+    uint32_t narrowing[CL_MAXCS];   // non-zero: the CTA has heard that there are too many candidates for the messages
+    __align__(16) uint32_t all[CL_CAND_MAX];      // candidates of all CTAs without gaps
     uint32_t thr[3];                // threshold key, ties to keep, ties in total
     __align__(16) uint32_t range[4];              // positive keys, zeros, smallest positive key, largest key
 };
@@ -621,7 +622,7 @@ __device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, C
         if (lane >= d) upto += t;
     }
 #pragma unroll 1
-    for (uint32_t g = threadIdx.x; g < CL_CAND_MAX; g += blockDim.x) {        // (at least 64 slots each: r is the same in a warp)
+    for (uint32_t g = threadIdx.x; g < CL_CAND_MAX; g += blockDim.x) {        // (at least 128 slots each: r is the same in a warp)
         const int r = (int)(g / slots);
         const uint32_t j = g - (uint32_t)r * slots, c = __shfl_sync(0xFFFFFFFFu, cnt, r), at = __shfl_sync(0xFFFFFFFFu, upto, r) - c;
         if (j < c) sm.all[at + j] = sm.pushed[g];
@@ -654,13 +655,13 @@ __device__ __forceinline__ void cluster_give_up(ClusterSmem& sm)
 
 // The short way of a gather: every CTA sends one message of fixed size to every CTA (st.async, counted by the receiver's mbarrier).
 // A cluster barrier would also wait for everything that its threads have under way in global memory (its release): 1.6 to 3.4
-// us for the gather and its block barriers against 0.8 to 1.3.  The candidates end up in sm.few; returns how many there are,
-// or TOO_MANY for a message or for sm.few, or GAVE_UP with the status set when the wait ran out.
+// us for the gather and its block barriers against 0.8 to 1.3.  Returns how many candidates there are, or GAVE_UP with the status set
+// when the wait ran out.  `few`: they are in sm.all.  Otherwise there are more than CL_FEW, or more from a CTA than a message holds.
 // st.async is left to launches with the cluster attribute (a lone CTA keeps its candidates): in a launch without it the store faulted
 // once, although st.shared::cluster to the own CTA works there.  Nothing documented says why.
 template <int KPT>
 __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, int crank, const uint32_t (&key)[KPT], uint32_t in_map, uint32_t lo,
-                                                     uint32_t hi, int warp, int lane)
+                                                     uint32_t hi, int warp, int lane, bool& few)
 {
     const bool alone = cs == 1;                        // (a launch without clusters)
     uint32_t in = 0u;
@@ -668,19 +669,21 @@ __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, in
     for (int i = 0; i < KPT; ++i) in |= (key[i] >= lo && key[i] <= hi) ? 1u << i : 0u;
     in &= in_map;
     if (__any_sync(0xFFFFFFFFu, in != 0u)) {
-        uint32_t* const list = alone ? sm.few : sm.out + 1;
-        const uint32_t most = alone ? CL_FEW : CL_MSG - 1;
-        uint32_t slot = most;
+        uint32_t* const list = alone ? sm.all : sm.out + 1;
+        uint32_t slot = CL_CAND_MAX;
         if (in) slot = atomicAdd(&sm.ncand, (uint32_t)__popc(in));
 #pragma unroll
         for (int i = 0; i < KPT; ++i)
             if (in & (1u << i)) {
-                if (slot < most) list[slot] = key[i];
+                if (slot < CL_CAND_MAX) list[slot] = key[i];
                 ++slot;
             }
     }
     __syncthreads();
-    if (alone) return sm.ncand <= CL_FEW ? sm.ncand : TOO_MANY;
+    if (alone) {
+        few = sm.ncand <= CL_FEW;
+        return sm.ncand;
+    }
     if ((int)threadIdx.x < cs * (CL_MSG / 4)) {        // sixteen bytes to one CTA per thread
         const int to = (int)threadIdx.x / (CL_MSG / 4), j = (int)threadIdx.x % (CL_MSG / 4);
         uint4 w = *reinterpret_cast<const uint4*>(&sm.out[4 * j]);
@@ -689,12 +692,13 @@ __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, in
                      " st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [ra], {%3, %4, %5, %6}, [rb];\n}\n"
                      ::"r"(tc::smem_u32(&sm.msg[crank][4 * j])), "r"(tc::smem_u32(&sm.msg_bar)), "r"(to), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w) : "memory");
     }
-    if (!__syncthreads_and(cluster_listen(sm) ? 1 : 0)) {        // (the same for the whole block)
+    if (__builtin_expect(!__syncthreads_and(cluster_listen(sm) ? 1 : 0), 0)) {        // (the same for the whole block)
         cluster_give_up(sm);
         return GAVE_UP;
     }
     const uint32_t cnt = lane < cs ? sm.msg[lane][0] : 0u, M = __reduce_add_sync(0xFFFFFFFFu, cnt);
-    if (__any_sync(0xFFFFFFFFu, cnt >= CL_MSG) || M > CL_FEW) return TOO_MANY;
+    few = !__any_sync(0xFFFFFFFFu, cnt >= CL_MSG) && M <= CL_FEW;
+    if (__builtin_expect(!few, 0)) return M;
     uint32_t upto = cnt;                               // of the CTAs up to `lane`
 #pragma unroll
     for (int d = 1; d < CL_MAXCS; d <<= 1) {
@@ -703,29 +707,24 @@ __device__ __forceinline__ uint32_t cluster_exchange(ClusterSmem& sm, int cs, in
     }
     for (int r = warp; r < cs; r += CL_THREADS / 32) {
         const uint32_t c = __shfl_sync(0xFFFFFFFFu, cnt, r), at = __shfl_sync(0xFFFFFFFFu, upto, r) - c;
-        for (uint32_t j = lane; j < c; j += 32) sm.few[at + j] = sm.msg[r][1 + j];
+        for (uint32_t j = lane; j < c; j += 32) sm.all[at + j] = sm.msg[r][1 + j];
     }
     __syncthreads();
     return M;
 }
 
-// The krem-th largest of the M candidates in sm.few, which agree with `base` in all but their low 15 bits (zeros: none).  Three bits a
-// round, a threshold per warp, until one candidate is left.
-__device__ __forceinline__ void few_rank(ClusterSmem& sm, uint32_t M, uint32_t krem, uint32_t base, int warp, int lane, uint32_t& key, uint32_t& need, uint32_t& equal)
+// Three bits of the key of rank krem a round, a threshold per warp, until one candidate is left: count(v) and below(v) are the number of
+// candidates of v or more and the largest one below v (the same in all lanes of a warp).  All candidates agree with `base` in all but 15 bits.
+template <typename Count, typename Below>
+__device__ __forceinline__ void rank_by_bits(ClusterSmem& sm, uint32_t M, uint32_t krem, uint32_t base, int warp, int lane, Count count, Below below,
+                                             uint32_t& key, uint32_t& need, uint32_t& equal)
 {
-    uint32_t c[CL_FEW / 32];
-#pragma unroll
-    for (int i = 0; i < CL_FEW / 32; ++i) c[i] = sm.few[32 * i + lane];
     uint32_t t = base, above = 0, all = M;             // the key is in [t, t + 2^bits): `all` are t or larger, `above` beyond
     int bits = 15;
 #pragma unroll 1
     for (int round = 0; bits > 0 && all - above > 1; ++round) {
         bits -= 3;
-        const uint32_t mine = t + ((uint32_t)warp << bits);
-        uint32_t n = 0;
-#pragma unroll
-        for (int i = 0; i < CL_FEW / 32; ++i) n += c[i] >= mine ? 1u : 0u;
-        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        const uint32_t n = count(t + ((uint32_t)warp << bits));
         if (lane == 0) sm.counts[round & 1][warp] = n;
         __syncthreads();
         const uint4 a = *reinterpret_cast<const uint4*>(&sm.counts[round & 1][0]), b = *reinterpret_cast<const uint4*>(&sm.counts[round & 1][4]);
@@ -740,13 +739,70 @@ __device__ __forceinline__ void few_rank(ClusterSmem& sm, uint32_t M, uint32_t k
             if (v[i] < krem) above = v[i];             // (counts fall with i: ends at the smallest threshold too large)
         t += w << bits;
     }
-    if (bits > 0) {                                    // one candidate left
+    if (bits > 0) t = below(t + (1u << bits));         // one candidate left
+    key = t; need = krem - above; equal = all - above;
+}
+
+// The krem-th largest of the M candidates in sm.all, at most CL_FEW (zeros: none), from registers.
+__device__ __forceinline__ void few_rank(ClusterSmem& sm, uint32_t M, uint32_t krem, uint32_t base, int warp, int lane, uint32_t& key, uint32_t& need, uint32_t& equal)
+{
+    uint32_t c[CL_FEW / 32];
+#pragma unroll
+    for (int i = 0; i < CL_FEW / 32; ++i) c[i] = sm.all[32 * i + lane];
+    auto count = [&](uint32_t v) {
+        uint32_t n = 0;
+#pragma unroll
+        for (int i = 0; i < CL_FEW / 32; ++i) n += c[i] >= v ? 1u : 0u;
+        return __reduce_add_sync(0xFFFFFFFFu, n);
+    };
+    auto below = [&](uint32_t v) {
         uint32_t m = 0;
 #pragma unroll
-        for (int i = 0; i < CL_FEW / 32; ++i) m = max(m, c[i] < t + (1u << bits) ? c[i] : 0u);
-        t = __reduce_max_sync(0xFFFFFFFFu, m);
+        for (int i = 0; i < CL_FEW / 32; ++i) m = max(m, c[i] < v ? c[i] : 0u);
+        return __reduce_max_sync(0xFFFFFFFFu, m);
+    };
+    rank_by_bits(sm, M, krem, base, warp, lane, count, below, key, need, equal);
+}
+
+// The longer way, for up to CL_CAND_MAX candidates that the messages have counted (M) but could not hold: every CTA writes its own to their
+// place in sm.all of every CTA, a warp to one CTA at a time (whole lines; a lane to each took 6 us more for 1920 candidates).  One
+// cluster barrier; false behind it if a CTA has given up.  The CTA has sent `narrowing`.  Then as few_rank, from shared memory -> sm.thr.
+// Histogram rounds over the cluster instead, as beyond CL_CAND_MAX: one constant map of 64 x 64 14.0 -> 20.7 us a layer, noise in 2 x 64 -> 32
+// channels of 256 x 512 bf16, half of it kept, 57.4 -> 61.7.  (Not inlined, so that the short way's code stays together: inlined, six-layer
+// chain 324.4 -> 326.7 us, C4 63.5 -> 63.8.)
+__device__ __noinline__ bool cluster_spread(ClusterSmem& sm, int cs, int crank, uint32_t M, uint32_t krem, uint32_t base)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x < 128 && M + threadIdx.x < CL_CAND_MAX) sm.all[M + threadIdx.x] = 0u;
+    if (cs == 1) {                                     // (they are there)
+        __syncthreads();
+    } else {
+        const uint32_t at = __reduce_add_sync(0xFFFFFFFFu, lane < crank ? sm.msg[lane & (CL_MAXCS - 1)][0] : 0u);      // candidates of the CTAs before
+        for (int to = warp; to < cs; to += CL_THREADS / 32)
+            for (uint32_t j = lane; j < sm.ncand && at + j < CL_CAND_MAX; j += 32) push_u32(&sm.all[at + j], to, sm.out[1 + j]);
+        cg::this_cluster().sync();
+        if (__any_sync(0xFFFFFFFFu, lane < cs && sm.narrowing[lane & (CL_MAXCS - 1)] == 0u)) return false;
     }
-    key = t; need = krem - above; equal = all - above;
+    if (M >= krem) {
+        auto count = [&](uint32_t v) {
+            uint32_t n = 0;
+            for (uint32_t i = 4u * lane; i < M; i += 128) {
+                const uint4 x = *reinterpret_cast<const uint4*>(&sm.all[i]);
+                n += (x.x >= v) + (x.y >= v) + (x.z >= v) + (x.w >= v);
+            }
+            return __reduce_add_sync(0xFFFFFFFFu, n);
+        };
+        auto below = [&](uint32_t v) {
+            uint32_t m = 0;
+            for (uint32_t i = lane; i < M; i += 32) m = max(m, sm.all[i] < v ? sm.all[i] : 0u);
+            return __reduce_max_sync(0xFFFFFFFFu, m);
+        };
+        uint32_t key, need, equal;
+        rank_by_bits(sm, M, krem, base, warp, lane, count, below, key, need, equal);
+        if (threadIdx.x == 0) { sm.thr[0] = key; sm.thr[1] = need; sm.thr[2] = equal; }
+        __syncthreads();
+    }
+    return true;
 }
 
 // The krem-th largest of the M candidates in sm.all, all of them in [lo, hi] -> sm.thr = {key, equal keys to keep, equal keys}.
@@ -854,7 +910,7 @@ __device__ __forceinline__ bool cluster_select(ClusterSmem& sm, const float* __r
         for (int i = threadIdx.x; i < SEL_BINS; i += CL_THREADS) sm.hist[i] = 0u;
     if (threadIdx.x < 4) sm.range[threadIdx.x] = threadIdx.x == 2 ? 0xFFFFFFFFu : 0u;
     if (threadIdx.x < CL_MSG) sm.out[threadIdx.x] = 0u;
-    for (int i = threadIdx.x; i < CL_FEW; i += CL_THREADS) sm.few[i] = 0u;
+    for (int i = threadIdx.x; i < CL_FEW; i += CL_THREADS) sm.all[i] = 0u;
     if (HIST && threadIdx.x < CL_MAXCS) { sm.kept_cnt[threadIdx.x].x = GAVE_UP; sm.narrowing[threadIdx.x] = 0u; }
     if (threadIdx.x == 0) {
         tc::mbar_init(tc::smem_u32(&sm.msg_bar), 1);
@@ -960,20 +1016,28 @@ __device__ __forceinline__ bool cluster_select(ClusterSmem& sm, const float* __r
     if (HIST && !found && krem == 0) { tkey = 0xFFFFFFFFu; found = true; }       // no such fine bin: keep nothing, as above
     if (HIST && !found) {
         if (amaxpos) { load_amax(lo); amax_loaded = true; }          // (on their way while the threshold is found)
-        const uint32_t M = cluster_exchange<KPT>(sm, cs, crank, key, in_map, lo, hi, warp, lane);
-        if (HIST && M == GAVE_UP) { return false; }
-        if (M != TOO_MANY) {
+        bool few;
+        const uint32_t M = cluster_exchange<KPT>(sm, cs, crank, key, in_map, lo, hi, warp, lane, few);
+        if (__builtin_expect(M == GAVE_UP, 0)) return false;
+        if (__builtin_expect(few, 1)) {
             tkey = 0xFFFFFFFFu;                        // keep nothing if there are fewer (histograms that do not match the keys)
             if (M >= krem) few_rank(sm, M, krem, hi & ~0x7FFFu, warp, lane, tkey, need_eq, total_eq);
             ranked = M;
             found = true;
         } else {
-            reads_remote = true;
-            __syncthreads();                           // (a lone CTA has just read its count)
             if ((int)threadIdx.x < cs) push_u32(&sm.narrowing[crank], (int)threadIdx.x, 1u);
-            if (threadIdx.x == 0) sm.ncand = 0u;
-            for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
-            __syncthreads();
+            if (M <= CL_CAND_MAX) {
+                if (!cluster_spread(sm, cs, crank, M, krem, hi & ~0x7FFFu)) return false;
+                tkey = sm.thr[0]; need_eq = sm.thr[1]; total_eq = sm.thr[2];
+                ranked = M;
+                found = true;
+            } else {
+                reads_remote = true;
+                __syncthreads();                       // (a lone CTA has just read its count)
+                if (threadIdx.x == 0) sm.ncand = 0u;
+                for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) sm.hist[i] = 0u;
+                __syncthreads();
+            }
         }
     }
     if (!HIST) {

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 # a CTA has 256 threads of 8, 16 or 32 keys, a cluster 1 to 16 CTAs: both sides of each step
 SIZES = [(2, 8), (32, 64), (34, 64), (64, 66), (96, 320), (256, 256), (256, 260), (256, 512)]
-CLOSE = [1, 2, 63, 64, 256, 257, 2000]       # keys in the threshold's bin
+CLOSE = [1, 2, 63, 64, 256, 257, 2000, 2048, 2049]       # keys in the threshold's bin
 
 
 def _map_of(v, H, W):

@@ -80,15 +80,18 @@ def test_histograms_of_something_else(wcc, P, want_rank):      # noqa: F811
 @pytest.mark.parametrize("P", [4096, 8192, 16384])     # clusters of two, four and eight
 def test_a_wait_that_runs_out(wcc, P, want_rank):      # noqa: F811
     """One CTA of the cluster gives up its wait for candidates.  It stays until its neighbours, which heard everything, have left or need
-    to hear from it: at the end of the threshold alone, in front of an ordered compaction (asked for, or ties kept in part), and in front
-    of the histogram rounds (more candidates than a message holds)."""
+    to hear from it: at the end of the threshold alone, in front of an ordered compaction (asked for, or ties kept in part), and where
+    there are more candidates than the messages hold, in front of their spreading and of the histogram rounds."""
     plain = _norms(P, P)
     ties = plain.copy()
     ties[:: P // 50] = 7.0                             # few enough for the messages
     crowd = (1.0 + np.arange(P) / 2.0 ** 23).astype(np.float32)
+    some = plain.copy()                                # too many for the messages, not for one CTA
+    some[: P // 4] = (20.0 + np.arange(P // 4) / 2.0 ** 18).astype(np.float32)[: P // 4]
+    some[1000:P // 4] = 0.5
     wcc.debug_set_wait_limit(300)
     try:
-        for nrm, k in ((plain, P // 4), (ties, int((ties > 7).sum()) + 20), (crowd, P // 2)):
+        for nrm, k in ((plain, P // 4), (ties, int((ties > 7).sum()) + 20), (some, int((some > 20).sum()) - 300), (crowd, P // 2)):
             h = _histograms(nrm)
             got = _select(wcc, nrm, k, *h, want_rank, late=True)
             right = np.sort(np.argsort(-nrm, kind="stable")[:k])
