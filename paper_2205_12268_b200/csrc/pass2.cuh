@@ -558,9 +558,13 @@ static wcc_status pass2_dispatch(const void* x, const void* Wq, const int32_t* r
     };
     // Two CTAs of eight warps to an SM leave a last wave of up to one CTA per SM at half speed.  Its groups get sixteen warps each, in a
     // launch of their own that takes the SMs as they fall free: 64 -> 64 channels fp32 on 12 x 96 x 320 (360 groups, 64 of them in
-    // the last wave) 65.3 -> 63.7 us a layer, 24 images of it (720, 128) 116.0 -> 109.6.
+    // the last wave) 65.3 -> 63.7 us a layer, 24 images of it (720, 128) 116.0 -> 109.6.  The launch costs up to 2.5 us, so a group must
+    // be work enough, of which the way in takes the larger part per channel.  36 layers of 301 to 445 groups, one launch / two: bf16
+    // 8 -> 32 channels 25.3 / 27.7, 64 -> 32 50.6 / 50.7, 32 -> 128 46.4 / 46.9, 96 -> 32 49.1 / 48.9, 128 -> 24 58.7 / 56.6, fp32 32 -> 32
+    // 36.9 / 37.0, 16 -> 96 49.6 / 48.0, 96 -> 32 72.8 / 68.8.
     const unsigned wave = 2u * (unsigned)sms, last = groups % wave;
-    if (first.wpt == 2 && groups > wave && last > 0 && last <= (unsigned)sms) {
+    const bool heavy = (int)sizeof(T) * (2 * Cin + Cout) >= 448;
+    if (first.wpt == 2 && heavy && groups > wave && last > 0 && last <= (unsigned)sms) {
         const P2Plan rest = p2_plan(false, Cout, krow, i8, L, last, sms);
         if (rest.ok) {
             if ((s = run(first, 0, groups - last)) != WCC_OK) return s;

@@ -30,9 +30,14 @@ def test_second_pass(wcc, cfg):                       # noqa: F811
 # per group and are compared with the oracle by the tests above: the same integers, so the same bits.
 SPLITS = [
     (3, 12, 20, 400, 256, "f32", 2, 0.2),             # 300 groups: 296 by one launch, 4 by the next
-    (9, 40, 24, 132, 376, "bf16", 2, 0.3),            # 446: nearly all the SMs once more
+    (9, 40, 24, 132, 376, "bf16", 2, 0.3),            # 446: 150 more than two for every SM, so one launch
     (5, 10, 50, 440, 272, "bf16", 3, 0.1),            # 619: two waves and 27 groups
     (4, 9, 12, 216, 360, "f32", 3, 0.25),             # 324 with a ragged width
+    # the same with channels enough for two launches (the four above are too light for it)
+    (3, 12, 100, 400, 256, "f32", 2, 0.2),
+    (9, 140, 24, 132, 376, "bf16", 2, 0.3),
+    (5, 110, 50, 440, 272, "bf16", 3, 0.1),
+    (4, 57, 12, 216, 360, "f32", 3, 0.25),
     (1, 20, 70, 60, 92, "bf16", 2, 0.25),             # 80 padded channels on few groups: shares of 16
     (2, 33, 112, 64, 128, "f32", 3, 0.25),            # seven units of sixteen
     (3, 24, 200, 96, 160, "bf16", 3, 0.25),           # thirteen units among three CTAs: the last one has fewer
@@ -71,18 +76,19 @@ def _map_of_groups(groups):
 @pytest.mark.parametrize("last", [lambda sms: 1, lambda sms: 100, lambda sms: sms - 1, lambda sms: sms, lambda sms: sms + 1],
                          ids=["1", "100", "sms-1", "sms", "sms+1"])
 def test_last_groups(wcc, last, opts):                # noqa: F811
-    """Last waves up to the size that is a launch of its own (one group per SM) and one beyond, shared among SMs and not, with every kind
-    of option; the call with taps is one launch.  Sixteen input channels: one K step, so unquantized sums have one order too."""
+    """Heavy groups (fp32, 16 -> 96 channels): last waves up to the size that is a launch of its own (one group per SM) and one beyond,
+    shared among SMs and not, with every kind of option; the call with taps is one launch.  Sixteen input channels: one K step, so
+    unquantized sums have one order too."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     N, H, W = _map_of_groups(2 * sms + last(sms))
     gen = torch.Generator(device="cuda").manual_seed(5)
-    x = torch.randn((N, 16, H, W), device="cuda", generator=gen).to(torch.bfloat16)
-    Wt = torch.randn((36, 16), device="cuda", generator=gen)
-    kw = dict(plain={}, residual=dict(residual=torch.randn((N, 36, H, W), device="cuda", generator=gen).to(torch.bfloat16), relu=True),
+    x = torch.randn((N, 16, H, W), device="cuda", generator=gen)
+    Wt = torch.randn((96, 16), device="cuda", generator=gen)
+    kw = dict(plain={}, residual=dict(residual=torch.randn((N, 96, H, W), device="cuda", generator=gen), relu=True),
               alpha=dict(alpha=2.0), bits0={})[opts]
     k, bits = inputs.keep_count(0.25, H * W), 0 if opts == "bits0" else 8
     want, _ = wcc.forward(x, Wt, 2, k, bits, taps=("Xb" if bits == 0 else "Xq", "acc"), **kw)
-    ws = wcc.Workspace.for_problem(x, 36, 2, k, bits)
+    ws = wcc.Workspace.for_problem(x, 96, 2, k, bits)
     for i in range(3):                                 # the workspace of the calls before holds their words
         assert torch.equal(wcc.forward(x, Wt, 2, k, bits, y=torch.full_like(want, 7.0), ws=ws, **kw), want)
     assert wcc.last_status() == 0
