@@ -621,11 +621,9 @@ __device__ __forceinline__ uint32_t cluster_gather(cg::cluster_group& cluster, C
         const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, upto, d);
         if (lane >= d) upto += t;
     }
-#pragma unroll 1
-    for (uint32_t g = threadIdx.x; g < CL_CAND_MAX; g += blockDim.x) {        // (at least 128 slots each: r is the same in a warp)
-        const int r = (int)(g / slots);
-        const uint32_t j = g - (uint32_t)r * slots, c = __shfl_sync(0xFFFFFFFFu, cnt, r), at = __shfl_sync(0xFFFFFFFFu, upto, r) - c;
-        if (j < c) sm.all[at + j] = sm.pushed[g];
+    for (int r = threadIdx.x >> 5; r < cs; r += CL_THREADS / 32) {
+        const uint32_t c = __shfl_sync(0xFFFFFFFFu, cnt, r), at = __shfl_sync(0xFFFFFFFFu, upto, r) - c;
+        for (uint32_t j = lane; j < c; j += 32) sm.all[at + j] = sm.pushed[(uint32_t)r * slots + j];
     }
     __syncthreads();
     return M;
