@@ -314,10 +314,9 @@ const char* wcc_status_str(wcc_status s);
 
 /*
  * Test hooks for the device-side timeout contract (no counterpart in the paper).  Every wait inside a kernel (on an
- * mbarrier of the tensor-core pipeline, of its TMA ring or of the hand-over between the warps of a tile, on the arrival counter
- * of the cooperative select) polls a
- * bounded number of times, then the kernel records WCC_ERR_TIMEOUT, lets its copies in flight land, frees its TMEM
- * and returns; nothing traps or faults.
+ * mbarrier of the tensor-core pipeline, of its TMA ring, of the hand-over between the warps of a tile or of the messages between
+ * the blocks of a selection, on the arrival counter of the cooperative select) polls a bounded number of times, then the kernel
+ * records WCC_ERR_TIMEOUT, lets its copies in flight land, frees its TMEM and returns; nothing traps or faults.
  *   wcc_debug_set_wait_limit  sets the number of polls (each suspends for up to about a microsecond) on the current
  *                             device; 0 restores the default (2,000,000).  Synchronous.
  *   wcc_debug_wait_selftest   enqueues one warp that waits on a barrier nobody arrives on; with a small limit it

@@ -887,7 +887,8 @@ __device__ __forceinline__ void block_rank(ClusterSmem& sm, uint32_t M, uint32_t
 // Blocks of 256 threads: what every warp has to do besides its keys (some 500 instructions) was most of the issue slots of 1024.
 // Measured, from the end of the first pass to the start of the second's threshold (us, blocks of up to 1024 threads that read each
 // other's candidates after a cluster barrier -> this): 2 x 131072 positions 14.3 -> 8.3, 12 x 30720 7.8 -> 5.3, 4 x 32768 8.0 -> 6.2.
-// KPT: keys per thread (8, 16 or 32).  HIST: the histograms are supplied.  LATE (a test's): the second CTA expects more than is sent to
+// KPT: keys per thread (8, 16 or 32; with 32 the 128 registers of two blocks per SM spill 12 bytes, with histograms 32).  HIST: the
+// histograms are supplied.  LATE (a test's): the second CTA expects more than is sent to
 // it, so its wait runs out.
 // False: this CTA has given up, or has not heard from one that has.
 template <int KPT, bool HIST, bool LATE>
@@ -1093,7 +1094,7 @@ __device__ __forceinline__ bool cluster_select(ClusterSmem& sm, const float* __r
             if (in) atomicAdd(&sm.hist[b], 1u);
         }
         uint32_t b, above;
-        if (!cluster_find_bin<HIST>(cluster, sm, cs, crank, krem, b, above)) { return false; }
+        if (!cluster_find_bin<HIST>(cluster, sm, cs, crank, krem, b, above)) return false;
         const uint32_t cnt = sm.res[2];
         if (HIST && cnt == 0) { tkey = 0xFFFFFFFFu; need_eq = total_eq = 0u; break; }    // fewer keys than the histograms say: keep nothing
         krem -= above;
@@ -1149,7 +1150,7 @@ __device__ __forceinline__ bool cluster_select(ClusterSmem& sm, const float* __r
         if ((int)threadIdx.x < cs) push_u64(&sm.kept_cnt[crank], (int)threadIdx.x, make_uint2(tot_gt, tot_eq));
         cluster.sync();
         const uint2 sent = lane < cs ? sm.kept_cnt[lane] : make_uint2(0u, 0u);
-        if (HIST && __any_sync(0xFFFFFFFFu, sent.x == GAVE_UP)) { return false; }
+        if (HIST && __any_sync(0xFFFFFFFFu, sent.x == GAVE_UP)) return false;
         gt_before += __reduce_add_sync(0xFFFFFFFFu, lane < crank ? sent.x : 0u);
         eq_before += __reduce_add_sync(0xFFFFFFFFu, lane < crank ? sent.y : 0u);
         const unsigned below = (1u << lane) - 1u;
